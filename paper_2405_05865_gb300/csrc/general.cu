@@ -18,7 +18,7 @@
 //              w = (r - A^T (A~ y)) / lam~  X = A~, Y = A
 // SolveM2's two level-3 solves apply W = A~^T A~ as its formed FP64 Gram
 // (s x s, cheaper than a pass over A~ and the same operator), both in one
-// two-block launch (k_level3_pcg).
+// launch of two clusters (k_level3_cluster).
 // The inner levels run a fixed number of PCG steps (t2, t3) with all scalars
 // on the device, so one application of SolveM1 is a fixed launch sequence;
 // it is captured once into a CUDA graph and replayed per level-1 iteration.
@@ -516,165 +516,124 @@ __global__ void k_dense_mv(const double* __restrict__ M, const float* __restrict
     if (lane == 0) out[row] = (float)s;
 }
 
-// Algorithm 5 steps 2-3 in one launch: block 0 runs t3 PCG steps on
-// W u = r preconditioned by M3a^{-1}, block 1 on (W + lam~ I) v = r with
-// M3b^{-1}; W = A~^T A~ is the formed FP64 Gram (the same operator as
-// A~^T (A~ .), applied as an s x s product). Thread i < s_pad owns component
-// i; every dense product is split over 1024 / s_pad threads per component
-// (j ranges, combined in a fixed order) and reads columns of the symmetric
-// matrices (coalesced across threads). FP64 throughout; s_pad <= 1024.
-__global__ void __launch_bounds__(1024) k_level3_pcg(const double* __restrict__ W, const double* __restrict__ Ma,
-                                                    const double* __restrict__ Mb, double lam_t, int sp, int t3,
-                                                    const float* __restrict__ b, float* __restrict__ u,
-                                                    float* __restrict__ v) {
-    __shared__ double red[33];
-    __shared__ double vec[1024], pbuf[1024];
-    const int tid = threadIdx.x;
-    const int parts = max(1, 1024 / sp);
-    const int per = (sp + parts - 1) / parts;
-    const int ci = tid % sp, part = tid / sp;
-    const bool own = tid < sp;
-    const double* M = blockIdx.x == 0 ? Ma : Mb;
-    const double shift = blockIdx.x == 0 ? 0.0 : lam_t;
-    float* out = blockIdx.x == 0 ? u : v;
-    // y = Mat vec for the owner threads (vec staged in shared memory by the caller)
-    auto mv = [&](const double* Mat) {
-        double s = 0.0;
-        if (part < parts) {
-            const int j0 = part * per, j1 = min(sp, j0 + per);
-#pragma unroll 8
-            for (int j = j0; j < j1; ++j) s = fma(Mat[(int64_t)j * sp + ci], vec[j], s);
-        }
-        pbuf[tid] = s;
-        __syncthreads();
-        double y = 0.0;
-        if (own)
-            for (int q = 0; q < parts; ++q) y += pbuf[ci + q * sp];
-        return y;
-    };
-    double x = 0.0, r = own ? (double)b[tid] : 0.0;
-    vec[tid] = r;
-    __syncthreads();
-    double z = mv(M);
-    double rz = block_sum(own ? r * z : 0.0, red);
-    double p = z;
-    for (int k = 0; k < t3; ++k) {
-        __syncthreads();
-        vec[tid] = own ? p : 0.0;
-        __syncthreads();
-        const double q = mv(W) + shift * p;
-        const double pq = block_sum(own ? p * q : 0.0, red);
-        const double alpha = (pq > 0.0 && rz != 0.0) ? rz / pq : 0.0;
-        x = fma(alpha, p, x);
-        r = fma(-alpha, q, r);
-        if (k + 1 < t3) {
-            __syncthreads();
-            vec[tid] = own ? r : 0.0;
-            __syncthreads();
-            z = mv(M);
-            const double rzn = block_sum(own ? r * z : 0.0, red);
-            const double beta = rz != 0.0 ? rzn / rz : 0.0;
-            p = fma(beta, p, z);
-            rz = rzn;
-        }
-    }
-    if (own) out[tid] = (float)x;
-}
-
-// The same two level-3 solves on two thread-block clusters of kCl CTAs
-// (cluster 0: W u = r with M3a^{-1}; cluster 1: (W + lam~ I) v = r with
-// M3b^{-1}). CTA `rank` owns components [rank s_pad / kCl, (rank + 1) s_pad /
-// kCl); each warp forms whole rows of the symmetric matrices (lanes over
-// columns, coalesced), so the FP64 products run on 2 kCl SMs instead of two.
-// Vector slices and dot partials are broadcast to every CTA of the cluster
-// through distributed shared memory; cluster barriers order the steps (no
-// spin-waits). The dot partials are summed in rank order, so every CTA takes
-// the same scalars. s_pad <= 1024, s_pad divisible by kCl.
+// Algorithm 5 steps 2-3 in one launch, on two thread-block clusters of kCl
+// CTAs: cluster 0 runs t3 PCG steps on W u = r preconditioned by M3a^{-1},
+// cluster 1 on (W + lam~ I) v = r with M3b^{-1}; W = A~^T A~ is the formed FP64
+// Gram (the same operator as A~^T (A~ .), applied as an s x s product). FP64
+// throughout; s_pad a multiple of 128, at most 1024.
+//
+// What bounds it is the FP64 pipe (2 lanes per clock per SM: a warp-wide FP64
+// instruction holds it for 16 cycles whether the lanes' results are needed or
+// not) and the latency of the serial chain product -> dot -> step, so every
+// FP64 instruction that is not the product itself is kept to the threads that
+// need it. A CTA has s_pad threads: 8 lanes form one of its s_pad / kCl rows
+// of a product (their slices of W and M3^{-1} in registers up to s_pad = 256,
+// E = s_pad / 8 values each, read from L1 / L2 beyond), and after the row's
+// butterfly each of the 8 lanes holds the sum and stores it into one CTA's copy
+// of the full result, so one cluster barrier per product is the only exchange
+// (two copies in turn: a CTA is never more than one barrier ahead). Thread t
+// then keeps component t of x, r, p redundantly in every CTA, the dots are
+// taken in each CTA from the full vectors in the same order, and one warp
+// forms each step's quotient. The former layout (1024 threads whatever s_pad,
+// every thread summing partials and dividing, two cluster barriers a product)
+// took 177 us at s_pad = 128, t3 = 8, most of a three-level solve; with this one
+// the solve at 16384 x 2048 went from 355 to 180 ms.
 constexpr int kCl = 8;
 
-__global__ void __cluster_dims__(kCl, 1, 1) __launch_bounds__(1024)
+template <int E>
+__global__ void __cluster_dims__(kCl, 1, 1) __launch_bounds__(E > 0 ? 8 * E : 1024)
     k_level3_cluster(const double* __restrict__ W, const double* __restrict__ Ma, const double* __restrict__ Mb,
                      double lam_t, int sp, int t3, const float* __restrict__ b, float* __restrict__ u,
                      float* __restrict__ v) {
     namespace cg = cooperative_groups;
     cg::cluster_group cl = cg::this_cluster();
-    __shared__ double vec[1024];          // the full vector of the next product
-    __shared__ double part[2][kCl];       // dot partials, one slot per rank
-    __shared__ double loc[32];
+    __shared__ __align__(16) double vec[1024];   // the vector of the next product
+    __shared__ double ybuf[2][1024];             // products, in turn
+    __shared__ double red[32];
+    __shared__ double s_sc;
     const int rank = (int)cl.block_rank();
     const int sys = blockIdx.x / kCl;
-    const double* M = sys == 0 ? Ma : Mb;
     const double shift = sys == 0 ? 0.0 : lam_t;
     float* out = sys == 0 ? u : v;
-    const int own = sp / kCl, i0 = rank * own;
-    const int tid = threadIdx.x, warp = tid >> 5, lane = tid & 31;
-    // owner state: thread c < own keeps component i0 + c
-    double x = 0.0, r = 0.0, z = 0.0, p = 0.0;
-    // y_c = (Mat vec)_(i0 + c) for the owned rows, into ys (shared)
-    __shared__ double ys[1024];
-    auto mv = [&](const double* Mat) {
-        for (int c = warp; c < own; c += 32) {
-            const double* row = Mat + (int64_t)(i0 + c) * sp;
-            double s = 0.0;
-            for (int j = lane; j < sp; j += 32) s = fma(row[j], vec[j], s);
+    const int tid = threadIdx.x, warp = tid >> 5, lane = tid & 31, l8 = tid & 7;
+    const int nw = sp >> 5, own = sp / kCl;
+    const int row = rank * own + (tid >> 3);
+    // this lane's elements of its row: the pairs 2 l8 + 16 k
+    const double2* Wr = reinterpret_cast<const double2*>(W + (int64_t)row * sp) + l8;
+    const double2* Mr = reinterpret_cast<const double2*>((sys == 0 ? Ma : Mb) + (int64_t)row * sp) + l8;
+    constexpr int ER = E > 0 ? E / 2 : 1;
+    double2 wreg[ER], mreg[ER];
+    if constexpr (E > 0) {
 #pragma unroll
-            for (int o = 16; o > 0; o >>= 1) s += __shfl_xor_sync(0xffffffffu, s, o);
-            if (lane == 0) ys[c] = s;
-        }
-        __syncthreads();
-    };
-    // every CTA's vec <- the owners' values (slices from all ranks)
-    auto broadcast = [&](double val) {
-        if (tid < own)
-            for (int q = 0; q < kCl; ++q) {
-                double* dst = cl.map_shared_rank(vec, q);
-                dst[i0 + tid] = val;
-            }
-        cl.sync();
-    };
-    // cluster-wide sum of one value per owner thread, fixed order
-    auto csum = [&](double val, int slot) {
-        double s = tid < own ? val : 0.0;
+        for (int k = 0; k < ER; ++k) mreg[k] = __ldg(Mr + 8 * k);
 #pragma unroll
-        for (int o = 16; o > 0; o >>= 1) s += __shfl_xor_sync(0xffffffffu, s, o);
-        if (lane == 0) loc[warp] = s;
-        __syncthreads();
-        if (tid == 0) {
-            double t = 0.0;
-            for (int w = 0; w < 32; ++w) t += loc[w];
-            for (int q = 0; q < kCl; ++q) cl.map_shared_rank(&part[slot][0], q)[rank] = t;
-        }
-        cl.sync();
-        double tot = 0.0;
-        for (int q = 0; q < kCl; ++q) tot += part[slot][q];
-        return tot;
-    };
-    if (tid < own) r = (double)b[i0 + tid];
-    broadcast(r);
-    mv(M);
-    if (tid < own) z = ys[tid];
-    double rz = csum(r * z, 0);
-    p = z;
-    for (int k = 0; k < t3; ++k) {
-        broadcast(p);
-        mv(W);
-        const double q = tid < own ? ys[tid] + shift * p : 0.0;
-        const double pq = csum(p * q, 1);
-        const double alpha = (pq > 0.0 && rz != 0.0) ? rz / pq : 0.0;
-        x = fma(alpha, p, x);
-        r = fma(-alpha, q, r);
-        if (k + 1 < t3) {
-            broadcast(r);
-            mv(M);
-            if (tid < own) z = ys[tid];
-            const double rzn = csum(r * z, 0);
-            const double beta = rz != 0.0 ? rzn / rz : 0.0;
-            p = fma(beta, p, z);
-            rz = rzn;
-        }
+        for (int k = 0; k < ER; ++k) wreg[k] = __ldg(Wr + 8 * k);
     }
-    if (tid < own) out[i0 + tid] = (float)x;
-    cl.sync();   // no CTA leaves while others may still write its shared memory
+    cl.sync();   // every CTA of the cluster runs before its shared memory is written
+    int turn = 0;
+    // component tid of (Mat val), val component tid of the vector
+    auto product = [&](const double2 (&reg)[ER], const double2* rows, double val) {
+        vec[tid] = val;
+        __syncthreads();
+        const double2* v2 = reinterpret_cast<const double2*>(vec) + l8;
+        double s0 = 0.0, s1 = 0.0;
+        if constexpr (E > 0) {
+#pragma unroll
+            for (int k = 0; k < ER; ++k) {
+                const double2 a = v2[8 * k];
+                s0 = fma(reg[k].x, a.x, s0);
+                s1 = fma(reg[k].y, a.y, s1);
+            }
+        } else {
+            const int n2 = sp >> 4;
+#pragma unroll 8
+            for (int k = 0; k < n2; ++k) {
+                const double2 m = __ldg(rows + 8 * k), a = v2[8 * k];
+                s0 = fma(m.x, a.x, s0);
+                s1 = fma(m.y, a.y, s1);
+            }
+        }
+        double s = s0 + s1;
+#pragma unroll
+        for (int o = 4; o > 0; o >>= 1) s += __shfl_xor_sync(0xffffffffu, s, o);
+        cl.map_shared_rank(&ybuf[turn][0], l8)[row] = s;
+        cl.sync();
+        const double y = ybuf[turn][tid];
+        turn ^= 1;
+        return y;
+    };
+    // sum over the components, in warp 0 only
+    auto dot0 = [&](double prod) {
+        prod = warp_sum_t(prod);
+        if (lane == 0) red[warp] = prod;
+        __syncthreads();
+        double t = 0.0;
+        if (warp == 0) t = warp_sum_t(lane < nw ? red[lane] : 0.0);
+        return t;
+    };
+    // warp 0's value to every thread
+    auto share = [&](double val) {
+        if (tid == 0) s_sc = val;
+        __syncthreads();
+        return s_sc;
+    };
+    double x = 0.0, r = (double)b[tid];
+    double p = product(mreg, Mr, r);
+    double rz = dot0(r * p);   // warp 0's, as every rz and quotient below
+    for (int k = 0; k < t3; ++k) {
+        const double q = product(wreg, Wr, p) + shift * p;
+        const double pq = dot0(p * q);
+        const double alpha = share(warp == 0 && pq > 0.0 && rz != 0.0 ? rz / pq : 0.0);
+        x = fma(alpha, p, x);
+        if (k + 1 == t3) break;
+        r = fma(-alpha, q, r);
+        const double z = product(mreg, Mr, r);
+        const double rzn = dot0(r * z);
+        const double beta = share(warp == 0 && rz != 0.0 ? rzn / rz : 0.0);
+        p = fma(beta, p, z);
+        rz = rzn;
+    }
+    if (tid / own == rank) out[tid] = (float)x;
 }
 
 // out = a x + b y
@@ -1036,11 +995,15 @@ struct Ops {
     msp_status solve_m2(const float* r, float* z, int t3) {
         if (t3 == 0) return dense(g->M2inv, r, z);
         const int sp = (int)g->s_pad;
-        if (sp % kCl == 0)
-            k_level3_cluster<<<2 * kCl, 1024, 0, strm>>>(g->W64, g->M3a, g->M3b, g->lam_tilde, sp, t3, r, g->u3,
-                                                         g->v3);
+        if (sp == 128)
+            k_level3_cluster<16><<<2 * kCl, sp, 0, strm>>>(g->W64, g->M3a, g->M3b, g->lam_tilde, sp, t3, r, g->u3,
+                                                           g->v3);
+        else if (sp == 256)
+            k_level3_cluster<32><<<2 * kCl, sp, 0, strm>>>(g->W64, g->M3a, g->M3b, g->lam_tilde, sp, t3, r, g->u3,
+                                                           g->v3);
         else
-            k_level3_pcg<<<2, 1024, 0, strm>>>(g->W64, g->M3a, g->M3b, g->lam_tilde, sp, t3, r, g->u3, g->v3);
+            k_level3_cluster<0><<<2 * kCl, sp, 0, strm>>>(g->W64, g->M3a, g->M3b, g->lam_tilde, sp, t3, r, g->u3,
+                                                          g->v3);
         MSP_CHECK_LAUNCH(ctx);
         if (count) ++*count;
         const float il = (float)(1.0 / g->lam_tilde);

@@ -315,21 +315,30 @@ __global__ void __launch_bounds__(kWorkerThreads + 32, 1) k_rowpass_ring(
 }
 
 // out[j] = alpha sum_g part[g][j] + beta w[j] + v[j] (w, v optional), the
-// partials summed in FP64 in a fixed order. Block 32 x 8: 32 columns, the
-// G partial rows split over 8 thread rows, combined in a fixed order.
+// partials summed in FP64 in a fixed order. The FP64 adds and widenings bound
+// it (2 lanes per clock per SM), so the columns are spread thin: 8 columns a
+// block (one 32-byte sector of each partial row), the G partial rows split over
+// 32 thread rows, which a warp's shuffles and one pass over the 8 warps combine.
+// 32 columns a block (4 blocks at 128 columns, 152 x 32 adds on each SM) took
+// 4.4 us at 4096 columns and 152 partial rows and 5.4 us on average in the three-level
+// solve, against 4.1 and 3.7 us.
 template <typename Acc>
-__global__ void k_colsum(const Acc* __restrict__ part, int64_t ldp, int G, int ny, double alpha,
-                         const Acc* __restrict__ w, double beta, const Acc* __restrict__ v,
-                         Acc* __restrict__ out) {
-    __shared__ double red[8][33];
-    const int tx = threadIdx.x & 31, ty = threadIdx.x >> 5;
-    const int j = blockIdx.x * 32 + tx;
+__global__ void __launch_bounds__(256) k_colsum(const Acc* __restrict__ part, int64_t ldp, int G, int ny,
+                                                double alpha, const Acc* __restrict__ w, double beta,
+                                                const Acc* __restrict__ v, Acc* __restrict__ out) {
+    __shared__ double red[8][8];
+    const int tx = threadIdx.x & 7, ty = threadIdx.x >> 3;
+    const int j = blockIdx.x * 8 + tx;
     double s = 0.0;
-    if (j < ny)
-        for (int g = ty; g < G; g += 8) s += (double)part[(int64_t)g * ldp + j];
-    red[ty][tx] = s;
+    if (j < ny) {
+#pragma unroll 5
+        for (int g = ty; g < G; g += 32) s += (double)part[(int64_t)g * ldp + j];
+    }
+    s += __shfl_xor_sync(0xffffffffu, s, 8);
+    s += __shfl_xor_sync(0xffffffffu, s, 16);
+    if ((threadIdx.x & 31) < 8) red[threadIdx.x >> 5][tx] = s;
     __syncthreads();
-    if (ty == 0 && j < ny) {
+    if (threadIdx.x < 8 && j < ny) {
         double tot = 0.0;
 #pragma unroll
         for (int q = 0; q < 8; ++q) tot += red[q][tx];
@@ -381,7 +390,10 @@ __device__ __forceinline__ void ff_add_prod(FF& acc, float a, float b) {
     acc.lo += e + pe;
 }
 
-__device__ double block_sum_ff(FF v, double* red) {
+// Sum of a pair per thread over the block, in warp 0 only (every lane of it):
+// the lanes of a warp combine their pairs, warp 0 adds the warps' sums in FP64.
+// red holds a value per warp; ends with the block past one barrier.
+__device__ double block_sum0_ff(FF v, double* red) {
 #pragma unroll
     for (int o = 16; o > 0; o >>= 1) {
         const float h = __shfl_xor_sync(0xffffffffu, v.hi, o);
@@ -391,31 +403,74 @@ __device__ double block_sum_ff(FF v, double* red) {
         v.hi = s;
         v.lo += l + e;
     }
-    const int warp = threadIdx.x >> 5, lane = threadIdx.x & 31;
-    __syncthreads();
+    const int warp = threadIdx.x >> 5, lane = threadIdx.x & 31, nw = (int)(blockDim.x >> 5);
     if (lane == 0) red[warp] = (double)v.hi + (double)v.lo;
     __syncthreads();
-    if (threadIdx.x == 0) {
-        double t = 0.0;
-        for (int q = 0; q < (int)(blockDim.x >> 5); ++q) t += red[q];
-        red[32] = t;
-    }
-    __syncthreads();
-    return red[32];
+    return warp == 0 ? warp_sum_t(lane < nw ? red[lane] : 0.0) : 0.0;
 }
 
-// x = 0, r = b, bb = b.b
-__global__ void k_pcg_init(int len, const float* __restrict__ b, float* __restrict__ x,
-                           float* __restrict__ r, Pcg* sc) {
-    __shared__ double red[33];
-    FF a{0.f, 0.f};
-    for (int i = threadIdx.x; i < len; i += blockDim.x) {
-        const float v = b[i];
-        x[i] = 0.f;
-        r[i] = v;
-        ff_add_prod(a, v, v);
+// The vector steps of a PCG iteration, one block each: thread t keeps the
+// float4 entries t, t + blockDim of the vectors (Q of them; a block has len / 4Q
+// threads, a whole number of warps), every load issued before the first dot, so
+// a step is one round trip to L2, the reductions, and the stores. The FP64
+// sums and quotients are formed by warp 0 alone (a warp-wide FP64 instruction
+// holds the SM's FP64 pipe for 16 cycles; with a running sum over 32 warp sums
+// in one thread and the quotient in all 1024 threads, and loads in a loop, the step
+// and the direction took 13.6 and 12.2 us at 4096 entries and take 4.8 and 5.2 us; about 10 and 3 us
+// at 128).
+template <int Q>
+struct Slice {
+    float4 v[Q];
+    __device__ __forceinline__ void load(const float* p, int n4) {
+#pragma unroll
+        for (int k = 0; k < Q; ++k) {
+            const int i = (int)(threadIdx.x + k * blockDim.x);
+            v[k] = i < n4 ? reinterpret_cast<const float4*>(p)[i] : make_float4(0.f, 0.f, 0.f, 0.f);
+        }
     }
-    const double s = block_sum_ff(a, red);
+    __device__ __forceinline__ void store(float* p, int n4) const {
+#pragma unroll
+        for (int k = 0; k < Q; ++k) {
+            const int i = (int)(threadIdx.x + k * blockDim.x);
+            if (i < n4) reinterpret_cast<float4*>(p)[i] = v[k];
+        }
+    }
+    // this += a s
+    __device__ __forceinline__ void axpy(float a, const Slice& s) {
+#pragma unroll
+        for (int k = 0; k < Q; ++k) {
+            v[k].x = fmaf(a, s.v[k].x, v[k].x);
+            v[k].y = fmaf(a, s.v[k].y, v[k].y);
+            v[k].z = fmaf(a, s.v[k].z, v[k].z);
+            v[k].w = fmaf(a, s.v[k].w, v[k].w);
+        }
+    }
+    __device__ __forceinline__ FF dot(const Slice& s) const {
+        FF a{0.f, 0.f};
+#pragma unroll
+        for (int k = 0; k < Q; ++k) {
+            ff_add_prod(a, v[k].x, s.v[k].x);
+            ff_add_prod(a, v[k].y, s.v[k].y);
+            ff_add_prod(a, v[k].z, s.v[k].z);
+            ff_add_prod(a, v[k].w, s.v[k].w);
+        }
+        return a;
+    }
+};
+
+// x = 0, r = b, bb = b.b
+template <int Q>
+__global__ void __launch_bounds__(kVecThreads) k_pcg_init(int len, const float* __restrict__ b, float* __restrict__ x,
+                           float* __restrict__ r, Pcg* sc) {
+    __shared__ double red[32];
+    const int n4 = len / 4;
+    Slice<Q> bv, zero;
+    bv.load(b, n4);
+#pragma unroll
+    for (int k = 0; k < Q; ++k) zero.v[k] = make_float4(0.f, 0.f, 0.f, 0.f);
+    zero.store(x, n4);
+    bv.store(r, n4);
+    const double s = block_sum0_ff(bv.dot(bv), red);
     if (threadIdx.x == 0) {
         sc->bb = s;
         sc->rr = s;
@@ -423,78 +478,89 @@ __global__ void k_pcg_init(int len, const float* __restrict__ b, float* __restri
 }
 
 // rz = r.z, p = z, zo = z
-__global__ void k_pcg_start(int len, const float* __restrict__ r, const float* __restrict__ z,
+template <int Q>
+__global__ void __launch_bounds__(kVecThreads) k_pcg_start(int len, const float* __restrict__ r, const float* __restrict__ z,
                             float* __restrict__ p, float* __restrict__ zo, Pcg* sc) {
-    __shared__ double red[33];
-    FF a{0.f, 0.f};
-    for (int i = threadIdx.x; i < len; i += blockDim.x) {
-        const float v = z[i];
-        p[i] = v;
-        zo[i] = v;
-        ff_add_prod(a, r[i], v);
-    }
-    const double s = block_sum_ff(a, red);
+    __shared__ double red[32];
+    const int n4 = len / 4;
+    Slice<Q> rv, zv;
+    rv.load(r, n4);
+    zv.load(z, n4);
+    zv.store(p, n4);
+    zv.store(zo, n4);
+    const double s = block_sum0_ff(rv.dot(zv), red);
     if (threadIdx.x == 0) sc->rz = s;
 }
 
 // pq = p.q; alpha = rz / pq (0 when the step is undefined); x += alpha p;
 // r -= alpha q; rr = r.r
-__global__ void k_pcg_step(int len, const float* __restrict__ p, const float* __restrict__ q,
+template <int Q>
+__global__ void __launch_bounds__(kVecThreads) k_pcg_step(int len, const float* __restrict__ p, const float* __restrict__ q,
                            float* __restrict__ x, float* __restrict__ r, Pcg* sc, int* err) {
-    __shared__ double red[33];
-    FF a{0.f, 0.f};
-    for (int i = threadIdx.x; i < len; i += blockDim.x) ff_add_prod(a, p[i], q[i]);
-    const double pq = block_sum_ff(a, red);
+    __shared__ double red[32], red2[32];
+    __shared__ float s_alpha;
+    const int n4 = len / 4;
+    Slice<Q> pv, qv, xv, rv;
+    pv.load(p, n4);
+    qv.load(q, n4);
+    xv.load(x, n4);
+    rv.load(r, n4);
     const double rz = sc->rz;
-    double alpha = 0.0;
-    if (pq > 0.0 && isfinite(pq) && isfinite(rz)) alpha = rz / pq;
-    else if (err && threadIdx.x == 0 && rz != 0.0 && sc->rr > sc->tol2)
-        atomicCAS(err, 0, isfinite(pq) ? (int)MSP_ENOTPD : (int)MSP_ENONFINITE);
-    const float af = (float)alpha;
-    FF a2{0.f, 0.f};
-    for (int i = threadIdx.x; i < len; i += blockDim.x) {
-        x[i] = fmaf(af, p[i], x[i]);
-        const float rv = fmaf(-af, q[i], r[i]);
-        r[i] = rv;
-        ff_add_prod(a2, rv, rv);
+    const double pq = block_sum0_ff(pv.dot(qv), red);
+    if (threadIdx.x < 32) {
+        double alpha = 0.0;
+        if (pq > 0.0 && isfinite(pq) && isfinite(rz)) alpha = rz / pq;
+        else if (err && threadIdx.x == 0 && rz != 0.0 && sc->rr > sc->tol2)
+            atomicCAS(err, 0, isfinite(pq) ? (int)MSP_ENOTPD : (int)MSP_ENONFINITE);
+        if (threadIdx.x == 0) {
+            s_alpha = (float)alpha;
+            sc->pq = pq;
+            sc->alpha = alpha;
+        }
     }
-    const double rr = block_sum_ff(a2, red);
-    if (threadIdx.x == 0) {
-        sc->pq = pq;
-        sc->alpha = alpha;
-        sc->rr = rr;
-    }
+    __syncthreads();
+    const float af = s_alpha;
+    xv.axpy(af, pv);
+    rv.axpy(-af, qv);
+    xv.store(x, n4);
+    rv.store(r, n4);
+    const double rr = block_sum0_ff(rv.dot(rv), red2);
+    if (threadIdx.x == 0) sc->rr = rr;
 }
 
 // rzn = r.z; flexible: beta = (rzn - r.zo) / rz, else rzn / rz; p = z + beta p;
 // zo = z; rz = rzn
-__global__ void k_pcg_dir(int len, const float* __restrict__ r, const float* __restrict__ z,
+template <int Q>
+__global__ void __launch_bounds__(kVecThreads) k_pcg_dir(int len, const float* __restrict__ r, const float* __restrict__ z,
                           float* __restrict__ zo, float* __restrict__ p, Pcg* sc, int flexible) {
-    __shared__ double red[33];
-    FF a1{0.f, 0.f}, a2{0.f, 0.f};
-    for (int i = threadIdx.x; i < len; i += blockDim.x) {
-        const float rv = r[i];
-        ff_add_prod(a1, rv, z[i]);
-        ff_add_prod(a2, rv, zo[i]);
-    }
-    const double rzn = block_sum_ff(a1, red);
-    const double rzo = flexible ? block_sum_ff(a2, red) : 0.0;
+    __shared__ double red[32], red2[32];
+    __shared__ float s_beta;
+    const int n4 = len / 4;
+    Slice<Q> rv, zv, zov, pv;
+    rv.load(r, n4);
+    zv.load(z, n4);
+    zov.load(zo, n4);
+    pv.load(p, n4);
     const double rz = sc->rz;
-    double beta = 0.0;
-    if (rz != 0.0 && isfinite(rz)) beta = (rzn - rzo) / rz;
-    if (!isfinite(beta)) beta = 0.0;
-    const float bf = (float)beta;
-    for (int i = threadIdx.x; i < len; i += blockDim.x) {
-        const float zv = z[i];
-        p[i] = fmaf(bf, p[i], zv);
-        zo[i] = zv;
+    const double rzn = block_sum0_ff(rv.dot(zv), red);
+    const double rzo = flexible ? block_sum0_ff(rv.dot(zov), red2) : 0.0;
+    if (threadIdx.x < 32) {
+        double beta = 0.0;
+        if (rz != 0.0 && isfinite(rz)) beta = (rzn - rzo) / rz;
+        if (!isfinite(beta)) beta = 0.0;
+        if (threadIdx.x == 0) {
+            s_beta = (float)beta;
+            sc->rzn = rzn;
+            sc->rzo = rzo;
+            sc->beta = beta;
+            sc->rz = rzn;
+        }
     }
-    if (threadIdx.x == 0) {
-        sc->rzn = rzn;
-        sc->rzo = rzo;
-        sc->beta = beta;
-        sc->rz = rzn;
-    }
+    __syncthreads();
+    Slice<Q> pn = zv;
+    pn.axpy(s_beta, pv);
+    pn.store(p, n4);
+    zv.store(zo, n4);
 }
 
 // out = M v for a dense s_pad x s_pad FP64 M (row-major), one warp per row
@@ -895,7 +961,7 @@ msp_status launch_same(msp_ctx* ctx, cudaStream_t strm, int max_ctas, int64_t ro
 template <typename Acc>
 msp_status colsum(msp_ctx* ctx, cudaStream_t strm, G_t* g, const Acc* part, int64_t ldp, int ny, double alpha, const Acc* w,
                   double beta, const Acc* v, Acc* out, int* count, int ctas = 0) {
-    k_colsum<Acc><<<(unsigned)((ny + 31) / 32), 256, 0, strm>>>(part, ldp, ctas ? ctas : g->G, ny, alpha, w, beta,
+    k_colsum<Acc><<<(unsigned)((ny + 7) / 8), 256, 0, strm>>>(part, ldp, ctas ? ctas : g->G, ny, alpha, w, beta,
                                                               v, out);
     MSP_CHECK_LAUNCH(ctx);
     if (count) ++*count;
@@ -976,15 +1042,23 @@ struct Ops {
         if (count) ++*count;
         return MSP_OK;
     }
+    template <int Q>
+    void launch_vec(int which, int len, const float* a0, const float* a1, float* a2, float* a3, Pcg* sc,
+                    int flexible) {
+        const unsigned nt = (unsigned)round_up((len / 4 + Q - 1) / Q, 32);
+        switch (which) {
+            case 0: k_pcg_init<Q><<<1, nt, 0, strm>>>(len, a0, a2, a3, sc); break;
+            case 1: k_pcg_start<Q><<<1, nt, 0, strm>>>(len, a0, a1, a2, a3, sc); break;
+            // the fixed-step inner levels only freeze a step with p.q <= 0
+            case 2: k_pcg_step<Q><<<1, nt, 0, strm>>>(len, a0, a1, a2, a3, sc, sc == g->sc ? g->err : nullptr); break;
+            default: k_pcg_dir<Q><<<1, nt, 0, strm>>>(len, a0, a1, a2, a3, sc, flexible); break;
+        }
+    }
     msp_status vec(int which, int len, const float* a0, const float* a1, float* a2, float* a3, Pcg* sc,
                    int flexible = 0) {
-        switch (which) {
-            case 0: k_pcg_init<<<1, kVecThreads, 0, strm>>>(len, a0, a2, a3, sc); break;
-            case 1: k_pcg_start<<<1, kVecThreads, 0, strm>>>(len, a0, a1, a2, a3, sc); break;
-            // the fixed-step inner levels only freeze a step with p.q <= 0
-            case 2: k_pcg_step<<<1, kVecThreads, 0, strm>>>(len, a0, a1, a2, a3, sc, sc == g->sc ? g->err : nullptr); break;
-            default: k_pcg_dir<<<1, kVecThreads, 0, strm>>>(len, a0, a1, a2, a3, sc, flexible); break;
-        }
+        // len is a multiple of 4, at most kMaxN
+        if (len <= 4 * kVecThreads) launch_vec<1>(which, len, a0, a1, a2, a3, sc, flexible);
+        else launch_vec<kMaxN / (4 * kVecThreads)>(which, len, a0, a1, a2, a3, sc, flexible);
         MSP_CHECK_LAUNCH(ctx);
         if (count) ++*count;
         return MSP_OK;

@@ -4,6 +4,8 @@
 // One level-1 (outer) iteration is two launches:
 //   k_gemv      q = (A + lam I) p, one pass over A, with the dot p^T q fused;
 //               the last block to finish forms alpha = (r^T z) / (p^T q).
+//               (With packed tiles k_symv_packed of symv.cu: it also forms the
+//               direction p = w + beta p, and leaves p^T q in block partials.)
 //   k_level2    persistent cooperative kernel: x += alpha p, r -= alpha q,
 //               convergence test on |r|, then SolveM1(r) (Algorithm 2):
 //               g = C^T r; level-2 PCG on (C^T C + lam~ W) y = g
@@ -13,6 +15,7 @@
 // memory; every block computes the same scalars from the same partial sums
 // in the same order, so all blocks take identical branches and the number of
 // grid barriers always matches. Reductions use fixed orders (deterministic).
+#include "bulk.cuh"
 #include "msp_internal.cuh"
 
 #include <cuda_bf16.h>
@@ -23,8 +26,10 @@
 
 namespace {
 
-constexpr int kNW = 8;             // warps per block in k_level2
+constexpr int kNW = 16;            // warps per block in k_level2
 constexpr int kThreads = kNW * 32;
+constexpr int kRowChunk = kThreads;          // rows of C whose r, w are staged at a time
+constexpr int kQScratch = 4 * kNW * 32;      // slot sums of the level-1 update
 
 enum { MODE_INIT = 0, MODE_ITER = 1, MODE_APPLY = 2 };
 
@@ -294,6 +299,7 @@ template <typename T, typename TC = T>
 struct L2Args {
     int64_t n, s_pad;
     int mode;
+    int res_rows;           // rows of C a block keeps in shared memory
     const TC* C;
     const TC* W;
     const T* B;
@@ -305,10 +311,13 @@ struct L2Args {
     T* x;
     T* r;
     const T* q;
-    T* p;
+    T* p;                   // direction (packed A pass: the two buffers p, p + p_ld in turn)
+    int64_t p_ld;
     T* z;                   // level-1 preconditioned residual (in/out)
     const float* qpart;     // packed A pass: q_i = sum_slot qpart[slot][i] + lam p_i
     int q_slots;
+    int n_dq;               // and the block partials of p^T q, n_dq of them in dq
+    const double* dq;
     int64_t q_ld;
     T lam;
     CtlBlock* ctl;
@@ -343,192 +352,193 @@ struct RowSlice {
     }
 };
 
-template <typename T, int PL, typename TS = T>
-__device__ inline void store_slice(T* dst, const T* src, int lane) {
-    constexpr int W = StoreW<TS>::W;
-#pragma unroll
-    for (int k = 0; k < PL / W; ++k)
-#pragma unroll
-        for (int e = 0; e < W; ++e) dst[k * 32 * W + lane * W + e] = src[k * W + e];
+// Two neighbouring values of a stored row, widened.
+__device__ inline void load_pair(const float* p, float& a, float& b) {
+    const float2 v = *reinterpret_cast<const float2*>(p);
+    a = v.x;
+    b = v.y;
+}
+__device__ inline void load_pair(const double* p, double& a, double& b) {
+    const double2 v = *reinterpret_cast<const double2*>(p);
+    a = v.x;
+    b = v.y;
+}
+__device__ inline void load_pair(const __nv_bfloat16* p, float& a, float& b) {
+    const uint32_t v = *reinterpret_cast<const uint32_t*>(p);
+    a = __uint_as_float(v << 16);
+    b = __uint_as_float(v & 0xFFFF0000u);
 }
 
-// Row pass over this block's rows of C.
-//   kind 0: acc += r_i c_i                     (g = C^T r)
-//   kind 1: acc += (c_i . d) c_i               (u = C^T C d)
-//   kind 2: w_i = (r_i - c_i . y) / lam~; dots r.w and r.z_old  (no acc)
-// Per-warp accumulators are combined through shared memory into part[b].
-constexpr int kRowChunk = 256;   // rows of C staged per round (r, z, w in shared memory)
-
+// Layout of the level-2 kernel for a padded sketch size 32 PL.
 template <typename T, typename TC, int PL>
-__device__ inline void row_one(const L2Args<T, TC>& a, int kind, int64_t il, const RowSlice<T, PL, TC>& c,
-                               const T* svec, T* acc, const T* sr, T* sw, int lane) {
-    T coef;
-    if (kind == 0) {
-        coef = sr[il];
-    } else {
-        T t = msp::warp_sum(c.dot_smem(svec, lane));
-        if (kind == 1) {
-            coef = t;
-        } else {
-            if (lane == 0) sw[il] = (sr[il] - t) / a.lam_t;
-            return;
-        }
-    }
-#pragma unroll
-    for (int k = 0; k < PL; ++k) acc[k] += coef * c.v[k];
-}
+struct L2Shape {
+    static constexpr int SP = 32 * PL;
+    static constexpr int U = SP / 2;                              // column pairs
+    static constexpr int NG = U >= kThreads ? 1 : kThreads / U;   // row groups of the column pass
+    static constexpr int KU = (U + kThreads - 1) / kThreads;      // pairs per thread
+    static constexpr int SCR = NG * SP > kQScratch ? NG * SP : kQScratch;
+    // four full vectors, the scratch of the reductions, r and the row results
+    static constexpr size_t fixed = ((size_t)4 * SP + SCR + 2 * kRowChunk) * sizeof(T) + 16;
+    static constexpr size_t row = (size_t)SP * sizeof(TC);
+};
 
-// Row pass over this block's rows of C, two rows in flight per warp, in
-// chunks of kRowChunk rows whose r (and z_old, w) live in shared memory so no
-// per-row global access sits on the critical path.
-//   kind 0: acc += r_i c_i                     (g = C^T r)
-//   kind 1: acc += (c_i . d) c_i               (u = C^T C d)
-//   kind 2: w_i = (r_i - c_i . y) / lam~ into z; per-thread dots r.w, r.z_old
-// Per-warp accumulators are combined through shared memory into part[b].
+// The rows [row0, row0 + nr) of C of one block: the first nres of them in
+// shared memory (copied once, when the kernel starts), the others read from L2.
+template <typename TC>
+struct BlockRows {
+    const TC* g;      // row row0 of C
+    const TC* s;      // the same rows, resident
+    int nr, nres;
+};
+
+// acc (a pair of columns per thread) += sum_i coef[i - cb] c_i over the rows
+// [cb, ce) of the block; the rows from L2 first (eight loads in flight), then the
+// resident ones.
 template <typename T, typename TC, int PL>
-__device__ void row_pass(const L2Args<T, TC>& a, int kind, int64_t row0, int64_t row1, const T* svec,
-                         T* swarp, T* srow, double* rw, double* rzo) {
-    const int lane = threadIdx.x & 31, w = threadIdx.x >> 5;
-    T* sr = srow;                 // kRowChunk
-    T* sw = srow + kRowChunk;     // kRowChunk
-    T acc[PL];
+__device__ __forceinline__ void cols_pass(const BlockRows<TC>& rows, int cb, int ce, const T* coef,
+                                          T (&acc)[L2Shape<T, TC, PL>::KU][2]) {
+    using S = L2Shape<T, TC, PL>;
+    const int grp = S::NG > 1 ? (int)threadIdx.x / S::U : 0;
+    const int u0 = S::NG > 1 ? (int)threadIdx.x % S::U : (int)threadIdx.x;
+    if (grp >= S::NG || u0 >= S::U) return;
+    int i = max(cb, rows.nres) + grp;
+    for (; i + 7 * S::NG < ce; i += 8 * S::NG) {
+        T c[8][S::KU][2];
 #pragma unroll
-    for (int k = 0; k < PL; ++k) acc[k] = T(0);
-    double d_rw = 0.0, d_rzo = 0.0;
-    for (int64_t base = row0; base < row1; base += kRowChunk) {
-        const int64_t end = min(row1, base + kRowChunk);
-        const int nr = (int)(end - base);
-        if (kind != 1) {
-            for (int e = threadIdx.x; e < nr; e += blockDim.x) sr[e] = a.r[base + e];
-            __syncthreads();
-        }
-        int il = w;
-        for (; il + kNW < nr; il += 2 * kNW) {
-            RowSlice<T, PL, TC> c0, c1;
-            c0.load(a.C + (base + il) * a.s_pad, lane);
-            c1.load(a.C + (base + il + kNW) * a.s_pad, lane);
-            row_one<T, TC, PL>(a, kind, il, c0, svec, acc, sr, sw, lane);
-            row_one<T, TC, PL>(a, kind, il + kNW, c1, svec, acc, sr, sw, lane);
-        }
-        if (il < nr) {
-            RowSlice<T, PL, TC> c0;
-            c0.load(a.C + (base + il) * a.s_pad, lane);
-            row_one<T, TC, PL>(a, kind, il, c0, svec, acc, sr, sw, lane);
-        }
-        if (kind != 1) __syncthreads();
-        if (kind == 2) {
-            for (int e = threadIdx.x; e < nr; e += blockDim.x) {
-                const T ri = sr[e], wi = sw[e];
-                const T zo = a.z[base + e];
-                d_rw += (double)ri * (double)wi;
-                d_rzo += (double)ri * (double)zo;
-                a.z[base + e] = wi;
+        for (int q = 0; q < 8; ++q)
+#pragma unroll
+            for (int k = 0; k < S::KU; ++k)
+                load_pair(rows.g + (int64_t)(i + q * S::NG) * S::SP + 2 * (u0 + k * kThreads), c[q][k][0], c[q][k][1]);
+#pragma unroll
+        for (int q = 0; q < 8; ++q) {
+            const T f = coef[i + q * S::NG - cb];
+#pragma unroll
+            for (int k = 0; k < S::KU; ++k) {
+                acc[k][0] += f * c[q][k][0];
+                acc[k][1] += f * c[q][k][1];
             }
-            __syncthreads();
         }
     }
-    if (kind == 2) {
-        *rw = d_rw;
-        *rzo = d_rzo;
-        return;
-    }
-    store_slice<T, PL, TC>(swarp + (int64_t)w * a.s_pad, acc, lane);
+    auto one = [&](const TC* row, T f) {
+#pragma unroll
+        for (int k = 0; k < S::KU; ++k) {
+            T c0, c1;
+            load_pair(row + 2 * (u0 + k * kThreads), c0, c1);
+            acc[k][0] += f * c0;
+            acc[k][1] += f * c1;
+        }
+    };
+#pragma unroll 4
+    for (; i < ce; i += S::NG) one(rows.g + (int64_t)i * S::SP, coef[i - cb]);
+    const int se = min(ce, rows.nres);
+#pragma unroll 8
+    for (i = cb + grp; i < se; i += S::NG) one(rows.s + (int64_t)i * S::SP, coef[i - cb]);
 }
 
-// Butterfly reduce-scatter: lane l ends with the sum over the 32 lanes of
-// v[l] (31 shuffles, v overwritten).
-template <typename T>
-__device__ inline T reduce_scatter32(T* v, int lane) {
+// part[b] = the threads' column sums (row groups added through scr, in order)
+template <typename T, typename TC, int PL>
+__device__ __forceinline__ void cols_store(T (&acc)[L2Shape<T, TC, PL>::KU][2], T* scr, T* part) {
+    using S = L2Shape<T, TC, PL>;
+    if constexpr (S::NG == 1) {
 #pragma unroll
-    for (int wd = 16; wd >= 1; wd >>= 1) {
+        for (int k = 0; k < S::KU; ++k) {
+            const int u = (int)threadIdx.x + k * kThreads;
+            if (u < S::U) {
+                part[2 * u] = acc[k][0];
+                part[2 * u + 1] = acc[k][1];
+            }
+        }
+    } else {
+        const int grp = (int)threadIdx.x / S::U, u = (int)threadIdx.x % S::U;
+        if (grp < S::NG) {
+            scr[grp * S::SP + 2 * u] = acc[0][0];
+            scr[grp * S::SP + 2 * u + 1] = acc[0][1];
+        }
+        __syncthreads();
+        for (int c = threadIdx.x; c < S::SP; c += kThreads) {
+            T v = T(0);
+#pragma unroll
+            for (int g = 0; g < S::NG; ++g) v += scr[g * S::SP + c];
+            part[c] = v;
+        }
+    }
+}
+
+// Butterfly reduce-scatter over 2^K lanes' groups: on entry v[0 .. 2^K), on
+// exit lane l holds in v[0] the sum over the warp of entry (l >> (5 - K)) of v.
+template <int K, typename T>
+__device__ __forceinline__ T reduce_scatter(T* v, int lane) {
+#pragma unroll
+    for (int s = 0; s < K; ++s) {
+        const int wd = 16 >> s, half = (1 << K) >> (s + 1);
         const bool upper = (lane & wd) != 0;
 #pragma unroll
-        for (int i = 0; i < wd; ++i) {
-            const T send = upper ? v[i] : v[i + wd];
-            const T keep = upper ? v[i + wd] : v[i];
+        for (int i = 0; i < half; ++i) {
+            const T send = upper ? v[i] : v[i + half];
+            const T keep = upper ? v[i + half] : v[i];
             v[i] = keep + __shfl_xor_sync(0xffffffffu, send, wd);
         }
     }
+#pragma unroll
+    for (int wd = 16 >> K; wd >= 1; wd >>= 1) v[0] += __shfl_xor_sync(0xffffffffu, v[0], wd);
     return v[0];
 }
 
-// Row pass of kind 2 (w_i = (r_i - c_i . y) / lam~, dots r.w and r.z_old)
-// for PL <= 32: a warp takes the rows w, w + kNW, ... of a chunk (at most 32
-// when kRowChunk = 32 kNW), holds its slice of y in registers, keeps one
-// partial dot per row and reduces all of them at once by a reduce-scatter, so
-// no per-row warp reduction sits in a dependency chain (the per-row
-// reductions of row_one held this pass to the latency of one shuffle chain
-// per row).
+// dot[i - cb] = c_i . vec over the rows [cb, ce) of the block (ce - cb <=
+// kRowChunk); vec in shared memory. A warp takes every kNW-th row. Up to PL =
+// 32 (FP64: 16) its slice of vec stays in registers and it reduces 8 or 16
+// rows' partial dots at once; the rows from L2 come first, two in flight.
 template <typename T, typename TC, int PL>
-__device__ void row_pass_w(const L2Args<T, TC>& a, int64_t row0, int64_t row1, const T* svec, T* srow,
-                           double* rw, double* rzo) {
-    static_assert(PL <= 32, "y slice and 32 partial dots in registers");
-    static_assert(kRowChunk == 32 * kNW, "a warp's rows of a chunk fit one reduce-scatter");
+__device__ __forceinline__ void dots_pass(const BlockRows<TC>& rows, int cb, int ce, const T* vec, T* dot) {
+    constexpr int SP = 32 * PL, W = StoreW<TC>::W;
     const int lane = threadIdx.x & 31, w = threadIdx.x >> 5;
-    constexpr int W = StoreW<TC>::W;
-    T* sr = srow;
-    T* sw = srow + kRowChunk;
-    T ys[PL];
+    if constexpr (PL <= (sizeof(T) == 4 ? 32 : 16)) {
+        T vs[PL];
 #pragma unroll
-    for (int k = 0; k < PL / W; ++k)
+        for (int k = 0; k < PL / W; ++k)
 #pragma unroll
-        for (int e = 0; e < W; ++e) ys[k * W + e] = svec[k * 32 * W + lane * W + e];
-    double d_rw = 0.0, d_rzo = 0.0;
-    for (int64_t base = row0; base < row1; base += kRowChunk) {
-        const int64_t end = min(row1, base + kRowChunk);
-        const int nr = (int)(end - base);
-        for (int e = threadIdx.x; e < nr; e += blockDim.x) sr[e] = a.r[base + e];
-        __syncthreads();
-        const int cnt = nr > w ? (nr - w + kNW - 1) / kNW : 0;   // this warp's rows: w + kNW t, t < cnt
-        T part[32];
+            for (int e = 0; e < W; ++e) vs[k * W + e] = vec[k * 32 * W + lane * W + e];
+        // this warp's rows in the order they are read: L2 rows, then resident ones
+        const int split = min(max(cb, rows.nres), ce);
+        const int ng = split + w < ce ? (ce - split - w + kNW - 1) / kNW : 0;
+        const int ns = cb + w < split ? (split - cb - w + kNW - 1) / kNW : 0;
+        const int cnt = ng + ns;
+        auto index = [&](int o) { return o < ng ? split + w + kNW * o : cb + w + kNW * (o - ng); };
+        auto ptr = [&](int o) {
+            const int i = index(o);
+            return o < ng ? rows.g + (int64_t)i * SP : rows.s + (int64_t)i * SP;
+        };
+        constexpr int KP = PL * sizeof(T) > 80 ? 3 : 4;      // 2^KP partial dots in registers
+        for (int o0 = 0; o0 < cnt; o0 += 1 << KP) {
+            T part[1 << KP];
 #pragma unroll
-        for (int t = 0; t < 32; ++t) part[t] = T(0);
+            for (int t = 0; t < 1 << KP; t += 2) {
+                part[t] = T(0);
+                part[t + 1] = T(0);
+                if (o0 + t < cnt) {
+                    RowSlice<T, PL, TC> c0, c1;
+                    c0.load(ptr(o0 + t), lane);
+                    const bool two = o0 + t + 1 < cnt;
+                    if (two) c1.load(ptr(o0 + t + 1), lane);
 #pragma unroll
-        for (int t = 0; t < 32; t += 2) {
-            if (t < cnt) {
-                RowSlice<T, PL, TC> c0, c1;
-                c0.load(a.C + (base + w + (int64_t)kNW * t) * a.s_pad, lane);
-                const bool two = t + 1 < cnt;
-                if (two) c1.load(a.C + (base + w + (int64_t)kNW * (t + 1)) * a.s_pad, lane);
-                T d0 = T(0), d1 = T(0);
+                    for (int k = 0; k < PL; ++k) part[t] += c0.v[k] * vs[k];
+                    if (two) {
 #pragma unroll
-                for (int k = 0; k < PL; ++k) d0 += c0.v[k] * ys[k];
-                part[t] = d0;
-                if (two) {
-#pragma unroll
-                    for (int k = 0; k < PL; ++k) d1 += c1.v[k] * ys[k];
-                    part[t + 1] = d1;
+                        for (int k = 0; k < PL; ++k) part[t + 1] += c1.v[k] * vs[k];
+                    }
                 }
             }
+            const T d = reduce_scatter<KP>(part, lane);
+            const int o = o0 + (lane >> (5 - KP));
+            if ((lane & ((32 >> KP) - 1)) == 0 && o < cnt) dot[index(o) - cb] = d;
         }
-        const T dot = reduce_scatter32<T>(part, lane);
-        if (lane < cnt) {
-            const int il = w + kNW * lane;
-            sw[il] = (sr[il] - dot) / a.lam_t;
+    } else {
+        for (int i = cb + w; i < ce; i += kNW) {
+            RowSlice<T, PL, TC> c;
+            c.load(i < rows.nres ? rows.s + (int64_t)i * SP : rows.g + (int64_t)i * SP, lane);
+            const T t = msp::warp_sum(c.dot_smem(vec, lane));
+            if (lane == 0) dot[i - cb] = t;
         }
-        __syncthreads();
-        for (int e = threadIdx.x; e < nr; e += blockDim.x) {
-            const T ri = sr[e], wi = sw[e];
-            const T zo = a.z[base + e];
-            d_rw += (double)ri * (double)wi;
-            d_rzo += (double)ri * (double)zo;
-            a.z[base + e] = wi;
-        }
-        __syncthreads();
-    }
-    *rw = d_rw;
-    *rzo = d_rzo;
-}
-
-// part[b][c] = sum over warps of swarp[w][c]
-template <typename T, typename TC>
-__device__ inline void combine_warps(const L2Args<T, TC>& a, const T* swarp, int b) {
-    __syncthreads();
-    for (int64_t c = threadIdx.x; c < a.s_pad; c += blockDim.x) {
-        T v = T(0);
-#pragma unroll
-        for (int w = 0; w < kNW; ++w) v += swarp[w * a.s_pad + c];
-        a.part[(int64_t)b * a.s_pad + c] = v;
     }
 }
 
@@ -545,66 +555,85 @@ __device__ inline void rows_dot(const TS* M, int64_t s_pad, int64_t c0, int64_t 
     }
 }
 
-// out[c] = sum_k part[k][c] (+ add_scale * addend[c]) for c in [c0, c1), k < G.
-// Fixed order: thread t sums k = t, t + blockDim, ...; then a warp tree; then
-// warps in index order. Returns sum_c out[c] * dvec[c] (dvec in shared memory,
-// may be null) and sum_c out[c]^2 through *sq (may be null). Columns are
-// processed 8 at a time so all loads of a chunk are in flight together.
-// With `pre` (stride pre_stride, G entries), its sum is formed alongside, its
-// loads in flight with the first chunk's, in the order of sum_parts (same
-// value), into *pre_out for every thread; red2 then holds 9 x 32 doubles.
+// out[c] = sum_k part[k][c] (+ add_scale * addend[c]) over the block's columns,
+// the groups of eight b, b + G, ...; k < G <= kThreads. Thread k reads the eight
+// columns of partial k (one or two sectors), a warp reduces them by a
+// reduce-scatter, and threads c < 8 add the warps' sums in order in FP64. With
+// dvec (shared memory) returns sum_c dvec[c] out[c], with sq sum_c out[c]^2, in
+// thread 0. red holds kNW x 8 values. Ends past a block barrier.
 template <typename T>
-__device__ inline void reduce_cols(const T* part, int G, int64_t sp, int64_t c0, int64_t c1,
-                                   const T* addend, T add_scale, T* out, const T* dvec,
-                                   double* dot_out, double* sq_out, double* red2 /*8*32*/,
-                                   const double* pre = nullptr, int pre_stride = 0,
-                                   double* pre_out = nullptr) {
-    const int lane = threadIdx.x & 31, w = threadIdx.x >> 5, nw = blockDim.x >> 5;
-    double dot = 0.0, sq = 0.0;
-    bool first = true;
-    for (int64_t cb = c0; first || cb < c1; cb += 8) {
-        const int nc = (int)max((int64_t)0, min((int64_t)8, c1 - cb));
-        const bool with_pre = first && pre != nullptr;
-        first = false;
-        T v[8];
-        double pv = 0.0;
+__device__ inline double reduce_cols(const T* part, int G, int64_t sp, const T* addend, T add_scale, T* out,
+                                     const T* dvec, bool sq, T* red) {
+    const int lane = threadIdx.x & 31, w = threadIdx.x >> 5, nw = (G + 31) >> 5;
+    constexpr int W = Vec16<T>::W;
+    double dot = 0.0;
+    int64_t cb = (int64_t)blockIdx.x * 8;
+    do {
+        if (w < nw && cb < sp) {
+            T v[8];
+            const T* row = part + (int64_t)threadIdx.x * sp + cb;
 #pragma unroll
-        for (int c = 0; c < 8; ++c) v[c] = T(0);
-        for (int k = threadIdx.x; k < G; k += blockDim.x) {
+            for (int k = 0; k < 8; k += W) {
+                if ((int)threadIdx.x < G) {
+                    const typename Vec16<T>::type q =
+                        __ldcg(reinterpret_cast<const typename Vec16<T>::type*>(row + k));
+                    if constexpr (W == 4) { v[k] = q.x; v[k + 1] = q.y; v[k + 2] = q.z; v[k + 3] = q.w; }
+                    else { v[k] = q.x; v[k + 1] = q.y; }
+                } else {
 #pragma unroll
-            for (int c = 0; c < 8; ++c)
-                if (c < nc) v[c] += __ldcg(&part[(int64_t)k * sp + cb + c]);
-            if (with_pre) pv += __ldcg(&pre[(int64_t)k * pre_stride]);
-        }
-#pragma unroll
-        for (int c = 0; c < 8; ++c) v[c] = msp::warp_sum(v[c]);
-        if (with_pre) pv = msp::warp_sum(pv);
-        __syncthreads();
-        if (lane == 0) {
-#pragma unroll
-            for (int c = 0; c < 8; ++c) red2[c * 32 + w] = (double)v[c];
-            if (with_pre) red2[8 * 32 + w] = pv;
+                    for (int e = 0; e < W; ++e) v[k + e] = T(0);
+                }
+            }
+            const T t = reduce_scatter<3>(v, lane);
+            if ((lane & 3) == 0) red[w * 8 + (lane >> 2)] = t;
         }
         __syncthreads();
-        if (with_pre) {
-            double t = 0.0;
-            for (int k = 0; k < nw; ++k) t += red2[8 * 32 + k];
-            *pre_out = t;
-        }
-        if (threadIdx.x < nc) {
-            const int c = threadIdx.x;
+        if (threadIdx.x < 8 && cb < sp) {
+            const int64_t c = cb + threadIdx.x;
             double acc = 0.0;
-            for (int k = 0; k < nw; ++k) acc += red2[c * 32 + k];
+            for (int k = 0; k < nw; ++k) acc += (double)red[k * 8 + threadIdx.x];
             T r = (T)acc;
-            if (addend) r += add_scale * __ldcg(&addend[cb + c]);
-            out[cb + c] = r;
-            if (dvec) dot += (double)dvec[cb + c] * (double)r;
-            sq += (double)r * (double)r;
+            if (addend) r += add_scale * __ldcg(&addend[c]);
+            out[c] = r;
+            if (dvec) dot += (double)dvec[c] * (double)r;
+            else if (sq) dot += (double)r * (double)r;
         }
+        cb += 8 * (int64_t)G;
+        if (cb < sp) __syncthreads();
+    } while (cb < sp);
+    if ((dvec || sq) && w == 0)
+#pragma unroll
+        for (int o = 4; o > 0; o >>= 1) dot += __shfl_xor_sync(0xffffffffu, dot, o);
+    return dot;
+}
+
+// Sum over the block in warp 0; `active`: this warp holds values (the same in
+// all its lanes; a warp without any adds nothing to the FP64 pipe). red: kNW.
+__device__ inline double block_sum0(double v, bool active, double* red) {
+    const int lane = threadIdx.x & 31, w = threadIdx.x >> 5;
+    if (active) v = msp::warp_sum(v);
+    if (lane == 0) red[w] = active ? v : 0.0;
+    __syncthreads();
+    if (w != 0) return 0.0;
+    return msp::warp_sum(lane < kNW ? red[lane] : 0.0);
+}
+
+// Sum of a per-block partial array by the calling warp, fixed order.
+__device__ inline double warp_sum_parts(const double* parts, int stride, int G) {
+    double v = 0.0;
+    for (int k = threadIdx.x & 31; k < G; k += 32) v += __ldcg(&parts[(int64_t)k * stride]);
+    return msp::warp_sum(v);
+}
+
+// The same for every thread: warp 0 sums, *slot hands the value on. A slot is
+// written again only after a later block barrier.
+__device__ inline double grid_sum(const double* parts, int G, double* slot) {
+    if ((threadIdx.x >> 5) == 0) {
+        const double v = warp_sum_parts(parts, 4, G);
+        if (threadIdx.x == 0) *slot = v;
     }
     __syncthreads();
-    if (dot_out) *dot_out = dot;   // per-thread partials; caller block-sums them
-    if (sq_out) *sq_out = sq;
+    return *slot;
 }
 
 template <typename T>
@@ -612,182 +641,278 @@ __device__ inline void load_full(const T* g, T* s, int64_t m) {
     for (int64_t c = threadIdx.x; c < m; c += blockDim.x) s[c] = __ldcg(&g[c]);
 }
 
+// One block of 16 warps per SM. What bounds it is latency: the grid barriers
+// and the serial phases between them; after those, the FP64 pipe (2 lanes a clock
+// an SM, a warp-wide FP64 instruction holds it for 16 cycles), so every FP64 sum
+// is formed by the warps that hold values and finished by one warp, and the two
+// passes over the block's rows of C. The first res_rows of those rows are copied
+// to shared memory by the copy engine when the kernel starts, beside the level-1
+// update, and serve every pass (at n = 8192, s = 512 all of them; at n = 16384,
+// s = 1024 a third). Two blocks of 8 warps per SM, every warp finishing every sum,
+// the rows read twice from L2, and the new direction formed here behind a fifth
+// barrier took 36.6 us (n = 16384, s = 1024) and 28.5 us (n = 8192, s = 512); now
+// 27.8 and 20.5 us.
 template <typename T, typename TC, int PL>
 __global__ void __launch_bounds__(kThreads, 1) k_level2(L2Args<T, TC> a) {
+    using S = L2Shape<T, TC, PL>;
     extern __shared__ __align__(16) unsigned char smem_raw[];
-    const int64_t sp = a.s_pad;
-    T* sd = reinterpret_cast<T*>(smem_raw);       // d (search direction)
+    constexpr int64_t sp = S::SP;
+    TC* cres = reinterpret_cast<TC*>(smem_raw);   // resident rows of C
+    T* sd = reinterpret_cast<T*>(smem_raw + (size_t)a.res_rows * S::row);   // d (search direction)
     T* sres = sd + sp;                            // level-2 residual
     T* sy = sres + sp;                            // level-2 iterate
     T* stmp = sy + sp;                            // scratch full vector
-    T* swarp = stmp + sp;                         // kNW x sp
-    T* srow = swarp + kNW * sp;                   // 2 x kRowChunk (row pass staging)
-    __shared__ double red[32];
-    __shared__ double red64[64];
-    __shared__ double red2[9 * 32];
-    __shared__ double s_rw, s_rzo;
+    T* scr = stmp + sp;                           // reduction scratch
+    T* srow = scr + S::SCR;                       // r of the block's rows (a chunk)
+    T* sw = srow + kRowChunk;                     // row results
+    uint64_t* bar = reinterpret_cast<uint64_t*>(sw + kRowChunk);
+    __shared__ double red[kNW], red_b[kNW], red_c[kNW];
+    __shared__ T redc[kNW * 8];
+    __shared__ double s_alpha, s_rr, s_val[4];
+    __shared__ int s_bad;
 
     CtlBlock* ctl = a.ctl;
     // the control words in one round trip
-    const int c_done = ctl->done, c_err = ctl->error;
-    const double alpha = ctl->alpha;
-    const double rz_outer = ctl->rz;
-    const double tol2 = ctl->tol2;
+    const int c_done = ctl->done, c_err = ctl->error, iter = ctl->iters;
+    const double c_alpha = ctl->alpha, c_rz = ctl->rz, tol2 = ctl->tol2;
+    const double c_rz0 = ctl->rzbuf[0], c_rz1 = ctl->rzbuf[1];
     if (c_done | c_err) return;
+    const int lane = threadIdx.x & 31, w = threadIdx.x >> 5;
     const int G = gridDim.x, b = blockIdx.x;
     const int64_t row0 = a.n * b / G, row1 = a.n * (b + 1) / G;
     const int64_t c0 = sp * b / G, c1 = sp * (b + 1) / G;
     unsigned int* bw = &ctl->bar_word;
     int* err = &ctl->error;
+    const bool packed = a.dq != nullptr;
+    BlockRows<TC> rows{a.C + row0 * sp, cres, (int)(row1 - row0), (int)min((int64_t)a.res_rows, row1 - row0)};
+    if (threadIdx.x == 0) {
+        msp::mbar_init(bar, 1);
+        asm volatile("fence.mbarrier_init.release.cluster;" ::: "memory");
+        uint32_t left = (uint32_t)(rows.nres * S::row);
+        msp::mbar_arrive_expect_tx(bar, left);
+        for (uint32_t o = 0; left > 0;) {
+            const uint32_t len = min(left, 32768u);
+            msp::bulk_g2s(smem_raw + o, reinterpret_cast<const unsigned char*>(rows.g) + o, len, bar);
+            o += len;
+            left -= len;
+        }
+        s_bad = 0;
+    }
+    __syncthreads();
 
-    // ---- level-1 update and g = C^T r partials
+    // ---- level-1 update
+    const T* p = a.p;
+    bool have_r = false;      // srow holds r of all the block's rows
     double rr = 0.0;
-    if (a.mode == MODE_ITER && a.qpart) {
+    if (a.mode == MODE_ITER && packed) {
         // q_i = sum over the packed A pass's slot partials + lam p_i, fixed
-        // summation order. Rounds of four 32-row groups: every thread sums
-        // its slot group for the four rows, the loads of all four rows in
-        // flight together (eight slots per row at a time), warp g finishes
-        // group g (its p_i, r_i, x_i loaded before the slot partials), and
-        // warp 0 adds the squares of the new r_i row by row in group order.
+        // summation order. Rounds of four 32-row groups: every warp sums its
+        // slots for the four rows of a lane, the loads in flight together
+        // (eight slots per row at a time), warp g finishes group g (its p_i,
+        // r_i, x_i loaded before the slot partials). The last warp takes no
+        // slots: it forms the step alpha = rz / p^T q meanwhile.
         constexpr int kGroups = 4;
-        T* sq = swarp;  // kGroups x 8 x 32 scratch (swarp holds 8 s_pad >= 1024 values; free here)
-        T* rnew = reinterpret_cast<T*>(red2);   // kGroups x 32 new r_i (red2 is free here)
-        const int rl = threadIdx.x & 31, grp = threadIdx.x >> 5;
+        p = a.p + (iter & 1) * a.p_ld;
+        T* sq = scr;          // kGroups x kNS x 32
+        constexpr int kNS = kNW - 1;
+        if (w == kNW - 1) {
+            const double pq = warp_sum_parts(a.dq, 1, a.n_dq);
+            if (lane == 0) {
+                s_alpha = ((iter & 1) ? c_rz1 : c_rz0) / pq;
+                if (!isfinite(pq)) s_bad = MSP_ENONFINITE;
+                else if (!(pq > 0.0)) s_bad = MSP_ENOTPD;
+            }
+        }
+        have_r = rows.nr <= kRowChunk;
         for (int64_t base = row0; base < row1; base += 32 * kGroups) {
-            const int64_t i_own = base + 32 * grp + rl;      // the row this thread finishes (grp < kGroups)
-            const bool own = grp < kGroups && i_own < row1;
+            const int64_t i_own = base + 32 * w + lane;      // the row this thread finishes (w < kGroups)
+            const bool own = w < kGroups && i_own < row1;
             T p_own = T(0), r_own = T(0), x_own = T(0);
             if (own) {
-                p_own = a.p[i_own];
+                p_own = p[i_own];
                 r_own = a.r[i_own];
                 x_own = a.x[i_own];
             }
             T v[kGroups];
 #pragma unroll
             for (int g = 0; g < kGroups; ++g) v[g] = T(0);
-            int sl = grp;
-            for (; sl + 7 * kNW < a.q_slots; sl += 8 * kNW) {
+            int sl = w < kNS ? w : a.q_slots;
+            for (; sl + 7 * kNS < a.q_slots; sl += 8 * kNS) {
                 T t8[kGroups][8];
 #pragma unroll
                 for (int g = 0; g < kGroups; ++g) {
-                    const int64_t i = base + 32 * g + rl;
+                    const int64_t i = base + 32 * g + lane;
 #pragma unroll
                     for (int u = 0; u < 8; ++u)
-                        t8[g][u] = (i < row1) ? __ldcg(&a.qpart[(int64_t)(sl + u * kNW) * a.q_ld + i]) : T(0);
+                        t8[g][u] = (i < row1) ? __ldcg(&a.qpart[(int64_t)(sl + u * kNS) * a.q_ld + i]) : T(0);
                 }
 #pragma unroll
                 for (int g = 0; g < kGroups; ++g)
 #pragma unroll
                     for (int u = 0; u < 8; ++u) v[g] += t8[g][u];
             }
-            for (; sl < a.q_slots; sl += kNW) {
+            for (; sl < a.q_slots; sl += 2 * kNS) {
+                const bool two = sl + kNS < a.q_slots;
+                T t0[kGroups], t1[kGroups];
 #pragma unroll
                 for (int g = 0; g < kGroups; ++g) {
-                    const int64_t i = base + 32 * g + rl;
-                    if (i < row1) v[g] += __ldcg(&a.qpart[(int64_t)sl * a.q_ld + i]);
+                    const int64_t i = base + 32 * g + lane;
+                    t0[g] = (i < row1) ? __ldcg(&a.qpart[(int64_t)sl * a.q_ld + i]) : T(0);
+                    t1[g] = (two && i < row1) ? __ldcg(&a.qpart[(int64_t)(sl + kNS) * a.q_ld + i]) : T(0);
                 }
+#pragma unroll
+                for (int g = 0; g < kGroups; ++g) v[g] = (v[g] + t0[g]) + t1[g];
             }
 #pragma unroll
-            for (int g = 0; g < kGroups; ++g) sq[(g * kNW + grp) * 32 + rl] = v[g];
+            for (int g = 0; g < kGroups; ++g)
+                if (w < kNS) sq[(g * kNS + w) * 32 + lane] = v[g];
             __syncthreads();
-            if (grp < kGroups) {
-                T ri = T(0);
-                if (own) {
-                    T qi = T(0);
-#pragma unroll
-                    for (int g = 0; g < kNW; ++g) qi += sq[(grp * kNW + g) * 32 + rl];
-                    qi += a.lam * p_own;
-                    ri = r_own;
-                    a.x[i_own] = x_own + (T)alpha * p_own;
-                    ri -= (T)alpha * qi;
-                    a.r[i_own] = ri;
+            if (s_bad) {
+                if (threadIdx.x == 0) {
+                    if (b == 0) atomicExch(err, s_bad);
+                    msp::mbar_wait_timed(bar, 0, err);   // the resident rows land before the block leaves
                 }
-                rnew[grp * 32 + rl] = ri;
+                return;       // the same in every block
             }
-            __syncthreads();
-            if (grp == 0) {
-                for (int g = 0; g < kGroups; ++g) {
-                    if (base + 32 * g + rl < row1) {
-                        const T ri = rnew[g * 32 + rl];
-                        rr += (double)ri * (double)ri;
-                    }
-                }
+            if (own) {
+                const T alpha = (T)s_alpha;
+                T qi = T(0);
+#pragma unroll
+                for (int g = 0; g < kNS; ++g) qi += sq[(w * kNS + g) * 32 + lane];
+                qi += a.lam * p_own;
+                T ri = r_own;
+                a.x[i_own] = x_own + alpha * p_own;
+                ri -= alpha * qi;
+                a.r[i_own] = ri;
+                if (have_r) srow[i_own - row0] = ri;
+                rr += (double)ri * (double)ri;
             }
             __syncthreads();
         }
-        rr = block_sum(rr, red);
-        if (threadIdx.x == 0) a.dpart[b * 4 + 0] = rr;
+        rr = block_sum0(rr, w < kGroups, red);
     } else if (a.mode != MODE_APPLY) {
         for (int64_t i = row0 + threadIdx.x; i < row1; i += blockDim.x) {
             T ri = a.r[i];
             if (a.mode == MODE_ITER) {
-                a.x[i] += (T)alpha * a.p[i];
-                ri -= (T)alpha * a.q[i];
+                const T alpha = (T)c_alpha;
+                a.x[i] += alpha * p[i];
+                ri -= alpha * a.q[i];
                 a.r[i] = ri;
             }
             rr += (double)ri * (double)ri;
         }
-        rr = block_sum(rr, red);
-        if (threadIdx.x == 0) a.dpart[b * 4 + 0] = rr;
+        rr = block_sum0(rr, 32 * w < rows.nr, red);
     }
-    __syncthreads();
-    row_pass<T, TC, PL>(a, 0, row0, row1, nullptr, swarp, srow, nullptr, nullptr);
-    combine_warps(a, swarp, b);
-    if (!msp::grid_barrier(bw, err)) return;
+    if (threadIdx.x == 0) a.dpart[b * 4 + 0] = rr;
 
-    // ---- g reduced over this block's columns, with |r|^2 (the convergence
-    // test) summed alongside; |g|^2 only where the level-2 iteration's
-    // tolerance needs it
+    // the block's rows of r (a chunk) in srow
+    auto load_r = [&](int cb, int ce) {
+        for (int e = cb + (int)threadIdx.x; e < ce; e += kThreads) srow[e - cb] = a.r[row0 + e];
+        __syncthreads();
+    };
+    // ---- g = C^T r partials. A copy that does not arrive is seen by every thread
+    // that waits for it; the block then leaves and the others' grid barrier runs out.
+    T acc[S::KU][2];
+#pragma unroll
+    for (int k = 0; k < S::KU; ++k) acc[k][0] = acc[k][1] = T(0);
+    if (!msp::mbar_wait_timed(bar, 0, err)) s_bad = MSP_ETIMEOUT;
+    for (int cb = 0; cb < rows.nr; cb += kRowChunk) {
+        const int ce = min(rows.nr, cb + kRowChunk);
+        if (!have_r) load_r(cb, ce);
+        cols_pass<T, TC, PL>(rows, cb, ce, srow, acc);
+        if (ce < rows.nr) __syncthreads();
+    }
+    have_r = rows.nr <= kRowChunk;   // srow is not written again below
+    cols_store<T, TC, PL>(acc, scr, a.part + (int64_t)b * sp);
+    // the block's rows of B and B^T on their way to registers during the barriers
+    const bool one_row = c1 - c0 <= kNW;
+    const bool my_row = one_row && c0 + w < c1;
+    RowSlice<T, PL> mB;
+    if (my_row) mB.load(a.B + (c0 + w) * sp, lane);
+    if (!msp::grid_barrier(bw, err) || s_bad) return;
+
+    // ---- g reduced over this block's columns, |r|^2 (the convergence test) by
+    // the last warp beside it; |g|^2 only where the level-2 iteration's tolerance needs it
     const bool inner = a.max_inner > 0;
-    double gg = 0.0;
-    reduce_cols<T>(a.part, G, sp, c0, c1, nullptr, T(0), a.gvec, nullptr, nullptr, inner ? &gg : nullptr, red2,
-                   a.mode != MODE_APPLY ? a.dpart + 0 : nullptr, 4, &rr);
+    if (a.mode != MODE_APPLY && w == kNW - 1) {
+        const double t = warp_sum_parts(a.dpart, 4, G);
+        if (lane == 0) s_rr = t;
+    }
+    double gg = reduce_cols<T>(a.part, G, sp, nullptr, T(0), a.gvec, nullptr, inner, redc);
     if (a.mode != MODE_APPLY) {
-        if (!isfinite(rr)) {
+        rr = s_rr;
+        bool stop = !isfinite(rr);
+        double t2 = tol2;
+        if (a.mode == MODE_INIT) t2 = a.tol_rel2 * rr;
+        if (stop) {
             if (b == 0 && threadIdx.x == 0) ctl->error = MSP_ENONFINITE;
             return;
         }
-        double t2 = tol2;
-        if (a.mode == MODE_INIT) t2 = a.tol_rel2 * rr;
         if (rr <= t2) {
             if (b == 0 && threadIdx.x == 0) {
                 ctl->rr = rr;
                 if (a.mode == MODE_INIT) { ctl->bb = rr; ctl->tol2 = t2; }
-                if (a.mode == MODE_ITER) ctl->iters += 1;
+                if (a.mode == MODE_ITER) ctl->iters = iter + 1;
                 ctl->done = 1;
             }
             return;
         }
     }
-    if (inner) {
-        gg = block_sum(gg, red);
-        if (threadIdx.x == 0) a.dpart[b * 4 + 1] = gg;
-    }
+    if (inner && threadIdx.x == 0) a.dpart[b * 4 + 1] = gg;
     if (!msp::grid_barrier(bw, err)) return;
-    if (inner) gg = sum_parts(a.dpart + 1, 4, G, red);
+    if (inner) gg = grid_sum(a.dpart + 1, G, &s_val[0]);
     load_full(a.gvec, sres, sp);
-    for (int64_t c = threadIdx.x; c < sp; c += blockDim.x) sy[c] = T(0);
+    if (inner)
+        for (int c = threadIdx.x; c < sp; c += kThreads) sy[c] = T(0);
     __syncthreads();
 
-    // ---- z = M2^{-1} res = B^T (B res)
+    // ---- z = M2^{-1} res = B^T (B res); z^T res only where the level-2
+    // iteration uses it (rz_out given; the same in every block)
+    int turn = 1;
+    bool fresh = my_row;      // mB holds the block's row of B
     auto precond = [&](double* rz_out) -> bool {
-        rows_dot<T, PL>(a.B, sp, c0, c1, sres, a.tvec);
+        RowSlice<T, PL> mT;
+        if (my_row) {
+            if (!fresh) mB.load(a.B + (c0 + w) * sp, lane);
+            fresh = false;
+            const T t = msp::warp_sum(mB.dot_smem(sres, lane));
+            if (lane == 0) a.tvec[c0 + w] = t;
+            mT.load(a.Bt + (c0 + w) * sp, lane);
+        } else if (!one_row) {
+            rows_dot<T, PL>(a.B, sp, c0, c1, sres, a.tvec);
+        }
         if (!msp::grid_barrier(bw, err)) return false;
         load_full(a.tvec, stmp, sp);
         __syncthreads();
-        rows_dot<T, PL>(a.Bt, sp, c0, c1, stmp, a.zvec);
-        __syncthreads();
-        // z^T res only where the level-2 iteration uses it (rz_out given;
-        // the same in every block)
+        double part = 0.0;
+        if (my_row) {
+            const T z = msp::warp_sum(mT.dot_smem(stmp, lane));
+            if (lane == 0) {
+                a.zvec[c0 + w] = z;
+                if (rz_out) part = (double)sres[c0 + w] * (double)z;
+            }
+        } else if (!one_row) {
+            rows_dot<T, PL>(a.Bt, sp, c0, c1, stmp, a.zvec);
+            __syncthreads();
+            if (rz_out)
+                for (int64_t c = c0 + threadIdx.x; c < c1; c += kThreads) part += (double)sres[c] * (double)a.zvec[c];
+        }
         if (rz_out) {
-            double part = 0.0;
-            for (int64_t c = c0 + threadIdx.x; c < c1; c += blockDim.x)
-                part += (double)sres[c] * (double)a.zvec[c];
-            part = block_sum(part, red);
+            // my_row: lane 0 of each warp holds a product
+            if (one_row) {
+                if (lane == 0) red_b[w] = part;
+                __syncthreads();
+                part = w == 0 ? msp::warp_sum(lane < kNW ? red_b[lane] : 0.0) : 0.0;
+            } else {
+                part = block_sum0(part, true, red_b);
+            }
             if (threadIdx.x == 0) a.dpart[b * 4 + 2] = part;
         }
         if (!msp::grid_barrier(bw, err)) return false;
-        if (rz_out) *rz_out = sum_parts(a.dpart + 2, 4, G, red);
+        if (rz_out) {
+            *rz_out = grid_sum(a.dpart + 2, G, &s_val[turn]);
+            turn = 3 - turn;
+        }
         return true;
     };
 
@@ -803,87 +928,130 @@ __global__ void __launch_bounds__(kThreads, 1) k_level2(L2Args<T, TC> a) {
     int k = 0;
     while (k < a.max_inner && rres > tin2) {
         // P1: partial u = C^T (C d) over this block's rows; wd = W d (columns)
-        row_pass<T, TC, PL>(a, 1, row0, row1, sd, swarp, srow, nullptr, nullptr);
-        combine_warps(a, swarp, b);
+#pragma unroll
+        for (int q = 0; q < S::KU; ++q) acc[q][0] = acc[q][1] = T(0);
+        for (int cb = 0; cb < rows.nr; cb += kRowChunk) {
+            const int ce = min(rows.nr, cb + kRowChunk);
+            dots_pass<T, TC, PL>(rows, cb, ce, sd, sw);
+            __syncthreads();
+            cols_pass<T, TC, PL>(rows, cb, ce, sw, acc);
+            if (ce < rows.nr) __syncthreads();
+        }
+        cols_store<T, TC, PL>(acc, scr, a.part + (int64_t)b * sp);
         rows_dot<T, PL, TC>(a.W, sp, c0, c1, sd, a.wdvec);
         if (!msp::grid_barrier(bw, err)) return;
         // P2: u over this block's columns; d.u partial
-        double du = 0.0;
-        reduce_cols<T>(a.part, G, sp, c0, c1, a.wdvec, a.lam_t, a.uvec, sd, &du, nullptr, red2);
-        du = block_sum(du, red);
+        double du = reduce_cols<T>(a.part, G, sp, a.wdvec, a.lam_t, a.uvec, sd, false, redc);
         if (threadIdx.x == 0) a.dpart[b * 4 + 3] = du;
         if (!msp::grid_barrier(bw, err)) return;
         // P3: step
-        du = sum_parts(a.dpart + 3, 4, G, red);
+        du = grid_sum(a.dpart + 3, G, &s_val[3]);
         if (!(du > 0.0)) break;   // breakdown (same decision in every block)
         const T ain = (T)(rz_in / du);
         double loc = 0.0;
-        for (int64_t c = threadIdx.x; c < sp; c += blockDim.x) {
+        for (int c = threadIdx.x; c < sp; c += kThreads) {
             T u = __ldcg(&a.uvec[c]);
             sy[c] += ain * sd[c];
             T rv = sres[c] - ain * u;
             sres[c] = rv;
             loc += (double)rv * (double)rv;
         }
-        rres = block_sum(loc, red);
+        rres = block_sum0(loc, 32 * w < sp, red_c);
+        if (threadIdx.x == 0) s_val[0] = rres;
+        __syncthreads();
+        rres = s_val[0];
         ++k;
         if (rres <= tin2) break;
         double rz_new = 0.0;
         if (!precond(&rz_new)) return;
         const T beta = (T)(rz_new / rz_in);
         rz_in = rz_new;
-        for (int64_t c = threadIdx.x; c < sp; c += blockDim.x) sd[c] = __ldcg(&a.zvec[c]) + beta * sd[c];
+        for (int c = threadIdx.x; c < sp; c += kThreads) sd[c] = __ldcg(&a.zvec[c]) + beta * sd[c];
         __syncthreads();
     }
 
-    // ---- w = (r - C y) / lam~ into z; dots for the level-1 beta
+    // ---- w = (r - C y) / lam~ into z; dots r.w and r.z_old for the level-1 beta
     __syncthreads();
     double rw = 0.0, rzo = 0.0;
-    if constexpr (PL <= 32 && (sizeof(T) == 4 || PL <= 16)) row_pass_w<T, TC, PL>(a, row0, row1, sy, srow, &rw, &rzo);
-    else row_pass<T, TC, PL>(a, 2, row0, row1, sy, swarp, srow, &rw, &rzo);
-    block_sum2(rw, rzo, red64);
-    if (threadIdx.x == 0) {
-        a.dpart[b * 4 + 0] = rw;
-        a.dpart[b * 4 + 1] = rzo;
+    for (int cb = 0; cb < rows.nr; cb += kRowChunk) {
+        const int ce = min(rows.nr, cb + kRowChunk);
+        if (!have_r) load_r(cb, ce);
+        T zo = T(0);
+        const int e = cb + (int)threadIdx.x;      // kRowChunk = kThreads: a row per thread
+        if (a.mode == MODE_ITER && e < ce) zo = a.z[row0 + e];
+        dots_pass<T, TC, PL>(rows, cb, ce, sy, sw);
+        __syncthreads();
+        if (e < ce) {
+            const T ri = srow[e - cb], wi = (ri - sw[e - cb]) / a.lam_t;
+            a.z[row0 + e] = wi;
+            if (a.mode != MODE_APPLY) {
+                rw += (double)ri * (double)wi;
+                rzo += (double)ri * (double)zo;
+            }
+        }
+        if (ce < rows.nr) __syncthreads();
     }
     if (a.mode == MODE_APPLY) {
         if (b == 0 && threadIdx.x == 0) atomicAdd(&ctl->inner_iters, k);
         return;
     }
-    if (!msp::grid_barrier(bw, err)) return;
-    // this thread's first row of z and p, in flight with the dot partials
-    const int64_t i_first = row0 + threadIdx.x;
-    T z_first = T(0), p_first = T(0);
-    if (i_first < row1) {
-        z_first = a.z[i_first];
-        p_first = a.p[i_first];
+    {
+        // rw by the warps that have rows, finished by warp 0; rzo by warp 1
+        if (32 * w < rows.nr) {
+            rw = msp::warp_sum(rw);
+            if (a.mode == MODE_ITER) rzo = msp::warp_sum(rzo);
+        }
+        if (lane == 0) {
+            red_b[w] = rw;
+            red_c[w] = rzo;
+        }
+        __syncthreads();
+        if (w < 2) {
+            const double t = msp::warp_sum(lane < kNW ? (w == 0 ? red_b[lane] : red_c[lane]) : 0.0);
+            if (lane == 0) a.dpart[b * 4 + w] = t;
+        }
     }
-    sum_parts2(a.dpart + 0, 4, G, red64, rw, rzo);
-    T beta = T(0);
-    if (a.mode == MODE_ITER) beta = (T)((rw - rzo) / rz_outer);
-    for (int64_t i = i_first; i < row1; i += blockDim.x) {
-        const T zi = (i == i_first) ? z_first : a.z[i];
-        const T pi = (i == i_first) ? p_first : a.p[i];
-        a.p[i] = zi + beta * (a.mode == MODE_ITER ? pi : T(0));
+    // packed A pass: the next launch (the A pass) is the barrier; it sums the
+    // partials, checks r^T w and forms beta and the new direction
+    if (!packed) {
+        if (!msp::grid_barrier(bw, err)) return;
+        if (w < 2) {
+            const double t = warp_sum_parts(a.dpart + w, 4, G);
+            if (lane == 0) s_val[w] = t;
+        }
+        __syncthreads();
+        rw = s_val[0];
+        rzo = s_val[1];
+        T beta = T(0);
+        if (a.mode == MODE_ITER) beta = (T)((rw - rzo) / c_rz);
+        for (int64_t i = row0 + threadIdx.x; i < row1; i += kThreads)
+            a.p[i] = a.z[i] + beta * (a.mode == MODE_ITER ? a.p[i] : T(0));
+        if (b == 0 && threadIdx.x == 0) {
+            ctl->rz = rw;
+            ctl->beta = (double)beta;
+            if (!(rw > 0.0) && isfinite(rw)) ctl->error = MSP_ENOTPD;
+            if (!isfinite(rw)) ctl->error = MSP_ENONFINITE;
+        }
     }
     if (b == 0 && threadIdx.x == 0) {
-        ctl->rz = rw;
-        ctl->beta = (double)beta;
         ctl->rr = rr;
         ctl->inner_iters += k;
-        if (a.mode == MODE_ITER) ctl->iters += 1;
+        if (a.mode == MODE_ITER) ctl->iters = iter + 1;
         if (a.mode == MODE_INIT) { ctl->bb = rr; ctl->tol2 = a.tol_rel2 * rr; }
-        if (!(rw > 0.0) && isfinite(rw)) ctl->error = MSP_ENOTPD;
-        if (!isfinite(rw)) ctl->error = MSP_ENONFINITE;
     }
-    (void)s_rw;
-    (void)s_rzo;
 }
 
 template <typename T, typename TC, int PL>
 msp_status launch_level2_pl(msp_ctx* ctx, L2Args<T, TC>& a, int G) {
+    using S = L2Shape<T, TC, PL>;
     auto kern = k_level2<T, TC, PL>;
-    size_t smem = ((size_t)(4 + kNW) * a.s_pad + 2 * kRowChunk) * sizeof(T);
+    // rows of C kept in shared memory: what the block's rows need, or what is
+    // left beside the vectors (4 KB aside for the kernel's static part)
+    const size_t left = ctx->smem_optin - 4096 - S::fixed;
+    const int64_t most = (a.n + G - 1) / G;
+    const int64_t fit = (int64_t)(left / S::row);
+    a.res_rows = (int)(fit >= most ? most : fit / kNW * kNW);
+    const size_t smem = S::fixed + (size_t)a.res_rows * S::row;
     MSP_CUDA_TRY(ctx, cudaFuncSetAttribute(kern, cudaFuncAttributeMaxDynamicSharedMemorySize,
                                            (int)smem));
     // co-residency is required by the grid barrier: never exceed what fits
@@ -891,7 +1059,6 @@ msp_status launch_level2_pl(msp_ctx* ctx, L2Args<T, TC>& a, int G) {
     MSP_CUDA_TRY(ctx, cudaOccupancyMaxActiveBlocksPerMultiprocessor(&per_sm, kern, kThreads, smem));
     if (per_sm < 1)
         return msp_set_error(ctx, MSP_EINVAL, "level-2 kernel does not fit on an SM");
-    G = std::min(G, per_sm * ctx->num_sms);
     void* args[] = {&a};
     ++ctx->launches;
     MSP_CUDA_TRY(ctx, cudaLaunchCooperativeKernel((const void*)kern, dim3(G), dim3(kThreads), args,
@@ -928,7 +1095,7 @@ struct Workspace {
     void* part;
     void* vecs;
     double* dpart;
-    void* level1;   // x r q p z (n_pad each)
+    void* level1;   // x r q p p' z (n_pad each)
     double* gpart;  // A-pass partials
     float* qpart;   // packed A pass: nt x n_pad slot partials (or null)
     int64_t n_pad;
@@ -943,7 +1110,7 @@ msp_status get_workspace(msp_ctx* ctx, int64_t n, int64_t sp, int G, int Gg, boo
     size_t b_part = round_up((int64_t)G * sp * ts, 256);
     size_t b_vecs = round_up(5 * sp * ts, 256);
     size_t b_dpart = round_up((int64_t)G * 4 * 8, 256);
-    size_t b_l1 = round_up(5 * n_pad * ts, 256);
+    size_t b_l1 = round_up(6 * n_pad * ts, 256);
     size_t b_gp = round_up((int64_t)Gg * 8, 256);
     size_t b_qp = packed ? round_up(nt * n_pad * 4, 256) : 0;
     void* scr = nullptr;
@@ -981,10 +1148,9 @@ void fill_l2(L2Args<T, TC>& a, const msp_factor_s* f, int64_t n, const Workspace
     a.dpart = ws.dpart;
 }
 
-// Upper bound on the level-2 grid (2 blocks per SM); launch_level2_pl lowers
-// it to what the occupancy calculator guarantees co-resident. The workspace is
-// sized for the upper bound.
-int level2_grid(msp_ctx* ctx) { return 2 * ctx->num_sms; }
+// The level-2 grid: one block per SM (a thread per block partial in the
+// column sums, so at most kThreads).
+int level2_grid(msp_ctx* ctx) { return std::min(ctx->num_sms, kThreads); }
 int gemv_grid(msp_ctx* ctx) { return ctx->num_sms * 8; }
 
 // ------------------------------------------------ level-1 graph replay
@@ -1127,11 +1293,11 @@ msp_status krylov_solve_t(msp_ctx* ctx, const msp_factor_s* f, const void* A, ms
     T* r = x + np;
     T* q = r + np;
     T* p = q + np;
-    T* z = p + np;
+    T* z = p + 2 * np;      // p: two buffers (the packed A pass writes them in turn)
     CtlBlock* ctl = (CtlBlock*)ctx->ctl;
     MSP_CUDA_TRY(ctx, cudaMemsetAsync(ctl, 0, sizeof(CtlBlock), ctx->stream));
-    // all five level-1 vectors, pads included (p must be zero past n)
-    MSP_CUDA_TRY(ctx, cudaMemsetAsync(x, 0, 5 * np * sizeof(T), ctx->stream));
+    // all the level-1 vectors, pads included (p and z must be zero past n)
+    MSP_CUDA_TRY(ctx, cudaMemsetAsync(x, 0, 6 * np * sizeof(T), ctx->stream));
     MSP_CUDA_TRY(ctx, cudaMemcpyAsync(r, rhs, n * sizeof(T), cudaMemcpyDeviceToDevice, ctx->stream));
 
     // zeroed bytes (padding included): the struct is part of the graph key
@@ -1145,6 +1311,9 @@ msp_status krylov_solve_t(msp_ctx* ctx, const msp_factor_s* f, const void* A, ms
     a.qpart = use_packed ? ws.qpart : nullptr;
     a.q_slots = (int)(np / 128);
     a.q_ld = np;
+    a.p_ld = np;
+    a.dq = use_packed ? ws.gpart : nullptr;
+    a.n_dq = ctx->num_sms;
     a.lam = (T)lambda;
     a.mode = MODE_INIT;
     MSP_TRY(launch_level2(ctx, a, G));
@@ -1168,7 +1337,7 @@ msp_status krylov_solve_t(msp_ctx* ctx, const msp_factor_s* f, const void* A, ms
     auto iteration = [&](bool cap) -> msp_status {
         MSP_TRY(mark(cap, 0));
         if (use_packed) {
-            MSP_TRY(msp_symv_packed(ctx, packed, n, (float)lambda, (const float*)p, ws.qpart,
+            MSP_TRY(msp_symv_packed(ctx, packed, n, (float)lambda, (const float*)z, (float*)p, ws.dpart, G, ws.qpart,
                                     ws.gpart, ctx->num_sms));
         } else {
             if (dt == MSP_F32) {
@@ -1237,6 +1406,12 @@ msp_status krylov_solve_t(msp_ctx* ctx, const msp_factor_s* f, const void* A, ms
         MSP_CUDA_TRY(ctx, cudaStreamSynchronize(ctx->stream));
         if (hf[0] || hf[1]) break;
         settled = pr.used;
+        // the packed A pass finds an indefinite or non-finite r^T w of the
+        // iteration before it: after the last allowed iteration one more pass
+        // looks at that one's
+        if (it >= max_outer && use_packed)
+            MSP_TRY(msp_symv_packed(ctx, packed, n, (float)lambda, (const float*)z, (float*)p, ws.dpart, G, ws.qpart,
+                                    ws.gpart, ctx->num_sms));
     }
     MSP_CUDA_TRY(ctx, cudaMemcpyAsync(hf, &ctl->done, 5 * sizeof(int), cudaMemcpyDeviceToHost,
                                       ctx->stream));

@@ -138,7 +138,8 @@ struct CtlBlock {
     double tol2;        // tol^2 |rhs|^2
     double pq;
     double beta;
-    double scratch[8];
+    double rzbuf[2];    // packed A pass: r^T z of the iterations, in turn
+    double scratch[6];
 };
 
 // ------------------------------------------------------------------ errors
@@ -368,8 +369,11 @@ msp_status msp_pack_upper_rows(msp_ctx* ctx, const float* A, int64_t lda, int64_
 // fill the strictly lower 128-tiles of tile rows [I0, I1) from the upper ones
 msp_status msp_mirror_lower_rows(msp_ctx* ctx, float* A, int64_t lda, int64_t n, int64_t I0, int64_t I1);
 msp_status msp_mirror_lower_cols(msp_ctx* ctx, float* A, int64_t lda, int64_t n, int64_t J0, int64_t J1);
-msp_status msp_symv_packed(msp_ctx* ctx, const float* packed, int64_t n, float lam, const float* p,
-                           float* part, double* dpart, int grid);
+// the level-1 direction and the A pass over it: p = z + beta p into the buffer
+// of p (two of n_pad) that ctl->iters selects, beta from the n_l2 block records
+// (r^T z, r^T z_old, 4 doubles apart) of the level-2 launch before it
+msp_status msp_symv_packed(msp_ctx* ctx, const float* packed, int64_t n, float lam, const float* z, float* p,
+                           const double* l2part, int n_l2, float* part, double* dpart, int grid);
 
 // krylov.cu
 msp_status msp_grid_wait_limit_krylov(msp_ctx* ctx, unsigned long long ns);

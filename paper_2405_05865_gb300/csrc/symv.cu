@@ -15,7 +15,12 @@
 // each (slot, segment) written exactly once, so q_i = sum_slot part[slot][i]
 // + lam p_i is formed deterministically by the consumer of q. The block
 // partials of p^T (A + lam I) p = sum_tiles (2 - [I==J]) p_I^T A_IJ p_J +
-// lam |p|^2 are combined by the last block, which writes alpha = rz / pq.
+// lam |p|^2 are summed by the consumer, which forms alpha = rz / pq.
+// The direction is formed here too: p = z + beta p_old, beta from the level-2
+// launch's block records, in registers from the staged segments of z and p_old
+// (the tile copies do not wait for beta); the blocks of the diagonal tiles
+// store it. That takes a grid barrier and a pass over the vectors (about 6 us at
+// n = 16384) off the level-2 kernel's end.
 // Every wait on an mbarrier is bounded in wall-clock time (MSP_ETIMEOUT).
 #include "msp_internal.cuh"
 
@@ -29,8 +34,9 @@ constexpr int kConsumerWarps = 8;
 constexpr int kSymvThreads = (kConsumerWarps + 1) * 32;
 constexpr int kTileBytes = kTile * kTile * 4;
 constexpr int kChunk = 16384;                 // bytes per bulk copy (4 per tile)
-// a stage holds the tile and the two 128-float segments p_I and p_J
-constexpr int kStageBytes = kTileBytes + 2 * kTile * 4;
+// a stage holds the tile and the 128-float segments z_I, z_J, p_I, p_J (of the
+// old p)
+constexpr int kStageBytes = kTileBytes + 4 * kTile * 4;
 constexpr size_t kSymvSmem =
     (size_t)kStages * kStageBytes + (size_t)kStages * kConsumerWarps * kTile * 4 + 1024;
 
@@ -165,7 +171,10 @@ struct SymvArgs {
     int64_t n;
     int64_t n_pad;          // nt * 128 (length of p, segment space of part)
     float lam;
-    const float* p;         // n_pad, zero past n
+    const float* z;         // n_pad, zero past n
+    float* p;               // two buffers of n_pad, zero past n
+    const double* l2part;   // n_l2 records of 4: r^T z, r^T z_old
+    int n_l2;
     float* part;            // nt x n_pad
     double* dpart;          // gridDim.x
     CtlBlock* ctl;
@@ -174,14 +183,16 @@ struct SymvArgs {
 __global__ void __launch_bounds__(kSymvThreads, 1) k_symv_packed(SymvArgs a) {
     CtlBlock* ctl = a.ctl;
     if (ctl->done | ctl->error) return;
+    const int iter = ctl->iters;
+    const float* p_old = a.p + ((iter & 1) ^ 1) * a.n_pad;
+    float* p_new = a.p + (iter & 1) * a.n_pad;
     extern __shared__ __align__(1024) unsigned char smem_raw[];
     unsigned char* ring = smem_raw;                                        // kStages stages
     float* colred = reinterpret_cast<float*>(smem_raw + (size_t)kStages * kStageBytes);
     uint64_t* full = reinterpret_cast<uint64_t*>(colred + (size_t)kStages * kConsumerWarps * kTile);
     uint64_t* empty = full + kStages;
-    __shared__ double red[32];
-    __shared__ bool am_last;
-    __shared__ int s_abort;
+    __shared__ double red[kConsumerWarps];
+    __shared__ float s_beta;
     __shared__ int col_count[kStages];
 
     const int warp = threadIdx.x >> 5, lane = threadIdx.x & 31;
@@ -192,7 +203,6 @@ __global__ void __launch_bounds__(kSymvThreads, 1) k_symv_packed(SymvArgs a) {
             col_count[s] = 0;
         }
         asm volatile("fence.mbarrier_init.release.cluster;" ::: "memory");
-        s_abort = 0;
     }
     __syncthreads();
 
@@ -211,7 +221,7 @@ __global__ void __launch_bounds__(kSymvThreads, 1) k_symv_packed(SymvArgs a) {
                 const uint32_t ph = (uint32_t)((k / kStages) & 1);
                 if (k >= kStages) {
                     // wait until the consumers released this stage (use k - kStages)
-                    if (!mbar_wait(&empty[s], ph ^ 1u, &ctl->error)) { s_abort = 1; break; }
+                    if (!mbar_wait(&empty[s], ph ^ 1u, &ctl->error)) break;
                 }
                 const int t = (int)blockIdx.x + k * G;
                 int I, J;
@@ -222,8 +232,11 @@ __global__ void __launch_bounds__(kSymvThreads, 1) k_symv_packed(SymvArgs a) {
 #pragma unroll
                 for (int c = 0; c < kTileBytes / kChunk; ++c)
                     bulk_g2s_hint(dst + c * kChunk, src + c * kChunk, kChunk, &full[s], pol);
-                bulk_g2s(dst + kTileBytes, a.p + (int64_t)I * kTile, kTile * 4, &full[s]);
-                bulk_g2s(dst + kTileBytes + kTile * 4, a.p + (int64_t)J * kTile, kTile * 4, &full[s]);
+                constexpr int kSeg = kTile * 4;
+                bulk_g2s(dst + kTileBytes, a.z + (int64_t)I * kTile, kSeg, &full[s]);
+                bulk_g2s(dst + kTileBytes + kSeg, a.z + (int64_t)J * kTile, kSeg, &full[s]);
+                bulk_g2s(dst + kTileBytes + 2 * kSeg, p_old + (int64_t)I * kTile, kSeg, &full[s]);
+                bulk_g2s(dst + kTileBytes + 3 * kSeg, p_old + (int64_t)J * kTile, kSeg, &full[s]);
                 issued = k + 1;
             }
             // drain: every issued copy must have landed before the block exits
@@ -235,17 +248,55 @@ __global__ void __launch_bounds__(kSymvThreads, 1) k_symv_packed(SymvArgs a) {
         }
     } else {
         // ---------------- consumers
-        const int ct = threadIdx.x;                 // 0..255
+        // beta = (r^T z - r^T z_old) / (r^T z of the iteration before), 0 at the
+        // first one: warp 0, while the first tiles are on their way. An r^T z that
+        // is not positive ends the iteration (the pass runs to its end, and what
+        // follows it returns at once).
+        if (warp == 0) {
+            double rw = 0.0, rzo = 0.0;
+            for (int b = lane; b < a.n_l2; b += 32) {
+                rw += __ldcg(&a.l2part[4 * b]);
+                rzo += __ldcg(&a.l2part[4 * b + 1]);
+            }
+            rw = msp::warp_sum(rw);
+            rzo = msp::warp_sum(rzo);
+            if (lane == 0) {
+                s_beta = iter == 0 ? 0.f : (float)((rw - rzo) / ctl->rzbuf[(iter & 1) ^ 1]);
+                if (blockIdx.x == 0) {
+                    ctl->rzbuf[iter & 1] = rw;
+                    if (!isfinite(rw)) ctl->error = MSP_ENONFINITE;
+                    else if (!(rw > 0.0)) ctl->error = MSP_ENOTPD;
+                }
+            }
+        }
+        asm volatile("bar.sync 1, %0;" ::"n"(kConsumerWarps * 32) : "memory");
+        const float beta = s_beta;
         for (int k = 0; k < my_tiles; ++k) {
             const int s = k % kStages;
             const uint32_t ph = (uint32_t)((k / kStages) & 1);
-            if (!mbar_wait(&full[s], ph, &ctl->error)) { s_abort = 1; break; }
+            if (!mbar_wait(&full[s], ph, &ctl->error)) break;
             const int t = (int)blockIdx.x + k * G;
             int I, J;
             tile_coords(t, a.nt, I, J);
             const float* tb = reinterpret_cast<const float*>(ring + (size_t)s * kStageBytes);
-            const float* pI = tb + kTile * kTile;            // p_I staged with the tile
-            const float4 pj = reinterpret_cast<const float4*>(pI + kTile)[lane];
+            const float* zI = tb + kTile * kTile;            // z_I, z_J, p_I, p_J staged with the tile
+            const float* oI = zI + 2 * kTile;
+            float4 pj = reinterpret_cast<const float4*>(zI + kTile)[lane];
+            {
+                const float4 oj = reinterpret_cast<const float4*>(oI + kTile)[lane];
+                pj.x = fmaf(beta, oj.x, pj.x);
+                pj.y = fmaf(beta, oj.y, pj.y);
+                pj.z = fmaf(beta, oj.z, pj.z);
+                pj.w = fmaf(beta, oj.w, pj.w);
+            }
+            if (I == J && warp == 0) {
+                reinterpret_cast<float4*>(p_new + (int64_t)I * kTile)[lane] = pj;
+                // lam |p_I|^2
+                const double pp = ((double)pj.x * (double)pj.x + (double)pj.y * (double)pj.y) +
+                                  ((double)pj.z * (double)pj.z + (double)pj.w * (double)pj.w);
+                const double t = msp::warp_sum(pp);
+                if (lane == 0) acc_dot += (double)a.lam * t;
+            }
             float rv[16];
             float c0 = 0.f, c1 = 0.f, c2 = 0.f, c3 = 0.f;
 #pragma unroll
@@ -253,7 +304,7 @@ __global__ void __launch_bounds__(kSymvThreads, 1) k_symv_packed(SymvArgs a) {
                 const int r = warp + kConsumerWarps * kk;
                 const float4 v = reinterpret_cast<const float4*>(tb + r * kTile)[lane];
                 rv[kk] = v.x * pj.x + v.y * pj.y + v.z * pj.z + v.w * pj.w;
-                const float pr = pI[r];
+                const float pr = fmaf(beta, oI[r], zI[r]);
                 c0 += v.x * pr;
                 c1 += v.y * pr;
                 c2 += v.z * pr;
@@ -321,7 +372,7 @@ __global__ void __launch_bounds__(kSymvThreads, 1) k_symv_packed(SymvArgs a) {
             if ((lane & 1) == 0) {
                 const int r = warp + kConsumerWarps * (lane >> 1);
                 a.part[(int64_t)J * a.n_pad + (int64_t)I * kTile + r] = rv[0];
-                tdot = pI[r] * rv[0];
+                tdot = fmaf(beta, oI[r], zI[r]) * rv[0];
             }
             // this warp's 16 rows of p_I^T A_IJ p_J: FP32 within the tile, one
             // FP64 add per warp and tile
@@ -331,47 +382,14 @@ __global__ void __launch_bounds__(kSymvThreads, 1) k_symv_packed(SymvArgs a) {
             __syncwarp();
             if (lane == 0) mbar_arrive(&empty[s]);
         }
-        // lam |p|^2 over a slice of p
-        const int64_t i0 = a.n * blockIdx.x / G, i1 = a.n * (blockIdx.x + 1) / G;
-        for (int64_t i = i0 + ct; i < i1; i += kConsumerWarps * 32) {
-            const double pv = (double)a.p[i];
-            acc_dot += (double)a.lam * pv * pv;
+        // block partial of p^T (A + lam I) p (lane 0 of each warp holds its sum)
+        if (lane == 0) red[warp] = acc_dot;
+        asm volatile("bar.sync 1, %0;" ::"n"(kConsumerWarps * 32) : "memory");
+        if (threadIdx.x == 0) {
+            double tot = 0.0;
+            for (int w = 0; w < kConsumerWarps; ++w) tot += red[w];
+            a.dpart[blockIdx.x] = tot;
         }
-    }
-    // block partial of p^T (A + lam I) p, then the last block forms alpha
-    double v = msp::warp_sum(acc_dot);
-    __syncthreads();
-    if (lane == 0) red[warp] = v;
-    __syncthreads();
-    if (threadIdx.x == 0) {
-        double tot = 0.0;
-        for (int w = 0; w < kConsumerWarps + 1; ++w) tot += red[w];
-        a.dpart[blockIdx.x] = tot;
-        __threadfence();
-        unsigned int tk = atomicAdd(&ctl->last_block_counter, 1u);
-        am_last = (tk == gridDim.x - 1);
-    }
-    __syncthreads();
-    if (!am_last) return;
-    __threadfence();
-    // the G block partials with all loads in flight together (not one
-    // thread's chain of L2 round trips): strided per thread, then the warp
-    // tree and the warps in order (a fixed order)
-    double all = 0.0;
-    for (int b = threadIdx.x; b < G; b += blockDim.x) all += __ldcg(&a.dpart[b]);
-    all = msp::warp_sum(all);
-    __syncthreads();
-    if (lane == 0) red[warp] = all;
-    __syncthreads();
-    if (threadIdx.x == 0) {
-        all = 0.0;
-        for (int w = 0; w < kConsumerWarps + 1; ++w) all += red[w];
-        ctl->last_block_counter = 0;
-        ctl->pq = all;
-        if (s_abort) { /* error already recorded */ }
-        else if (!isfinite(all)) ctl->error = MSP_ENONFINITE;
-        else if (!(all > 0.0)) ctl->error = MSP_ENOTPD;
-        else ctl->alpha = ctl->rz / all;
     }
 }
 
@@ -452,8 +470,8 @@ msp_status msp_pack_upper_rows(msp_ctx* ctx, const float* A, int64_t lda, int64_
     return MSP_OK;
 }
 
-msp_status msp_symv_packed(msp_ctx* ctx, const float* packed, int64_t n, float lam, const float* p,
-                           float* part, double* dpart, int grid) {
+msp_status msp_symv_packed(msp_ctx* ctx, const float* packed, int64_t n, float lam, const float* z, float* p,
+                           const double* l2part, int n_l2, float* part, double* dpart, int grid) {
     // the attribute belongs to a device: set once per device (bit of a mask)
     static std::atomic<uint64_t> attr_set{0};
     const uint64_t bit = 1ull << (ctx->device & 63);
@@ -470,7 +488,10 @@ msp_status msp_symv_packed(msp_ctx* ctx, const float* packed, int64_t n, float l
     a.n = n;
     a.n_pad = (int64_t)a.nt * kTile;
     a.lam = lam;
+    a.z = z;
     a.p = p;
+    a.l2part = l2part;
+    a.n_l2 = n_l2;
     a.part = part;
     a.dpart = dpart;
     a.ctl = (CtlBlock*)ctx->ctl;

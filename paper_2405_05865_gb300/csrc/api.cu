@@ -498,7 +498,7 @@ msp_status msp_sketch_get_C(msp_ctx* ctx, const msp_sketch_t* sk, void* C, int64
 
 void msp_factor_destroy(msp_factor_t* f) {
     if (!f) return;
-    for (void* p : {f->W, f->B, f->Bt, (void*)f->W64, (void*)f->M2, (void*)f->Linv64, f->Cb, f->Wb})
+    for (void* p : {f->W, f->B, f->Bt, (void*)f->W64, (void*)f->M2, (void*)f->Linv64, f->Cb, f->Wb, f->H})
         if (p) cudaFreeAsync(p, f->stream);
     delete f;
 }
@@ -599,6 +599,11 @@ msp_status msp_nystrom_impl(msp_ctx* ctx, const msp_sketch_s* sk, double lambda,
         phi_rows = phi;
     }
     if ((st = msp_build_factor(ctx, f, Ct, phi_rows)) != MSP_OK) return fail(st);
+    // a sketched level 2 iterates on C^T C + lam~ W: formed once where the whole
+    // iteration then runs on one cluster
+    if (phi > 0 && f->data == MSP_F32 && msp_inner_ok(ctx, f->dtype, sp) &&
+        (st = msp_form_level2(ctx, f, Csrc, n)) != MSP_OK)
+        return fail(st);
     if (f->data == MSP_BF16) {
         // Wb = bf16 of the symmetrised W (for the iterative level 2)
         k_round_bf16<<<(unsigned)((sp * sp + 255) / 256), 256, 0, ctx->stream>>>((const float*)f->W, sp * sp,

@@ -18,6 +18,7 @@
 #include "bulk.cuh"
 #include "msp_internal.cuh"
 
+#include <cooperative_groups.h>
 #include <cuda_bf16.h>
 
 #include <algorithm>
@@ -32,6 +33,7 @@ constexpr int kRowChunk = kThreads;          // rows of C whose r, w are staged 
 constexpr int kQScratch = 4 * kNW * 32;      // slot sums of the level-1 update
 
 enum { MODE_INIT = 0, MODE_ITER = 1, MODE_APPLY = 2 };
+enum { PHASE_ALL = 0, PHASE_FRONT = 1, PHASE_BACK = 2 };
 
 template <typename T> struct Vec16;
 template <> struct Vec16<float> { using type = float4; static constexpr int W = 4; };
@@ -299,6 +301,7 @@ template <typename T, typename TC = T>
 struct L2Args {
     int64_t n, s_pad;
     int mode;
+    int phase;              // PHASE_ALL, or the part before / after a k_inner launch
     int res_rows;           // rows of C a block keeps in shared memory
     const TC* C;
     const TC* W;
@@ -704,7 +707,8 @@ __global__ void __launch_bounds__(kThreads, 1) k_level2(L2Args<T, TC> a) {
     const T* p = a.p;
     bool have_r = false;      // srow holds r of all the block's rows
     double rr = 0.0;
-    if (a.mode == MODE_ITER && packed) {
+    if (a.phase == PHASE_BACK) {
+    } else if (a.mode == MODE_ITER && packed) {
         // q_i = sum over the packed A pass's slot partials + lam p_i, fixed
         // summation order. Rounds of four 32-row groups: every warp sums its
         // slots for the four rows of a lane, the loads in flight together
@@ -803,7 +807,7 @@ __global__ void __launch_bounds__(kThreads, 1) k_level2(L2Args<T, TC> a) {
         }
         rr = block_sum0(rr, 32 * w < rows.nr, red);
     }
-    if (threadIdx.x == 0) a.dpart[b * 4 + 0] = rr;
+    if (threadIdx.x == 0 && a.phase != PHASE_BACK) a.dpart[b * 4 + 0] = rr;
 
     // the block's rows of r (a chunk) in srow
     auto load_r = [&](int cb, int ce) {
@@ -816,158 +820,168 @@ __global__ void __launch_bounds__(kThreads, 1) k_level2(L2Args<T, TC> a) {
 #pragma unroll
     for (int k = 0; k < S::KU; ++k) acc[k][0] = acc[k][1] = T(0);
     if (!msp::mbar_wait_timed(bar, 0, err)) s_bad = MSP_ETIMEOUT;
-    for (int cb = 0; cb < rows.nr; cb += kRowChunk) {
-        const int ce = min(rows.nr, cb + kRowChunk);
-        if (!have_r) load_r(cb, ce);
-        cols_pass<T, TC, PL>(rows, cb, ce, srow, acc);
-        if (ce < rows.nr) __syncthreads();
-    }
-    have_r = rows.nr <= kRowChunk;   // srow is not written again below
-    cols_store<T, TC, PL>(acc, scr, a.part + (int64_t)b * sp);
-    // the block's rows of B and B^T on their way to registers during the barriers
-    const bool one_row = c1 - c0 <= kNW;
-    const bool my_row = one_row && c0 + w < c1;
-    RowSlice<T, PL> mB;
-    if (my_row) mB.load(a.B + (c0 + w) * sp, lane);
-    if (!msp::grid_barrier(bw, err) || s_bad) return;
-
-    // ---- g reduced over this block's columns, |r|^2 (the convergence test) by
-    // the last warp beside it; |g|^2 only where the level-2 iteration's tolerance needs it
-    const bool inner = a.max_inner > 0;
-    if (a.mode != MODE_APPLY && w == kNW - 1) {
-        const double t = warp_sum_parts(a.dpart, 4, G);
-        if (lane == 0) s_rr = t;
-    }
-    double gg = reduce_cols<T>(a.part, G, sp, nullptr, T(0), a.gvec, nullptr, inner, redc);
-    if (a.mode != MODE_APPLY) {
-        rr = s_rr;
-        bool stop = !isfinite(rr);
-        double t2 = tol2;
-        if (a.mode == MODE_INIT) t2 = a.tol_rel2 * rr;
-        if (stop) {
-            if (b == 0 && threadIdx.x == 0) ctl->error = MSP_ENONFINITE;
-            return;
-        }
-        if (rr <= t2) {
-            if (b == 0 && threadIdx.x == 0) {
-                ctl->rr = rr;
-                if (a.mode == MODE_INIT) { ctl->bb = rr; ctl->tol2 = t2; }
-                if (a.mode == MODE_ITER) ctl->iters = iter + 1;
-                ctl->done = 1;
-            }
-            return;
-        }
-    }
-    if (inner && threadIdx.x == 0) a.dpart[b * 4 + 1] = gg;
-    if (!msp::grid_barrier(bw, err)) return;
-    if (inner) gg = grid_sum(a.dpart + 1, G, &s_val[0]);
-    load_full(a.gvec, sres, sp);
-    if (inner)
-        for (int c = threadIdx.x; c < sp; c += kThreads) sy[c] = T(0);
-    __syncthreads();
-
-    // ---- z = M2^{-1} res = B^T (B res); z^T res only where the level-2
-    // iteration uses it (rz_out given; the same in every block)
-    int turn = 1;
-    bool fresh = my_row;      // mB holds the block's row of B
-    auto precond = [&](double* rz_out) -> bool {
-        RowSlice<T, PL> mT;
-        if (my_row) {
-            if (!fresh) mB.load(a.B + (c0 + w) * sp, lane);
-            fresh = false;
-            const T t = msp::warp_sum(mB.dot_smem(sres, lane));
-            if (lane == 0) a.tvec[c0 + w] = t;
-            mT.load(a.Bt + (c0 + w) * sp, lane);
-        } else if (!one_row) {
-            rows_dot<T, PL>(a.B, sp, c0, c1, sres, a.tvec);
-        }
-        if (!msp::grid_barrier(bw, err)) return false;
-        load_full(a.tvec, stmp, sp);
-        __syncthreads();
-        double part = 0.0;
-        if (my_row) {
-            const T z = msp::warp_sum(mT.dot_smem(stmp, lane));
-            if (lane == 0) {
-                a.zvec[c0 + w] = z;
-                if (rz_out) part = (double)sres[c0 + w] * (double)z;
-            }
-        } else if (!one_row) {
-            rows_dot<T, PL>(a.Bt, sp, c0, c1, stmp, a.zvec);
-            __syncthreads();
-            if (rz_out)
-                for (int64_t c = c0 + threadIdx.x; c < c1; c += kThreads) part += (double)sres[c] * (double)a.zvec[c];
-        }
-        if (rz_out) {
-            // my_row: lane 0 of each warp holds a product
-            if (one_row) {
-                if (lane == 0) red_b[w] = part;
-                __syncthreads();
-                part = w == 0 ? msp::warp_sum(lane < kNW ? red_b[lane] : 0.0) : 0.0;
-            } else {
-                part = block_sum0(part, true, red_b);
-            }
-            if (threadIdx.x == 0) a.dpart[b * 4 + 2] = part;
-        }
-        if (!msp::grid_barrier(bw, err)) return false;
-        if (rz_out) {
-            *rz_out = grid_sum(a.dpart + 2, G, &s_val[turn]);
-            turn = 3 - turn;
-        }
-        return true;
-    };
-
-    // direct level 2 (max_inner == 0) has no level-2 iteration: z^T res unused
-    double rz_in = 0.0;
-    if (!precond(inner ? &rz_in : nullptr)) return;
-    // direct level 2: M2 is the level-2 operator itself (Phi = I), so
-    // y = M2^{-1} C^T r with no correction steps
-    load_full(a.zvec, inner ? sd : sy, sp);
-    __syncthreads();
-    double rres = gg;
-    const double tin2 = a.inner_tol2 * gg;
-    int k = 0;
-    while (k < a.max_inner && rres > tin2) {
-        // P1: partial u = C^T (C d) over this block's rows; wd = W d (columns)
-#pragma unroll
-        for (int q = 0; q < S::KU; ++q) acc[q][0] = acc[q][1] = T(0);
+    int k = 0;                // level-2 iterations
+    if (a.phase != PHASE_BACK) {
         for (int cb = 0; cb < rows.nr; cb += kRowChunk) {
             const int ce = min(rows.nr, cb + kRowChunk);
-            dots_pass<T, TC, PL>(rows, cb, ce, sd, sw);
-            __syncthreads();
-            cols_pass<T, TC, PL>(rows, cb, ce, sw, acc);
+            if (!have_r) load_r(cb, ce);
+            cols_pass<T, TC, PL>(rows, cb, ce, srow, acc);
             if (ce < rows.nr) __syncthreads();
         }
+        have_r = rows.nr <= kRowChunk;   // srow is not written again below
         cols_store<T, TC, PL>(acc, scr, a.part + (int64_t)b * sp);
-        rows_dot<T, PL, TC>(a.W, sp, c0, c1, sd, a.wdvec);
-        if (!msp::grid_barrier(bw, err)) return;
-        // P2: u over this block's columns; d.u partial
-        double du = reduce_cols<T>(a.part, G, sp, a.wdvec, a.lam_t, a.uvec, sd, false, redc);
-        if (threadIdx.x == 0) a.dpart[b * 4 + 3] = du;
-        if (!msp::grid_barrier(bw, err)) return;
-        // P3: step
-        du = grid_sum(a.dpart + 3, G, &s_val[3]);
-        if (!(du > 0.0)) break;   // breakdown (same decision in every block)
-        const T ain = (T)(rz_in / du);
-        double loc = 0.0;
-        for (int c = threadIdx.x; c < sp; c += kThreads) {
-            T u = __ldcg(&a.uvec[c]);
-            sy[c] += ain * sd[c];
-            T rv = sres[c] - ain * u;
-            sres[c] = rv;
-            loc += (double)rv * (double)rv;
+        // the block's rows of B and B^T on their way to registers during the barriers
+        const bool one_row = c1 - c0 <= kNW;
+        const bool my_row = one_row && c0 + w < c1 && a.phase == PHASE_ALL;
+        RowSlice<T, PL> mB;
+        if (my_row) mB.load(a.B + (c0 + w) * sp, lane);
+        if (!msp::grid_barrier(bw, err) || s_bad) return;
+
+        // ---- g reduced over this block's columns, |r|^2 (the convergence test) by
+        // the last warp beside it; |g|^2 only where the level-2 iteration's tolerance needs it
+        const bool inner = a.max_inner > 0 && a.phase == PHASE_ALL;
+        if (a.mode != MODE_APPLY && w == kNW - 1) {
+            const double t = warp_sum_parts(a.dpart, 4, G);
+            if (lane == 0) s_rr = t;
         }
-        rres = block_sum0(loc, 32 * w < sp, red_c);
-        if (threadIdx.x == 0) s_val[0] = rres;
+        double gg = reduce_cols<T>(a.part, G, sp, nullptr, T(0), a.gvec, nullptr, inner, redc);
+        if (a.mode != MODE_APPLY) {
+            rr = s_rr;
+            bool stop = !isfinite(rr);
+            double t2 = tol2;
+            if (a.mode == MODE_INIT) t2 = a.tol_rel2 * rr;
+            if (stop) {
+                if (b == 0 && threadIdx.x == 0) ctl->error = MSP_ENONFINITE;
+                return;
+            }
+            if (rr <= t2) {
+                if (b == 0 && threadIdx.x == 0) {
+                    ctl->rr = rr;
+                    if (a.mode == MODE_INIT) { ctl->bb = rr; ctl->tol2 = t2; }
+                    if (a.mode == MODE_ITER) ctl->iters = iter + 1;
+                    ctl->done = 1;
+                }
+                return;
+            }
+        }
+        if (a.mode != MODE_APPLY && b == 0 && threadIdx.x == 0) {
+            ctl->rr = rr;
+            if (a.mode == MODE_INIT) { ctl->bb = rr; ctl->tol2 = a.tol_rel2 * rr; }
+        }
+        if (a.phase == PHASE_FRONT) return;
+        if (inner && threadIdx.x == 0) a.dpart[b * 4 + 1] = gg;
+        if (!msp::grid_barrier(bw, err)) return;
+        if (inner) gg = grid_sum(a.dpart + 1, G, &s_val[0]);
+        load_full(a.gvec, sres, sp);
+        if (inner)
+            for (int c = threadIdx.x; c < sp; c += kThreads) sy[c] = T(0);
         __syncthreads();
-        rres = s_val[0];
-        ++k;
-        if (rres <= tin2) break;
-        double rz_new = 0.0;
-        if (!precond(&rz_new)) return;
-        const T beta = (T)(rz_new / rz_in);
-        rz_in = rz_new;
-        for (int c = threadIdx.x; c < sp; c += kThreads) sd[c] = __ldcg(&a.zvec[c]) + beta * sd[c];
+
+        // ---- z = M2^{-1} res = B^T (B res); z^T res only where the level-2
+        // iteration uses it (rz_out given; the same in every block)
+        int turn = 1;
+        bool fresh = my_row;      // mB holds the block's row of B
+        auto precond = [&](double* rz_out) -> bool {
+            RowSlice<T, PL> mT;
+            if (my_row) {
+                if (!fresh) mB.load(a.B + (c0 + w) * sp, lane);
+                fresh = false;
+                const T t = msp::warp_sum(mB.dot_smem(sres, lane));
+                if (lane == 0) a.tvec[c0 + w] = t;
+                mT.load(a.Bt + (c0 + w) * sp, lane);
+            } else if (!one_row) {
+                rows_dot<T, PL>(a.B, sp, c0, c1, sres, a.tvec);
+            }
+            if (!msp::grid_barrier(bw, err)) return false;
+            load_full(a.tvec, stmp, sp);
+            __syncthreads();
+            double part = 0.0;
+            if (my_row) {
+                const T z = msp::warp_sum(mT.dot_smem(stmp, lane));
+                if (lane == 0) {
+                    a.zvec[c0 + w] = z;
+                    if (rz_out) part = (double)sres[c0 + w] * (double)z;
+                }
+            } else if (!one_row) {
+                rows_dot<T, PL>(a.Bt, sp, c0, c1, stmp, a.zvec);
+                __syncthreads();
+                if (rz_out)
+                    for (int64_t c = c0 + threadIdx.x; c < c1; c += kThreads) part += (double)sres[c] * (double)a.zvec[c];
+            }
+            if (rz_out) {
+                // my_row: lane 0 of each warp holds a product
+                if (one_row) {
+                    if (lane == 0) red_b[w] = part;
+                    __syncthreads();
+                    part = w == 0 ? msp::warp_sum(lane < kNW ? red_b[lane] : 0.0) : 0.0;
+                } else {
+                    part = block_sum0(part, true, red_b);
+                }
+                if (threadIdx.x == 0) a.dpart[b * 4 + 2] = part;
+            }
+            if (!msp::grid_barrier(bw, err)) return false;
+            if (rz_out) {
+                *rz_out = grid_sum(a.dpart + 2, G, &s_val[turn]);
+                turn = 3 - turn;
+            }
+            return true;
+        };
+
+        // direct level 2 (max_inner == 0) has no level-2 iteration: z^T res unused
+        double rz_in = 0.0;
+        if (!precond(inner ? &rz_in : nullptr)) return;
+        // direct level 2: M2 is the level-2 operator itself (Phi = I), so
+        // y = M2^{-1} C^T r with no correction steps
+        load_full(a.zvec, inner ? sd : sy, sp);
         __syncthreads();
+        double rres = gg;
+        const double tin2 = a.inner_tol2 * gg;
+        while (k < a.max_inner && rres > tin2) {
+            // P1: partial u = C^T (C d) over this block's rows; wd = W d (columns)
+#pragma unroll
+            for (int q = 0; q < S::KU; ++q) acc[q][0] = acc[q][1] = T(0);
+            for (int cb = 0; cb < rows.nr; cb += kRowChunk) {
+                const int ce = min(rows.nr, cb + kRowChunk);
+                dots_pass<T, TC, PL>(rows, cb, ce, sd, sw);
+                __syncthreads();
+                cols_pass<T, TC, PL>(rows, cb, ce, sw, acc);
+                if (ce < rows.nr) __syncthreads();
+            }
+            cols_store<T, TC, PL>(acc, scr, a.part + (int64_t)b * sp);
+            rows_dot<T, PL, TC>(a.W, sp, c0, c1, sd, a.wdvec);
+            if (!msp::grid_barrier(bw, err)) return;
+            // P2: u over this block's columns; d.u partial
+            double du = reduce_cols<T>(a.part, G, sp, a.wdvec, a.lam_t, a.uvec, sd, false, redc);
+            if (threadIdx.x == 0) a.dpart[b * 4 + 3] = du;
+            if (!msp::grid_barrier(bw, err)) return;
+            // P3: step
+            du = grid_sum(a.dpart + 3, G, &s_val[3]);
+            if (!(du > 0.0)) break;   // breakdown (same decision in every block)
+            const T ain = (T)(rz_in / du);
+            double loc = 0.0;
+            for (int c = threadIdx.x; c < sp; c += kThreads) {
+                T u = __ldcg(&a.uvec[c]);
+                sy[c] += ain * sd[c];
+                T rv = sres[c] - ain * u;
+                sres[c] = rv;
+                loc += (double)rv * (double)rv;
+            }
+            rres = block_sum0(loc, 32 * w < sp, red_c);
+            if (threadIdx.x == 0) s_val[0] = rres;
+            __syncthreads();
+            rres = s_val[0];
+            ++k;
+            if (rres <= tin2) break;
+            double rz_new = 0.0;
+            if (!precond(&rz_new)) return;
+            const T beta = (T)(rz_new / rz_in);
+            rz_in = rz_new;
+            for (int c = threadIdx.x; c < sp; c += kThreads) sd[c] = __ldcg(&a.zvec[c]) + beta * sd[c];
+            __syncthreads();
+        }
+    } else {
+        if (s_bad) return;
+        load_full(a.zvec, sy, sp);     // y of the k_inner launch
     }
 
     // ---- w = (r - C y) / lam~ into z; dots r.w and r.z_old for the level-1 beta
@@ -992,7 +1006,7 @@ __global__ void __launch_bounds__(kThreads, 1) k_level2(L2Args<T, TC> a) {
         if (ce < rows.nr) __syncthreads();
     }
     if (a.mode == MODE_APPLY) {
-        if (b == 0 && threadIdx.x == 0) atomicAdd(&ctl->inner_iters, k);
+        if (b == 0 && threadIdx.x == 0) ctl->inner_iters += k;
         return;
     }
     {
@@ -1034,10 +1048,8 @@ __global__ void __launch_bounds__(kThreads, 1) k_level2(L2Args<T, TC> a) {
         }
     }
     if (b == 0 && threadIdx.x == 0) {
-        ctl->rr = rr;
         ctl->inner_iters += k;
         if (a.mode == MODE_ITER) ctl->iters = iter + 1;
-        if (a.mode == MODE_INIT) { ctl->bb = rr; ctl->tol2 = a.tol_rel2 * rr; }
     }
 }
 
@@ -1089,6 +1101,200 @@ msp_status launch_level2(msp_ctx* ctx, L2Args<T, TC>& a, int G) {
     }
     return msp_set_error(ctx, MSP_EINVAL, "level-2: unsupported padded sketch size %lld",
                          (long long)a.s_pad);
+}
+
+// ------------------------------------------------ level-2 iteration on a formed operator
+
+template <typename T>
+struct InnerArgs {
+    const T* H;             // C^T C + lam~ W, s_pad x s_pad (FP32: rounded), null: not formed
+    const float* Hlo;       // FP32: what the rounding left
+    const T* B;
+    const T* Bt;
+    const T* g;             // C^T r
+    T* y;
+    double inner_tol2;
+    int max_inner;
+    CtlBlock* ctl;
+};
+
+// The level-2 PCG of Algorithm 2 on (C^T C + lam~ W) y = g, preconditioned by
+// M2^{-1} v = B^T (B v), as products with the formed s_pad x s_pad operator, on one
+// cluster of 16 CTAs. In k_level2 an iteration is a pass over C and four grid
+// barriers (18 us at n = 4999, s = 312; 18 us in FP64 at n = 1024, s = 64); here it is
+// three products on data that stays on the SMs, with a cluster barrier each: 6 us
+// and 5.6 us.
+//
+// A CTA has s_pad threads and s_pad / 16 rows of H, B and B^T, 16 lanes a row,
+// E = s_pad / 16 values of a row a lane, all in registers for the whole launch.
+// After a row's butterfly each of its lanes holds the sum and stores it into one
+// CTA's copy of the result (two copies in turn: a CTA is never more than one barrier
+// ahead), so thread t of every CTA has component t. Vectors, dots and scalars are
+// formed in every CTA from the same values in the same order; the FP64 dots are
+// taken by four warps (one per FP64 unit) from the vectors in shared memory and
+// finished, like the quotients, by one warp. FP32: H as a pair of floats, so the
+// operator is that of the compensated Gram, not its FP32 rounding.
+constexpr int kInnerCtas = 16;
+
+template <typename T, int E>
+__global__ void __launch_bounds__(16 * E, 1) k_inner(InnerArgs<T> a) {
+    namespace cg = cooperative_groups;
+    constexpr int SP = 16 * E, OWN = SP / kInnerCtas, W = Vec16<T>::W, NV = E / W;
+    cg::cluster_group cl = cg::this_cluster();
+    __shared__ __align__(16) T va[SP], vb[SP], ybuf[2][SP];
+    __shared__ double red[4], s_sc;
+    CtlBlock* ctl = a.ctl;
+    if (ctl->done | ctl->error) return;       // the same in every CTA: nothing writes them here
+    const int tid = threadIdx.x, warp = tid >> 5, lane = tid & 31, l16 = tid & 15;
+    const int rank = (int)cl.block_rank();
+    const int row = rank * OWN + (tid >> 4);
+    constexpr int NP = sizeof(T) == 4 ? 2 : 1;
+    T h[E], hl[NP == 2 ? E : 1], bm[E], bt[E];
+    auto load_row = [&](const T* M, T* dst) {
+#pragma unroll
+        for (int k = 0; k < NV; ++k) load16(M + (int64_t)row * SP + W * (l16 + 16 * k), dst + k * W);
+    };
+    load_row(a.B, bm);
+    load_row(a.Bt, bt);
+    load_row(a.H, h);
+    if constexpr (NP == 2) load_row(a.Hlo, hl);
+    T res = a.g[tid], y = T(0), d = T(0);
+    cl.sync();   // every CTA runs before its shared memory is written
+    int turn = 0;
+    // component tid of M v, v in shared memory (visible to the block); the full
+    // result is in the returned copy
+    auto product = [&](const T* m, const T* mlo, const T* v) -> const T* {
+        T s0 = T(0), s1 = T(0);
+#pragma unroll
+        for (int k = 0; k < NV; ++k) {
+            T x[W];
+            load16(v + W * (l16 + 16 * k), x);
+#pragma unroll
+            for (int e = 0; e < W; ++e) {
+                s0 = fma(m[k * W + e], x[e], s0);
+                if (mlo) s1 = fma(mlo[k * W + e], x[e], s1);
+            }
+        }
+        s0 += s1;
+#pragma unroll
+        for (int o = 8; o > 0; o >>= 1) s0 += __shfl_xor_sync(0xffffffffu, s0, o);
+        cl.map_shared_rank(&ybuf[turn][0], l16)[row] = s0;
+        cl.sync();
+        const T* out = ybuf[turn];
+        turn ^= 1;
+        return out;
+    };
+    // u . v (shared memory), in warp 0; ends past a block barrier
+    auto dot0 = [&](const T* u, const T* v) -> double {
+        if (warp < 4) {
+            double t = 0.0;
+#pragma unroll
+            for (int c = tid; c < SP; c += 128) t = fma((double)u[c], (double)v[c], t);
+            t = msp::warp_sum(t);
+            if (lane == 0) red[warp] = t;
+        }
+        __syncthreads();
+        return warp == 0 ? (red[0] + red[1]) + (red[2] + red[3]) : 0.0;
+    };
+    auto share = [&](double v) -> double {
+        if (tid == 0) s_sc = v;
+        __syncthreads();
+        return s_sc;
+    };
+    va[tid] = res;
+    __syncthreads();
+    const double gg = share(dot0(va, va)), tin2 = a.inner_tol2 * gg;
+    const T* z = nullptr;
+    // z = B^T (B res), res in va
+    auto precond = [&]() {
+        vb[tid] = product(bm, nullptr, va)[tid];
+        __syncthreads();
+        z = product(bt, nullptr, vb);
+    };
+    precond();
+    double rz = dot0(va, z);           // warp 0's
+    d = z[tid];
+    int k = 0;
+    while (k < a.max_inner && gg > tin2) {
+        vb[tid] = d;
+        __syncthreads();
+        const T* u = product(h, NP == 2 ? hl : nullptr, vb);
+        const double du = dot0(vb, u);
+        // the step, -1 for a breakdown (d . u not positive)
+        const double q = share(warp == 0 ? (du > 0.0 ? rz / du : nan("")) : 0.0);
+        if (!(q == q)) break;
+        const T ain = (T)q;
+        y += ain * d;
+        res -= ain * u[tid];
+        va[tid] = res;
+        __syncthreads();
+        const double rres = share(dot0(va, va));
+        ++k;
+        if (rres <= tin2 || k == a.max_inner) break;
+        precond();
+        const double rzn = dot0(va, z);
+        const T beta = (T)share(warp == 0 ? rzn / rz : 0.0);
+        rz = rzn;
+        d = z[tid] + beta * d;
+    }
+    if (rank == 0) {
+        a.y[tid] = y;
+        if (tid == 0) ctl->inner_iters += k;
+    }
+}
+
+// The kernel for a padded sketch size (its data fits the cluster's registers),
+// null where there is none.
+template <typename T>
+const void* inner_kernel(int64_t sp) {
+    switch (sp) {
+        case 128: return (const void*)k_inner<T, 8>;
+        case 256: return (const void*)k_inner<T, 16>;
+        case 384:
+            if constexpr (sizeof(T) == 4) return (const void*)k_inner<T, 24>;
+            return nullptr;
+        default: return nullptr;
+    }
+}
+
+cudaLaunchConfig_t inner_config(msp_ctx* ctx, int64_t sp, cudaLaunchAttribute* attr) {
+    cudaLaunchConfig_t cfg{};
+    cfg.gridDim = dim3(kInnerCtas);
+    cfg.blockDim = dim3((unsigned)sp);
+    cfg.stream = ctx->stream;
+    attr->id = cudaLaunchAttributeClusterDimension;
+    attr->val.clusterDim.x = kInnerCtas;
+    attr->val.clusterDim.y = 1;
+    attr->val.clusterDim.z = 1;
+    cfg.attrs = attr;
+    cfg.numAttrs = 1;
+    return cfg;
+}
+
+template <typename T>
+msp_status launch_inner(msp_ctx* ctx, InnerArgs<T>& a, int64_t sp) {
+    const void* kern = inner_kernel<T>(sp);
+    MSP_CUDA_TRY(ctx, cudaFuncSetAttribute(kern, cudaFuncAttributeNonPortableClusterSizeAllowed, 1));
+    cudaLaunchAttribute attr;
+    const cudaLaunchConfig_t cfg = inner_config(ctx, sp, &attr);
+    void* args[] = {&a};
+    ++ctx->launches;
+    MSP_CUDA_TRY(ctx, cudaLaunchKernelExC(&cfg, kern, args));
+    return MSP_OK;
+}
+
+// The level-2 step of an iteration: k_level2 whole (a direct level 2, no formed
+// operator), or k_inner between its two parts.
+template <typename T, typename TC>
+msp_status launch_level2(msp_ctx* ctx, L2Args<T, TC>& a, int G, InnerArgs<T>& in) {
+    if (!in.H || a.max_inner <= 0) return launch_level2(ctx, a, G);
+    a.phase = PHASE_FRONT;
+    msp_status st = launch_level2(ctx, a, G);
+    if (st == MSP_OK) st = launch_inner<T>(ctx, in, a.s_pad);
+    a.phase = PHASE_BACK;
+    if (st == MSP_OK) st = launch_level2(ctx, a, G);
+    a.phase = PHASE_ALL;
+    return st;
 }
 
 struct Workspace {
@@ -1146,6 +1352,24 @@ void fill_l2(L2Args<T, TC>& a, const msp_factor_s* f, int64_t n, const Workspace
     a.zvec = v + 3 * sp;
     a.wdvec = v + 4 * sp;
     a.dpart = ws.dpart;
+}
+
+// after the options are in `a`
+template <typename T, typename TC>
+InnerArgs<T> fill_inner(const msp_factor_s* f, const L2Args<T, TC>& a) {
+    InnerArgs<T> in;
+    std::memset(&in, 0, sizeof in);
+    if (!f->H || f->data == MSP_BF16) return in;
+    in.H = (const T*)f->H;
+    in.Hlo = sizeof(T) == 4 ? (const float*)f->H + f->s_pad * f->s_pad : nullptr;
+    in.B = a.B;
+    in.Bt = a.Bt;
+    in.g = a.gvec;
+    in.y = a.zvec;
+    in.inner_tol2 = a.inner_tol2;
+    in.max_inner = a.max_inner;
+    in.ctl = a.ctl;
+    return in;
 }
 
 // The level-2 grid: one block per SM (a thread per block partial in the
@@ -1316,7 +1540,8 @@ msp_status krylov_solve_t(msp_ctx* ctx, const msp_factor_s* f, const void* A, ms
     a.n_dq = ctx->num_sms;
     a.lam = (T)lambda;
     a.mode = MODE_INIT;
-    MSP_TRY(launch_level2(ctx, a, G));
+    InnerArgs<T> in = fill_inner(f, a);
+    MSP_TRY(launch_level2(ctx, a, G, in));
     a.mode = MODE_ITER;
 
     const bool vec = (lda % (16 / dtype_size(dt)) == 0) &&
@@ -1351,7 +1576,7 @@ msp_status krylov_solve_t(msp_ctx* ctx, const msp_factor_s* f, const void* A, ms
         }
         MSP_TRY(mark(cap, 1));
         MSP_TRY(mark(cap, 2));
-        MSP_TRY(launch_level2(ctx, a, G));
+        MSP_TRY(launch_level2(ctx, a, G, in));
         MSP_TRY(mark(cap, 3));
         return MSP_OK;
     };
@@ -1365,6 +1590,7 @@ msp_status krylov_solve_t(msp_ctx* ctx, const msp_factor_s* f, const void* A, ms
             double lambda;
             const void* qpart;
             const void* gpart;
+            const void* H;
             L2Args<T, TC> a;
         } key;
         static_assert(sizeof(Key) <= sizeof(ctx->l1_key), "level-1 graph key too large");
@@ -1382,6 +1608,7 @@ msp_status krylov_solve_t(msp_ctx* ctx, const msp_factor_s* f, const void* A, ms
         key.lambda = lambda;
         key.qpart = ws.qpart;
         key.gpart = ws.gpart;
+        key.H = in.H;
         std::memcpy(&key.a, &a, sizeof a);
         MSP_TRY(ensure_l1_graph(ctx, &key, sizeof key, pr.on, iteration));
         graphed = ctx->l1_exec != nullptr;
@@ -1458,6 +1685,22 @@ msp_status msp_grid_wait_limit_krylov(msp_ctx* ctx, unsigned long long ns) {
     const unsigned long long v = ns ? ns : msp::kWaitLimitNs;
     MSP_CUDA_TRY(ctx, cudaMemcpyToSymbol(msp::g_grid_wait_limit_ns, &v, sizeof v));
     return MSP_OK;
+}
+
+// Whether the level-2 iteration of a factor of this size runs on a formed
+// operator (k_inner): a kernel for the size, and room for its cluster.
+bool msp_inner_ok(msp_ctx* ctx, msp_dtype dt, int64_t sp) {
+    const void* kern = dt == MSP_F32 ? inner_kernel<float>(sp) : inner_kernel<double>(sp);
+    if (!kern) return false;
+    cudaLaunchAttribute attr;
+    const cudaLaunchConfig_t cfg = inner_config(ctx, sp, &attr);
+    int clusters = 0;
+    if (cudaFuncSetAttribute(kern, cudaFuncAttributeNonPortableClusterSizeAllowed, 1) != cudaSuccess ||
+        cudaOccupancyMaxActiveClusters(&clusters, kern, &cfg) != cudaSuccess) {
+        cudaGetLastError();
+        return false;
+    }
+    return clusters >= 1;
 }
 
 msp_status msp_krylov_solve(msp_ctx* ctx, const msp_factor_s* f, const void* A, msp_dtype dt,
@@ -1568,7 +1811,8 @@ msp_status msp_solve_m1_impl(msp_ctx* ctx, const msp_factor_s* f, const void* r,
         a.r = (float*)r;
         a.z = (float*)w;
         a.mode = MODE_APPLY;
-        MSP_TRY(launch_level2(ctx, a, G));
+        auto in = fill_inner(f, a);
+        MSP_TRY(launch_level2(ctx, a, G, in));
     } else if (f->dtype == MSP_F32) {
         Workspace ws;
         MSP_TRY(get_workspace<float>(ctx, n, f->s_pad, G, Gg, false, &ws));
@@ -1579,7 +1823,8 @@ msp_status msp_solve_m1_impl(msp_ctx* ctx, const msp_factor_s* f, const void* r,
         a.r = (float*)r;
         a.z = (float*)w;
         a.mode = MODE_APPLY;
-        MSP_TRY(launch_level2(ctx, a, G));
+        auto in = fill_inner(f, a);
+        MSP_TRY(launch_level2(ctx, a, G, in));
     } else {
         Workspace ws;
         MSP_TRY(get_workspace<double>(ctx, n, f->s_pad, G, Gg, false, &ws));
@@ -1590,7 +1835,8 @@ msp_status msp_solve_m1_impl(msp_ctx* ctx, const msp_factor_s* f, const void* r,
         a.r = (double*)r;
         a.z = (double*)w;
         a.mode = MODE_APPLY;
-        MSP_TRY(launch_level2(ctx, a, G));
+        auto in = fill_inner(f, a);
+        MSP_TRY(launch_level2(ctx, a, G, in));
     }
     MSP_CUDA_TRY(ctx, cudaMemcpyAsync(hf, &ctl->done, 5 * sizeof(int), cudaMemcpyDeviceToHost,
                                       ctx->stream));

@@ -119,6 +119,9 @@ struct msp_factor_s {
     msp_dtype data = MSP_F32;
     void* Cb = nullptr;         // n x s_pad BF16
     void* Wb = nullptr;         // s_pad x s_pad BF16
+    // the level-2 operator C^T C + lam~ W formed (phi > 0 and a size k_inner
+    // takes): FP64, or two FP32 matrices, the rounded entries and what that left
+    void* H = nullptr;
 };
 
 // Device control block layout (one per context).
@@ -348,6 +351,8 @@ bool msp_gram_tc_ok(int64_t s_pad);
 
 // factor.cu
 msp_status msp_build_factor(msp_ctx* ctx, msp_factor_s* f, const void* Ct, int64_t phi_rows);
+// f->H = C^T C + lam~ W, C of n rows
+msp_status msp_form_level2(msp_ctx* ctx, msp_factor_s* f, const void* C, int64_t n);
 // G64 = X^T X + diag I (FP64, pad identity); M^{-1} of an SPD FP64 matrix;
 // C = X^T Y (FP32, compensated) -- see factor.cu
 msp_status msp_gram64(msp_ctx* ctx, const float* X, int64_t rows, int64_t ld, int64_t s, int64_t sp,
@@ -376,6 +381,7 @@ msp_status msp_symv_packed(msp_ctx* ctx, const float* packed, int64_t n, float l
                            const double* l2part, int n_l2, float* part, double* dpart, int grid);
 
 // krylov.cu
+bool msp_inner_ok(msp_ctx* ctx, msp_dtype dt, int64_t sp);
 msp_status msp_grid_wait_limit_krylov(msp_ctx* ctx, unsigned long long ns);
 // prof: null, or two slots (A-pass GEMV, level-2 kernel) to accumulate
 // event-timed durations into (opts->profile).

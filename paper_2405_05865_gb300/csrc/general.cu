@@ -592,48 +592,49 @@ __global__ void k_dense_mv(const double* __restrict__ M, const float* __restrict
 // instruction holds it for 16 cycles whether the lanes' results are needed or
 // not) and the latency of the serial chain product -> dot -> step, so every
 // FP64 instruction that is not the product itself is kept to the threads that
-// need it. A CTA has s_pad threads: 8 lanes form one of its s_pad / kCl rows
-// of a product (their slices of W and M3^{-1} in registers up to s_pad = 256,
-// E = s_pad / 8 values each, read from L1 / L2 beyond), and after the row's
-// butterfly each of the 8 lanes holds the sum and stores it into one CTA's copy
-// of the full result, so one cluster barrier per product is the only exchange
-// (two copies in turn: a CTA is never more than one barrier ahead). Thread t
-// then keeps component t of x, r, p redundantly in every CTA, the dots are
+// need it. A CTA has s_pad threads: 16 lanes form one of its s_pad / kCl rows
+// of a product (their slices of W and M3^{-1} in registers up to s_pad = 384,
+// E = s_pad / kCl values each, read from L1 / L2 beyond). The CTA's row sums are
+// gathered in shared memory and stored to every CTA's copy of the full result by
+// 16-byte pieces (one word per lane and CTA costs twice the barrier), so one
+// cluster barrier per product is the only exchange (two copies in turn: a CTA
+// is never more than one barrier ahead). Thread t then keeps component t of x, r, p redundantly in every CTA, the dots are
 // taken in each CTA from the full vectors in the same order, and one warp
 // forms each step's quotient. The former layout (1024 threads whatever s_pad,
 // every thread summing partials and dividing, two cluster barriers a product)
 // took 177 us at s_pad = 128, t3 = 8, most of a three-level solve; with this one
 // the solve at 16384 x 2048 went from 355 to 180 ms.
-constexpr int kCl = 8;
+constexpr int kCl = 16;
 
 template <int E>
-__global__ void __cluster_dims__(kCl, 1, 1) __launch_bounds__(E > 0 ? 8 * E : 1024)
+__global__ void __cluster_dims__(kCl, 1, 1) __launch_bounds__(E > 0 ? kCl * E : 1024)
     k_level3_cluster(const double* __restrict__ W, const double* __restrict__ Ma, const double* __restrict__ Mb,
                      double lam_t, int sp, int t3, const float* __restrict__ b, float* __restrict__ u,
                      float* __restrict__ v) {
     namespace cg = cooperative_groups;
     cg::cluster_group cl = cg::this_cluster();
     __shared__ __align__(16) double vec[1024];   // the vector of the next product
-    __shared__ double ybuf[2][1024];             // products, in turn
+    __shared__ __align__(16) double ybuf[2][1024];   // products, in turn
+    __shared__ __align__(16) double stage[1024 / kCl];   // this CTA's part
     __shared__ double red[32];
     __shared__ double s_sc;
     const int rank = (int)cl.block_rank();
     const int sys = blockIdx.x / kCl;
     const double shift = sys == 0 ? 0.0 : lam_t;
     float* out = sys == 0 ? u : v;
-    const int tid = threadIdx.x, warp = tid >> 5, lane = tid & 31, l8 = tid & 7;
+    const int tid = threadIdx.x, warp = tid >> 5, lane = tid & 31, l16 = tid & 15;
     const int nw = sp >> 5, own = sp / kCl;
-    const int row = rank * own + (tid >> 3);
-    // this lane's elements of its row: the pairs 2 l8 + 16 k
-    const double2* Wr = reinterpret_cast<const double2*>(W + (int64_t)row * sp) + l8;
-    const double2* Mr = reinterpret_cast<const double2*>((sys == 0 ? Ma : Mb) + (int64_t)row * sp) + l8;
+    const int row = rank * own + (tid >> 4);
+    // this lane's elements of its row: the pairs 2 l16 + 32 k
+    const double2* Wr = reinterpret_cast<const double2*>(W + (int64_t)row * sp) + l16;
+    const double2* Mr = reinterpret_cast<const double2*>((sys == 0 ? Ma : Mb) + (int64_t)row * sp) + l16;
     constexpr int ER = E > 0 ? E / 2 : 1;
     double2 wreg[ER], mreg[ER];
     if constexpr (E > 0) {
 #pragma unroll
-        for (int k = 0; k < ER; ++k) mreg[k] = __ldg(Mr + 8 * k);
+        for (int k = 0; k < ER; ++k) mreg[k] = __ldg(Mr + kCl * k);
 #pragma unroll
-        for (int k = 0; k < ER; ++k) wreg[k] = __ldg(Wr + 8 * k);
+        for (int k = 0; k < ER; ++k) wreg[k] = __ldg(Wr + kCl * k);
     }
     cl.sync();   // every CTA of the cluster runs before its shared memory is written
     int turn = 0;
@@ -641,28 +642,34 @@ __global__ void __cluster_dims__(kCl, 1, 1) __launch_bounds__(E > 0 ? 8 * E : 10
     auto product = [&](const double2 (&reg)[ER], const double2* rows, double val) {
         vec[tid] = val;
         __syncthreads();
-        const double2* v2 = reinterpret_cast<const double2*>(vec) + l8;
+        const double2* v2 = reinterpret_cast<const double2*>(vec) + l16;
         double s0 = 0.0, s1 = 0.0;
         if constexpr (E > 0) {
 #pragma unroll
             for (int k = 0; k < ER; ++k) {
-                const double2 a = v2[8 * k];
+                const double2 a = v2[kCl * k];
                 s0 = fma(reg[k].x, a.x, s0);
                 s1 = fma(reg[k].y, a.y, s1);
             }
         } else {
-            const int n2 = sp >> 4;
+            const int n2 = sp / (2 * kCl);
 #pragma unroll 8
             for (int k = 0; k < n2; ++k) {
-                const double2 m = __ldg(rows + 8 * k), a = v2[8 * k];
+                const double2 m = __ldg(rows + kCl * k), a = v2[kCl * k];
                 s0 = fma(m.x, a.x, s0);
                 s1 = fma(m.y, a.y, s1);
             }
         }
         double s = s0 + s1;
 #pragma unroll
-        for (int o = 4; o > 0; o >>= 1) s += __shfl_xor_sync(0xffffffffu, s, o);
-        cl.map_shared_rank(&ybuf[turn][0], l8)[row] = s;
+        for (int o = kCl / 2; o > 0; o >>= 1) s += __shfl_xor_sync(0xffffffffu, s, o);
+        if (l16 == 0) stage[tid >> 4] = s;
+        __syncthreads();
+        if (tid < own / 2 * kCl) {
+            const int to = tid / (own / 2), piece = tid % (own / 2);
+            reinterpret_cast<double2*>(cl.map_shared_rank(&ybuf[turn][0], to) + rank * own)[piece] =
+                reinterpret_cast<const double2*>(stage)[piece];
+        }
         cl.sync();
         const double y = ybuf[turn][tid];
         turn ^= 1;
@@ -674,7 +681,7 @@ __global__ void __cluster_dims__(kCl, 1, 1) __launch_bounds__(E > 0 ? 8 * E : 10
         if (lane == 0) red[warp] = prod;
         __syncthreads();
         double t = 0.0;
-        if (warp == 0) t = warp_sum_t(lane < nw ? red[lane] : 0.0);
+        if (warp == 0) t = nw == 4 ? (red[0] + red[1]) + (red[2] + red[3]) : warp_sum_t(lane < nw ? red[lane] : 0.0);
         return t;
     };
     // warp 0's value to every thread
@@ -1069,15 +1076,10 @@ struct Ops {
     msp_status solve_m2(const float* r, float* z, int t3) {
         if (t3 == 0) return dense(g->M2inv, r, z);
         const int sp = (int)g->s_pad;
-        if (sp == 128)
-            k_level3_cluster<16><<<2 * kCl, sp, 0, strm>>>(g->W64, g->M3a, g->M3b, g->lam_tilde, sp, t3, r, g->u3,
-                                                           g->v3);
-        else if (sp == 256)
-            k_level3_cluster<32><<<2 * kCl, sp, 0, strm>>>(g->W64, g->M3a, g->M3b, g->lam_tilde, sp, t3, r, g->u3,
-                                                           g->v3);
-        else
-            k_level3_cluster<0><<<2 * kCl, sp, 0, strm>>>(g->W64, g->M3a, g->M3b, g->lam_tilde, sp, t3, r, g->u3,
-                                                          g->v3);
+        auto kern = sp == 128 ? k_level3_cluster<8> : sp == 256 ? k_level3_cluster<16>
+                    : sp == 384 ? k_level3_cluster<24> : k_level3_cluster<0>;
+        MSP_CUDA_TRY(ctx, cudaFuncSetAttribute(kern, cudaFuncAttributeNonPortableClusterSizeAllowed, 1));
+        kern<<<2 * kCl, sp, 0, strm>>>(g->W64, g->M3a, g->M3b, g->lam_tilde, sp, t3, r, g->u3, g->v3);
         MSP_CHECK_LAUNCH(ctx);
         if (count) ++*count;
         const float il = (float)(1.0 / g->lam_tilde);

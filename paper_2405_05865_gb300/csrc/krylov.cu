@@ -1125,119 +1125,182 @@ struct InnerArgs {
 // three products on data that stays on the SMs, with a cluster barrier each: 6 us
 // and 5.6 us.
 //
-// A CTA has s_pad threads and s_pad / 16 rows of H, B and B^T, 16 lanes a row,
-// E = s_pad / 16 values of a row a lane, all in registers for the whole launch.
-// After a row's butterfly each of its lanes holds the sum and stores it into one
-// CTA's copy of the result (two copies in turn: a CTA is never more than one barrier
-// ahead), so thread t of every CTA has component t. Vectors, dots and scalars are
-// formed in every CTA from the same values in the same order; the FP64 dots are
-// taken by four warps (one per FP64 unit) from the vectors in shared memory and
-// finished, like the quotients, by one warp. FP32: H as a pair of floats, so the
-// operator is that of the compensated Gram, not its FP32 rounding.
+// A CTA has s_pad / 16 rows of H, B and B^T, 16 lanes a row, E = s_pad / 16 values of
+// a row a lane, all in registers for the whole launch. The row sums are gathered
+// in shared memory and sent to every CTA's copy of the result by 16-byte st.async
+// pieces that count on that CTA's mbarrier (two copies in turn: a CTA sends product
+// k + 2 only after it has every CTA's part of k + 1, sent after the reads of k);
+// thread t of every CTA has component t. What bounds it is the latency of that
+// chain, so the dots and quotients, formed in every CTA from the same values in
+// the same order, belong to four more warps (one per FP64 unit: a warp-wide FP64
+// sum takes 520 cycles, a quotient 560 in one warp and 1540 in four), and
+// |res|^2 is taken while the product with B that follows it is under way. One thread
+// polls the mbarrier and the others wait at the block barrier: with a cluster
+// barrier instead, the waiting warps' polls slowed the others' shuffles (a
+// FP64 sum 2700 cycles, four FP32 steps 950) and an iteration took 6 us. FP32: H as a
+// pair of floats, so the operator is that of the compensated Gram, not its rounding.
 constexpr int kInnerCtas = 16;
+constexpr int kDotThreads = 128;
+
+// Exact widening without the FP64 pipe for normal numbers.
+__device__ __forceinline__ double widen_exact(double v) { return v; }
+__device__ __forceinline__ double widen_exact(float x) {
+    const uint32_t b = __float_as_uint(x);
+    if (((b >> 23) & 0xFFu) - 1u >= 254u) return (double)x;     // zero, subnormal, infinity, NaN
+    return __hiloint2double((int)((b & 0x80000000u) | (((b & 0x7FFFFFFFu) >> 3) + (896u << 20))), (int)(b << 29));
+}
+
+// 16 bytes of this CTA's shared memory to the same place as `dst` in CTA `to` of the
+// cluster, counted on that CTA's `bar`
+template <typename T>
+__device__ __forceinline__ void st_async16(T* dst, const T* src, uint64_t* bar, int to) {
+    uint32_t d, b;
+    asm("mapa.shared::cluster.u32 %0, %1, %2;" : "=r"(d) : "r"(msp::smem_u32(dst)), "r"(to));
+    asm("mapa.shared::cluster.u32 %0, %1, %2;" : "=r"(b) : "r"(msp::smem_u32(bar)), "r"(to));
+    const uint4 v = *reinterpret_cast<const uint4*>(src);
+    asm volatile("st.async.weak.shared::cluster.mbarrier::complete_tx::bytes.v4.b32 [%0], {%1, %2, %3, %4}, [%5];" ::"r"(d),
+                 "r"(v.x), "r"(v.y), "r"(v.z), "r"(v.w), "r"(b)
+                 : "memory");
+}
 
 template <typename T, int E>
-__global__ void __launch_bounds__(16 * E, 1) k_inner(InnerArgs<T> a) {
+__global__ void __launch_bounds__(16 * E + kDotThreads, 1) k_inner(InnerArgs<T> a) {
     namespace cg = cooperative_groups;
     constexpr int SP = 16 * E, OWN = SP / kInnerCtas, W = Vec16<T>::W, NV = E / W;
+    constexpr int VPD = OWN / W;              // 16-byte pieces of a CTA's rows
+    static_assert(VPD * kInnerCtas <= SP, "a piece per thread");
     cg::cluster_group cl = cg::this_cluster();
-    __shared__ __align__(16) T va[SP], vb[SP], ybuf[2][SP];
-    __shared__ double red[4], s_sc;
+    __shared__ __align__(16) T va[SP], vb[SP], ybuf[2][SP], stage[OWN];
+    __shared__ __align__(8) uint64_t full[2];
+    __shared__ double red[4], s_sc, s_rres;
+    __shared__ int s_bad;
     CtlBlock* ctl = a.ctl;
     if (ctl->done | ctl->error) return;       // the same in every CTA: nothing writes them here
-    const int tid = threadIdx.x, warp = tid >> 5, lane = tid & 31, l16 = tid & 15;
+    const int tid = threadIdx.x, lane = tid & 31, l16 = tid & 15;
+    const bool dots = tid >= SP;              // the warps of the dots
     const int rank = (int)cl.block_rank();
     const int row = rank * OWN + (tid >> 4);
     constexpr int NP = sizeof(T) == 4 ? 2 : 1;
     T h[E], hl[NP == 2 ? E : 1], bm[E], bt[E];
-    auto load_row = [&](const T* M, T* dst) {
+    T res = T(0), y = T(0), d = T(0);
+    if (!dots) {
+        auto load_row = [&](const T* M, T* dst) {
 #pragma unroll
-        for (int k = 0; k < NV; ++k) load16(M + (int64_t)row * SP + W * (l16 + 16 * k), dst + k * W);
+            for (int k = 0; k < NV; ++k) load16(M + (int64_t)row * SP + W * (l16 + 16 * k), dst + k * W);
+        };
+        load_row(a.B, bm);
+        load_row(a.Bt, bt);
+        load_row(a.H, h);
+        if constexpr (NP == 2) load_row(a.Hlo, hl);
+        res = a.g[tid];
+        va[tid] = res;
+    }
+    if (tid == 0) {
+        msp::mbar_init(&full[0], 1);
+        msp::mbar_init(&full[1], 1);
+        asm volatile("fence.mbarrier_init.release.cluster;" ::: "memory");
+        s_bad = 0;
+    }
+    cl.sync();   // every CTA runs, its mbarriers ready, before it is written to
+    uint32_t sent = 0;                        // products so far
+    // u . v (shared memory) in the first of the dots' warps
+    auto dot = [&](const T* u, const T* v) -> double {
+        double t = 0.0;
+#pragma unroll
+        for (int c = tid - SP; c < SP; c += kDotThreads) t = fma(widen_exact(u[c]), widen_exact(v[c]), t);
+        t = msp::warp_sum(t);
+        if (lane == 0) red[(tid - SP) >> 5] = t;
+        asm volatile("bar.sync 2, %0;" ::"n"(kDotThreads) : "memory");
+        return (red[0] + red[1]) + (red[2] + red[3]);
     };
-    load_row(a.B, bm);
-    load_row(a.Bt, bt);
-    load_row(a.H, h);
-    if constexpr (NP == 2) load_row(a.Hlo, hl);
-    T res = a.g[tid], y = T(0), d = T(0);
-    cl.sync();   // every CTA runs before its shared memory is written
-    int turn = 0;
-    // component tid of M v, v in shared memory (visible to the block); the full
-    // result is in the returned copy
-    auto product = [&](const T* m, const T* mlo, const T* v) -> const T* {
-        T s0 = T(0), s1 = T(0);
-#pragma unroll
-        for (int k = 0; k < NV; ++k) {
-            T x[W];
-            load16(v + W * (l16 + 16 * k), x);
-#pragma unroll
-            for (int e = 0; e < W; ++e) {
-                s0 = fma(m[k * W + e], x[e], s0);
-                if (mlo) s1 = fma(mlo[k * W + e], x[e], s1);
+    // f(u . v) for every thread; ends past a block barrier
+    auto scalar = [&](const T* u, const T* v, auto f) -> double {
+        if (dots) {
+            const double t = dot(u, v);
+            if (tid < SP + 32) {
+                const double q = f(t);
+                if (lane == 0) s_sc = q;
             }
         }
-        s0 += s1;
-#pragma unroll
-        for (int o = 8; o > 0; o >>= 1) s0 += __shfl_xor_sync(0xffffffffu, s0, o);
-        cl.map_shared_rank(&ybuf[turn][0], l16)[row] = s0;
-        cl.sync();
-        const T* out = ybuf[turn];
-        turn ^= 1;
-        return out;
-    };
-    // u . v (shared memory), in warp 0; ends past a block barrier
-    auto dot0 = [&](const T* u, const T* v) -> double {
-        if (warp < 4) {
-            double t = 0.0;
-#pragma unroll
-            for (int c = tid; c < SP; c += 128) t = fma((double)u[c], (double)v[c], t);
-            t = msp::warp_sum(t);
-            if (lane == 0) red[warp] = t;
-        }
-        __syncthreads();
-        return warp == 0 ? (red[0] + red[1]) + (red[2] + red[3]) : 0.0;
-    };
-    auto share = [&](double v) -> double {
-        if (tid == 0) s_sc = v;
         __syncthreads();
         return s_sc;
     };
-    va[tid] = res;
-    __syncthreads();
-    const double gg = share(dot0(va, va)), tin2 = a.inner_tol2 * gg;
-    const T* z = nullptr;
-    // z = B^T (B res), res in va
-    auto precond = [&]() {
-        vb[tid] = product(bm, nullptr, va)[tid];
+    // M v, v in shared memory (visible to the block): the copy of the full
+    // result. with_rr: |v|^2 into s_rres meanwhile. Ends past a block barrier.
+    auto product = [&](const T* m, const T* mlo, const T* v, bool with_rr) -> const T* {
+        if (!dots) {
+            T s0 = T(0), s1 = T(0);
+#pragma unroll
+            for (int k = 0; k < NV; ++k) {
+                T x[W];
+                load16(v + W * (l16 + 16 * k), x);
+#pragma unroll
+                for (int e = 0; e < W; ++e) {
+                    s0 = fma(m[k * W + e], x[e], s0);
+                    if (mlo) s1 = fma(mlo[k * W + e], x[e], s1);
+                }
+            }
+            s0 += s1;
+#pragma unroll
+            for (int o = 8; o > 0; o >>= 1) s0 += __shfl_xor_sync(0xffffffffu, s0, o);
+            if (l16 == 0) stage[tid >> 4] = s0;
+            asm volatile("bar.sync 1, %0;" ::"n"(SP) : "memory");
+            if (tid < VPD * kInnerCtas) {
+                const int to = tid / VPD, piece = tid % VPD;
+                st_async16(&ybuf[sent & 1][rank * OWN + piece * W], stage + piece * W, &full[sent & 1], to);
+            }
+            if (tid == 0) {
+                msp::mbar_arrive_expect_tx(&full[sent & 1], SP * (uint32_t)sizeof(T));
+                if (!msp::mbar_wait_timed(&full[sent & 1], (sent >> 1) & 1u, &ctl->error)) s_bad = 1;
+            }
+        } else if (with_rr) {
+            const double t = dot(v, v);
+            if (tid == SP) s_rres = t;
+        }
         __syncthreads();
-        z = product(bt, nullptr, vb);
+        return ybuf[sent++ & 1];
     };
-    precond();
-    double rz = dot0(va, z);           // warp 0's
-    d = z[tid];
+    const T* z = nullptr;
+    double rz = 0.0;             // r^T z, in the dots' first warp
     int k = 0;
-    while (k < a.max_inner && gg > tin2) {
-        vb[tid] = d;
+    // t = B res (res in va) and |res|^2; with t in vb, z = B^T t
+    auto half = [&]() {
+        const T* t = product(bm, nullptr, va, true);
+        if (!dots) vb[tid] = t[tid];
         __syncthreads();
-        const T* u = product(h, NP == 2 ? hl : nullptr, vb);
-        const double du = dot0(vb, u);
-        // the step, -1 for a breakdown (d . u not positive)
-        const double q = share(warp == 0 ? (du > 0.0 ? rz / du : nan("")) : 0.0);
-        if (!(q == q)) break;
-        const T ain = (T)q;
-        y += ain * d;
-        res -= ain * u[tid];
-        va[tid] = res;
-        __syncthreads();
-        const double rres = share(dot0(va, va));
-        ++k;
-        if (rres <= tin2 || k == a.max_inner) break;
-        precond();
-        const double rzn = dot0(va, z);
-        const T beta = (T)share(warp == 0 ? rzn / rz : 0.0);
-        rz = rzn;
-        d = z[tid] + beta * d;
+        return s_rres;
+    };
+    const double gg = half(), tin2 = a.inner_tol2 * gg;
+    if (gg > tin2 && a.max_inner > 0) {
+        z = product(bt, nullptr, vb, false);
+        scalar(va, z, [&](double t) { return rz = t; });
+        if (!dots) d = z[tid];
+        while (true) {
+            if (!dots) vb[tid] = d;
+            __syncthreads();
+            const T* u = product(h, NP == 2 ? hl : nullptr, vb, false);
+            // the step, NaN for a breakdown (d . u not positive)
+            const double q = scalar(vb, u, [&](double du) { return du > 0.0 ? rz / du : nan(""); });
+            if (!(q == q)) break;
+            if (!dots) {
+                const T ain = (T)q;
+                y += ain * d;
+                res -= ain * u[tid];
+                va[tid] = res;
+            }
+            __syncthreads();
+            if (++k == a.max_inner) break;
+            if (half() <= tin2 || s_bad) break;
+            z = product(bt, nullptr, vb, false);
+            const double beta = scalar(va, z, [&](double rzn) {
+                const double v = rzn / rz;
+                rz = rzn;
+                return v;
+            });
+            if (!dots) d = z[tid] + (T)beta * d;
+        }
     }
-    if (rank == 0) {
+    if (rank == 0 && !dots) {
         a.y[tid] = y;
         if (tid == 0) ctl->inner_iters += k;
     }
@@ -1260,7 +1323,7 @@ const void* inner_kernel(int64_t sp) {
 cudaLaunchConfig_t inner_config(msp_ctx* ctx, int64_t sp, cudaLaunchAttribute* attr) {
     cudaLaunchConfig_t cfg{};
     cfg.gridDim = dim3(kInnerCtas);
-    cfg.blockDim = dim3((unsigned)sp);
+    cfg.blockDim = dim3((unsigned)(sp + kDotThreads));
     cfg.stream = ctx->stream;
     attr->id = cudaLaunchAttributeClusterDimension;
     attr->val.clusterDim.x = kInnerCtas;

@@ -40,22 +40,32 @@ __device__ inline void two_sum_add(TA& hi, TA& lo, TA v) {
     lo += err;
 }
 
-constexpr int kGramSlices = 4;   // split-K slices of the Gram (combined in FP64)
+// Split-K slices of the Gram (combined in FP64): at least 4, and as many as give
+// each SM about a block, 64 rows or more a slice, up to 32. The Grams of the sketch
+// sizes below 512 have 1 to 10 tiles: with 4 slices whatever the size, that of 4999 x
+// 384 (FP32) took 208 us on 24 blocks and that of 1024 x 128 in FP64 425 us on
+// 12; they take 66 and 110 us.
+constexpr int kGramSlicesMax = 32;
+constexpr int kGemmSlices = 4;   // split-K slices of k_gemm_tn
+
+int gram_slices(const msp_ctx* ctx, int64_t tiles, int64_t K) {
+    const int64_t want = std::min<int64_t>(kGramSlicesMax, std::min<int64_t>(ctx->num_sms / tiles, K / 64));
+    return (int)std::max<int64_t>(4, want);
+}
 
 // Partial Gram of one K slice: P[slice][a][b] = sum_{k in slice} Ct[k][a] Ct[k][b]
-// for the upper-triangular 64 x 64 tile pairs (mirrored), FP64 output (hi + lo).
-// blockIdx.x = tile pair, blockIdx.y = K slice.
+// for the upper-triangular 64 x 64 tile pairs (mirrored) of the first nt tiles a side,
+// FP64 output (hi + lo). blockIdx.x = tile pair, blockIdx.y = K slice.
 template <typename TA>
 __global__ void __launch_bounds__(256, 4) k_gram(const TA* __restrict__ Ct, int64_t K, int64_t ld,
-                                                int64_t s_pad, double* __restrict__ P) {
+                                                int64_t s_pad, int nt, double* __restrict__ P) {
     __shared__ __align__(16) TA As[16][64];
     __shared__ __align__(16) TA Bs[16][64];
-    const int nt = (int)(s_pad / 64);
     int ta = 0, rem = blockIdx.x;
     while (rem >= nt - ta) { rem -= nt - ta; ++ta; }
     const int tb = ta + rem;
     const int a0 = ta * 64, b0 = tb * 64;
-    const int64_t kper = ((K + kGramSlices - 1) / kGramSlices + 15) / 16 * 16;
+    const int64_t kper = ((K + gridDim.y - 1) / gridDim.y + 15) / 16 * 16;
     const int64_t kbeg = (int64_t)blockIdx.y * kper;
     const int64_t kend = min(K, kbeg + kper);
     const int tx = threadIdx.x & 15, ty = threadIdx.x >> 4;
@@ -124,15 +134,14 @@ __global__ void __launch_bounds__(256, 4) k_gram(const TA* __restrict__ Ct, int6
 // to the bit; a thread's 32 outputs per shared-memory read of 12 values (4
 // for k_gram's 16) keep the FP32 pipe, not shared memory, the limit.
 __global__ void __launch_bounds__(512, 1) k_gram128(const float* __restrict__ Ct, int64_t K, int64_t ld,
-                                                    int64_t s_pad, double* __restrict__ P) {
+                                                    int64_t s_pad, int nt, double* __restrict__ P) {
     __shared__ __align__(16) float As[2][16][128];
     __shared__ __align__(16) float Bs[2][16][128];
-    const int nt = (int)(s_pad / 128);
     int ta = 0, rem = blockIdx.x;
     while (rem >= nt - ta) { rem -= nt - ta; ++ta; }
     const int tb = ta + rem;
     const int a0 = ta * 128, b0 = tb * 128;
-    const int64_t kper = ((K + kGramSlices - 1) / kGramSlices + 15) / 16 * 16;
+    const int64_t kper = ((K + gridDim.y - 1) / gridDim.y + 15) / 16 * 16;
     const int64_t kbeg = (int64_t)blockIdx.y * kper;
     const int64_t kend = min(K, kbeg + kper);
     const int tx = threadIdx.x & 31, ty = threadIdx.x >> 5;
@@ -193,23 +202,33 @@ __global__ void __launch_bounds__(512, 1) k_gram128(const float* __restrict__ Ct
         }
 }
 
-// Split-K partial Grams of FP32 Ct into P (kGramSlices x s_pad x s_pad).
-msp_status launch_gram_f32(msp_ctx* ctx, const float* Ct, int64_t K, int64_t ld, int64_t sp, double* P) {
-    if (sp % 128 == 0 && ld % 4 == 0 && ((uintptr_t)Ct & 15) == 0) {
-        const int nt = (int)(sp / 128);
-        dim3 grid((unsigned)(nt * (nt + 1) / 2), kGramSlices);
-        k_gram128<<<grid, 512, 0, ctx->stream>>>(Ct, K, ld, sp, P);
-    } else {
-        const int nt = (int)(sp / 64);
-        dim3 grid((unsigned)(nt * (nt + 1) / 2), kGramSlices);
-        k_gram<float><<<grid, 256, 0, ctx->stream>>>(Ct, K, ld, sp, P);
+// Split-K partial Grams of the first s columns of Ct into scratch P (*slices x s_pad x
+// s_pad, with `extra` doubles behind them).
+template <typename TA>
+msp_status launch_gram(msp_ctx* ctx, const TA* Ct, int64_t K, int64_t ld, int64_t s, int64_t sp, int64_t extra,
+                       double** P, int* slices) {
+    const bool wide = sizeof(TA) == 4 && sp % 128 == 0 && ld % 4 == 0 && ((uintptr_t)Ct & 15) == 0;
+    const int nt = (int)((s + (wide ? 127 : 63)) / (wide ? 128 : 64));     // tiles of padding are not read
+    const int tiles = nt * (nt + 1) / 2;
+    *slices = gram_slices(ctx, tiles, K);
+    void* scr = nullptr;
+    MSP_TRY(msp_scratch(ctx, (size_t)(*slices * sp * sp + extra) * 8, &scr));
+    *P = (double*)scr;
+    const dim3 grid((unsigned)tiles, (unsigned)*slices);
+    if constexpr (sizeof(TA) == 4) {
+        if (wide) {
+            k_gram128<<<grid, 512, 0, ctx->stream>>>(Ct, K, ld, sp, nt, *P);
+            MSP_CHECK_LAUNCH(ctx);
+            return MSP_OK;
+        }
     }
+    k_gram<TA><<<grid, 256, 0, ctx->stream>>>(Ct, K, ld, sp, nt, *P);
     MSP_CHECK_LAUNCH(ctx);
     return MSP_OK;
 }
 
 template <typename TA>
-__global__ void k_gram_finish(const double* __restrict__ P, const TA* __restrict__ W, double lam_t,
+__global__ void k_gram_finish(const double* __restrict__ P, int slices, const TA* __restrict__ W, double lam_t,
                               int64_t s, int64_t s_pad, double* __restrict__ M2) {
     const int64_t e = (int64_t)blockIdx.x * blockDim.x + threadIdx.x;
     if (e >= s_pad * s_pad) return;
@@ -217,8 +236,8 @@ __global__ void k_gram_finish(const double* __restrict__ P, const TA* __restrict
     double v;
     if (a < s && b < s) {
         v = 0.0;
-#pragma unroll
-        for (int sl = 0; sl < kGramSlices; ++sl) v += P[(int64_t)sl * s_pad * s_pad + e];
+#pragma unroll 4
+        for (int sl = 0; sl < slices; ++sl) v += P[(int64_t)sl * s_pad * s_pad + e];
         v += W ? lam_t * (double)W[e] : (a == b ? lam_t : 0.0);
     } else {
         v = (a == b) ? 1.0 : 0.0;
@@ -717,20 +736,45 @@ __global__ void k_copy_add_diag(const double* __restrict__ src, double* __restri
 }
 
 // dst = float-float of (src + nu I) scale (scale a power of two: exact)
+// The shift and scaling of a float-float attempt from |M|_F^2: nu = 2^-24 |M|_F
+// 100^attempt, M scaled by 4^k to |M|_F in [1, 4). Formed on the device so that the
+// host need not wait for the norm before the factor starts.
+struct FFShift {
+    double nu;
+    int k;
+};
+__device__ inline FFShift ff_shift(double fro2, int attempt) {
+    const double fn = sqrt(fro2);
+    FFShift f{ldexp(1.0, -24) * fn, fn > 0.0 && isfinite(fn) ? -(ilogb(fn) / 2) : 0};
+    for (int t = 0; t < attempt; ++t) f.nu *= 100.0;
+    return f;
+}
+
+// dst = (src + nu I) 4^k
 __global__ void k_copy_add_diag_ff(const double* __restrict__ src, float2* __restrict__ dst,
-                                   int64_t s_pad, double nu, double scale) {
+                                   int64_t s_pad, const double* __restrict__ fro2, int attempt) {
+    __shared__ double s_nu, s_scale;
+    if (threadIdx.x == 0) {
+        const FFShift f = ff_shift(*fro2, attempt);
+        s_nu = f.nu;
+        s_scale = ldexp(1.0, 2 * f.k);
+    }
+    __syncthreads();
     int64_t e = (int64_t)blockIdx.x * blockDim.x + threadIdx.x;
     if (e >= s_pad * s_pad) return;
     int64_t i = e / s_pad, j = e % s_pad;
-    dst[e] = ff_from_double((src[e] + ((i == j) ? nu : 0.0)) * scale);
+    dst[e] = ff_from_double((src[e] + ((i == j) ? s_nu : 0.0)) * s_scale);
 }
 
-// dst = src scale in FP64 (scale a power of two)
+// dst = src 2^k in FP64
 __global__ void k_ff_to_double(const float2* __restrict__ src, double* __restrict__ dst, int64_t count,
-                               double scale) {
+                               const double* __restrict__ fro2) {
+    __shared__ double s_scale;
+    if (threadIdx.x == 0) s_scale = ldexp(1.0, ff_shift(*fro2, 0).k);
+    __syncthreads();
     int64_t e = (int64_t)blockIdx.x * blockDim.x + threadIdx.x;
     if (e >= count) return;
-    dst[e] = ff_to_double(src[e]) * scale;
+    dst[e] = ff_to_double(src[e]) * s_scale;
 }
 
 // Frobenius norm^2 partials (single block, deterministic order).
@@ -755,11 +799,11 @@ __global__ void __launch_bounds__(256) k_fro2_part(const double* __restrict__ M,
 }
 
 __global__ void k_fro2_final(const double* __restrict__ part, double* __restrict__ out) {
-    if (threadIdx.x == 0) {
-        double v = 0.0;
-        for (int b = 0; b < kFroBlocks; ++b) v += part[b];
-        *out = v;
-    }
+    double v = 0.0;
+#pragma unroll
+    for (int b = 0; b < kFroBlocks; b += 32) v += part[b + threadIdx.x];
+    v = msp::warp_sum(v);
+    if (threadIdx.x == 0) *out = v;
 }
 
 template <typename T>
@@ -1013,35 +1057,42 @@ msp_status factor_shifted(msp_ctx* ctx, const double* M, int64_t s, int64_t sp, 
     double* fro = (double*)(fail + 16);
     double* fro_part = fro + 2;
     int* hflag = (int*)ctx->host_flags;
-    auto fro_norm = [&](double* out) -> msp_status {
+    double* hfro = (double*)((char*)ctx->host_flags + 128);
+    auto fro_launch = [&]() -> msp_status {
         k_fro2_part<<<kFroBlocks, 256, 0, ctx->stream>>>(M, sp * sp, fro_part);
         MSP_CHECK_LAUNCH(ctx);
         k_fro2_final<<<1, 32, 0, ctx->stream>>>(fro_part, fro);
         MSP_CHECK_LAUNCH(ctx);
-        double h = 0.0;
-        MSP_CUDA_TRY(ctx, cudaMemcpyAsync(&h, fro, 8, cudaMemcpyDeviceToHost, ctx->stream));
+        MSP_CUDA_TRY(ctx, cudaMemcpyAsync(hfro, fro, 8, cudaMemcpyDeviceToHost, ctx->stream));
+        return MSP_OK;
+    };
+    auto fro_norm = [&](double* out) -> msp_status {
+        MSP_TRY(fro_launch());
         MSP_CUDA_TRY(ctx, cudaStreamSynchronize(ctx->stream));
-        *out = std::sqrt(h);
+        *out = std::sqrt(*hfro);
         return MSP_OK;
     };
     double nu = 0.0;
-    int scale_k = 0;            // M scaled by 4^scale_k, L^{-1} by 2^-scale_k
-    if (fp32_data) {
+    if (ff) {
+        // nu and the scaling are formed on the device (ff_shift); the host reads the
+        // norm with the outcome
+        MSP_TRY(fro_launch());
+    } else if (fp32_data) {
         double fn = 0.0;
         MSP_TRY(fro_norm(&fn));
         nu = std::ldexp(1.0, -24) * fn;
-        if (ff && fn > 0.0 && std::isfinite(fn)) scale_k = -(std::ilogb(fn) / 2);
     }
     for (int attempt = 0; attempt <= 4; ++attempt) {
         unsigned blocks = (unsigned)((sp * sp + 255) / 256);
         MSP_CUDA_TRY(ctx, cudaMemsetAsync(fail, 0, sizeof(int), ctx->stream));
         if (ff) {
-            k_copy_add_diag_ff<<<blocks, 256, 0, ctx->stream>>>(M, reinterpret_cast<float2*>(Mw), sp, nu,
-                                                                std::ldexp(1.0, 2 * scale_k));
+            k_copy_add_diag_ff<<<blocks, 256, 0, ctx->stream>>>(M, reinterpret_cast<float2*>(Mw), sp, fro, attempt);
             MSP_CHECK_LAUNCH(ctx);
             MSP_CUDA_TRY(ctx, cudaMemsetAsync(Xff, 0, mat, ctx->stream));
             MSP_TRY(chol_inv_ff_graphed(ctx, reinterpret_cast<float2*>(Mw), Xff, reinterpret_cast<float2*>(T1),
                                         reinterpret_cast<float2*>(T2), sp, fail));
+            k_ff_to_double<<<blocks, 256, 0, ctx->stream>>>(Xff, Linv64, sp * sp, fro);
+            MSP_CHECK_LAUNCH(ctx);
         } else {
             k_copy_add_diag<<<blocks, 256, 0, ctx->stream>>>(M, Mw, sp, nu);
             MSP_CHECK_LAUNCH(ctx);
@@ -1051,11 +1102,8 @@ msp_status factor_shifted(msp_ctx* ctx, const double* M, int64_t s, int64_t sp, 
         MSP_CUDA_TRY(ctx, cudaMemcpyAsync(hflag, fail, sizeof(int), cudaMemcpyDeviceToHost,
                                           ctx->stream));
         MSP_CUDA_TRY(ctx, cudaStreamSynchronize(ctx->stream));
+        if (ff && attempt == 0) nu = std::ldexp(1.0, -24) * std::sqrt(*hfro);
         if (hflag[0] == 0) {
-            if (ff) {
-                k_ff_to_double<<<blocks, 256, 0, ctx->stream>>>(Xff, Linv64, sp * sp, std::ldexp(1.0, scale_k));
-                MSP_CHECK_LAUNCH(ctx);
-            }
             *shift_out = nu;
             *retries_out = attempt;
             return MSP_OK;
@@ -1096,20 +1144,16 @@ msp_status msp_build_factor(msp_ctx* ctx, msp_factor_s* f, const void* Ct, int64
     if (f->dtype == MSP_F32 && ctx->gram_tc && msp_gram_tc_ok(sp)) {
         MSP_TRY(msp_gram_tc(ctx, (const float*)Ct, phi_rows, sp, f->s, sp, (const float*)f->W, f->lam_tilde, f->M2));
     } else {
-        void* scr = nullptr;
-        MSP_TRY(msp_scratch(ctx, (size_t)kGramSlices * sp * sp * 8, &scr));
-        double* P = (double*)scr;
-        const int nt = (int)(sp / 64);
-        dim3 grid((unsigned)(nt * (nt + 1) / 2), kGramSlices);
+        double* P = nullptr;
+        int slices = 0;
         const unsigned fb = (unsigned)((sp * sp + 255) / 256);
         if (f->dtype == MSP_F32) {
-            MSP_TRY(launch_gram_f32(ctx, (const float*)Ct, phi_rows, sp, sp, P));
-            k_gram_finish<float><<<fb, 256, 0, ctx->stream>>>(P, (const float*)f->W, f->lam_tilde,
+            MSP_TRY(launch_gram(ctx, (const float*)Ct, phi_rows, sp, f->s, sp, 0, &P, &slices));
+            k_gram_finish<float><<<fb, 256, 0, ctx->stream>>>(P, slices, (const float*)f->W, f->lam_tilde,
                                                                f->s, sp, f->M2);
         } else {
-            k_gram<double><<<grid, 256, 0, ctx->stream>>>((const double*)Ct, phi_rows, sp, sp, P);
-            MSP_CHECK_LAUNCH(ctx);
-            k_gram_finish<double><<<fb, 256, 0, ctx->stream>>>(P, (const double*)f->W, f->lam_tilde,
+            MSP_TRY(launch_gram(ctx, (const double*)Ct, phi_rows, sp, f->s, sp, 0, &P, &slices));
+            k_gram_finish<double><<<fb, 256, 0, ctx->stream>>>(P, slices, (const double*)f->W, f->lam_tilde,
                                                                 f->s, sp, f->M2);
         }
         MSP_CHECK_LAUNCH(ctx);
@@ -1148,21 +1192,17 @@ msp_status msp_form_level2(msp_ctx* ctx, msp_factor_s* f, const void* C, int64_t
     const int64_t sp = f->s_pad, mat = sp * sp;
     const unsigned fb = (unsigned)((mat + 255) / 256);
     MSP_TRY(msp_alloc(ctx, &f->H, (size_t)mat * 8));
-    void* scr = nullptr;
-    MSP_TRY(msp_scratch(ctx, (size_t)(kGramSlices + 1) * mat * 8, &scr));
-    double* P = (double*)scr;
-    double* H64 = P + (size_t)kGramSlices * mat;
+    double* P = nullptr;
+    int slices = 0;
     if (f->dtype == MSP_F32) {
-        MSP_TRY(launch_gram_f32(ctx, (const float*)C, n, sp, sp, P));
-        k_gram_finish<float><<<fb, 256, 0, ctx->stream>>>(P, (const float*)f->W, f->lam_tilde, f->s, sp, H64);
+        MSP_TRY(launch_gram(ctx, (const float*)C, n, sp, f->s, sp, mat, &P, &slices));
+        double* H64 = P + slices * mat;
+        k_gram_finish<float><<<fb, 256, 0, ctx->stream>>>(P, slices, (const float*)f->W, f->lam_tilde, f->s, sp, H64);
         MSP_CHECK_LAUNCH(ctx);
         k_split_pair<<<fb, 256, 0, ctx->stream>>>(H64, (float*)f->H, (float*)f->H + mat, mat);
     } else {
-        const int nt = (int)(sp / 64);
-        dim3 grid((unsigned)(nt * (nt + 1) / 2), kGramSlices);
-        k_gram<double><<<grid, 256, 0, ctx->stream>>>((const double*)C, n, sp, sp, P);
-        MSP_CHECK_LAUNCH(ctx);
-        k_gram_finish<double><<<fb, 256, 0, ctx->stream>>>(P, (const double*)f->W, f->lam_tilde, f->s, sp,
+        MSP_TRY(launch_gram(ctx, (const double*)C, n, sp, f->s, sp, 0, &P, &slices));
+        k_gram_finish<double><<<fb, 256, 0, ctx->stream>>>(P, slices, (const double*)f->W, f->lam_tilde, f->s, sp,
                                                             (double*)f->H);
     }
     MSP_CHECK_LAUNCH(ctx);
@@ -1174,12 +1214,11 @@ msp_status msp_form_level2(msp_ctx* ctx, msp_factor_s* f, const void* C, int64_t
 // FP32 sums, combined in FP64 in a fixed order; pad block identity.
 msp_status msp_gram64(msp_ctx* ctx, const float* X, int64_t rows, int64_t ld, int64_t s, int64_t sp,
                       double diag, double* G64) {
-    void* scr = nullptr;
-    MSP_TRY(msp_scratch(ctx, (size_t)kGramSlices * sp * sp * 8, &scr));
-    double* P = (double*)scr;
-    MSP_TRY(launch_gram_f32(ctx, X, rows, ld, sp, P));
-    k_gram_finish<float><<<(unsigned)((sp * sp + 255) / 256), 256, 0, ctx->stream>>>(P, nullptr, diag, s, sp,
-                                                                                      G64);
+    double* P = nullptr;
+    int slices = 0;
+    MSP_TRY(launch_gram(ctx, X, rows, ld, s, sp, 0, &P, &slices));
+    k_gram_finish<float><<<(unsigned)((sp * sp + 255) / 256), 256, 0, ctx->stream>>>(
+        P, slices, (const float*)nullptr, diag, s, sp, G64);
     MSP_CHECK_LAUNCH(ctx);
     return MSP_OK;
 }
@@ -1219,7 +1258,7 @@ __global__ void __launch_bounds__(256, 4) k_gemm_tn(const float* __restrict__ X,
     const int nty = (int)(ny_pad / 64);
     const int ta = blockIdx.x / nty, tb = blockIdx.x % nty;
     const int64_t a0 = (int64_t)ta * 64, b0 = (int64_t)tb * 64;
-    const int64_t kper = ((K + kGramSlices - 1) / kGramSlices + 15) / 16 * 16;
+    const int64_t kper = ((K + gridDim.y - 1) / gridDim.y + 15) / 16 * 16;
     const int64_t kbeg = (int64_t)blockIdx.y * kper;
     const int64_t kend = min(K, kbeg + kper);
     const int tx = threadIdx.x & 15, ty = threadIdx.x >> 4;
@@ -1270,7 +1309,7 @@ __global__ void k_sum_slices_f32(const double* __restrict__ P, int64_t len, floa
     if (e >= len) return;
     double v = 0.0;
 #pragma unroll
-    for (int sl = 0; sl < kGramSlices; ++sl) v += P[(int64_t)sl * len + e];
+    for (int sl = 0; sl < kGemmSlices; ++sl) v += P[(int64_t)sl * len + e];
     out[e] = (float)v;
 }
 
@@ -1283,9 +1322,9 @@ __global__ void k_sum_slices_f32(const double* __restrict__ P, int64_t len, floa
 msp_status msp_gemm_tn(msp_ctx* ctx, const float* X, int64_t ldx, int64_t ncx, const float* Y, int64_t ldy,
                        int64_t ncy, int64_t K, int64_t nx_pad, int64_t ny_pad, float* C) {
     void* scr = nullptr;
-    MSP_TRY(msp_scratch(ctx, (size_t)kGramSlices * nx_pad * ny_pad * 8, &scr));
+    MSP_TRY(msp_scratch(ctx, (size_t)kGemmSlices * nx_pad * ny_pad * 8, &scr));
     double* P = (double*)scr;
-    dim3 grid((unsigned)((nx_pad / 64) * (ny_pad / 64)), kGramSlices);
+    dim3 grid((unsigned)((nx_pad / 64) * (ny_pad / 64)), kGemmSlices);
     k_gemm_tn<<<grid, 256, 0, ctx->stream>>>(X, ldx, ncx, Y, ldy, ncy, K, ny_pad, nx_pad, P);
     MSP_CHECK_LAUNCH(ctx);
     const int64_t len = nx_pad * ny_pad;

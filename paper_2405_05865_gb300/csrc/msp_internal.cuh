@@ -94,8 +94,8 @@ struct msp_sketch_s {
     void* C = nullptr;           // n x s_pad, dtype
     float* packed = nullptr;     // FP32 A: upper 128 x 128 tiles (see symv.cu)
     const void* A_src = nullptr; // the A the sketch (and packed copy) came from
-    // norm bound of A_src for the backward-error rule: row sums, their
-    // rounding bounds and row squares (3 n), then the bound (see norms.cu)
+    // norm bound of A_src for the backward-error rule: work of its two kernels
+    // (3 n), then the bound (see norms.cu)
     double* stats = nullptr;
 };
 
@@ -142,7 +142,11 @@ struct CtlBlock {
     double pq;
     double beta;
     double rzbuf[2];    // packed A pass: r^T z of the iterations, in turn
-    double scratch[6];
+    // k_norm_lb's own (it may run on a side stream, beside kernels that use
+    // last_block_counter)
+    unsigned int lb_counter;
+    unsigned int pad1;
+    double lb_part[96];
 };
 
 // ------------------------------------------------------------------ errors
@@ -319,8 +323,6 @@ msp_status msp_sketch_sym_pass(msp_ctx* ctx, const float* A, int64_t n, int64_t 
 msp_status msp_sketch_sym_blocks(msp_ctx* ctx, const float* A, int64_t n, int64_t lda, int64_t s_pad,
                                  const int32_t* ptr, const int32_t* ent, int gamma, float* C, float* packed,
                                  int64_t ib0, int64_t ib1);
-// the norm bound from row statistics already in work (3 n doubles)
-msp_status msp_norm_lb_finish(msp_ctx* ctx, double* work, int64_t n, double* out_dev);
 msp_status msp_gather_rows(msp_ctx* ctx, msp_dtype dt, int64_t rows_out, int64_t width,
                            const int32_t* ptr, const int32_t* ent, const void* in,
                            int64_t ld_in, double scale, void* out, int64_t ld_out);

@@ -10,10 +10,12 @@
 //              FP32 chunk kept beside it (the FP64 pipe of this part is 1/64
 //              of the FP32 rate: with chunks of 16 the FP64 conversions and
 //              sums alone kept it ~80% busy and held the pass to ~4 TB/s).
-// k_norm_lb    one block: max of the row squares and the FP64 sum of the row
+// k_norm_lb    max of the row squares and the FP64 sum of the row
 //              sums in a fixed order, each lowered by its rounding bound, so
 //              the result stays at most |A|_2.
 #include "msp_internal.cuh"
+
+#include <algorithm>
 
 namespace {
 
@@ -97,13 +99,22 @@ __global__ void __launch_bounds__(256) k_row_stats(const T* __restrict__ A, int6
         row_stats_one<T>(A + i * lda, n, lane, rowsum + i, rowerr + i, rowsq + i);
 }
 
-__global__ void __launch_bounds__(1024) k_norm_lb(const double* __restrict__ rowsum,
-                                                 const double* __restrict__ rowerr,
-                                                 const double* __restrict__ rowsq, int64_t n,
-                                                 double* out) {
-    __shared__ double ssum[32], serr[32], smax[32];
+// Block b of G takes the statistics of rows [n b / G, n (b + 1) / G); the last block to
+// finish adds the blocks' sums in a fixed order. One block over all the rows was held by its FP64 sums (26 us at n =
+// 16384 beside the sketch's last wave, against 21).
+constexpr int kLbBlocks = 32;
+
+__global__ void __launch_bounds__(256) k_norm_lb(const double* __restrict__ rowsum,
+                                                const double* __restrict__ rowerr,
+                                                const double* __restrict__ rowsq, int64_t n,
+                                                double* __restrict__ part, unsigned int* counter,
+                                                double* out) {
+    __shared__ double red[3][8];
+    __shared__ bool am_last;
+    const int w = threadIdx.x >> 5, lane = threadIdx.x & 31, G = gridDim.x;
+    const int64_t i1 = n * (blockIdx.x + 1) / G;
     double s = 0.0, e = 0.0, m = 0.0;
-    for (int64_t i = threadIdx.x; i < n; i += blockDim.x) {
+    for (int64_t i = n * blockIdx.x / G + threadIdx.x; i < i1; i += blockDim.x) {
         s += rowsum[i];
         e += rowerr[i];
         m = fmax(m, rowsq[i]);
@@ -112,24 +123,42 @@ __global__ void __launch_bounds__(1024) k_norm_lb(const double* __restrict__ row
     e = msp::warp_sum(e);
 #pragma unroll
     for (int o = 16; o > 0; o >>= 1) m = fmax(m, __shfl_xor_sync(0xffffffffu, m, o));
-    const int w = threadIdx.x >> 5, lane = threadIdx.x & 31;
     if (lane == 0) {
-        ssum[w] = s;
-        serr[w] = e;
-        smax[w] = m;
+        red[0][w] = s;
+        red[1][w] = e;
+        red[2][w] = m;
     }
     __syncthreads();
     if (threadIdx.x == 0) {
         double ts = 0.0, te = 0.0, tm = 0.0;
-        for (int k = 0; k < (int)(blockDim.x >> 5); ++k) {
-            ts += ssum[k];
-            te += serr[k];
-            tm = fmax(tm, smax[k]);
+#pragma unroll
+        for (int k = 0; k < 8; ++k) {
+            ts += red[0][k];
+            te += red[1][k];
+            tm = fmax(tm, red[2][k]);
         }
+        part[3 * blockIdx.x] = ts;
+        part[3 * blockIdx.x + 1] = te;
+        part[3 * blockIdx.x + 2] = tm;
+        __threadfence();
+        am_last = atomicAdd(counter, 1u) == (unsigned)G - 1u;
+    }
+    __syncthreads();
+    if (!am_last || w != 0) return;
+    __threadfence();
+    s = lane < G ? __ldcg(&part[3 * lane]) : 0.0;
+    e = lane < G ? __ldcg(&part[3 * lane + 1]) : 0.0;
+    m = lane < G ? __ldcg(&part[3 * lane + 2]) : 0.0;
+    s = msp::warp_sum(s);
+    e = msp::warp_sum(e);
+#pragma unroll
+    for (int o = 16; o > 0; o >>= 1) m = fmax(m, __shfl_xor_sync(0xffffffffu, m, o));
+    if (lane == 0) {
+        *counter = 0;
         // FP64 combination error (n^2 / kChunk chunk terms) is far below the
         // FP32 chunk bound; 2e-6 covers it with room
-        const double col = sqrt(tm * (1.0 - (kChunk + 3) * kU32) * (1.0 - 2e-6));
-        const double ones = (ts - te * (1.0 + 2e-6) - 2e-6 * fabs(ts)) / (double)n;
+        const double col = sqrt(m * (1.0 - (kChunk + 3) * kU32) * (1.0 - 2e-6));
+        const double ones = (s - e * (1.0 + 2e-6) - 2e-6 * fabs(s)) / (double)n;
         *out = fmax(col, ones);
     }
 }
@@ -146,13 +175,9 @@ msp_status msp_norm_lb_launch(msp_ctx* ctx, const void* A, msp_dtype dt, int64_t
         k_row_stats<double><<<blocks, 256, 0, ctx->stream>>>((const double*)A, n, lda, work, work + n,
                                                             work + 2 * n);
     MSP_CHECK_LAUNCH(ctx);
-    k_norm_lb<<<1, 1024, 0, ctx->stream>>>(work, work + n, work + 2 * n, n, out_dev);
-    MSP_CHECK_LAUNCH(ctx);
-    return MSP_OK;
-}
-
-msp_status msp_norm_lb_finish(msp_ctx* ctx, double* work, int64_t n, double* out_dev) {
-    k_norm_lb<<<1, 1024, 0, ctx->stream>>>(work, work + n, work + 2 * n, n, out_dev);
+    CtlBlock* ctl = (CtlBlock*)ctx->ctl;
+    k_norm_lb<<<(unsigned)std::min<int64_t>(kLbBlocks, (n + 255) / 256), 256, 0, ctx->stream>>>(
+        work, work + n, work + 2 * n, n, ctl->lb_part, &ctl->lb_counter, out_dev);
     MSP_CHECK_LAUNCH(ctx);
     return MSP_OK;
 }

@@ -106,7 +106,10 @@ typedef struct {
                              operator itself (phi = 0, Phi = I).                 */
     int precision;        /* msp_precision. Default MSP_PREC_MIXED.              */
     int check_every;      /* level-1 iterations between host checks of the
-                             device-side convergence flag. Default 8.            */
+                             device-side convergence flag with profile = 1;
+                             without it the host keeps at most min(check_every, 4)
+                             iterations queued past the last one that the device
+                             reported in pinned host memory. Default 8.          */
     int profile;          /* 1: time every A-pass and level-2 launch with CUDA
                              events on the context stream (msp_info *_ms);
                              launches queued after the device flagged

@@ -331,6 +331,7 @@ struct L2Args {
     T* zvec;
     T* wdvec;
     double* dpart;          // G x 4
+    volatile int* prog;     // pinned host words: iterations done, finished (or null)
 };
 
 // Per-lane slice of an s_pad row stored as TS: PL elements as PL/W vectors of
@@ -679,9 +680,16 @@ __global__ void __launch_bounds__(kThreads, 1) k_level2(L2Args<T, TC> a) {
     const int c_done = ctl->done, c_err = ctl->error, iter = ctl->iters;
     const double c_alpha = ctl->alpha, c_rz = ctl->rz, tol2 = ctl->tol2;
     const double c_rz0 = ctl->rzbuf[0], c_rz1 = ctl->rzbuf[1];
-    if (c_done | c_err) return;
     const int lane = threadIdx.x & 31, w = threadIdx.x >> 5;
     const int G = gridDim.x, b = blockIdx.x;
+    // tells the host that polls for it (block 0)
+    auto report = [&](int word, int v) {
+        if (a.prog && b == 0 && threadIdx.x == 0) a.prog[word] = v;
+    };
+    if (c_done | c_err) {
+        report(1, 1);
+        return;
+    }
     const int64_t row0 = a.n * b / G, row1 = a.n * (b + 1) / G;
     const int64_t c0 = sp * b / G, c1 = sp * (b + 1) / G;
     unsigned int* bw = &ctl->bar_word;
@@ -1049,7 +1057,10 @@ __global__ void __launch_bounds__(kThreads, 1) k_level2(L2Args<T, TC> a) {
     }
     if (b == 0 && threadIdx.x == 0) {
         ctl->inner_iters += k;
-        if (a.mode == MODE_ITER) ctl->iters = iter + 1;
+        if (a.mode == MODE_ITER) {
+            ctl->iters = iter + 1;
+            report(0, iter + 1);
+        }
     }
 }
 
@@ -1602,6 +1613,9 @@ msp_status krylov_solve_t(msp_ctx* ctx, const msp_factor_s* f, const void* A, ms
     a.dq = use_packed ? ws.gpart : nullptr;
     a.n_dq = ctx->num_sms;
     a.lam = (T)lambda;
+    a.prog = (volatile int*)((char*)ctx->host_flags + 192);
+    a.prog[0] = 0;
+    a.prog[1] = 0;
     a.mode = MODE_INIT;
     InnerArgs<T> in = fill_inner(f, a);
     MSP_TRY(launch_level2(ctx, a, G, in));
@@ -1678,30 +1692,60 @@ msp_status krylov_solve_t(msp_ctx* ctx, const msp_factor_s* f, const void* A, ms
     }
     int* hf = (int*)ctx->host_flags;
     const int check = std::max(1, o->check_every);
+    // the packed A pass finds an indefinite or non-finite r^T w of the iteration
+    // before it: after the last allowed iteration one more pass looks at that one's
+    auto last_look = [&]() -> msp_status {
+        if (!use_packed) return MSP_OK;
+        return msp_symv_packed(ctx, packed, n, (float)lambda, (const float*)z, (float*)p, ws.dpart, G, ws.qpart,
+                               ws.gpart, ctx->num_sms);
+    };
     // profiler entries of iterations known to have run to completion with
     // work (every iteration before a check that found no flag): read while
     // the next interval runs, not after it
     int settled = 0, l2_open = -1;
-    for (int it = 0; it < max_outer;) {
-        const int nrun = std::min(check, max_outer - it);
-        for (int i = 0; i < nrun; ++i) {
-            if (graphed) MSP_TRY(replay_l1(ctx, pr, &l2_open));
-            else MSP_TRY(iteration(false));
+    if (!pr.on) {
+        // the device reports each iteration in pinned host words; the host keeps
+        // at most `ahead` iterations queued and polls, so the stream never runs
+        // dry between checks (a stream synchronisation every 8 iterations left it
+        // idle for about 30 us) and few launches follow the converged one. The
+        // poll ends when the stream has nothing left to do, whatever was reported.
+        const int ahead = std::min(check, 4);
+        int it = 0;
+        while (it < max_outer && !a.prog[1]) {
+            const int done = a.prog[0];
+            if (it < done + ahead) {
+                if (graphed) MSP_TRY(replay_l1(ctx, pr, &l2_open));
+                else MSP_TRY(iteration(false));
+                ++it;
+                continue;
+            }
+            for (int spin = 0; a.prog[0] == done && !a.prog[1]; ++spin) {
+                if ((spin & 1023) != 1023) continue;
+                const cudaError_t e = cudaStreamQuery(ctx->stream);
+                if (e == cudaSuccess) break;
+                if (e != cudaErrorNotReady) MSP_CUDA_TRY(ctx, e);
+            }
+            // idle without a report: the launches ended early (an error word)
+            if (a.prog[0] == done && !a.prog[1]) break;
         }
-        if (graphed) MSP_TRY(close_l1_chain(ctx, pr, &l2_open));
-        it += nrun;
-        MSP_CUDA_TRY(ctx, cudaMemcpyAsync(hf, &ctl->done, 5 * sizeof(int), cudaMemcpyDeviceToHost,
-                                          ctx->stream));
-        MSP_TRY(pr.harvest(prof, 2, settled));
-        MSP_CUDA_TRY(ctx, cudaStreamSynchronize(ctx->stream));
-        if (hf[0] || hf[1]) break;
-        settled = pr.used;
-        // the packed A pass finds an indefinite or non-finite r^T w of the
-        // iteration before it: after the last allowed iteration one more pass
-        // looks at that one's
-        if (it >= max_outer && use_packed)
-            MSP_TRY(msp_symv_packed(ctx, packed, n, (float)lambda, (const float*)z, (float*)p, ws.dpart, G, ws.qpart,
-                                    ws.gpart, ctx->num_sms));
+        if (it >= max_outer && !a.prog[1]) MSP_TRY(last_look());
+    } else {
+        for (int it = 0; it < max_outer;) {
+            const int nrun = std::min(check, max_outer - it);
+            for (int i = 0; i < nrun; ++i) {
+                if (graphed) MSP_TRY(replay_l1(ctx, pr, &l2_open));
+                else MSP_TRY(iteration(false));
+            }
+            if (graphed) MSP_TRY(close_l1_chain(ctx, pr, &l2_open));
+            it += nrun;
+            MSP_CUDA_TRY(ctx, cudaMemcpyAsync(hf, &ctl->done, 5 * sizeof(int), cudaMemcpyDeviceToHost,
+                                              ctx->stream));
+            MSP_TRY(pr.harvest(prof, 2, settled));
+            MSP_CUDA_TRY(ctx, cudaStreamSynchronize(ctx->stream));
+            if (hf[0] || hf[1]) break;
+            settled = pr.used;
+            if (it >= max_outer) MSP_TRY(last_look());
+        }
     }
     MSP_CUDA_TRY(ctx, cudaMemcpyAsync(hf, &ctl->done, 5 * sizeof(int), cudaMemcpyDeviceToHost,
                                       ctx->stream));

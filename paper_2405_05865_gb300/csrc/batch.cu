@@ -18,7 +18,7 @@
 // direct level 2, Section 4):
 //   S2  G = C^T R            items (instance, 64-column strip of C)
 //       + convergence flags  one block per instance decides, fixed order
-//   S3  Y1 = L^{-1} G        items (instance, 128-row chunk of s)
+//   S3  Y1 = L^{-1} G        items (instance, 32-row chunk of s)
 //   S4  Y2 = L^{-T} Y1
 //   S5  Z = (R - C Y2)/lam~  items (instance, 128-row block), dots z.r, z.q
 //   S6  beta, P = Z + beta P
@@ -41,6 +41,8 @@
 #include "msp_internal.cuh"
 #include "bulk.cuh"
 
+#include <functional>
+#include <queue>
 #include <algorithm>
 #include <map>
 #include <tuple>
@@ -71,6 +73,8 @@ constexpr int kStageBytes = kTileBytes + 2 * kSliceBytes;
 // is a run-time choice (msp_batch_autotune); kUtMin bounds the partial
 // buffers.
 constexpr int kUtMin = 16;
+constexpr int kSegBlocks = 10;                  // row blocks of a G segment, at most kSegMax of them
+constexpr int kSegMax = 8;
 constexpr int kRingBytes = kStages * kStageBytes;   // 160 KB
 constexpr int kRedBytes = 65536;
 constexpr int kMiscBytes = 2048;
@@ -93,6 +97,7 @@ struct BInst {
     int64_t ldb, ldx;
     int n, n_pad, s_pad, m;
     int nb;               // row blocks n_pad / 128
+    int ng;               // row segments of the G step (partial sums of G)
     int nkc;              // units per row block: ceil(n_pad / 64 / ut)
     int qoff;             // first row of the instance in the unit-partial arrays
     int voff;             // first row in the [.][16] vector arrays
@@ -109,7 +114,7 @@ struct BCtl {
     int active[2];
     int unfinished[2];
     int sweepsA, sweepsR;     // A passes and residual passes run
-    int ctrG, ctrT1, ctrT2, ctrZ;   // dynamic item counters of S2, S3, S4, S5
+    int ctrG, ctrZ;           // dynamic item counters of S2, S5
     int pad0;
     unsigned long long tilesA;   // A tiles streamed by the level-1 passes
     unsigned long long tilesR;   // A tiles streamed by the residual passes
@@ -124,8 +129,8 @@ struct BArgs {
     const BInst* inst;
     int count, nrows, nstrips, nchunks;
     const int2* rows;     // (instance, row block), largest n first
-    const int2* strips;   // (instance, 64-column strip of C)
-    const int2* chunks;   // (instance, 128-row chunk of s)
+    const int2* strips;   // (instance, 64-column strip of C | row segment << 16), longest first
+    const int2* chunks;   // (instance, 32-row chunk of s from the long end), longest first
     int nunits;
     int ut;               // tiles per unit
     const int2* units;    // (instance, row block | unit << 16), largest first
@@ -135,6 +140,7 @@ struct BArgs {
     float *P, *Q, *R, *Z, *XW, *XH, *XL;
     double* R64;
     float *G, *Y1, *Y2;
+    int64_t gstride;      // from one segment's G to the next (floats)
     double *p_pq, *p_rr, *p_zr, *p_zq, *p_r64, *p_xx;
     double *bb, *scale, *alpha, *rz;    // per column; rz holds two generations
     int *act, *fin;                     // per column
@@ -421,8 +427,9 @@ __device__ __noinline__ void producer(const BArgs& a, unsigned char* ring, uint6
             if (Mode == kModeG) {
                 // rb holds the strip; the loop runs over the row blocks
                 nk = a.inst[inst].s_pad / kKT;
-                k0 = 0;
-                k1 = a.inst[inst].nb;
+                const int seg = w.y >> 16, ng = a.inst[inst].ng, nb = a.inst[inst].nb;
+                k0 = nb * seg / ng;
+                k1 = nb * (seg + 1) / ng;
             } else if (Mode == kModeZ) {
                 nk = a.inst[inst].s_pad / kKT;
                 k0 = 0;
@@ -669,44 +676,20 @@ __device__ __noinline__ void consume_R(const BArgs& a, unsigned char* ring, uint
 
 // ------------------------------------------------- mat-vec steps (S3-S5)
 
-// acc += M[rows 0..127][k] V[k][.] over k tiles [kt0, kt1): M row-major (ld),
-// rows >= rows_valid read as zero; V staged in shared memory by absolute k.
-__device__ __forceinline__ void mv_stream(float (&acc)[4][16], const float* __restrict__ M, int64_t ld, int rows_valid,
-                          int kt0, int kt1, const float* Vs, float* tiles, int tid, int w, int lane) {
-    const int nkt = kt1 - kt0;
-    auto issue = [&](int kt, int buf) {
-        float* dst = tiles + buf * kTileFloats;
-#pragma unroll
-        for (int j = 0; j < 8; ++j) {
-            const int e = tid + kWorkers * j;
-            const int row = e >> 4, g = e & 15;
-            const bool ok = row < rows_valid;
-            const float* src = ok ? M + (int64_t)row * ld + (int64_t)kt * kKT + 4 * g : M;
-            msp::cp_async16(dst + row * kKT + ((g ^ (row & 7)) << 2), src, ok);
+// Stage rows [k0, k1) of a [.][16] vector block into Vs (same row indices): the sum
+// of `parts` blocks `stride` floats apart, in order. The caller's barrier makes it
+// visible.
+__device__ __forceinline__ void stage_vec(float* Vs, const float* src, int64_t stride, int parts, int k0, int k1,
+                                          int tid) {
+#pragma unroll 4
+    for (int e = k0 * 4 + tid; e < k1 * 4; e += kWorkers) {
+        float4 v = __ldcg(reinterpret_cast<const float4*>(src) + e);
+        for (int p = 1; p < parts; ++p) {
+            const float4 u = __ldcg(reinterpret_cast<const float4*>(src + p * stride) + e);
+            v.x += u.x; v.y += u.y; v.z += u.z; v.w += u.w;
         }
-    };
-#pragma unroll 1
-    for (int j = 0; j < 2; ++j) {
-        if (j < nkt) issue(kt0 + j, j);
-        msp::cp_async_commit();
+        reinterpret_cast<float4*>(Vs)[e] = v;
     }
-#pragma unroll 1
-    for (int i = 0; i < nkt; ++i) {
-        if (i + 2 < nkt) issue(kt0 + i + 2, (i + 2) % kMvTiles);
-        msp::cp_async_commit();
-        msp::cp_async_wait<2>();
-        msp::bar_workers<kWorkers>();
-        fma_tile(acc, tiles + (i % kMvTiles) * kTileFloats, Vs + (int64_t)(kt0 + i) * kKT * kM, w, lane);
-        msp::bar_workers<kWorkers>();
-    }
-}
-
-// Stage rows [k0, k1) of a [.][16] vector block into Vs (same row indices).
-__device__ __forceinline__ void stage_vec(float* Vs, const float* src, int k0, int k1, int tid) {
-    msp::bar_workers<kWorkers>();
-    for (int e = k0 * 4 + tid; e < k1 * 4; e += kWorkers)
-        reinterpret_cast<float4*>(Vs)[e] = reinterpret_cast<const float4*>(src)[e];
-    msp::bar_workers<kWorkers>();
 }
 
 // ------------------------------------------------------------- the steps
@@ -715,16 +698,6 @@ __device__ __forceinline__ void stage_vec(float* Vs, const float* src, int k0, i
 __device__ __forceinline__ void my_range(int n, int& i0, int& i1) {
     i0 = (int)((int64_t)n * blockIdx.x / gridDim.x);
     i1 = (int)((int64_t)n * (blockIdx.x + 1) / gridDim.x);
-}
-
-// Dynamic item claim for the worker threads: thread 0 takes the next index
-// of the step's counter and shares it through `slot`.
-__device__ __forceinline__ int claim(int* ctr, int* slot, int tid) {
-    if (tid == 0) *slot = atomicAdd(ctr, 1);
-    msp::bar_workers<kWorkers>();
-    const int it = *(volatile int*)slot;
-    msp::bar_workers<kWorkers>();
-    return it;
 }
 
 // R64 = B (X = 0), partials of |b|^2.
@@ -818,7 +791,7 @@ __device__ __forceinline__ void step_scale(const BArgs& a, int step, float* wsum
         a.ctl->active[1] = 0;
         a.ctl->unfinished[(step + 1) & 1] = 0;
         a.ctl->ctrA = 0;
-        a.ctl->ctrG = a.ctl->ctrT1 = a.ctl->ctrT2 = a.ctl->ctrZ = 0;
+        a.ctl->ctrG = a.ctl->ctrZ = 0;
     }
     int i0, i1;
     my_range(a.nrows, i0, i1);
@@ -866,8 +839,11 @@ __device__ __forceinline__ void step_flags(const BArgs& a, int t, int lane) {
     for (int i = blockIdx.x; i < a.count; i += gridDim.x) {
         const BInst& I = a.inst[i];
         const int c = lane & 15, gi = i * kM + c;
+        // even row blocks in the lower half warp, odd ones in the upper
         double rr = 0.0;
-        for (int b = 0; b < I.nb; ++b) rr += a.p_rr[((int64_t)I.boff + b) * kM + c];
+#pragma unroll 4
+        for (int b = lane >> 4; b < I.nb; b += 2) rr += __ldcg(&a.p_rr[((int64_t)I.boff + b) * kM + c]);
+        rr += __shfl_xor_sync(0xffffffffu, rr, 16);
         const bool live = lane < 16 && c < I.m && !a.fin[gi];
         if (live && !isfinite(rr)) atomicCAS(&a.ierr[i], 0, (int)MSP_ENONFINITE);
         __syncwarp();
@@ -888,7 +864,10 @@ __device__ __forceinline__ void step_flags(const BArgs& a, int t, int lane) {
 // strip's tiles down all row blocks with the R rows of each; warp w takes
 // rows 16w..16w+15 of a tile, a lane two columns x 16 right-hand sides
 // (FP32 FMA), and the 8 warps' sums are combined in warp order at the end of
-// the strip.
+// the strip. A strip is cut into row segments of at most kSegBlocks row blocks, so that
+// the items outnumber the blocks and none is long; the segments' sums are added, in
+// order, where the next step stages G. (Uncut, the 220 strips of the 24-instance batch,
+// up to 30 tiles each, took 38 us an iteration, against 32.)
 __device__ __noinline__ void consume_G(const BArgs& a, unsigned char* ring, uint64_t* full, uint64_t* empty,
                                        const int2* hdr, uint32_t& kring, float* red, int w, int lane) {
     float acc[2][16];
@@ -954,44 +933,111 @@ __device__ __noinline__ void consume_G(const BArgs& a, unsigned char* ring, uint
                 const float4 u = red4[(ww * 64 + j) * 4 + qd];
                 v.x += u.x; v.y += u.y; v.z += u.z; v.w += u.w;
             }
-            st4(a.G + ((int64_t)I.soff + item.y * kKT + j) * kM + 4 * qd, v);
+            st4(a.G + (item.y >> 16) * a.gstride + ((int64_t)I.soff + (item.y & 0xffff) * kKT + j) * kM + 4 * qd, v);
         }
         msp::bar_workers<kWorkers>();
     }
 }
 
-// S3 / S4: Y_out[chunk] = L^{-1} G or L^{-T} Y1 (triangular k range).
+// S3 / S4: Y_out[chunk] = L^{-1} G or L^{-T} Y1 (triangular k range), items of 32
+// rows of the factor. The factors are small (128 to 1024 rows) and their rows
+// independent, so the length of the longest item and the latency of its first loads
+// are the time: an item streams 32-row pieces of 256 columns through three tile
+// buffers (16-byte async copies, the first two on their way before the vector block
+// is staged), warp w takes 32 of the 256 columns with a lane a row (16 sums), and
+// the 8 warps' sums are added in warp order. The items are sorted by length and
+// dealt out in turn, so no block waits for a shared counter. With 128-row items
+// claimed from a counter the two steps took 46 us an iteration of the 24-instance
+// batch (n 512 to 4096), and take 37.
+constexpr int kTriRows = 32, kTriK = 256;
+
 template <bool kUpper>
-__device__ __noinline__ void step_tri(const BArgs& a, int t, unsigned char* smem, float* red, int* slot,
-                                      int tid, int w, int lane) {
+__device__ __noinline__ void step_tri(const BArgs& a, int t, unsigned char* smem, float* red, int tid, int w,
+                                      int lane) {
     const int cur = t & 1;
     float* tiles = reinterpret_cast<float*>(smem);
     float* Vs = reinterpret_cast<float*>(smem + kVsOffset);
-    for (;;) {
-        const int it = claim(kUpper ? &a.ctl->ctrT2 : &a.ctl->ctrT1, slot, tid);
-        if (it >= a.nchunks) break;
+    for (int turn = 0;; ++turn) {
+        // longest first, there and back over the blocks
+        const int G = (int)gridDim.x, b = (int)blockIdx.x;
+        const int it = turn * G + ((turn & 1) ? G - 1 - b : b);
+        if (turn * G >= a.nchunks) break;
+        if (it >= a.nchunks) continue;
         const int2 item = a.chunks[it];
         const BInst& I = a.inst[item.x];
         if (!ld_volatile(&a.iact[cur * a.count + item.x])) continue;
-        const int kt0 = kUpper ? 2 * item.y : 0;
-        const int kt1 = kUpper ? I.s_pad / kKT : 2 * (item.y + 1);
-        const float* V = (kUpper ? a.Y1 : a.G) + (int64_t)I.soff * kM;
-        stage_vec(Vs, V, kt0 * kKT, kt1 * kKT, tid);
-        float acc[4][16];
+        // the item's rows, counted so that the longest come first in both steps: from
+        // the end for L^{-1} (k < row + 1), from the start for L^{-T} (k >= row)
+        const int r0 = (kUpper ? item.y : I.s_pad / kTriRows - 1 - item.y) * kTriRows;
+        const int k0 = kUpper ? r0 : 0, k1 = kUpper ? I.s_pad : r0 + kTriRows;
+        const float* M = (kUpper ? I.Bu : I.Bl) + (int64_t)r0 * I.s_pad;
+        const int nt = (k1 - k0 + kTriK - 1) / kTriK;
+        auto issue = [&](int i) {
+            if (i < nt) {
+                float* dst = tiles + (i % kMvTiles) * kTileFloats;
+                const int kb = k0 + i * kTriK;
 #pragma unroll
-        for (int i = 0; i < 4; ++i)
+                for (int j = 0; j < 8; ++j) {
+                    // row e / 64, granule e % 64 of the piece; granule g of row r at
+                    // g ^ (r & 7): lanes over rows then read distinct banks
+                    const int e = tid + kWorkers * j, row = e >> 6, g = e & 63;
+                    const bool ok = kb + 4 * g < k1;
+                    msp::cp_async16(dst + row * kTriK + ((g ^ (row & 7)) << 2),
+                                    M + (int64_t)row * I.s_pad + (ok ? kb + 4 * g : k0), ok);
+                }
+            }
+            msp::cp_async_commit();
+        };
+        msp::bar_workers<kWorkers>();        // the item before: Vs, tiles and red are free
+        issue(0);
+        issue(1);
+        stage_vec(Vs, (kUpper ? a.Y1 : a.G) + (int64_t)I.soff * kM, a.gstride, kUpper ? 1 : I.ng, k0, k1, tid);
+        float acc[16];
 #pragma unroll
-            for (int c = 0; c < 16; ++c) acc[i][c] = 0.f;
-        const float* M = (kUpper ? I.Bu : I.Bl) + (int64_t)item.y * kRB * I.s_pad;
-        mv_stream(acc, M, I.s_pad, kRB, kt0, kt1, Vs, tiles, tid, w, lane);
-        float out[8];
-        reduce_scatter_fma(acc, red, out, w, lane);
-        const int ch = lane >> 4;
-        float* Y = (kUpper ? a.Y2 : a.Y1) + ((int64_t)I.soff + item.y * kRB + 16 * w + (lane & 15)) * kM + 8 * ch;
-        st4(Y, make_float4(out[0], out[1], out[2], out[3]));
-        st4(Y + 4, make_float4(out[4], out[5], out[6], out[7]));
+        for (int c = 0; c < 16; ++c) acc[c] = 0.f;
+#pragma unroll 1
+        for (int i = 0; i < nt; ++i) {
+            issue(i + 2);
+            msp::cp_async_wait<2>();
+            msp::bar_workers<kWorkers>();
+            const float4* T4 = reinterpret_cast<const float4*>(tiles + (i % kMvTiles) * kTileFloats) + lane * (kTriK / 4);
+            const int kw = k0 + i * kTriK + 32 * w;      // this warp's columns
+            const float4* V4 = reinterpret_cast<const float4*>(Vs) + (int64_t)kw * 4;
+            const int gn = min(8, (k1 - kw + 3) / 4);    // granules of it (the ranges are multiples of 32)
+#pragma unroll 2
+            for (int g = 0; g < gn; ++g) {
+                const float4 m = T4[(8 * w + g) ^ (lane & 7)];
+#pragma unroll
+                for (int kk = 0; kk < 4; ++kk) {
+                    const float mv = comp(m, kk);
+#pragma unroll
+                    for (int j = 0; j < 4; ++j) {
+                        const float4 v = V4[(4 * g + kk) * 4 + j];
+                        acc[4 * j + 0] = fmaf(mv, v.x, acc[4 * j + 0]);
+                        acc[4 * j + 1] = fmaf(mv, v.y, acc[4 * j + 1]);
+                        acc[4 * j + 2] = fmaf(mv, v.z, acc[4 * j + 2]);
+                        acc[4 * j + 3] = fmaf(mv, v.w, acc[4 * j + 3]);
+                    }
+                }
+            }
+            msp::bar_workers<kWorkers>();
+        }
+#pragma unroll
+        for (int c = 0; c < 16; ++c) red[(w * 16 + c) * 32 + lane] = acc[c];
         msp::bar_workers<kWorkers>();
+        // thread: row tid >> 3, columns 2 (tid & 7), + 1
+        const int row = tid >> 3, c = 2 * (tid & 7);
+        float o0 = 0.f, o1 = 0.f;
+#pragma unroll
+        for (int ww = 0; ww < kWorkWarps; ++ww) {
+            o0 += red[(ww * 16 + c) * 32 + row];
+            o1 += red[(ww * 16 + c + 1) * 32 + row];
+        }
+        float* Y = (kUpper ? a.Y2 : a.Y1) + ((int64_t)I.soff + r0 + row) * kM + c;
+        *reinterpret_cast<float2*>(Y) = make_float2(o0, o1);
     }
+    msp::cp_async_wait<0>();
+    msp::bar_workers<kWorkers>();
 }
 
 // S5: Z = (R - C Y2) / lam~ by row blocks, partials of z.r and z.q: the
@@ -1053,9 +1099,37 @@ __device__ __noinline__ void consume_Z(const BArgs& a, unsigned char* ring, uint
     }
 }
 
+// Sums over an instance's row blocks of the partials p (and q) for the 16 columns:
+// thread (block group tid >> 4, column tid & 15) adds every 16th row block, and warp 0
+// (q: warp 1) adds the 16 groups, two halves and a shuffle, for its lanes < 16. All
+// worker threads call it; buf holds 2 x 16 x 16 doubles and is free on entry after a
+// barrier. (One lane a column over all the row blocks, 30 dependent FP64 adds, was most
+// of the vector steps: 23 us an iteration, against 20.)
+__device__ __forceinline__ double block_partials(const double* p, const double* q, const BInst& I, double* buf, int tid,
+                                                 int w, int lane) {
+    const int c = tid & 15, g = tid >> 4;
+    double sp = 0.0, sq = 0.0;
+    for (int b = g; b < I.nb; b += 16) {
+        sp += __ldcg(&p[((int64_t)I.boff + b) * kM + c]);
+        if (q) sq += __ldcg(&q[((int64_t)I.boff + b) * kM + c]);
+    }
+    buf[tid] = sp;
+    if (q) buf[256 + tid] = sq;
+    msp::bar_workers<kWorkers>();
+    double t = 0.0;
+    if (w == 0 || (q && w == 1)) {
+        const double* v = buf + 256 * w + 128 * (lane >> 4) + (lane & 15);
+        t = ((v[0] + v[16]) + (v[32] + v[48])) + ((v[64] + v[80]) + (v[96] + v[112]));
+        t += __shfl_xor_sync(0xffffffffu, t, 16);
+        if (w == 1 && lane < 16) buf[256 + lane] = t;
+    }
+    if (q) msp::bar_workers<kWorkers>();
+    return t;      // warp 0: the sum of p; the sum of q is buf[256 + column]
+}
+
 // S6: beta = -alpha z^T q / rz_old (flexible Polak-Ribiere with
 // r_new - r_old = -alpha q), P = Z + beta P; rz_new kept for S1.
-__device__ __forceinline__ void step_P(const BArgs& a, int t, float* sv, int tid, int w, int lane) {
+__device__ __forceinline__ void step_P(const BArgs& a, int t, float* sv, double* buf, int tid, int w, int lane) {
     const int cur = t & 1, prev = cur ^ 1;
     int i0, i1;
     my_range(a.nrows, i0, i1);
@@ -1067,13 +1141,10 @@ __device__ __forceinline__ void step_P(const BArgs& a, int t, float* sv, int tid
         // beta of the instance: once per instance met by this block
         if (item.x != cached || item.y == 0) {
             msp::bar_workers<kWorkers>();     // the previous item's readers of sv are done
+            const double rzn = block_partials(a.p_zr, a.p_zq, I, buf, tid, w, lane);
             if (w == 0 && lane < 16) {
                 const int c = lane, gi = item.x * kM + c;
-                double rzn = 0.0, zq = 0.0;
-                for (int b = 0; b < I.nb; ++b) {
-                    rzn += a.p_zr[((int64_t)I.boff + b) * kM + c];
-                    zq += a.p_zq[((int64_t)I.boff + b) * kM + c];
-                }
+                const double zq = buf[256 + c];
                 const double rzo = a.rz[(int64_t)prev * a.count * kM + gi];
                 double beta = 0.0;
                 if (t > 0 && a.act[gi] && rzo > 0.0 && isfinite(rzo)) beta = -a.alpha[gi] * zq / rzo;
@@ -1102,11 +1173,12 @@ __device__ __forceinline__ void step_P(const BArgs& a, int t, float* sv, int tid
 }
 
 // S1: alpha = rz / p^T q, X_w += alpha P, R -= alpha Q, partials of |r|^2.
-__device__ __forceinline__ void step_X(const BArgs& a, int t, float* wsum, float* sv, int tid, int w, int lane) {
+__device__ __forceinline__ void step_X(const BArgs& a, int t, float* wsum, float* sv, double* buf, int tid, int w,
+                                       int lane) {
     const int cur = t & 1;
     if (blockIdx.x == 0 && tid == 0) {
         a.ctl->ctrA = 0;
-        a.ctl->ctrG = a.ctl->ctrT1 = a.ctl->ctrT2 = a.ctl->ctrZ = 0;
+        a.ctl->ctrG = a.ctl->ctrZ = 0;
     }
     int i0, i1;
     my_range(a.nrows, i0, i1);
@@ -1117,12 +1189,11 @@ __device__ __forceinline__ void step_X(const BArgs& a, int t, float* wsum, float
         if (!ld_volatile(&a.iact[cur * a.count + item.x])) continue;
         // alpha of the instance: once per instance met by this block
         if (item.x != cached || item.y == 0) {
+            const double pq = block_partials(a.p_pq, nullptr, I, buf, tid, w, lane);
             if (w == 0 && lane < 16) {
                 const int c = lane, gi = item.x * kM + c;
                 double al = 0.0;
                 if (a.act[gi]) {
-                    double pq = 0.0;
-                    for (int b = 0; b < I.nb; ++b) pq += a.p_pq[((int64_t)I.boff + b) * kM + c];
                     const double rz = a.rz[(int64_t)cur * a.count * kM + gi];
                     if (pq > 0.0 && isfinite(pq)) al = rz / pq;
                     else atomicCAS(&a.ierr[item.x], 0, isfinite(pq) ? (int)MSP_ENOTPD : (int)MSP_ENONFINITE);
@@ -1218,7 +1289,6 @@ __global__ void __launch_bounds__(kThreads, 1) k_batch_solve(BArgs a) {
     double* wsumd = reinterpret_cast<double*>(misc + 128);
     float* sv = reinterpret_cast<float*>(misc + 1152);        // 16 per-column scalars
     double* sd = reinterpret_cast<double*>(misc + 1280);      // 16 per-column scalars
-    int* slot = reinterpret_cast<int*>(misc + 1408);          // claimed item index
     int* sflag = reinterpret_cast<int*>(misc + 1412);         // last-unit flag
 
     const int tid = threadIdx.x, w = tid >> 5, lane = tid & 31;
@@ -1268,21 +1338,21 @@ __global__ void __launch_bounds__(kThreads, 1) k_batch_solve(BArgs a) {
                 ctl->active[(t + 1) & 1] = 0;
                 ctl->sweepsA += 1;
             }
-            if (worker) step_tri<false>(a, t, smem, red, slot, tid, w, lane);
+            if (worker) step_tri<false>(a, t, smem, red, tid, w, lane);
             MSP_GBAR(kTTri);
-            if (worker) step_tri<true>(a, t, smem, red, slot, tid, w, lane);
+            if (worker) step_tri<true>(a, t, smem, red, tid, w, lane);
             MSP_GBAR(kTTri);
             if (worker) consume_Z(a, ring, full, empty, hdr, kring, red, wsum, w, lane);
             else if (lane == 0)
                 producer<kModeZ>(a, ring, full, empty, hdr, kring, &ctl->ctrZ, a.iact + (t & 1) * a.count);
             MSP_GBAR(kTZ);
-            if (worker) step_P(a, t, sv, tid, w, lane);
+            if (worker) step_P(a, t, sv, reinterpret_cast<double*>(red), tid, w, lane);
             MSP_GBAR(kTVec);
             if (worker) consume_A(a, ring, full, empty, hdr, kring, red, wsum, sflag, w, lane);
             else if (lane == 0)
                 producer<kModeA>(a, ring, full, empty, hdr, kring, &ctl->ctrA, a.iact + (t & 1) * a.count);
             MSP_GBAR(kTA);
-            if (worker) step_X(a, t, wsum, sv, tid, w, lane);
+            if (worker) step_X(a, t, wsum, sv, reinterpret_cast<double*>(red), tid, w, lane);
             MSP_GBAR(kTVec);
         }
         if (worker) step_back(a, wsumd, tid, w, lane);
@@ -1600,6 +1670,7 @@ msp_status msp_batch_create(msp_ctx* ctx, int count, const msp_instance* inst, m
         H.voff = (int)nv;
         H.soff = (int)ns;
         H.boff = (int)nbt;
+        H.ng = std::min((H.nb + kSegBlocks - 1) / kSegBlocks, kSegMax);
         H.nkc = (H.n_pad / kKT + kUtMin - 1) / kUtMin;   // the most units (smallest width)
         H.qoff = (int)nq;
         H.lam = (float)I.lambda;
@@ -1623,10 +1694,25 @@ msp_status msp_batch_create(msp_ctx* ctx, int count, const msp_instance* inst, m
     std::stable_sort(by_n.begin(), by_n.end(), [&](int x, int y) { return inst[x].n > inst[y].n; });
     for (int k : by_n)
         for (int r = 0; r < b->hinst[k].nb; ++r) b->rows.push_back(make_int2(k, r));
+    int segs = 1;
+    for (int k : by_n) {
+        segs = std::max(segs, b->hinst[k].ng);
+        for (int s = 0; s < b->hinst[k].s_pad / kKT; ++s)
+            for (int g = 0; g < b->hinst[k].ng; ++g) b->strips.push_back(make_int2(k, s | (g << 16)));
+    }
+    auto seg_len = [&](const int2& x) {
+        const BInst& H = b->hinst[x.x];
+        const int g = x.y >> 16;
+        return H.nb * (g + 1) / H.ng - H.nb * g / H.ng;
+    };
+    std::stable_sort(b->strips.begin(), b->strips.end(),
+                     [&](const int2& x, const int2& y) { return seg_len(x) > seg_len(y); });
+    // longest first: chunk c of an instance has s_pad - 32 c columns
     for (int k : by_n)
-        for (int s = 0; s < b->hinst[k].s_pad / kKT; ++s) b->strips.push_back(make_int2(k, s));
-    for (int k : by_n)
-        for (int s = 0; s < b->hinst[k].s_pad / kRB; ++s) b->chunks.push_back(make_int2(k, s));
+        for (int s = 0; s < b->hinst[k].s_pad / kTriRows; ++s) b->chunks.push_back(make_int2(k, s));
+    std::stable_sort(b->chunks.begin(), b->chunks.end(), [&](const int2& x, const int2& y) {
+        return b->hinst[x.x].s_pad - kTriRows * x.y > b->hinst[y.x].s_pad - kTriRows * y.y;
+    });
     b->by_n = by_n;
     // room for the units list at the smallest width
     size_t max_units = 0;
@@ -1655,7 +1741,7 @@ msp_status msp_batch_create(msp_ctx* ctx, int count, const msp_instance* inst, m
     for (int q = 0; q < 7; ++q) o_v[q] = take(vbytes);
     const size_t o_r64 = take((size_t)nv * kM * 8);
     const size_t sbytes = (size_t)ns * kM * 4;
-    const size_t o_g = take(sbytes), o_y1 = take(sbytes), o_y2 = take(sbytes);
+    const size_t o_g = take((size_t)segs * sbytes), o_y1 = take(sbytes), o_y2 = take(sbytes);
     const size_t pbytes = (size_t)nbt * kM * 8;
     size_t o_p[6];
     for (int q = 0; q < 6; ++q) o_p[q] = take(pbytes);
@@ -1740,6 +1826,7 @@ msp_status msp_batch_create(msp_ctx* ctx, int count, const msp_instance* inst, m
     for (int q = 0; q < 7; ++q) *vp[q] = (float*)(base + o_v[q]);
     A.R64 = (double*)(base + o_r64);
     A.G = (float*)(base + o_g);
+    A.gstride = (int64_t)(sbytes / 4);
     A.Y1 = (float*)(base + o_y1);
     A.Y2 = (float*)(base + o_y2);
     double** pp[6] = {&A.p_pq, &A.p_rr, &A.p_zr, &A.p_zq, &A.p_r64, &A.p_xx};
@@ -1772,14 +1859,39 @@ msp_status msp_batch_create(msp_ctx* ctx, int count, const msp_instance* inst, m
         if (st != MSP_OK) return fail(st);
     }
     {
-        // default width: the widest whose units still number 8 per SM
+        // default width: the one whose units, dealt out largest first, finish first
+        // (in tiles: a unit also costs about 2.5 for its reduction, and one more where
+        // its sums go through the unit partials). On 24 instances of n 512 to 4096 the A
+        // passes take 25.8, 22.1 and 20.7 ms at 16, 32 and 64 tiles, as this orders
+        // them; a floor of 8 units per SM chose 16.
         int ut = kUtMin;
+        double best = 0.0;
         for (int cand : {256, 128, 64, 32, 16}) {
-            size_t nu = 0;
-            for (const BInst& H : b->hinst) nu += (size_t)H.nb * ((H.n_pad / kKT + cand - 1) / cand);
-            if (nu >= (size_t)8 * ctx->num_sms) {
+            std::vector<double> cost;
+            double total = 0.0;
+            for (const BInst& H : b->hinst) {
+                const int nk = H.n_pad / kKT, nkc = (nk + cand - 1) / cand;
+                for (int c = 0; c < nkc; ++c) {
+                    const double u = std::min(nk, (c + 1) * cand) - c * cand + 2.5 + (nkc > 1 ? 1.0 : 0.0);
+                    cost.insert(cost.end(), H.nb, u);
+                    total += u * H.nb;
+                }
+            }
+            double end = total / ctx->num_sms;
+            if (cost.size() < (size_t)64 * ctx->num_sms) {
+                std::sort(cost.begin(), cost.end(), std::greater<double>());
+                std::priority_queue<double, std::vector<double>, std::greater<double>> load;
+                for (int q = 0; q < ctx->num_sms; ++q) load.push(0.0);
+                for (double u : cost) {
+                    const double t = load.top() + u;
+                    load.pop();
+                    load.push(t);
+                    end = std::max(end, t);
+                }
+            }
+            if (best == 0.0 || end < best) {
+                best = end;
                 ut = cand;
-                break;
             }
         }
         const msp_status st = set_units(ctx, b, ut);

@@ -1315,6 +1315,7 @@ __global__ void __launch_bounds__(16 * E + kDotThreads, 1) k_inner(InnerArgs<T> 
         a.y[tid] = y;
         if (tid == 0) ctl->inner_iters += k;
     }
+    cl.sync();   // a CTA whose wait ran out stays until nobody sends to it (the others' waits end too)
 }
 
 // The kernel for a padded sketch size (its data fits the cluster's registers),

@@ -388,102 +388,6 @@ __device__ __forceinline__ float2 ff_from_double(double v) {
 
 __device__ __forceinline__ double ff_to_double(float2 a) { return (double)a.x + (double)a.y; }
 
-// k_dgemm in float-float: the same tiling, triangular limits and lower_out,
-// operands and result stored as float2 (hi, lo). alpha is +-1 and beta 0 or
-// 1 (what the recursion uses): Cm = beta Cm +- op(A) op(B). The accumulators
-// are renormalised after every K chunk of 16.
-template <bool TA_, bool TB_, int TS>
-__global__ void __launch_bounds__(256) k_ffgemm(int64_t m, int64_t n, int64_t k, float alpha,
-                                               const float2* __restrict__ A, int64_t lda,
-                                               const float2* __restrict__ B, int64_t ldb,
-                                               int beta, float2* __restrict__ Cm, int64_t ldc,
-                                               int tri_a, int tri_b, int lower_out) {
-    constexpr int PT = TS / 16;
-    __shared__ float2 As[16][TS + 1];
-    __shared__ float2 Bs[16][TS + 1];
-    const int64_t i0 = (int64_t)blockIdx.y * TS, j0 = (int64_t)blockIdx.x * TS;
-    if (lower_out && j0 > i0 + TS - 1) return;
-    int64_t kbeg = 0, kend = k;
-    if (tri_a == 1) kend = min(kend, i0 + TS);
-    if (tri_b == 1) kend = min(kend, j0 + TS);
-    if (tri_b == 2) kbeg = (j0 / 16) * 16;
-    const int tx = threadIdx.x & 15, ty = threadIdx.x >> 4;
-    float sh[PT][PT], sl[PT][PT];
-#pragma unroll
-    for (int i = 0; i < PT; ++i)
-#pragma unroll
-        for (int j = 0; j < PT; ++j) sh[i][j] = sl[i][j] = 0.f;
-    const float2 zero = make_float2(0.f, 0.f);
-    // the K chunk's operands, loaded into registers one chunk ahead
-    constexpr int LD = 16 * TS / 256;        // elements per thread per operand
-    float2 ra[LD], rb[LD];
-    auto fetch = [&](int64_t k0) {
-#pragma unroll
-        for (int u = 0; u < LD; ++u) {
-            const int e = threadIdx.x + 256 * u;
-            int kk, ii;
-            if (TA_) { ii = e % TS; kk = e / TS; }
-            else { kk = e & 15; ii = e >> 4; }
-            const int64_t gi = i0 + ii, gk = k0 + kk;
-            ra[u] = (gi < m && gk < kend) ? (TA_ ? A[gk * lda + gi] : A[gi * lda + gk]) : zero;
-            int jj;
-            if (TB_) { kk = e & 15; jj = e >> 4; }
-            else { jj = e % TS; kk = e / TS; }
-            const int64_t gj = j0 + jj, gk2 = k0 + kk;
-            rb[u] = (gj < n && gk2 < kend) ? (TB_ ? B[gj * ldb + gk2] : B[gk2 * ldb + gj]) : zero;
-        }
-    };
-    if (kbeg < kend) fetch(kbeg);
-    for (int64_t k0 = kbeg; k0 < kend; k0 += 16) {
-#pragma unroll
-        for (int u = 0; u < LD; ++u) {
-            const int e = threadIdx.x + 256 * u;
-            int kk, ii, jj;
-            if (TA_) { ii = e % TS; kk = e / TS; }
-            else { kk = e & 15; ii = e >> 4; }
-            As[kk][ii] = ra[u];
-            if (TB_) { kk = e & 15; jj = e >> 4; }
-            else { jj = e % TS; kk = e / TS; }
-            Bs[kk][jj] = rb[u];
-        }
-        __syncthreads();
-        if (k0 + 16 < kend) fetch(k0 + 16);
-#pragma unroll
-        for (int kk = 0; kk < 16; ++kk) {
-            float2 av[PT], bv[PT];
-#pragma unroll
-            for (int i = 0; i < PT; ++i) av[i] = As[kk][ty * PT + i];
-#pragma unroll
-            for (int j = 0; j < PT; ++j) bv[j] = Bs[kk][tx * PT + j];
-#pragma unroll
-            for (int i = 0; i < PT; ++i)
-#pragma unroll
-                for (int j = 0; j < PT; ++j) ff_fma_acc(sh[i][j], sl[i][j], av[i], bv[j]);
-        }
-#pragma unroll
-        for (int i = 0; i < PT; ++i)
-#pragma unroll
-            for (int j = 0; j < PT; ++j) {
-                const float2 t = ff_norm(sh[i][j], sl[i][j]);
-                sh[i][j] = t.x;
-                sl[i][j] = t.y;
-            }
-        __syncthreads();
-    }
-#pragma unroll
-    for (int i = 0; i < PT; ++i)
-#pragma unroll
-        for (int j = 0; j < PT; ++j) {
-            const int64_t gi = i0 + ty * PT + i, gj = j0 + tx * PT + j;
-            if (gi < m && gj < n) {
-                float2 r = make_float2(sh[i][j], sl[i][j]);
-                if (alpha < 0.f) r = ff_neg(r);
-                if (beta) r = ff_add(Cm[gi * ldc + gj], r);
-                Cm[gi * ldc + gj] = r;
-            }
-        }
-}
-
 constexpr int kLeafSmem = 2 * 64 * 65 * (int)sizeof(double);
 constexpr int kLeafUpd = 256;                 // eight update warps (32 x 8 thread grid)
 constexpr int kLeafThreads = kLeafUpd + 32;   // and the pivot warp
@@ -628,103 +532,215 @@ __device__ __forceinline__ float2 ff_rsqrt(float2 d) {
     return ff_fast2sum(r0, __fmul_rn(__fmul_rn(0.5f, r0), res));
 }
 
-// k_chol_leaf in float-float (the same elimination and pivot warp; the
-// block and its inverse in shared memory as float2; 31 update warps take a
-// row each, a lane per element, so that a step of a 32-wide leaf is one
-// dependent chain per lane, where the FP64 version is bound by the FP64
-// pipe): M = L L^T,
-// X = L^{-1}, both float2 with leading dimension ld.
-constexpr int kFFUpd = 31 * 32;              // update warps of the float-float leaf
-constexpr int kFFThreads = kFFUpd + 32;       // and its pivot warp
+// Element (i, j) of a float-float matrix kept as 32 x 32 row-major tiles.
+__device__ __forceinline__ int64_t ff_tile_at(int64_t i, int64_t j, int64_t s_pad) {
+    return (((i >> 5) * (s_pad >> 5) + (j >> 5)) << 10) + ((i & 31) << 5) + (j & 31);
+}
 
-__global__ void __launch_bounds__(kFFThreads) k_chol_leaf_ff(float2* __restrict__ M, float2* __restrict__ X,
-                                                              int64_t ld, int nb, int* __restrict__ fail) {
-    extern __shared__ __align__(16) float2 leaf_smem_ff[];
-    float2 (*a)[65] = reinterpret_cast<float2 (*)[65]>(leaf_smem_ff);
-    float2 (*x)[65] = reinterpret_cast<float2 (*)[65]>(leaf_smem_ff + 64 * 65);
-    __shared__ float2 piv[64], rinv[64], rs[64];
-    __shared__ int bad;
-    const int tid = threadIdx.x, lane = tid & 31;
-    const bool pivot_warp = tid >= kFFUpd;
+constexpr int kFFThreads = 256;
+
+struct FFShared {
+    float4 L[512], R[512];            // a tile's operands, k-major: [k][row or column]
+    float2 T[32][33];                 // the leaf, or the pivot tile's inverse
+    float2 col[2][32], rk[2], piv[32];
+    int bad;
+};
+
+// Cholesky inverse of the 32 x 32 tile in sh.T (lower triangle), left there: the
+// elimination of k_chol_leaf (LDL^T on the tile and the identity at once). A lane has
+// a row, warp w the columns w + 8 q in registers, X where the column is done and
+// A where it is not. A step needs column k and 1 / d_k from shared memory; the
+// warp of column k + 1 updates that one first and publishes it with its pivot's
+// reciprocal, so a step is one chain of a product, an update and a reciprocal and
+// one barrier.
+__device__ void ff_leaf(FFShared& sh) {
+    const int lane = threadIdx.x & 31, w = threadIdx.x >> 5;
     const float2 zero = make_float2(0.f, 0.f), one = make_float2(1.f, 0.f);
-    if (tid == 0) bad = 0;
-    for (int e = tid; e < nb * nb; e += kFFThreads) {
-        const int i = e / nb, j = e % nb;
-        a[i][j] = (j <= i) ? M[i * ld + j] : zero;
-        x[i][j] = (i == j) ? one : zero;
-    }
-    __syncthreads();
-    auto pivot_ok = [](float2 d) { return d.x > 0.f && isfinite(d.x); };
-    float2 dg0 = one, dg1 = one;
-    if (pivot_warp) {
-        if (lane < nb) dg0 = a[lane][lane];
-        if (lane + 32 < nb) dg1 = a[lane + 32][lane + 32];
-        if (lane == 0) {
-            float2 d = dg0;
-            if (!pivot_ok(d)) {
-                bad = 1;
-                d = one;
+    auto publish = [&](int k, float2 v) {
+        sh.col[k & 1][lane] = v;
+        if (lane == k) {
+            if (!(v.x > 0.f) || !isfinite(v.x)) {
+                sh.bad = 1;
+                v = one;
             }
-            piv[0] = d;
-            rinv[0] = ff_rcp(d);
+            sh.piv[k] = v;
+            sh.rk[k & 1] = ff_rcp(v);
+        }
+    };
+    float2 v[4];
+#pragma unroll
+    for (int q = 0; q < 4; ++q) v[q] = sh.T[lane][w + 8 * q];
+    if (w == 0) publish(0, v[0]);
+    __syncthreads();
+#pragma unroll
+    for (int kb = 0; kb < 4; ++kb) {
+#pragma unroll 1
+        for (int k = 8 * kb; k < min(8 * kb + 8, 31); ++k) {
+            const float2* col = sh.col[k & 1];
+            const float2 nti = ff_neg(ff_mul(col[lane], sh.rk[k & 1]));
+            auto update = [&](int q) {
+                const int j = w + 8 * q;
+                float2 src = col[j];
+                if (q <= kb) {          // a column that is done has row k of X in lane k
+                    const float xh = __shfl_sync(0xffffffffu, v[q].x, k), xl = __shfl_sync(0xffffffffu, v[q].y, k);
+                    if (j <= k) src = make_float2(xh, xl);
+                }
+                float h = v[q].x, l = v[q].y;
+                ff_fma_acc(h, l, nti, src);
+                const float2 u = j == k ? nti : ff_norm(h, l);
+                if (lane > k) v[q] = u;
+            };
+            update(kb);
+            if (kb < 3) update(kb + 1);
+            if (w == ((k + 1) & 7)) publish(k + 1, k < 8 * kb + 7 ? v[kb] : v[kb < 3 ? kb + 1 : 3]);
+#pragma unroll
+            for (int q = 0; q < 4; ++q)
+                if (q < kb || q > kb + 1) update(q);
+            __syncthreads();
         }
     }
+    const float2 rs = ff_rsqrt(sh.piv[lane]);
+#pragma unroll
+    for (int q = 0; q < 4; ++q) {
+        const int j = w + 8 * q;
+        sh.T[lane][j] = j < lane ? ff_mul(v[q], rs) : j == lane ? rs : zero;
+    }
     __syncthreads();
-    const int warp = tid >> 5;
-    for (int k = 0; k < nb; ++k) {
-        const float2 rk = rinv[k];
-        if (!pivot_warp) {
-            // one warp per row i = k + 1 + w, + 31, ...: lane j < i updates
-            // its element of the row, x[i][j] (j <= k) or a[i][j] (k < j <
-            // i), so the step's updates spread evenly over the lanes (no
-            // store of the step touches row k or column k)
-            for (int i = k + 1 + warp; i < nb; i += kFFUpd / 32) {
-                const float2 nti = ff_neg(ff_mul(a[i][k], rk));
-                for (int j = lane; j < i; j += 32) {
-                    const bool xs = j <= k;
-                    const float2 src = xs ? x[k][j] : a[j][k];
-                    float2* dst = xs ? &x[i][j] : &a[i][j];
-                    const float2 v = *dst;
-                    float h = v.x, l = v.y;
-                    ff_fma_acc(h, l, nti, src);
-                    *dst = ff_norm(h, l);
-                }
-            }
-        } else if (k + 1 < nb) {
-            if (lane > k && lane < nb) {
-                const float2 nti = ff_neg(ff_mul(a[lane][k], rk));
-                float h = dg0.x, l = dg0.y;
-                ff_fma_acc(h, l, nti, a[lane][k]);
-                dg0 = ff_norm(h, l);
-            }
-            if (lane + 32 > k && lane + 32 < nb) {
-                const float2 nti = ff_neg(ff_mul(a[lane + 32][k], rk));
-                float h = dg1.x, l = dg1.y;
-                ff_fma_acc(h, l, nti, a[lane + 32][k]);
-                dg1 = ff_norm(h, l);
-            }
-            const int kn = k + 1;
-            if (lane == (kn & 31)) {
-                float2 d = kn < 32 ? dg0 : dg1;
-                if (!pivot_ok(d)) {
-                    bad = 1;
-                    d = one;
-                }
-                piv[kn] = d;
-                rinv[kn] = ff_rcp(d);
-            }
+}
+
+// L^{-1} of the Cholesky factor of an SPD float-float matrix of nt x nt tiles
+// (tile-major, S; both triangles of the diagonal tiles), left in S's lower
+// tiles: block Gauss-Jordan elimination on the matrix and the identity at once, in
+// place, as tile column k is done with A before X needs it. Step k has X_kk, the
+// inverse of the factor of tile (k, k), and
+//   1. forms the panel L_ik = A_ik X_kk^T (i > k) into Lp, transposed, and row k of X,
+//      X_kj = X_kk X_kj (j < k): a quarter of a tile a block;
+//   2. updates every tile of the rows below, A_ij -= L_ik L_jk^T (j > k) and
+//      X_ij -= L_ik X_kj (j <= k), a tile a block, 2 x 2 entries a thread; block 0
+//      takes tile (k + 1, k + 1) and its leaf, the next step's pivot.
+// One cooperative launch, two grid barriers a step. The chain of the leaves bounds it
+// up to s_pad of about 1024 (the updates are s_pad^3 / 3 products of 14 FP32
+// operations over all SMs, 135 us there).
+// sync: failure, barrier and error words, zero at the launch.
+__global__ void __launch_bounds__(kFFThreads, 2) k_chol_inv_ff(float2* S, float2* Lp, int nt, int* sync) {
+    __shared__ __align__(16) FFShared sh;
+    const int tid = threadIdx.x, G = (int)gridDim.x, b = (int)blockIdx.x;
+    const int tx = tid & 15, ty = tid >> 4, lo = tid & 7, hi = tid >> 3;
+    unsigned int* word = reinterpret_cast<unsigned int*>(sync + 1);
+    auto tile = [&](int i, int j) { return S + (((int64_t)i * nt + j) << 10); };
+    auto load4 = [](const float2* p, int e) { return __ldcg(reinterpret_cast<const float4*>(p) + e); };
+    auto tile_to_T = [&](const float2* p) {
+#pragma unroll
+        for (int u = 0; u < 2; ++u) {
+            const float4 f = load4(p, 2 * tid + u);
+            sh.T[hi][4 * lo + 2 * u] = make_float2(f.x, f.y);
+            sh.T[hi][4 * lo + 2 * u + 1] = make_float2(f.z, f.w);
         }
+    };
+    auto leaf = [&](int k) {          // of the tile in T, to tile (k, k)
+        ff_leaf(sh);
+#pragma unroll
+        for (int u = 0; u < 4; ++u) tile(k, k)[hi * 32 + 4 * lo + u] = sh.T[hi][4 * lo + u];
+    };
+    if (tid == 0) sh.bad = 0;
+    if (b == 0) {
+        tile_to_T(tile(0, 0));
         __syncthreads();
+        leaf(0);
     }
-    for (int k = tid; k < nb; k += kFFThreads) rs[k] = ff_rsqrt(piv[k]);
-    __syncthreads();
-    for (int e = tid; e < nb * nb; e += kFFThreads) {
-        const int i = e / nb, j = e % nb;
-        if (j < i) M[i * ld + j] = ff_mul(a[i][j], rs[j]);
-        else if (j == i) M[i * ld + j] = ff_mul(piv[i], rs[i]);
-        X[i * ld + j] = (j <= i) ? ff_mul(x[i][j], rs[i]) : zero;
+    for (int k = 0; k < nt; ++k) {
+        if (!msp::grid_barrier(word, sync + 2)) return;
+        // ---- panel
+        if (b < 4 * (nt - 1)) tile_to_T(tile(k, k));
+        float2* sub = reinterpret_cast<float2*>(sh.L);
+        for (int it = b; it < 4 * (nt - 1); it += G) {
+            const int q = it & 3, below = nt - 1 - k, t = it >> 2;
+            const bool is_l = t < below;
+            // rows 8 q .. of A_ik, or columns 8 q .. of X_kj
+            float2* src = is_l ? tile(k + 1 + t, k) : tile(k, t - below);
+            if (is_l) sub[(tid >> 5) * 33 + (tid & 31)] = __ldcg(src + 256 * q + tid);
+            else sub[tid] = __ldcg(src + hi * 32 + 8 * q + lo);
+            __syncthreads();
+            const float2* a = sub + (is_l ? 33 * lo : lo);
+            const int step = is_l ? 1 : 8;
+            float s = 0.f, e = 0.f;
+#pragma unroll
+            for (int m0 = 0; m0 < 32; m0 += 16) {
+#pragma unroll
+                for (int m = m0; m < m0 + 16; ++m) ff_fma_acc(s, e, sh.T[hi][m], a[m * step]);
+                const float2 n = ff_norm(s, e);
+                s = n.x;
+                e = n.y;
+            }
+            (is_l ? Lp + ((int64_t)(k + 1 + t) << 10) : src)[hi * 32 + 8 * q + lo] = make_float2(s, e);
+            __syncthreads();
+        }
+        if (k == nt - 1) break;
+        if (!msp::grid_barrier(word, sync + 2)) return;
+        // ---- update: row i = k + 1, .. has tiles j = i, .., 0
+        const int tiles = nt * (nt + 1) / 2 - (k + 1) * (k + 2) / 2;
+        int i = k + 1, j = i - b;
+        for (int t = b; t < tiles; t += G - 1) {
+            while (j < 0) j += ++i + 1;
+            const float2* Rg = j > k ? Lp + ((int64_t)j << 10) : tile(k, j);
+            const float2* Lg = Lp + ((int64_t)i << 10);
+            float2* D = tile(i, j);
+            const float4 l0 = load4(Lg, tid), l1 = load4(Lg, tid + 256);
+            const float4 r0 = load4(Rg, tid), r1 = load4(Rg, tid + 256);
+            float4 d[2] = {};
+            if (j != k) {
+                d[0] = load4(D, (2 * ty) * 16 + tx);
+                d[1] = load4(D, (2 * ty + 1) * 16 + tx);
+            }
+            __syncthreads();          // the tile before is done with its operands
+            sh.L[tid] = l0;
+            sh.L[tid + 256] = l1;
+            sh.R[tid] = r0;
+            sh.R[tid + 256] = r1;
+            __syncthreads();
+            float s[4] = {}, e[4] = {};
+#pragma unroll
+            for (int k0 = 0; k0 < 2; ++k0) {
+#pragma unroll 8
+                for (int kk = 16 * k0; kk < 16 * k0 + 16; ++kk) {
+                    const float4 a = sh.L[kk * 16 + ty], c = sh.R[kk * 16 + tx];
+                    const float2 a0 = make_float2(a.x, a.y), a1 = make_float2(a.z, a.w);
+                    const float2 c0 = make_float2(c.x, c.y), c1 = make_float2(c.z, c.w);
+                    ff_fma_acc(s[0], e[0], a0, c0);
+                    ff_fma_acc(s[1], e[1], a0, c1);
+                    ff_fma_acc(s[2], e[2], a1, c0);
+                    ff_fma_acc(s[3], e[3], a1, c1);
+                }
+#pragma unroll
+                for (int u = 0; u < 4; ++u) {
+                    const float2 n = ff_norm(s[u], e[u]);
+                    s[u] = n.x;
+                    e[u] = n.y;
+                }
+            }
+            float4 o[2];
+#pragma unroll
+            for (int u = 0; u < 2; ++u) {
+                const float2 x = ff_add(make_float2(d[u].x, d[u].y), make_float2(-s[2 * u], -e[2 * u]));
+                const float2 y = ff_add(make_float2(d[u].z, d[u].w), make_float2(-s[2 * u + 1], -e[2 * u + 1]));
+                o[u] = make_float4(x.x, x.y, y.x, y.y);
+            }
+            if (b == 0) {
+#pragma unroll
+                for (int u = 0; u < 2; ++u) {
+                    sh.T[2 * ty + u][2 * tx] = make_float2(o[u].x, o[u].y);
+                    sh.T[2 * ty + u][2 * tx + 1] = make_float2(o[u].z, o[u].w);
+                }
+                __syncthreads();
+                leaf(k + 1);
+                break;
+            }
+#pragma unroll
+            for (int u = 0; u < 2; ++u) reinterpret_cast<float4*>(D)[(2 * ty + u) * 16 + tx] = o[u];
+            j -= G - 1;
+        }
     }
-    if (tid == 0 && bad) atomicExch(fail, 1);
+    if (b == 0 && tid == 0 && sh.bad) sync[0] = 1;
 }
 
 __global__ void k_copy_add_diag(const double* __restrict__ src, double* __restrict__ dst,
@@ -735,7 +751,6 @@ __global__ void k_copy_add_diag(const double* __restrict__ src, double* __restri
     dst[e] = src[e] + ((i == j) ? nu : 0.0);
 }
 
-// dst = float-float of (src + nu I) scale (scale a power of two: exact)
 // The shift and scaling of a float-float attempt from |M|_F^2: nu = 2^-24 |M|_F
 // 100^attempt, M scaled by 4^k to |M|_F in [1, 4). Formed on the device so that the
 // host need not wait for the norm before the factor starts.
@@ -750,7 +765,7 @@ __device__ inline FFShift ff_shift(double fro2, int attempt) {
     return f;
 }
 
-// dst = (src + nu I) 4^k
+// dst = (src + nu I) 4^k, row-major to 32 x 32 tiles
 __global__ void k_copy_add_diag_ff(const double* __restrict__ src, float2* __restrict__ dst,
                                    int64_t s_pad, const double* __restrict__ fro2, int attempt) {
     __shared__ double s_nu, s_scale;
@@ -763,18 +778,19 @@ __global__ void k_copy_add_diag_ff(const double* __restrict__ src, float2* __res
     int64_t e = (int64_t)blockIdx.x * blockDim.x + threadIdx.x;
     if (e >= s_pad * s_pad) return;
     int64_t i = e / s_pad, j = e % s_pad;
-    dst[e] = ff_from_double((src[e] + ((i == j) ? s_nu : 0.0)) * s_scale);
+    dst[ff_tile_at(i, j, s_pad)] = ff_from_double((src[e] + ((i == j) ? s_nu : 0.0)) * s_scale);
 }
 
-// dst = src 2^k in FP64
-__global__ void k_ff_to_double(const float2* __restrict__ src, double* __restrict__ dst, int64_t count,
+// dst = the lower triangle of src 2^k in FP64, tiles to row-major
+__global__ void k_ff_to_double(const float2* __restrict__ src, double* __restrict__ dst, int64_t s_pad,
                                const double* __restrict__ fro2) {
     __shared__ double s_scale;
     if (threadIdx.x == 0) s_scale = ldexp(1.0, ff_shift(*fro2, 0).k);
     __syncthreads();
     int64_t e = (int64_t)blockIdx.x * blockDim.x + threadIdx.x;
-    if (e >= count) return;
-    dst[e] = ff_to_double(src[e]) * s_scale;
+    if (e >= s_pad * s_pad) return;
+    const int64_t i = e / s_pad, j = e % s_pad;
+    dst[e] = j <= i ? ff_to_double(src[ff_tile_at(i, j, s_pad)]) * s_scale : 0.0;
 }
 
 // Frobenius norm^2 partials (single block, deterministic order).
@@ -842,63 +858,15 @@ msp_status dgemm(msp_ctx* ctx, bool ta, bool tb, int64_t m, int64_t n, int64_t k
     return MSP_OK;
 }
 
-template <int TS>
-void launch_ffgemm_ts(msp_ctx* ctx, bool ta, bool tb, int64_t m, int64_t n, int64_t k, float alpha,
-                      const float2* A, int64_t lda, const float2* B, int64_t ldb, int beta,
-                      float2* Cm, int64_t ldc, int tri_a, int tri_b, int lower_out) {
-    dim3 grid((unsigned)((n + TS - 1) / TS), (unsigned)((m + TS - 1) / TS));
-    if (!ta && !tb) k_ffgemm<false, false, TS><<<grid, 256, 0, ctx->stream>>>(m, n, k, alpha, A, lda, B, ldb, beta, Cm, ldc, tri_a, tri_b, lower_out);
-    else if (!ta && tb) k_ffgemm<false, true, TS><<<grid, 256, 0, ctx->stream>>>(m, n, k, alpha, A, lda, B, ldb, beta, Cm, ldc, tri_a, tri_b, lower_out);
-    else if (ta && !tb) k_ffgemm<true, false, TS><<<grid, 256, 0, ctx->stream>>>(m, n, k, alpha, A, lda, B, ldb, beta, Cm, ldc, tri_a, tri_b, lower_out);
-    else k_ffgemm<true, true, TS><<<grid, 256, 0, ctx->stream>>>(m, n, k, alpha, A, lda, B, ldb, beta, Cm, ldc, tri_a, tri_b, lower_out);
-}
-
-// The recursion's products on the two storages: FP64, or float-float
-// (alpha +-1, beta 0 or 1).
-msp_status gemm_s(msp_ctx* ctx, bool ta, bool tb, int64_t m, int64_t n, int64_t k, double alpha,
-                  const double* A, int64_t lda, const double* B, int64_t ldb, double beta,
-                  double* Cm, int64_t ldc, int tri_a, int tri_b, int lower_out) {
-    return dgemm(ctx, ta, tb, m, n, k, alpha, A, lda, B, ldb, beta, Cm, ldc, tri_a, tri_b, lower_out);
-}
-
-msp_status gemm_s(msp_ctx* ctx, bool ta, bool tb, int64_t m, int64_t n, int64_t k, double alpha,
-                  const float2* A, int64_t lda, const float2* B, int64_t ldb, double beta,
-                  float2* Cm, int64_t ldc, int tri_a, int tri_b, int lower_out) {
-    if (!(alpha == 1.0 || alpha == -1.0) || !(beta == 0.0 || beta == 1.0))
-        return msp_set_error(ctx, MSP_EINVAL, "factor: float-float product needs alpha = +-1, beta = 0 or 1");
-    // the FP32 pipe has room for the larger tile once it fills the SMs
-    const int64_t tiles32 = ((m + 31) / 32) * ((n + 31) / 32);
-    if (tiles32 >= ctx->num_sms)
-        launch_ffgemm_ts<32>(ctx, ta, tb, m, n, k, (float)alpha, A, lda, B, ldb, (int)beta, Cm, ldc, tri_a, tri_b, lower_out);
-    else
-        launch_ffgemm_ts<16>(ctx, ta, tb, m, n, k, (float)alpha, A, lda, B, ldb, (int)beta, Cm, ldc, tri_a, tri_b, lower_out);
-    MSP_CHECK_LAUNCH(ctx);
-    return MSP_OK;
-}
-
-template <typename Kern>
-msp_status leaf_attr(msp_ctx* ctx, Kern kern, std::atomic<bool>* attr_set) {
+msp_status leaf(msp_ctx* ctx, double* M, double* X, int64_t ld, int64_t n, int* fail) {
     // set once per device; batch set-up calls this from several threads
+    static std::atomic<bool> attr_set[64];
     const int d = ctx->device;
     if (d < 0 || d >= 64 || !attr_set[d].load()) {
-        MSP_CUDA_TRY(ctx, cudaFuncSetAttribute(kern, cudaFuncAttributeMaxDynamicSharedMemorySize, kLeafSmem));
+        MSP_CUDA_TRY(ctx, cudaFuncSetAttribute(k_chol_leaf, cudaFuncAttributeMaxDynamicSharedMemorySize, kLeafSmem));
         if (d >= 0 && d < 64) attr_set[d] = true;
     }
-    return MSP_OK;
-}
-
-msp_status leaf_s(msp_ctx* ctx, double* M, double* X, int64_t ld, int64_t n, int* fail) {
-    static std::atomic<bool> attr_set[64];
-    MSP_TRY(leaf_attr(ctx, k_chol_leaf, attr_set));
     k_chol_leaf<<<1, kLeafThreads, kLeafSmem, ctx->stream>>>(M, X, ld, (int)n, fail);
-    MSP_CHECK_LAUNCH(ctx);
-    return MSP_OK;
-}
-
-msp_status leaf_s(msp_ctx* ctx, float2* M, float2* X, int64_t ld, int64_t n, int* fail) {
-    static std::atomic<bool> attr_set[64];
-    MSP_TRY(leaf_attr(ctx, k_chol_leaf_ff, attr_set));
-    k_chol_leaf_ff<<<1, kFFThreads, kLeafSmem, ctx->stream>>>(M, X, ld, (int)n, fail);
     MSP_CHECK_LAUNCH(ctx);
     return MSP_OK;
 }
@@ -909,20 +877,19 @@ msp_status leaf_s(msp_ctx* ctx, float2* M, float2* X, int64_t ld, int64_t n, int
 // triangle, the leaves leave their L blocks there, L21 is not stored). Leaves
 // of at most 32: a leaf runs on one SM, whose FP64 pipe bounds it (its work
 // grows as nb^3), while the products of the recursion spread over all SMs.
-template <typename S>
-msp_status chol_inv(msp_ctx* ctx, S* M, S* X, S* T1, S* T2, int64_t ld,
-                    int64_t off, int64_t n, int* fail, int depth) {
-    if (n <= 32) return leaf_s(ctx, M + off * ld + off, X + off * ld + off, ld, n, fail);
+msp_status chol_inv(msp_ctx* ctx, double* M, double* X, double* T1, double* T2, int64_t ld, int64_t off,
+                    int64_t n, int* fail, int depth) {
+    if (n <= 32) return leaf(ctx, M + off * ld + off, X + off * ld + off, ld, n, fail);
     int64_t n1 = std::max<int64_t>(32, (n / 2) / 32 * 32);
     int64_t n2 = n - n1;
-    S* A21 = M + (off + n1) * ld + off;
-    S* A22 = M + (off + n1) * ld + off + n1;
-    S* X11 = X + off * ld + off;
-    S* X21 = X + (off + n1) * ld + off;
-    S* X22 = X + (off + n1) * ld + off + n1;
+    double* A21 = M + (off + n1) * ld + off;
+    double* A22 = M + (off + n1) * ld + off + n1;
+    double* X11 = X + off * ld + off;
+    double* X21 = X + (off + n1) * ld + off;
+    double* X22 = X + (off + n1) * ld + off + n1;
     MSP_TRY(chol_inv(ctx, M, X, T1, T2, ld, off, n1, fail, depth + 1));
     // T1 = L21 = A21 X11^T   (n2 x n1; X11^T is upper triangular)
-    MSP_TRY(gemm_s(ctx, false, true, n2, n1, n1, 1.0, A21, ld, X11, ld, 0.0, T1, ld, 0, 1, 0));
+    MSP_TRY(dgemm(ctx, false, true, n2, n1, n1, 1.0, A21, ld, X11, ld, 0.0, T1, ld, 0, 1, 0));
     // T2 = L21 X11 (X11 lower) needs only T1 and X11, so it runs on the side
     // stream of this depth while A22 is updated and factored on the main
     // stream. Disjoint memory: T1 and T2 hold columns [0, n1) of the
@@ -953,83 +920,42 @@ msp_status chol_inv(msp_ctx* ctx, S* M, S* X, S* T1, S* T2, int64_t ld,
     if (side) {
         cudaStream_t main_stream = ctx->stream;
         ctx->stream = side;
-        st = gemm_s(ctx, false, false, n2, n1, n1, 1.0, T1, ld, X11, ld, 0.0, T2, ld, 0, 2, 0);
+        st = dgemm(ctx, false, false, n2, n1, n1, 1.0, T1, ld, X11, ld, 0.0, T2, ld, 0, 2, 0);
         ctx->stream = main_stream;
         if (st == MSP_OK && cudaEventRecord(ev_t2, side) != cudaSuccess)
             st = msp_set_error(ctx, MSP_ECUDA, "factor: side stream record failed");
     }
     // A22 -= L21 L21^T (lower triangle is all the recursion reads)
     if (st == MSP_OK)
-        st = gemm_s(ctx, false, true, n2, n2, n1, -1.0, T1, ld, T1, ld, 1.0, A22, ld, 0, 0, 1);
+        st = dgemm(ctx, false, true, n2, n2, n1, -1.0, T1, ld, T1, ld, 1.0, A22, ld, 0, 0, 1);
     if (st == MSP_OK) st = chol_inv(ctx, M, X, T1 + n1, T2 + n1, ld, off + n1, n2, fail, depth + 1);
     if (st == MSP_OK) {
         if (side) {
             if (cudaStreamWaitEvent(ctx->stream, ev_t2, 0) != cudaSuccess)
                 st = msp_set_error(ctx, MSP_ECUDA, "factor: side stream join failed");
         } else {
-            st = gemm_s(ctx, false, false, n2, n1, n1, 1.0, T1, ld, X11, ld, 0.0, T2, ld, 0, 2, 0);
+            st = dgemm(ctx, false, false, n2, n1, n1, 1.0, T1, ld, X11, ld, 0.0, T2, ld, 0, 2, 0);
         }
     }
     if (side && st != MSP_OK) cudaStreamSynchronize(side);
     MSP_TRY(st);
     // X21 = -X22 T2 (X22 lower)
-    MSP_TRY(gemm_s(ctx, false, false, n2, n1, n2, -1.0, X22, ld, T2, ld, 0.0, X21, ld, 1, 0, 0));
+    MSP_TRY(dgemm(ctx, false, false, n2, n1, n2, -1.0, X22, ld, T2, ld, 0.0, X21, ld, 1, 0, 0));
     return MSP_OK;
 }
 
-// One float-float factor attempt (chol_inv on scratch buffers) replayed
-// from a CUDA graph: the recursion issues about 130 launches of a few
-// microseconds each, whose host-side cost would otherwise pace the GPU. The
-// executable is keyed by the buffers and the size; the side-stream forks of
-// the recursion become parallel branches of the graph. Where capture is
-// not possible the recursion launches on the stream.
-msp_status chol_inv_ff_graphed(msp_ctx* ctx, float2* M, float2* X, float2* T1, float2* T2, int64_t sp,
-                               int* fail) {
-    struct Key {
-        const void *M, *X, *T1, *T2, *fail;
-        int64_t sp;
-        int overlap, device;
-    } key;
-    std::memset(&key, 0, sizeof key);
-    key.M = M; key.X = X; key.T1 = T1; key.T2 = T2; key.fail = fail;
-    key.sp = sp;
-    key.overlap = ctx->fac_overlap;
-    key.device = ctx->device;
-    static_assert(sizeof(Key) <= sizeof(ctx->fac_key), "factor graph key too large");
-    const bool hit = ctx->fac_exec && ctx->fac_key_len == sizeof key &&
-                     std::memcmp(ctx->fac_key, &key, sizeof key) == 0;
-    if (!hit) {
-        msp_fac_graph_release(ctx);
-        bool ok = ctx->cap_stream != nullptr ||
-                  cudaStreamCreateWithFlags(&ctx->cap_stream, cudaStreamNonBlocking) == cudaSuccess;
-        if (ok) ok = cudaStreamBeginCapture(ctx->cap_stream, cudaStreamCaptureModeRelaxed) == cudaSuccess;
-        if (ok) {
-            const cudaStream_t saved = ctx->stream;
-            const int64_t l0 = ctx->launches;
-            ctx->stream = ctx->cap_stream;
-            const msp_status st = chol_inv(ctx, M, X, T1, T2, sp, 0, sp, fail, 0);
-            ctx->stream = saved;
-            cudaGraph_t graph = nullptr;
-            const cudaError_t ce = cudaStreamEndCapture(ctx->cap_stream, &graph);
-            const int kernels = (int)(ctx->launches - l0);
-            ctx->launches = l0;
-            ok = st == MSP_OK && ce == cudaSuccess && graph != nullptr &&
-                 cudaGraphInstantiate(&ctx->fac_exec, graph, 0) == cudaSuccess;
-            if (ok) {
-                ctx->fac_graph = graph;
-                std::memcpy(ctx->fac_key, &key, sizeof key);
-                ctx->fac_key_len = sizeof key;
-                ctx->fac_kernels = kernels;
-            } else {
-                ctx->fac_exec = nullptr;
-                if (graph) cudaGraphDestroy(graph);
-            }
-        }
-        cudaGetLastError();
-        if (!ok) return chol_inv(ctx, M, X, T1, T2, sp, 0, sp, fail, 0);
-    }
-    MSP_CUDA_TRY(ctx, cudaGraphLaunch(ctx->fac_exec, ctx->stream));
-    ctx->launches += ctx->fac_kernels;
+// One float-float attempt: k_chol_inv_ff on as many blocks as its widest step has
+// work for, two an SM at most. sync: its failure word, barrier word and error word.
+msp_status chol_inv_ff(msp_ctx* ctx, float2* S, float2* Lp, int64_t sp, int* sync) {
+    int nt = (int)(sp / 32), per_sm = 0;
+    MSP_CUDA_TRY(ctx, cudaOccupancyMaxActiveBlocksPerMultiprocessor(&per_sm, k_chol_inv_ff, kFFThreads, 0));
+    if (per_sm < 1) return msp_set_error(ctx, MSP_ECUDA, "factor: kernel does not fit on an SM");
+    const int work = std::max(nt * (nt + 1) / 2 - 1, 4 * (nt - 1));
+    const int grid = std::max(2, std::min(work, std::min(per_sm, 2) * ctx->num_sms));
+    void* args[] = {&S, &Lp, &nt, &sync};
+    ++ctx->launches;
+    MSP_CUDA_TRY(ctx, cudaLaunchCooperativeKernel((const void*)k_chol_inv_ff, dim3(grid), dim3(kFFThreads), args, 0,
+                                                  ctx->stream));
     return MSP_OK;
 }
 
@@ -1048,12 +974,11 @@ msp_status factor_shifted(msp_ctx* ctx, const double* M, int64_t s, int64_t sp, 
     const bool ff = fp32_data && ctx->factor_ff;
     void* scr = nullptr;
     size_t mat = (size_t)sp * sp * 8;
-    MSP_TRY(msp_scratch(ctx, (ff ? 4 : 3) * mat + 2048, &scr));
+    MSP_TRY(msp_scratch(ctx, (ff ? mat + (size_t)sp * 32 * 8 : 3 * mat) + 2048, &scr));
     double* Mw = (double*)scr;
-    double* T1 = Mw + sp * sp;
+    double* T1 = Mw + sp * sp;                       // ff: 32 columns, the panel
     double* T2 = T1 + sp * sp;
-    float2* Xff = reinterpret_cast<float2*>(T2 + sp * sp);       // ff only
-    int* fail = (int*)(T2 + (ff ? 2 : 1) * sp * sp);
+    int* fail = (int*)(ff ? T1 + 32 * sp : T2 + sp * sp);        // and, ff, a barrier and an error word
     double* fro = (double*)(fail + 16);
     double* fro_part = fro + 2;
     int* hflag = (int*)ctx->host_flags;
@@ -1084,14 +1009,12 @@ msp_status factor_shifted(msp_ctx* ctx, const double* M, int64_t s, int64_t sp, 
     }
     for (int attempt = 0; attempt <= 4; ++attempt) {
         unsigned blocks = (unsigned)((sp * sp + 255) / 256);
-        MSP_CUDA_TRY(ctx, cudaMemsetAsync(fail, 0, sizeof(int), ctx->stream));
+        MSP_CUDA_TRY(ctx, cudaMemsetAsync(fail, 0, 3 * sizeof(int), ctx->stream));
         if (ff) {
             k_copy_add_diag_ff<<<blocks, 256, 0, ctx->stream>>>(M, reinterpret_cast<float2*>(Mw), sp, fro, attempt);
             MSP_CHECK_LAUNCH(ctx);
-            MSP_CUDA_TRY(ctx, cudaMemsetAsync(Xff, 0, mat, ctx->stream));
-            MSP_TRY(chol_inv_ff_graphed(ctx, reinterpret_cast<float2*>(Mw), Xff, reinterpret_cast<float2*>(T1),
-                                        reinterpret_cast<float2*>(T2), sp, fail));
-            k_ff_to_double<<<blocks, 256, 0, ctx->stream>>>(Xff, Linv64, sp * sp, fro);
+            MSP_TRY(chol_inv_ff(ctx, reinterpret_cast<float2*>(Mw), reinterpret_cast<float2*>(T1), sp, fail));
+            k_ff_to_double<<<blocks, 256, 0, ctx->stream>>>(reinterpret_cast<float2*>(Mw), Linv64, sp, fro);
             MSP_CHECK_LAUNCH(ctx);
         } else {
             k_copy_add_diag<<<blocks, 256, 0, ctx->stream>>>(M, Mw, sp, nu);
@@ -1099,9 +1022,10 @@ msp_status factor_shifted(msp_ctx* ctx, const double* M, int64_t s, int64_t sp, 
             MSP_CUDA_TRY(ctx, cudaMemsetAsync(Linv64, 0, mat, ctx->stream));
             MSP_TRY(chol_inv(ctx, Mw, Linv64, T1, T2, sp, 0, sp, fail, 0));
         }
-        MSP_CUDA_TRY(ctx, cudaMemcpyAsync(hflag, fail, sizeof(int), cudaMemcpyDeviceToHost,
+        MSP_CUDA_TRY(ctx, cudaMemcpyAsync(hflag, fail, 3 * sizeof(int), cudaMemcpyDeviceToHost,
                                           ctx->stream));
         MSP_CUDA_TRY(ctx, cudaStreamSynchronize(ctx->stream));
+        if (hflag[2]) return msp_set_error(ctx, (msp_status)hflag[2], "factor: grid barrier timed out");
         if (ff && attempt == 0) nu = std::ldexp(1.0, -24) * std::sqrt(*hfro);
         if (hflag[0] == 0) {
             *shift_out = nu;
@@ -1337,13 +1261,4 @@ extern "C" msp_status msp_set_factor_float_float(msp_ctx* ctx, int on) {
     if (!ctx) return msp_set_error(nullptr, MSP_EINVAL, "ctx is NULL");
     ctx->factor_ff = on != 0;
     return MSP_OK;
-}
-
-void msp_fac_graph_release(msp_ctx* ctx) {
-    if (ctx->fac_exec) cudaGraphExecDestroy(ctx->fac_exec);
-    if (ctx->fac_graph) cudaGraphDestroy(ctx->fac_graph);
-    ctx->fac_exec = nullptr;
-    ctx->fac_graph = nullptr;
-    ctx->fac_key_len = 0;
-    ctx->fac_kernels = 0;
 }

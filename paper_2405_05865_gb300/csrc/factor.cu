@@ -379,8 +379,6 @@ __device__ __forceinline__ float2 ff_add(float2 a, float2 b) {
     return ff_fast2sum(s.x, __fadd_rn(s.y, __fadd_rn(a.y, b.y)));
 }
 
-__device__ __forceinline__ float2 ff_neg(float2 a) { return make_float2(-a.x, -a.y); }
-
 __device__ __forceinline__ float2 ff_from_double(double v) {
     const float h = __double2float_rn(v);
     return make_float2(h, __double2float_rn(v - (double)h));
@@ -507,18 +505,6 @@ __global__ void __launch_bounds__(kLeafThreads) k_chol_leaf(double* __restrict__
     if (tid == 0 && bad) atomicExch(fail, 1);
 }
 
-// 1/d in float-float for a positive normal d: the FP32 reciprocal r0, then
-// one Newton-Raphson step r = r0 + r0 (1 - d r0) with the residual 1 - d r0
-// formed exactly to first order (1 - hi(d r0) is exact: d r0 is within
-// 2^-23 of 1), ~2^-46 relative.
-__device__ __forceinline__ float2 ff_rcp(float2 d) {
-    const float r0 = __frcp_rn(d.x);
-    const float p = __fmul_rn(d.x, r0);
-    const float pe = __fmaf_rn(d.y, r0, __fmaf_rn(d.x, r0, -p));
-    const float res = __fsub_rn(__fsub_rn(1.0f, p), pe);
-    return ff_fast2sum(r0, __fmul_rn(r0, res));
-}
-
 // d^{-1/2} in float-float for a positive normal d: the FP32 rsqrtf r0, then
 // one Newton-Raphson step r = r0 + r0 (1 - d r0^2) / 2 with the residual
 // 1 - d r0^2 formed to first order exactly (r0^2 and d r0^2 by TwoProduct;
@@ -537,75 +523,140 @@ __device__ __forceinline__ int64_t ff_tile_at(int64_t i, int64_t j, int64_t s_pa
     return (((i >> 5) * (s_pad >> 5) + (j >> 5)) << 10) + ((i & 31) << 5) + (j & 31);
 }
 
-constexpr int kFFThreads = 256;
+constexpr int kFFThreads = 288;     // eight warps of the tiles, and the leaf's pivot warp
 
 struct FFShared {
     float4 L[512], R[512];            // a tile's operands, k-major: [k][row or column]
     float2 T[32][33];                 // the leaf, or the pivot tile's inverse
-    float2 col[2][32], rk[2], piv[32];
+    float2 A[32][33];                 // block 0: the tile below the pivot
+    float2 row[2][32], rk[2], piv[32];
     int bad;
 };
 
-// Cholesky inverse of the 32 x 32 tile in sh.T (lower triangle), left there: the
-// elimination of k_chol_leaf (LDL^T on the tile and the identity at once). A lane has
-// a row, warp w the columns w + 8 q in registers, X where the column is done and
-// A where it is not. A step needs column k and 1 / d_k from shared memory; the
-// warp of column k + 1 updates that one first and publishes it with its pivot's
-// reciprocal, so a step is one chain of a product, an update and a reciprocal and
-// one barrier.
-__device__ void ff_leaf(FFShared& sh) {
+// 1/d in float-float for a positive normal d: r0, the hardware's approximation
+// (2^-23 relative), then r = r0 + r0 (e + e^2) with the residual e = 1 - d r0 formed to
+// first order exactly (1 - hi(d r0) is exact), ~2^-46 relative. The low part may
+// overlap the high one by a bit or two.
+__device__ __forceinline__ float2 ff_rcp(float2 d) {
+    float r0;
+    asm("rcp.approx.ftz.f32 %0, %1;" : "=f"(r0) : "f"(d.x));
+    const float p = __fmul_rn(d.x, r0);
+    const float pe = __fmaf_rn(d.y, r0, __fmaf_rn(d.x, r0, -p));
+    const float res = __fsub_rn(__fsub_rn(1.0f, p), pe);
+    return make_float2(r0, __fmul_rn(r0, __fmaf_rn(res, res, res)));
+}
+
+// -a b, the parts not renormalised (what ff_fma_acc takes as well)
+__device__ __forceinline__ float2 ff_nmul(float2 a, float2 b) {
+    const float p = __fmul_rn(a.x, -b.x);
+    float e = __fmaf_rn(a.x, -b.x, -p);
+    e = __fmaf_rn(a.x, -b.y, e);
+    e = __fmaf_rn(a.y, -b.x, e);
+    return make_float2(p, e);
+}
+
+// Cholesky inverse of the 32 x 32 tile in sh.T (both triangles), left there: the
+// elimination of k_chol_leaf (LDL^T on the tile and the identity at once) in place,
+// X in the columns that are done and A in the others. A lane has a column, warp w
+// the rows w + 8 r in registers. Row k then is what step k adds to the rows below
+// it, a_ki = a_ik times -1 / d_k the factor of row i, so a step reads the row and 1 / d_k
+// from shared memory and its updates are independent of each other. A ninth warp
+// keeps the diagonal and forms the next 1 / d: that chain (a product, an update, a
+// reciprocal, a barrier) is what a step takes, so its products stay unnormalised
+// and the test of the pivot is beside the reciprocal.
+__device__ __forceinline__ void ff_leaf(FFShared& sh) {
     const int lane = threadIdx.x & 31, w = threadIdx.x >> 5;
     const float2 zero = make_float2(0.f, 0.f), one = make_float2(1.f, 0.f);
-    auto publish = [&](int k, float2 v) {
-        sh.col[k & 1][lane] = v;
+    const bool pivots = w == 8;
+    float2 v[4], dg = sh.T[lane][lane];
+    auto pivot = [&](int k) {
+        const float2 r = ff_rcp(dg);
         if (lane == k) {
-            if (!(v.x > 0.f) || !isfinite(v.x)) {
-                sh.bad = 1;
-                v = one;
-            }
-            sh.piv[k] = v;
-            sh.rk[k & 1] = ff_rcp(v);
+            const bool ok = dg.x > 0.f && isfinite(dg.x);
+            sh.rk[k & 1] = ok ? r : one;
+            sh.piv[k] = ok ? dg : one;
+            if (!ok) sh.bad = 1;
         }
     };
-    float2 v[4];
+    if (pivots) {
+        pivot(0);
+    } else {
 #pragma unroll
-    for (int q = 0; q < 4; ++q) v[q] = sh.T[lane][w + 8 * q];
-    if (w == 0) publish(0, v[0]);
+        for (int r = 0; r < 4; ++r) v[r] = sh.T[w + 8 * r][lane];
+        if (w == 0) sh.row[0][lane] = lane == 0 ? one : v[0];
+    }
     __syncthreads();
 #pragma unroll
     for (int kb = 0; kb < 4; ++kb) {
 #pragma unroll 1
-        for (int k = 8 * kb; k < min(8 * kb + 8, 31); ++k) {
-            const float2* col = sh.col[k & 1];
-            const float2 nti = ff_neg(ff_mul(col[lane], sh.rk[k & 1]));
-            auto update = [&](int q) {
-                const int j = w + 8 * q;
-                float2 src = col[j];
-                if (q <= kb) {          // a column that is done has row k of X in lane k
-                    const float xh = __shfl_sync(0xffffffffu, v[q].x, k), xl = __shfl_sync(0xffffffffu, v[q].y, k);
-                    if (j <= k) src = make_float2(xh, xl);
-                }
-                float h = v[q].x, l = v[q].y;
+        for (int kr = 0; kr < (kb < 3 ? 8 : 7); ++kr) {
+            const int k = 8 * kb + kr;
+            const float2* row = sh.row[k & 1];
+            const float2 src = row[lane], rk = sh.rk[k & 1];
+            if (pivots) {
+                const float2 nti = ff_nmul(src, rk);
+                float h = dg.x, l = dg.y;
                 ff_fma_acc(h, l, nti, src);
-                const float2 u = j == k ? nti : ff_norm(h, l);
-                if (lane > k) v[q] = u;
-            };
-            update(kb);
-            if (kb < 3) update(kb + 1);
-            if (w == ((k + 1) & 7)) publish(k + 1, k < 8 * kb + 7 ? v[kb] : v[kb < 3 ? kb + 1 : 3]);
+                dg = ff_norm(h, l);
+                pivot(k + 1);
+            } else {
 #pragma unroll
-            for (int q = 0; q < 4; ++q)
-                if (q < kb || q > kb + 1) update(q);
+                for (int r = kb; r < 4; ++r) {
+                    const float2 nti = ff_nmul(row[w + 8 * r], rk);
+                    float h = v[r].x, l = v[r].y;
+                    ff_fma_acc(h, l, nti, src);
+                    const float2 u = lane == k ? nti : ff_norm(h, l);
+                    if (r > kb || w > kr) v[r] = u;
+                }
+                const float2 next = kr < 7 ? v[kb] : v[kb < 3 ? kb + 1 : 3];
+                if (w == ((k + 1) & 7)) sh.row[(k + 1) & 1][lane] = lane == k + 1 ? one : next;
+            }
             __syncthreads();
         }
     }
-    const float2 rs = ff_rsqrt(sh.piv[lane]);
+    if (!pivots) {
 #pragma unroll
-    for (int q = 0; q < 4; ++q) {
-        const int j = w + 8 * q;
-        sh.T[lane][j] = j < lane ? ff_mul(v[q], rs) : j == lane ? rs : zero;
+        for (int r = 0; r < 4; ++r) {
+            const int i = w + 8 * r;
+            const float2 rs = ff_rsqrt(sh.piv[i]);
+            sh.T[i][lane] = lane < i ? ff_mul(v[r], rs) : lane == i ? rs : zero;
+        }
     }
     __syncthreads();
+}
+
+// Monotonic counters between the blocks of a cooperative launch: arrive adds one after
+// the block's writes (and reads), wait_for returns once the count has reached
+// `target` (false: the wait limit ran out, MSP_ETIMEOUT in *err).
+__device__ __forceinline__ void arrive(unsigned int* count) {
+    __syncthreads();
+    if (threadIdx.x == 0) {
+        __threadfence();
+        asm volatile("red.release.gpu.global.add.u32 [%0], 1;" ::"l"(count) : "memory");
+    }
+}
+
+__device__ __forceinline__ bool reached(const unsigned int* count, unsigned int target, int* err) {
+    const uint64_t t0 = msp::globaltimer_ns();
+    const unsigned long long limit = msp::grid_wait_limit_ns();
+    while (true) {
+        unsigned int cur;
+        asm volatile("ld.acquire.gpu.global.u32 %0, [%1];" : "=r"(cur) : "l"(count) : "memory");
+        if (cur >= target) return true;
+        if (msp::globaltimer_ns() - t0 > limit) {
+            atomicExch(err, (int)MSP_ETIMEOUT);
+            return false;
+        }
+    }
+}
+
+__device__ __forceinline__ bool wait_for(const unsigned int* a, unsigned int target_a, const unsigned int* b,
+                                         unsigned int target_b, int* err) {
+    __shared__ int ok;
+    __syncthreads();
+    if (threadIdx.x == 0) ok = reached(a, target_a, err) && reached(b, target_b, err);
+    __syncthreads();
+    return ok != 0;
 }
 
 // L^{-1} of the Cholesky factor of an SPD float-float matrix of nt x nt tiles
@@ -616,131 +667,184 @@ __device__ void ff_leaf(FFShared& sh) {
 //   1. forms the panel L_ik = A_ik X_kk^T (i > k) into Lp, transposed, and row k of X,
 //      X_kj = X_kk X_kj (j < k): a quarter of a tile a block;
 //   2. updates every tile of the rows below, A_ij -= L_ik L_jk^T (j > k) and
-//      X_ij -= L_ik X_kj (j <= k), a tile a block, 2 x 2 entries a thread; block 0
-//      takes tile (k + 1, k + 1) and its leaf, the next step's pivot.
-// One cooperative launch, two grid barriers a step. The chain of the leaves bounds it
-// up to s_pad of about 1024 (the updates are s_pad^3 / 3 products of 14 FP32
-// operations over all SMs, 135 us there).
-// sync: failure, barrier and error words, zero at the launch.
-__global__ void __launch_bounds__(kFFThreads, 2) k_chol_inv_ff(float2* S, float2* Lp, int nt, int* sync) {
+//      X_ij -= L_ik X_kj (j <= k), a tile a block, 2 x 2 entries a thread.
+// Block 0 runs one step ahead of the others: it forms L_k+1,k for itself, updates
+// tile (k + 1, k + 1) and inverts its factor (ff_leaf), the next step's pivot, while they
+// take the rest of step k, so that a step takes the longer of the two.
+// What bounds it: block 0's chain (a leaf of about 15 thousand cycles, half of
+// a step) up to s_pad = 512, the updates (14 FP32 operations a product, s_pad^3 / 3 of
+// them, 135 us at s_pad = 1024 over all SMs) and the two waits beside it above. At
+// s_pad = 128, 256, 512 and 1024: 55, 106, 213 and 438 us (with block 0 in step with the
+// others, two grid barriers a step: 61, 121, 241 and 489 us; the recursion it
+// replaced, 32 leaves and 90 dependent products at 1024: about 1200 us).
+// sync (zero at the launch): failure word, -, error word, pivots published, panel
+// arrivals (all blocks), update arrivals (all but block 0).
+__global__ void __launch_bounds__(kFFThreads, 1) k_chol_inv_ff(float2* S, float2* Lp, int nt, int* sync) {
     __shared__ __align__(16) FFShared sh;
-    const int tid = threadIdx.x, G = (int)gridDim.x, b = (int)blockIdx.x;
+    const int tid = threadIdx.x, G = (int)gridDim.x, b = (int)blockIdx.x, NW = G - 1;
     const int tx = tid & 15, ty = tid >> 4, lo = tid & 7, hi = tid >> 3;
-    unsigned int* word = reinterpret_cast<unsigned int*>(sync + 1);
+    const bool on = tid < 256;
+    int* err = sync + 2;
+    unsigned int* pivots = reinterpret_cast<unsigned int*>(sync + 3);
+    unsigned int *panels = pivots + 1, *updates = pivots + 2;
     auto tile = [&](int i, int j) { return S + (((int64_t)i * nt + j) << 10); };
     auto load4 = [](const float2* p, int e) { return __ldcg(reinterpret_cast<const float4*>(p) + e); };
-    auto tile_to_T = [&](const float2* p) {
+    auto stage = [&](float2 (*dst)[33], const float2* p) {
 #pragma unroll
-        for (int u = 0; u < 2; ++u) {
+        for (int u = 0; u < 2 && on; ++u) {
             const float4 f = load4(p, 2 * tid + u);
-            sh.T[hi][4 * lo + 2 * u] = make_float2(f.x, f.y);
-            sh.T[hi][4 * lo + 2 * u + 1] = make_float2(f.z, f.w);
+            dst[hi][4 * lo + 2 * u] = make_float2(f.x, f.y);
+            dst[hi][4 * lo + 2 * u + 1] = make_float2(f.z, f.w);
         }
     };
-    auto leaf = [&](int k) {          // of the tile in T, to tile (k, k)
-        ff_leaf(sh);
+    // d -= Ls Rs (k-major): rows 2 ty, + 1, columns 2 tx, + 1
+    auto update = [&](const float4* Ls, const float4* Rs, float4* d) {
+        float s[4] = {}, e[4] = {};
 #pragma unroll
-        for (int u = 0; u < 4; ++u) tile(k, k)[hi * 32 + 4 * lo + u] = sh.T[hi][4 * lo + u];
+        for (int k0 = 0; k0 < 2; ++k0) {
+#pragma unroll 8
+            for (int kk = 16 * k0; kk < 16 * k0 + 16; ++kk) {
+                const float4 a = Ls[kk * 16 + ty], c = Rs[kk * 16 + tx];
+                const float2 a0 = make_float2(a.x, a.y), a1 = make_float2(a.z, a.w);
+                const float2 c0 = make_float2(c.x, c.y), c1 = make_float2(c.z, c.w);
+                ff_fma_acc(s[0], e[0], a0, c0);
+                ff_fma_acc(s[1], e[1], a0, c1);
+                ff_fma_acc(s[2], e[2], a1, c0);
+                ff_fma_acc(s[3], e[3], a1, c1);
+            }
+#pragma unroll
+            for (int u = 0; u < 4; ++u) {
+                const float2 n = ff_norm(s[u], e[u]);
+                s[u] = n.x;
+                e[u] = n.y;
+            }
+        }
+#pragma unroll
+        for (int u = 0; u < 2; ++u) {
+            const float2 x = ff_add(make_float2(d[u].x, d[u].y), make_float2(-s[2 * u], -e[2 * u]));
+            const float2 y = ff_add(make_float2(d[u].z, d[u].w), make_float2(-s[2 * u + 1], -e[2 * u + 1]));
+            d[u] = make_float4(x.x, x.y, y.x, y.y);
+        }
     };
-    if (tid == 0) sh.bad = 0;
+    float2* sub = reinterpret_cast<float2*>(sh.L);
     if (b == 0) {
-        tile_to_T(tile(0, 0));
+        if (tid == 0) sh.bad = 0;
+        stage(sh.T, tile(0, 0));
         __syncthreads();
-        leaf(0);
+        for (int k = 0;; ++k) {
+            ff_leaf(sh);
+#pragma unroll
+            for (int u = 0; u < 4 && on; ++u) tile(k, k)[hi * 32 + 4 * lo + u] = sh.T[hi][4 * lo + u];
+            arrive(pivots);
+            if (k == nt - 1) break;
+            if (!wait_for(updates, (unsigned)(NW * k), updates, 0u, err)) return;
+            stage(sh.A, tile(k + 1, k));
+            float4 d[2] = {};
+#pragma unroll
+            for (int u = 0; u < 2 && on; ++u) d[u] = load4(tile(k + 1, k + 1), (2 * ty + u) * 16 + tx);
+            arrive(panels);           // tile (k + 1, k) is read (the others' update overwrites it)
+            if (on) {
+                // L_k+1,k transposed: row hi, columns lo + 8 q; X_kk is lower triangular
+                float s[4] = {}, e[4] = {};
+#pragma unroll
+                for (int m0 = 0; m0 < 32; m0 += 16) {
+                    if (m0 <= hi)
+#pragma unroll 4
+                        for (int m = m0; m < m0 + 16; ++m)
+#pragma unroll
+                            for (int q = 0; q < 4; ++q) ff_fma_acc(s[q], e[q], sh.T[hi][m], sh.A[lo + 8 * q][m]);
+#pragma unroll
+                    for (int q = 0; q < 4; ++q) {
+                        const float2 n = ff_norm(s[q], e[q]);
+                        s[q] = n.x;
+                        e[q] = n.y;
+                    }
+                }
+#pragma unroll
+                for (int q = 0; q < 4; ++q) sub[hi * 32 + lo + 8 * q] = make_float2(s[q], e[q]);
+            }
+            __syncthreads();
+            if (on) {
+                update(sh.L, sh.L, d);
+#pragma unroll
+                for (int u = 0; u < 2; ++u) {
+                    sh.T[2 * ty + u][2 * tx] = make_float2(d[u].x, d[u].y);
+                    sh.T[2 * ty + u][2 * tx + 1] = make_float2(d[u].z, d[u].w);
+                }
+            }
+            __syncthreads();
+        }
+        if (tid == 0 && sh.bad) sync[0] = 1;
+        return;
     }
     for (int k = 0; k < nt; ++k) {
-        if (!msp::grid_barrier(word, sync + 2)) return;
+        // the tiles of step k - 1 and this step's pivot
+        if (!wait_for(updates, (unsigned)(NW * k), pivots, (unsigned)(k + 1), err)) return;
         // ---- panel
-        if (b < 4 * (nt - 1)) tile_to_T(tile(k, k));
-        float2* sub = reinterpret_cast<float2*>(sh.L);
-        for (int it = b; it < 4 * (nt - 1); it += G) {
+        if (b <= 4 * (nt - 1)) stage(sh.T, tile(k, k));
+        for (int it = b - 1; it < 4 * (nt - 1); it += NW) {
             const int q = it & 3, below = nt - 1 - k, t = it >> 2;
             const bool is_l = t < below;
             // rows 8 q .. of A_ik, or columns 8 q .. of X_kj
             float2* src = is_l ? tile(k + 1 + t, k) : tile(k, t - below);
-            if (is_l) sub[(tid >> 5) * 33 + (tid & 31)] = __ldcg(src + 256 * q + tid);
+            if (!on) {
+            } else if (is_l) sub[(tid >> 5) * 33 + (tid & 31)] = __ldcg(src + 256 * q + tid);
             else sub[tid] = __ldcg(src + hi * 32 + 8 * q + lo);
             __syncthreads();
             const float2* a = sub + (is_l ? 33 * lo : lo);
             const int step = is_l ? 1 : 8;
-            float s = 0.f, e = 0.f;
+            if (on) {
+                float s = 0.f, e = 0.f;
 #pragma unroll
-            for (int m0 = 0; m0 < 32; m0 += 16) {
+                for (int m0 = 0; m0 < 32; m0 += 16) {
 #pragma unroll
-                for (int m = m0; m < m0 + 16; ++m) ff_fma_acc(s, e, sh.T[hi][m], a[m * step]);
-                const float2 n = ff_norm(s, e);
-                s = n.x;
-                e = n.y;
+                    for (int m = m0; m < m0 + 16; ++m) ff_fma_acc(s, e, sh.T[hi][m], a[m * step]);
+                    const float2 n = ff_norm(s, e);
+                    s = n.x;
+                    e = n.y;
+                }
+                (is_l ? Lp + ((int64_t)(k + 1 + t) << 10) : src)[hi * 32 + 8 * q + lo] = make_float2(s, e);
             }
-            (is_l ? Lp + ((int64_t)(k + 1 + t) << 10) : src)[hi * 32 + 8 * q + lo] = make_float2(s, e);
             __syncthreads();
         }
-        if (k == nt - 1) break;
-        if (!msp::grid_barrier(word, sync + 2)) return;
-        // ---- update: row i = k + 1, .. has tiles j = i, .., 0
+        if (k == nt - 1) return;
+        arrive(panels);
+        if (!wait_for(panels, (unsigned)(G * (k + 1)), updates, 0u, err)) return;
+        // ---- update: row i = k + 1, .. has tiles j = i, .., 0; the first is block 0's
         const int tiles = nt * (nt + 1) / 2 - (k + 1) * (k + 2) / 2;
         int i = k + 1, j = i - b;
-        for (int t = b; t < tiles; t += G - 1) {
+        float4 l[2], r[2], dn[2];     // operands, one tile ahead
+        auto fetch = [&]() {
             while (j < 0) j += ++i + 1;
             const float2* Rg = j > k ? Lp + ((int64_t)j << 10) : tile(k, j);
             const float2* Lg = Lp + ((int64_t)i << 10);
-            float2* D = tile(i, j);
-            const float4 l0 = load4(Lg, tid), l1 = load4(Lg, tid + 256);
-            const float4 r0 = load4(Rg, tid), r1 = load4(Rg, tid + 256);
-            float4 d[2] = {};
-            if (j != k) {
-                d[0] = load4(D, (2 * ty) * 16 + tx);
-                d[1] = load4(D, (2 * ty + 1) * 16 + tx);
-            }
-            __syncthreads();          // the tile before is done with its operands
-            sh.L[tid] = l0;
-            sh.L[tid + 256] = l1;
-            sh.R[tid] = r0;
-            sh.R[tid + 256] = r1;
-            __syncthreads();
-            float s[4] = {}, e[4] = {};
-#pragma unroll
-            for (int k0 = 0; k0 < 2; ++k0) {
-#pragma unroll 8
-                for (int kk = 16 * k0; kk < 16 * k0 + 16; ++kk) {
-                    const float4 a = sh.L[kk * 16 + ty], c = sh.R[kk * 16 + tx];
-                    const float2 a0 = make_float2(a.x, a.y), a1 = make_float2(a.z, a.w);
-                    const float2 c0 = make_float2(c.x, c.y), c1 = make_float2(c.z, c.w);
-                    ff_fma_acc(s[0], e[0], a0, c0);
-                    ff_fma_acc(s[1], e[1], a0, c1);
-                    ff_fma_acc(s[2], e[2], a1, c0);
-                    ff_fma_acc(s[3], e[3], a1, c1);
-                }
-#pragma unroll
-                for (int u = 0; u < 4; ++u) {
-                    const float2 n = ff_norm(s[u], e[u]);
-                    s[u] = n.x;
-                    e[u] = n.y;
-                }
-            }
-            float4 o[2];
 #pragma unroll
             for (int u = 0; u < 2; ++u) {
-                const float2 x = ff_add(make_float2(d[u].x, d[u].y), make_float2(-s[2 * u], -e[2 * u]));
-                const float2 y = ff_add(make_float2(d[u].z, d[u].w), make_float2(-s[2 * u + 1], -e[2 * u + 1]));
-                o[u] = make_float4(x.x, x.y, y.x, y.y);
+                l[u] = load4(Lg, tid + 256 * u);
+                r[u] = load4(Rg, tid + 256 * u);
+                dn[u] = j == k ? make_float4(0.f, 0.f, 0.f, 0.f) : load4(tile(i, j), (2 * ty + u) * 16 + tx);
             }
-            if (b == 0) {
+        };
+        if (on && b < tiles) fetch();
+        for (int t = b; t < tiles; t += NW) {
+            float2* D = tile(i, j);
+            float4 d[2] = {dn[0], dn[1]};
+            __syncthreads();          // the tile before is done with its operands
 #pragma unroll
-                for (int u = 0; u < 2; ++u) {
-                    sh.T[2 * ty + u][2 * tx] = make_float2(o[u].x, o[u].y);
-                    sh.T[2 * ty + u][2 * tx + 1] = make_float2(o[u].z, o[u].w);
-                }
-                __syncthreads();
-                leaf(k + 1);
-                break;
+            for (int u = 0; u < 2 && on; ++u) {
+                sh.L[tid + 256 * u] = l[u];
+                sh.R[tid + 256 * u] = r[u];
             }
+            __syncthreads();
+            j -= NW;
+            if (!on) continue;
+            if (t + NW < tiles) fetch();
+            update(sh.L, sh.R, d);
 #pragma unroll
-            for (int u = 0; u < 2; ++u) reinterpret_cast<float4*>(D)[(2 * ty + u) * 16 + tx] = o[u];
-            j -= G - 1;
+            for (int u = 0; u < 2; ++u) reinterpret_cast<float4*>(D)[(2 * ty + u) * 16 + tx] = d[u];
         }
+        arrive(updates);
     }
-    if (b == 0 && tid == 0 && sh.bad) sync[0] = 1;
 }
 
 __global__ void k_copy_add_diag(const double* __restrict__ src, double* __restrict__ dst,
@@ -945,13 +1049,13 @@ msp_status chol_inv(msp_ctx* ctx, double* M, double* X, double* T1, double* T2, 
 }
 
 // One float-float attempt: k_chol_inv_ff on as many blocks as its widest step has
-// work for, two an SM at most. sync: its failure word, barrier word and error word.
+// work for and one more, one an SM at most. sync: six words, see there.
 msp_status chol_inv_ff(msp_ctx* ctx, float2* S, float2* Lp, int64_t sp, int* sync) {
     int nt = (int)(sp / 32), per_sm = 0;
     MSP_CUDA_TRY(ctx, cudaOccupancyMaxActiveBlocksPerMultiprocessor(&per_sm, k_chol_inv_ff, kFFThreads, 0));
     if (per_sm < 1) return msp_set_error(ctx, MSP_ECUDA, "factor: kernel does not fit on an SM");
     const int work = std::max(nt * (nt + 1) / 2 - 1, 4 * (nt - 1));
-    const int grid = std::max(2, std::min(work, std::min(per_sm, 2) * ctx->num_sms));
+    const int grid = std::max(2, std::min(work + 1, ctx->num_sms));
     void* args[] = {&S, &Lp, &nt, &sync};
     ++ctx->launches;
     MSP_CUDA_TRY(ctx, cudaLaunchCooperativeKernel((const void*)k_chol_inv_ff, dim3(grid), dim3(kFFThreads), args, 0,
@@ -978,7 +1082,7 @@ msp_status factor_shifted(msp_ctx* ctx, const double* M, int64_t s, int64_t sp, 
     double* Mw = (double*)scr;
     double* T1 = Mw + sp * sp;                       // ff: 32 columns, the panel
     double* T2 = T1 + sp * sp;
-    int* fail = (int*)(ff ? T1 + 32 * sp : T2 + sp * sp);        // and, ff, a barrier and an error word
+    int* fail = (int*)(ff ? T1 + 32 * sp : T2 + sp * sp);        // and, ff, the words of k_chol_inv_ff
     double* fro = (double*)(fail + 16);
     double* fro_part = fro + 2;
     int* hflag = (int*)ctx->host_flags;
@@ -1009,7 +1113,7 @@ msp_status factor_shifted(msp_ctx* ctx, const double* M, int64_t s, int64_t sp, 
     }
     for (int attempt = 0; attempt <= 4; ++attempt) {
         unsigned blocks = (unsigned)((sp * sp + 255) / 256);
-        MSP_CUDA_TRY(ctx, cudaMemsetAsync(fail, 0, 3 * sizeof(int), ctx->stream));
+        MSP_CUDA_TRY(ctx, cudaMemsetAsync(fail, 0, 6 * sizeof(int), ctx->stream));
         if (ff) {
             k_copy_add_diag_ff<<<blocks, 256, 0, ctx->stream>>>(M, reinterpret_cast<float2*>(Mw), sp, fro, attempt);
             MSP_CHECK_LAUNCH(ctx);

@@ -104,6 +104,19 @@ static msp_status stage_alloc(msp_ctx* ctx, size_t bytes) {
     return MSP_OK;
 }
 
+// Forks the context's side stream (created once, lazily) from its main stream; false:
+// not possible, the work stays on the main stream.
+static bool aux_fork(msp_ctx* ctx) {
+    if ((ctx->aux_stream || cudaStreamCreateWithFlags(&ctx->aux_stream, cudaStreamNonBlocking) == cudaSuccess) &&
+        (ctx->aux_ev[0] || cudaEventCreateWithFlags(&ctx->aux_ev[0], cudaEventDisableTiming) == cudaSuccess) &&
+        (ctx->aux_ev[1] || cudaEventCreateWithFlags(&ctx->aux_ev[1], cudaEventDisableTiming) == cudaSuccess) &&
+        cudaEventRecord(ctx->aux_ev[0], ctx->stream) == cudaSuccess &&
+        cudaStreamWaitEvent(ctx->aux_stream, ctx->aux_ev[0], 0) == cudaSuccess)
+        return true;
+    cudaGetLastError();
+    return false;
+}
+
 extern "C" {
 
 const char* msp_version(void) { return "msp-gb300 0.1 sm_103a"; }
@@ -224,15 +237,7 @@ static msp_status sym_pass_and_stats(msp_ctx* ctx, const float* A, msp_dtype dty
                                      float* packed, double* stats) {
     cudaStream_t side = nullptr;
     if (stats) {
-        if ((ctx->aux_stream ||
-             cudaStreamCreateWithFlags(&ctx->aux_stream, cudaStreamNonBlocking) == cudaSuccess) &&
-            (ctx->aux_ev[0] || cudaEventCreateWithFlags(&ctx->aux_ev[0], cudaEventDisableTiming) == cudaSuccess) &&
-            (ctx->aux_ev[1] || cudaEventCreateWithFlags(&ctx->aux_ev[1], cudaEventDisableTiming) == cudaSuccess) &&
-            cudaEventRecord(ctx->aux_ev[0], ctx->stream) == cudaSuccess &&
-            cudaStreamWaitEvent(ctx->aux_stream, ctx->aux_ev[0], 0) == cudaSuccess)
-            side = ctx->aux_stream;
-        else
-            cudaGetLastError();   // the statistics stay on the main stream
+        if (aux_fork(ctx)) side = ctx->aux_stream;   // else the statistics stay on the main stream
     }
     msp_status st = msp_sketch_sym_pass(ctx, A, n, lda, sp, ptr, ent, gamma, C, packed);
     if (stats && st == MSP_OK) {
@@ -572,7 +577,9 @@ msp_status msp_nystrom_impl(msp_ctx* ctx, const msp_sketch_s* sk, double lambda,
     msp_status st = MSP_OK;
     void* phi_mem = nullptr;
     float* Cr = nullptr;         // BF16 data: float(bf16(C)), the C every later step uses
+    cudaStream_t side = nullptr;      // W beside the Gram
     auto fail = [&](msp_status s2) {
+        if (side) cudaStreamSynchronize(side);
         cudaStreamSynchronize(ctx->stream);
         if (phi_mem) free_on(ctx, phi_mem);
         if (Cr) free_on(ctx, Cr);
@@ -597,11 +604,20 @@ msp_status msp_nystrom_impl(msp_ctx* ctx, const msp_sketch_s* sk, double lambda,
         (st = msp_alloc(ctx, (void**)&f->M2, mat_d)) != MSP_OK ||
         (st = msp_alloc(ctx, (void**)&f->Linv64, mat_d)) != MSP_OK)
         return fail(st);
-    // W = S C = Pi^T C: row c of W gathers the rows j of C listed for column c
+    // W = S C = Pi^T C: row c of W gathers the rows j of C listed for column c. Nothing
+    // reads it before the Gram's last kernel, so it is formed on the side stream
+    // (95 us, mostly reads from L2, at n = 16384, s = 1024) while the Gram's operands are split
+    // and multiplied; the worker contexts of a batch keep to their own stream.
+    if (ctx->fac_overlap && aux_fork(ctx)) side = ctx->aux_stream;
     const double sc = 1.0 / std::sqrt((double)sk->gamma);
-    if ((st = msp_gather_rows(ctx, sk->dtype, sp, sp, sk->csr_ptr, sk->csr_ent, Csrc, sp, sc, f->W,
-                              sp)) != MSP_OK)
-        return fail(st);
+    const cudaStream_t main_stream = ctx->stream;
+    if (side) ctx->stream = side;
+    st = msp_gather_rows(ctx, sk->dtype, sp, sp, sk->csr_ptr, sk->csr_ent, Csrc, sp, sc, f->W, sp);
+    if (st == MSP_OK) st = msp_symmetrize_w(ctx, f);
+    ctx->stream = main_stream;
+    if (st == MSP_OK && side && cudaEventRecord(ctx->aux_ev[1], side) != cudaSuccess)
+        st = msp_set_error(ctx, MSP_ECUDA, "nystrom: side stream record failed");
+    if (st != MSP_OK) return fail(st);
     const void* Ct = Csrc;
     int64_t phi_rows = n;
     if (phi > 0) {
@@ -627,7 +643,7 @@ msp_status msp_nystrom_impl(msp_ctx* ctx, const msp_sketch_s* sk, double lambda,
         Ct = ct;
         phi_rows = phi;
     }
-    if ((st = msp_build_factor(ctx, f, Ct, phi_rows)) != MSP_OK) return fail(st);
+    if ((st = msp_build_factor(ctx, f, Ct, phi_rows, side ? ctx->aux_ev[1] : nullptr)) != MSP_OK) return fail(st);
     // a sketched level 2 iterates on C^T C + lam~ W: formed once where the whole
     // iteration then runs on one cluster
     if (phi > 0 && f->data == MSP_F32 && msp_inner_ok(ctx, f->dtype, sp) &&

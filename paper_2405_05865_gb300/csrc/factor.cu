@@ -855,46 +855,67 @@ __global__ void k_copy_add_diag(const double* __restrict__ src, double* __restri
     dst[e] = src[e] + ((i == j) ? nu : 0.0);
 }
 
-// The shift and scaling of a float-float attempt from |M|_F^2: nu = 2^-24 |M|_F
-// 100^attempt, M scaled by 4^k to |M|_F in [1, 4). Formed on the device so that the
-// host need not wait for the norm before the factor starts.
-struct FFShift {
-    double nu;
-    int k;
+// What a float-float attempt takes from |M|_F, formed on the device so that the host
+// need not wait for the norm: the shift nu = 2^-24 |M|_F (times 100 per retry),
+// and 4^k and 2^k with |M|_F 4^k in [1, 4).
+struct FFScale {
+    double fro2, nu, up, out;
 };
-__device__ inline FFShift ff_shift(double fro2, int attempt) {
-    const double fn = sqrt(fro2);
-    FFShift f{ldexp(1.0, -24) * fn, fn > 0.0 && isfinite(fn) ? -(ilogb(fn) / 2) : 0};
-    for (int t = 0; t < attempt; ++t) f.nu *= 100.0;
-    return f;
-}
 
-// dst = (src + nu I) 4^k, row-major to 32 x 32 tiles
-__global__ void k_copy_add_diag_ff(const double* __restrict__ src, float2* __restrict__ dst,
-                                   int64_t s_pad, const double* __restrict__ fro2, int attempt) {
-    __shared__ double s_nu, s_scale;
-    if (threadIdx.x == 0) {
-        const FFShift f = ff_shift(*fro2, attempt);
-        s_nu = f.nu;
-        s_scale = ldexp(1.0, 2 * f.k);
+// The lower tiles of dst = (src + nu 100^attempt I) 4^k, row-major to 32 x 32 tiles
+// (a block (32, 8) a tile); the pivots need both triangles of theirs. Over the whole
+// square, each block forming the shift itself, 20 us at s_pad = 1024; now 12.
+__global__ void k_copy_add_diag_ff(const double* __restrict__ src, float2* __restrict__ dst, int64_t s_pad,
+                                   const FFScale* __restrict__ f, int attempt) {
+    if (blockIdx.x > blockIdx.y) return;
+    double nu = f->nu;
+    for (int t = 0; t < attempt; ++t) nu *= 100.0;
+    const double up = f->up;
+    const int64_t j = (int64_t)blockIdx.x * 32 + threadIdx.x;
+#pragma unroll
+    for (int r = 0; r < 4; ++r) {
+        const int64_t i = (int64_t)blockIdx.y * 32 + threadIdx.y + 8 * r;
+        double v = src[i * s_pad + j];
+        if (i == j) v += nu;
+        dst[ff_tile_at(i, j, s_pad)] = ff_from_double(v * up);
     }
-    __syncthreads();
-    int64_t e = (int64_t)blockIdx.x * blockDim.x + threadIdx.x;
-    if (e >= s_pad * s_pad) return;
-    int64_t i = e / s_pad, j = e % s_pad;
-    dst[ff_tile_at(i, j, s_pad)] = ff_from_double((src[e] + ((i == j) ? s_nu : 0.0)) * s_scale);
 }
 
-// dst = the lower triangle of src 2^k in FP64, tiles to row-major
-__global__ void k_ff_to_double(const float2* __restrict__ src, double* __restrict__ dst, int64_t s_pad,
-                               const double* __restrict__ fro2) {
-    __shared__ double s_scale;
-    if (threadIdx.x == 0) s_scale = ldexp(1.0, ff_shift(*fro2, 0).k);
+// L^{-1} = src 2^k from lower tiles: FP64 X, and FP32 B = X and Bt = X^T (null: not
+// asked for), zeros above (below) the diagonal. A block (32, 8) per tile pair (i, j),
+// (j, i): 11 us at s_pad = 1024, 22 as two kernels over rows.
+__global__ void __launch_bounds__(256) k_ff_unpack(const float2* __restrict__ src, int64_t s_pad,
+                                                   const FFScale* __restrict__ f, double* __restrict__ X,
+                                                   float* __restrict__ B, float* __restrict__ Bt) {
+    if (blockIdx.x > blockIdx.y) return;
+    __shared__ float tile[32][33];
+    const double out = f->out;
+    const bool diag = blockIdx.x == blockIdx.y;
+    const int64_t i0 = (int64_t)blockIdx.y * 32, j0 = (int64_t)blockIdx.x * 32;
+    const int x = threadIdx.x;
+#pragma unroll
+    for (int r = 0; r < 4; ++r) {
+        const int y = threadIdx.y + 8 * r;
+        const int64_t at = (i0 + y) * s_pad + j0 + x, up = (j0 + y) * s_pad + i0 + x;
+        const double v = diag && x > y ? 0.0 : ff_to_double(src[ff_tile_at(i0 + y, j0 + x, s_pad)]) * out;
+        X[at] = v;
+        if (!diag) X[up] = 0.0;
+        if (B) {
+            B[at] = (float)v;
+            if (!diag) {
+                B[up] = 0.f;
+                Bt[at] = 0.f;
+            }
+            tile[y][x] = (float)v;
+        }
+    }
+    if (!B) return;
     __syncthreads();
-    int64_t e = (int64_t)blockIdx.x * blockDim.x + threadIdx.x;
-    if (e >= s_pad * s_pad) return;
-    const int64_t i = e / s_pad, j = e % s_pad;
-    dst[e] = j <= i ? ff_to_double(src[ff_tile_at(i, j, s_pad)]) * s_scale : 0.0;
+#pragma unroll
+    for (int r = 0; r < 4; ++r) {
+        const int y = threadIdx.y + 8 * r;
+        Bt[(j0 + y) * s_pad + i0 + x] = tile[x][y];
+    }
 }
 
 // Frobenius norm^2 partials (single block, deterministic order).
@@ -918,12 +939,16 @@ __global__ void __launch_bounds__(256) k_fro2_part(const double* __restrict__ M,
     }
 }
 
-__global__ void k_fro2_final(const double* __restrict__ part, double* __restrict__ out) {
+__global__ void k_fro2_final(const double* __restrict__ part, FFScale* __restrict__ out) {
     double v = 0.0;
 #pragma unroll
     for (int b = 0; b < kFroBlocks; b += 32) v += part[b + threadIdx.x];
     v = msp::warp_sum(v);
-    if (threadIdx.x == 0) *out = v;
+    if (threadIdx.x == 0) {
+        const double fn = sqrt(v);
+        const int k = fn > 0.0 && isfinite(fn) ? -(ilogb(fn) / 2) : 0;
+        *out = FFScale{v, ldexp(1.0, -24) * fn, ldexp(1.0, 2 * k), ldexp(1.0, k)};
+    }
 }
 
 template <typename T>
@@ -1070,7 +1095,8 @@ msp_status chol_inv_ff(msp_ctx* ctx, float2* S, float2* Lp, int64_t sp, int* syn
 // second factorisation. FP64 data: unshifted first, then s 2^-52 |M|_F.
 // Then nu x 100 per retry, at most 4 retries, else MSP_ENOTPD.
 msp_status factor_shifted(msp_ctx* ctx, const double* M, int64_t s, int64_t sp, bool fp32_data,
-                          double* Linv64, double* shift_out, int* retries_out) {
+                          double* Linv64, double* shift_out, int* retries_out, float* B = nullptr,
+                          float* Bt = nullptr) {
     // FP32 data: the factorisation in float-float (its backward error, a
     // small multiple of s 2^-46 |M|, stays far below the shift 2^-24 |M|_F
     // the data needs), on M scaled by a power of four to |M|_F in [1, 4) so
@@ -1083,8 +1109,8 @@ msp_status factor_shifted(msp_ctx* ctx, const double* M, int64_t s, int64_t sp, 
     double* T1 = Mw + sp * sp;                       // ff: 32 columns, the panel
     double* T2 = T1 + sp * sp;
     int* fail = (int*)(ff ? T1 + 32 * sp : T2 + sp * sp);        // and, ff, the words of k_chol_inv_ff
-    double* fro = (double*)(fail + 16);
-    double* fro_part = fro + 2;
+    FFScale* fro = (FFScale*)(fail + 16);
+    double* fro_part = (double*)(fro + 1);
     int* hflag = (int*)ctx->host_flags;
     double* hfro = (double*)((char*)ctx->host_flags + 128);
     auto fro_launch = [&]() -> msp_status {
@@ -1092,7 +1118,7 @@ msp_status factor_shifted(msp_ctx* ctx, const double* M, int64_t s, int64_t sp, 
         MSP_CHECK_LAUNCH(ctx);
         k_fro2_final<<<1, 32, 0, ctx->stream>>>(fro_part, fro);
         MSP_CHECK_LAUNCH(ctx);
-        MSP_CUDA_TRY(ctx, cudaMemcpyAsync(hfro, fro, 8, cudaMemcpyDeviceToHost, ctx->stream));
+        MSP_CUDA_TRY(ctx, cudaMemcpyAsync(hfro, &fro->fro2, 8, cudaMemcpyDeviceToHost, ctx->stream));
         return MSP_OK;
     };
     auto fro_norm = [&](double* out) -> msp_status {
@@ -1103,7 +1129,7 @@ msp_status factor_shifted(msp_ctx* ctx, const double* M, int64_t s, int64_t sp, 
     };
     double nu = 0.0;
     if (ff) {
-        // nu and the scaling are formed on the device (ff_shift); the host reads the
+        // nu and the scaling are formed on the device (FFScale); the host reads the
         // norm with the outcome
         MSP_TRY(fro_launch());
     } else if (fp32_data) {
@@ -1115,10 +1141,11 @@ msp_status factor_shifted(msp_ctx* ctx, const double* M, int64_t s, int64_t sp, 
         unsigned blocks = (unsigned)((sp * sp + 255) / 256);
         MSP_CUDA_TRY(ctx, cudaMemsetAsync(fail, 0, 6 * sizeof(int), ctx->stream));
         if (ff) {
-            k_copy_add_diag_ff<<<blocks, 256, 0, ctx->stream>>>(M, reinterpret_cast<float2*>(Mw), sp, fro, attempt);
+            const dim3 tiles((unsigned)(sp / 32), (unsigned)(sp / 32)), thr(32, 8);
+            k_copy_add_diag_ff<<<tiles, thr, 0, ctx->stream>>>(M, reinterpret_cast<float2*>(Mw), sp, fro, attempt);
             MSP_CHECK_LAUNCH(ctx);
             MSP_TRY(chol_inv_ff(ctx, reinterpret_cast<float2*>(Mw), reinterpret_cast<float2*>(T1), sp, fail));
-            k_ff_to_double<<<blocks, 256, 0, ctx->stream>>>(reinterpret_cast<float2*>(Mw), Linv64, sp, fro);
+            k_ff_unpack<<<tiles, thr, 0, ctx->stream>>>(reinterpret_cast<float2*>(Mw), sp, fro, Linv64, B, Bt);
             MSP_CHECK_LAUNCH(ctx);
         } else {
             k_copy_add_diag<<<blocks, 256, 0, ctx->stream>>>(M, Mw, sp, nu);
@@ -1152,26 +1179,30 @@ msp_status factor_shifted(msp_ctx* ctx, const double* M, int64_t s, int64_t sp, 
 
 }  // namespace
 
-// Build W (symmetrised), M2, its shifted Cholesky inverse, and the working
-// copies B, Bt. `Ct` is C~ (phi_rows x s_pad, dtype of the sketch).
-msp_status msp_build_factor(msp_ctx* ctx, msp_factor_s* f, const void* Ct, int64_t phi_rows) {
+// W symmetrised, and its FP64 copy.
+msp_status msp_symmetrize_w(msp_ctx* ctx, msp_factor_s* f) {
     const int64_t sp = f->s_pad;
-    const size_t ts = dtype_size(f->dtype);
-    // W symmetrise + FP64 copy
-    {
-        dim3 blk(32, 32), grid((unsigned)((sp + 31) / 32), (unsigned)((sp + 31) / 32));
-        if (f->dtype == MSP_F32)
-            k_symmetrize<float><<<grid, blk, 0, ctx->stream>>>((float*)f->W, f->W64, sp);
-        else
-            k_symmetrize<double><<<grid, blk, 0, ctx->stream>>>((double*)f->W, f->W64, sp);
-        MSP_CHECK_LAUNCH(ctx);
-    }
+    const dim3 blk(32, 32), grid((unsigned)((sp + 31) / 32), (unsigned)((sp + 31) / 32));
+    if (f->dtype == MSP_F32)
+        k_symmetrize<float><<<grid, blk, 0, ctx->stream>>>((float*)f->W, f->W64, sp);
+    else
+        k_symmetrize<double><<<grid, blk, 0, ctx->stream>>>((double*)f->W, f->W64, sp);
+    MSP_CHECK_LAUNCH(ctx);
+    return MSP_OK;
+}
+
+// Build M2, its shifted Cholesky inverse, and the working copies B, Bt. `Ct` is C~
+// (phi_rows x s_pad, dtype of the sketch); W symmetrised, by w_ready.
+msp_status msp_build_factor(msp_ctx* ctx, msp_factor_s* f, const void* Ct, int64_t phi_rows, cudaEvent_t w_ready) {
+    const int64_t sp = f->s_pad;
     // M2 = Ct^T Ct + lam_t W: on the tensor cores (FP32 data), else split-K
     // partial Grams (upper tiles, mirrored) then the fixed-order FP64
     // combination
     if (f->dtype == MSP_F32 && ctx->gram_tc && msp_gram_tc_ok(sp)) {
-        MSP_TRY(msp_gram_tc(ctx, (const float*)Ct, phi_rows, sp, f->s, sp, (const float*)f->W, f->lam_tilde, f->M2));
+        MSP_TRY(msp_gram_tc(ctx, (const float*)Ct, phi_rows, sp, f->s, sp, (const float*)f->W, f->lam_tilde, f->M2,
+                            w_ready));
     } else {
+        if (w_ready) MSP_CUDA_TRY(ctx, cudaStreamWaitEvent(ctx->stream, w_ready, 0));
         double* P = nullptr;
         int slices = 0;
         const unsigned fb = (unsigned)((sp * sp + 255) / 256);
@@ -1186,14 +1217,16 @@ msp_status msp_build_factor(msp_ctx* ctx, msp_factor_s* f, const void* Ct, int64
         }
         MSP_CHECK_LAUNCH(ctx);
     }
-    MSP_TRY(factor_shifted(ctx, f->M2, f->s, sp, f->dtype == MSP_F32, f->Linv64, &f->shift, &f->retries));
+    const bool f32 = f->dtype == MSP_F32;
+    MSP_TRY(factor_shifted(ctx, f->M2, f->s, sp, f32, f->Linv64, &f->shift, &f->retries,
+                           f32 ? (float*)f->B : nullptr, f32 ? (float*)f->Bt : nullptr));
+    if (f32 && ctx->factor_ff) return MSP_OK;       // B and Bt are there
     unsigned b2 = (unsigned)((sp * sp + 255) / 256);
-    if (f->dtype == MSP_F32)
+    if (f32)
         k_cast_tri<float><<<b2, 256, 0, ctx->stream>>>(f->Linv64, (float*)f->B, (float*)f->Bt, sp);
     else
         k_cast_tri<double><<<b2, 256, 0, ctx->stream>>>(f->Linv64, (double*)f->B, (double*)f->Bt, sp);
     MSP_CHECK_LAUNCH(ctx);
-    (void)ts;
     return MSP_OK;
 }
 

@@ -22,7 +22,7 @@
 //                    the MMA steps between drains (measured): 4 for hh. The
 //                    item's 128 x 128 partial is written in FP64;
 //   k_gram_tc_finish M2 = (sum over slices, in order, in FP64) / q^2 + lam W,
-//                    mirrored, identity on the padding.
+//                    upper tiles mirrored, identity on the padding.
 // Warp roles in k_gram_tc: 0 TMA producer (and tensor-memory owner), 1 MMA
 // issuer, 2..9 drain (tensor-memory lane quarter = warp mod 4, 64 columns
 // each).
@@ -67,44 +67,55 @@ __global__ void k_absmax(const float* __restrict__ X, int64_t K, int64_t ld, int
                          unsigned int* __restrict__ out) {
     float m = 0.f;
     for (int64_t r = blockIdx.x; r < K; r += gridDim.x)
+#pragma unroll 4
         for (int64_t c = threadIdx.x; c < s; c += blockDim.x) m = fmaxf(m, fabsf(X[r * ld + c]));
 #pragma unroll
     for (int o = 16; o > 0; o >>= 1) m = fmaxf(m, __shfl_xor_sync(0xffffffffu, m, o));
     if ((threadIdx.x & 31) == 0 && m > 0.f) atomicMax(out, __float_as_uint(m));
 }
 
-// q = 2^(14 - e) with max < 2^e (1 for an all-zero X)
-__global__ void k_scale_of(const unsigned int* __restrict__ mx, float* __restrict__ q) {
+// q = 2^(14 - e) with max < 2^e (1 for an all-zero X), and q^-2
+__global__ void k_scale_of(const unsigned int* __restrict__ mx, float* __restrict__ q, double* __restrict__ unscale) {
     const float m = __uint_as_float(*mx);
     int e = 0;
     if (m > 0.f && isfinite(m)) frexpf(m, &e);
     *q = ldexpf(1.0f, 14 - max(e, -100));   // q m < 2^14; q finite
+    *unscale = ldexp(1.0, -2 * (14 - max(e, -100)));
 }
 
 // H^T, M^T, L^T (s_t x K_pad FP16, zero beyond K and s) from v = q x:
 // h = fp16(v), m = fp16(v - h), l = fp16(v - h - m) (both differences exact
-// in FP32); 32 x 32 tiles, block (32, 8).
+// in FP32); tiles of 64 rows and 32 columns, block (32, 8): a lane writes two rows, a
+// warp 128 bytes of each term.
 __global__ void k_split_t(const float* __restrict__ X, int64_t K, int64_t ld, int64_t s, int64_t K_pad,
                           const float* __restrict__ qp, __half* __restrict__ Ht, __half* __restrict__ Mt,
                           __half* __restrict__ Lt) {
-    __shared__ float tile[32][33];
+    __shared__ float tile[64][33];
     const float q = *qp;
-    const int64_t k0 = (int64_t)blockIdx.x * 32, c0 = (int64_t)blockIdx.y * 32;
-    for (int i = threadIdx.y; i < 32; i += 8) {
+    const int64_t k0 = (int64_t)blockIdx.x * 64, c0 = (int64_t)blockIdx.y * 32;
+#pragma unroll
+    for (int i = threadIdx.y; i < 64; i += 8) {
         const int64_t k = k0 + i, c = c0 + threadIdx.x;
         tile[i][threadIdx.x] = (k < K && c < s) ? q * X[k * ld + c] : 0.f;
     }
     __syncthreads();
+    const int64_t k = k0 + 2 * threadIdx.x;       // K_pad is a multiple of 32
+    if (k >= K_pad) return;
+#pragma unroll
     for (int i = threadIdx.y; i < 32; i += 8) {
-        const int64_t c = c0 + i, k = k0 + threadIdx.x;
-        const float v = tile[threadIdx.x][i];
-        const __half h = __float2half_rn(v);
-        const float r1 = __fsub_rn(v, __half2float(h));
-        const __half m = __float2half_rn(r1);
-        const __half l = __float2half_rn(__fsub_rn(r1, __half2float(m)));
-        Ht[c * K_pad + k] = h;
-        Mt[c * K_pad + k] = m;
-        Lt[c * K_pad + k] = l;
+        __half2 h, m, l;
+        auto split = [](float v, __half& a, __half& b, __half& c) {
+            a = __float2half_rn(v);
+            const float r1 = __fsub_rn(v, __half2float(a));
+            b = __float2half_rn(r1);
+            c = __float2half_rn(__fsub_rn(r1, __half2float(b)));
+        };
+        split(tile[2 * threadIdx.x][i], h.x, m.x, l.x);
+        split(tile[2 * threadIdx.x + 1][i], h.y, m.y, l.y);
+        const int64_t at = (c0 + i) * K_pad + k;
+        *reinterpret_cast<__half2*>(Ht + at) = h;
+        *reinterpret_cast<__half2*>(Mt + at) = m;
+        *reinterpret_cast<__half2*>(Lt + at) = l;
     }
 }
 
@@ -305,30 +316,50 @@ k_gram_tc(const __grid_constant__ CUtensorMap tmH, const __grid_constant__ CUten
 }
 
 // M2[a][b] = (sum over slices of the tile partial, FP64, slice order) / q^2
-//            + lam (W ? W[a][b] : [a == b]); the upper partial mirrored;
-//            identity on the padding.
-template <typename TW>
-__global__ void k_gram_tc_finish(const double* __restrict__ P, int nt, int ns, const float* __restrict__ qp,
-                                 const TW* __restrict__ W, double lam, int64_t s, int64_t s_pad,
-                                 double* __restrict__ M2) {
-    const int64_t e = (int64_t)blockIdx.x * blockDim.x + threadIdx.x;
-    if (e >= s_pad * s_pad) return;
-    const int64_t a = e / s_pad, b = e % s_pad;
-    if (a >= s || b >= s) {
-        M2[e] = (a == b) ? 1.0 : 0.0;
-        return;
-    }
-    const int64_t lo = a < b ? a : b, hi = a < b ? b : a;
-    const int ta = (int)(lo / kGT), tb = (int)(hi / kGT);
+//            + lam (W ? W[a][b] : [a == b]), W symmetric; identity on the
+//            padding. A block (32, 8) forms a 32 x 32 tile of the upper triangle
+//            and stores it at both places; q^-2 is a power of two, so its product is
+//            the quotient. FP64-issue-bound an entry at a time over the whole square,
+//            with a division and column reads of the mirrored partials, it took
+//            36 us at s = 1024, and takes 16.
+__global__ void __launch_bounds__(256) k_gram_tc_finish(const double* __restrict__ P, int nt, int ns,
+                                                        const double* __restrict__ unscale,
+                                                        const float* __restrict__ W, double lam, int64_t s,
+                                                        int64_t s_pad, double* __restrict__ M2) {
+    if (blockIdx.x < blockIdx.y) return;
+    __shared__ double tile[32][33];
+    const double u = *unscale;
+    const int64_t a0 = (int64_t)blockIdx.y * 32, b0 = (int64_t)blockIdx.x * 32, b = b0 + threadIdx.x;
+    const int ta = (int)(a0 / kGT), tb = (int)(b0 / kGT);
     const int64_t p = (int64_t)ta * nt - (int64_t)ta * (ta - 1) / 2 + (tb - ta);
-    // within the pair's tile: row from the first tile, column from the second
-    const int64_t r = lo % kGT, c = hi % kGT;
-    double v = 0.0;
-    for (int sl = 0; sl < ns; ++sl) v += P[((p * ns + sl) * kGT + r) * kGT + c];
-    const double q = (double)*qp;
-    v /= q * q;
-    v += W ? lam * (double)W[e] : (a == b ? lam : 0.0);
-    M2[e] = v;
+    double v[4];
+#pragma unroll
+    for (int i = 0; i < 4; ++i) {
+        const int64_t a = a0 + threadIdx.y + 8 * i;
+        // within the pair's tile: row from the first tile, column from the second
+        const double* src = P + (p * ns * kGT + a % kGT) * kGT + b % kGT;
+        v[i] = 0.0;
+        if (a > b || b >= s) {
+            if (a == b) v[i] = 1.0;
+        } else {
+            for (int sl = 0; sl < ns; ++sl) v[i] += src[(int64_t)sl * kGT * kGT];
+            v[i] *= u;
+            v[i] += W ? lam * (double)W[a * s_pad + b] : (a == b ? lam : 0.0);
+        }
+        tile[threadIdx.y + 8 * i][threadIdx.x] = v[i];
+    }
+    __syncthreads();
+#pragma unroll
+    for (int i = 0; i < 4; ++i) {
+        const int y = threadIdx.y + 8 * i, x = threadIdx.x;
+        const int64_t a = a0 + y;
+        if (a0 == b0) {
+            M2[a * s_pad + b] = x < y ? tile[x][y] : v[i];
+        } else {
+            M2[a * s_pad + b] = v[i];
+            M2[(b0 + y) * s_pad + a0 + x] = tile[x][y];
+        }
+    }
 }
 
 }  // namespace
@@ -336,12 +367,12 @@ __global__ void k_gram_tc_finish(const double* __restrict__ P, int nt, int ns, c
 // M2 = X^T X + lam W (W: s_pad x s_pad; null: + lam I) for X: K x s FP32
 // (leading dimension ld, no alignment needed), FP64 s_pad x s_pad out with
 // the identity on the padding. The tiles cover s_t = s_pad rounded up to 128
-// (zero columns beyond s). Callers check msp_gram_tc_ok first (the
+// (zero columns beyond s). W is read after w_ready (null: at once). Callers check msp_gram_tc_ok first (the
 // tensor-map encoder exists); otherwise they use the FP32-pipe Gram.
 bool msp_gram_tc_ok(int64_t s_pad) { return s_pad % 32 == 0 && msp_tensor_map_encoder() != nullptr; }
 
 msp_status msp_gram_tc(msp_ctx* ctx, const float* X, int64_t K, int64_t ld, int64_t s, int64_t s_pad,
-                       const float* W, double lam, double* M2) {
+                       const float* W, double lam, double* M2, cudaEvent_t w_ready) {
     auto enc = msp_tensor_map_encoder();
     if (!enc || s_pad % 32 != 0 || K < 1 || s < 1 || s > s_pad || ld < s || K >= (1ll << 30))
         return msp_set_error(ctx, MSP_EINVAL, "gram_tc: unsupported arguments");
@@ -382,12 +413,13 @@ msp_status msp_gram_tc(msp_ctx* ctx, const float* X, int64_t K, int64_t ld, int6
     double* P = (double*)c; c += b_p;
     unsigned int* mx = (unsigned int*)c;
     float* q = (float*)(c + 16);
+    double* unscale = (double*)(c + 24);
     MSP_CUDA_TRY(ctx, cudaMemsetAsync(mx, 0, 4, ctx->stream));
     k_absmax<<<(unsigned)std::min<int64_t>(K, 4 * ctx->num_sms), 256, 0, ctx->stream>>>(X, K, ld, s, mx);
     MSP_CHECK_LAUNCH(ctx);
-    k_scale_of<<<1, 1, 0, ctx->stream>>>(mx, q);
+    k_scale_of<<<1, 1, 0, ctx->stream>>>(mx, q, unscale);
     MSP_CHECK_LAUNCH(ctx);
-    k_split_t<<<dim3((unsigned)(K_pad / 32), (unsigned)(s_t / 32)), dim3(32, 8), 0, ctx->stream>>>(
+    k_split_t<<<dim3((unsigned)((K_pad + 63) / 64), (unsigned)(s_t / 32)), dim3(32, 8), 0, ctx->stream>>>(
         X, K, ld, s, K_pad, q, T[0], T[1], T[2]);
     MSP_CHECK_LAUNCH(ctx);
     CUtensorMap tm[kGTerms];
@@ -408,8 +440,9 @@ msp_status msp_gram_tc(msp_ctx* ctx, const float* X, int64_t K, int64_t ld, int6
     k_gram_tc<<<(unsigned)items, kGThreads, kGSmem, ctx->stream>>>(tm[0], tm[1], tm[2], nt, K_pad, slice_k, ns, P,
                                                                      &ctl->error);
     MSP_CHECK_LAUNCH(ctx);
-    const unsigned fb = (unsigned)((s_pad * s_pad + 255) / 256);
-    k_gram_tc_finish<float><<<fb, 256, 0, ctx->stream>>>(P, nt, ns, q, W, lam, s, s_pad, M2);
+    if (w_ready) MSP_CUDA_TRY(ctx, cudaStreamWaitEvent(ctx->stream, w_ready, 0));
+    const unsigned sub = (unsigned)(s_pad / 32);
+    k_gram_tc_finish<<<dim3(sub, sub), dim3(32, 8), 0, ctx->stream>>>(P, nt, ns, unscale, W, lam, s, s_pad, M2);
     MSP_CHECK_LAUNCH(ctx);
     return MSP_OK;
 }

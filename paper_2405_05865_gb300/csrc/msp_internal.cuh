@@ -42,8 +42,8 @@ struct msp_ctx {
     // only after every wait on its previous record has been enqueued)
     cudaStream_t fac_side[8] = {};
     cudaEvent_t fac_ev[8][2] = {};
-    // side stream and fork/join events of the sketch's row statistics
-    // (created once, lazily)
+    // side stream and fork/join events of the sketch's row statistics and of the
+    // factor's W (created once, lazily)
     cudaStream_t aux_stream = nullptr;
     cudaEvent_t aux_ev[2] = {};
     bool fac_overlap = true;     // false: the factor's products stay on the main stream
@@ -338,13 +338,15 @@ msp_status msp_norm_lb_launch(msp_ctx* ctx, const void* A, msp_dtype dt, int64_t
 
 // gram_tc.cu: M2 = X^T X + lam W (W null: + lam I) on the tensor cores
 // (two FP16 terms per entry, FP64 across K slices); MSP_EINVAL when the
-// tensor-core path is unavailable
+// tensor-core path is unavailable. W is read after w_ready (null: at once)
 msp_status msp_gram_tc(msp_ctx* ctx, const float* X, int64_t K, int64_t ld, int64_t s, int64_t s_pad,
-                       const float* W, double lam, double* M2);
+                       const float* W, double lam, double* M2, cudaEvent_t w_ready);
 bool msp_gram_tc_ok(int64_t s_pad);
 
 // factor.cu
-msp_status msp_build_factor(msp_ctx* ctx, msp_factor_s* f, const void* Ct, int64_t phi_rows);
+msp_status msp_symmetrize_w(msp_ctx* ctx, msp_factor_s* f);
+// w_ready: the event after which the symmetrised W may be read (null: at once)
+msp_status msp_build_factor(msp_ctx* ctx, msp_factor_s* f, const void* Ct, int64_t phi_rows, cudaEvent_t w_ready);
 // f->H = C^T C + lam~ W, C of n rows
 msp_status msp_form_level2(msp_ctx* ctx, msp_factor_s* f, const void* C, int64_t n);
 // G64 = X^T X + diag I (FP64, pad identity); M^{-1} of an SPD FP64 matrix;

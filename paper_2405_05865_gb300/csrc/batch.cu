@@ -128,9 +128,10 @@ struct BCtl {
 struct BArgs {
     const BInst* inst;
     int count, nrows, nstrips, nchunks;
+    int tri_wide;         // factor chunks of 64 rows, not 32
     const int2* rows;     // (instance, row block), largest n first
     const int2* strips;   // (instance, 64-column strip of C | row segment << 16), longest first
-    const int2* chunks;   // (instance, 32-row chunk of s from the long end), longest first
+    const int2* chunks;   // (instance, chunk of s from the long end), longest first
     int nunits;
     int ut;               // tiles per unit
     const int2* units;    // (instance, row block | unit << 16), largest first
@@ -957,11 +958,18 @@ __device__ __noinline__ void consume_G(const BArgs& a, unsigned char* ring, uint
 // dealt out in turn, so no block waits for a shared counter. With 128-row items
 // claimed from a counter the two steps took 46 us an iteration of the 24-instance
 // batch (n 512 to 4096), and take 37.
-constexpr int kTriRows = 32, kTriK = 256;
+//
+// With many instances the items' number is no concern and the vector block's
+// shared-memory reads are: from kTriMany 32-row chunks for each block on, items have
+// 64 rows, two a lane (R = 2), in pieces of 128 columns: 64 instances of
+// the benchmark (10 or so chunks a block) 17.9 ms of a solve in these steps, 23.0 with 32
+// rows; the batch of 24 has 3 chunks a block and keeps the shorter items.
+constexpr int kTriMany = 6;
 
-template <bool kUpper>
+template <bool kUpper, int R>
 __device__ __noinline__ void step_tri(const BArgs& a, int t, unsigned char* smem, float* red, int tid, int w,
                                       int lane) {
+    constexpr int kTriRows = 32 * R, kTriK = 256 / R, kRowG = kTriK / 4;     // a piece, granules a row
     const int cur = t & 1;
     float* tiles = reinterpret_cast<float*>(smem);
     float* Vs = reinterpret_cast<float*>(smem + kVsOffset);
@@ -986,9 +994,9 @@ __device__ __noinline__ void step_tri(const BArgs& a, int t, unsigned char* smem
                 const int kb = k0 + i * kTriK;
 #pragma unroll
                 for (int j = 0; j < 8; ++j) {
-                    // row e / 64, granule e % 64 of the piece; granule g of row r at
+                    // row e / kRowG, granule e % kRowG of the piece; granule g of row r at
                     // g ^ (r & 7): lanes over rows then read distinct banks
-                    const int e = tid + kWorkers * j, row = e >> 6, g = e & 63;
+                    const int e = tid + kWorkers * j, row = e / kRowG, g = e % kRowG;
                     const bool ok = kb + 4 * g < k1;
                     msp::cp_async16(dst + row * kTriK + ((g ^ (row & 7)) << 2),
                                     M + (int64_t)row * I.s_pad + (ok ? kb + 4 * g : k0), ok);
@@ -1000,43 +1008,58 @@ __device__ __noinline__ void step_tri(const BArgs& a, int t, unsigned char* smem
         issue(0);
         issue(1);
         stage_vec(Vs, (kUpper ? a.Y1 : a.G) + (int64_t)I.soff * kM, a.gstride, kUpper ? 1 : I.ng, k0, k1, tid);
-        float acc[16];
+        float acc[R][16];
 #pragma unroll
-        for (int c = 0; c < 16; ++c) acc[c] = 0.f;
+        for (int q = 0; q < R; ++q)
+#pragma unroll
+            for (int c = 0; c < 16; ++c) acc[q][c] = 0.f;
 #pragma unroll 1
         for (int i = 0; i < nt; ++i) {
             issue(i + 2);
             msp::cp_async_wait<2>();
             msp::bar_workers<kWorkers>();
-            const float4* T4 = reinterpret_cast<const float4*>(tiles + (i % kMvTiles) * kTileFloats) + lane * (kTriK / 4);
-            const int kw = k0 + i * kTriK + 32 * w;      // this warp's columns
+            const float4* T4 = reinterpret_cast<const float4*>(tiles + (i % kMvTiles) * kTileFloats) + lane * kRowG;
+            const int kw = k0 + i * kTriK + kTriK / 8 * w;      // this warp's columns
             const ulonglong2* V4 = reinterpret_cast<const ulonglong2*>(Vs) + (int64_t)kw * 4;
-            const int gn = min(8, (k1 - kw + 3) / 4);    // granules of it (the ranges are multiples of 32)
+            const int gn = min(kRowG / 8, (k1 - kw + 3) / 4);    // granules of it (the ranges are multiples of 32)
 #pragma unroll 2
             for (int g = 0; g < gn; ++g) {
-                const float4 m = T4[(8 * w + g) ^ (lane & 7)];
+                float4 m[R];
+#pragma unroll
+                for (int q = 0; q < R; ++q) m[q] = T4[32 * q * kRowG + ((kRowG / 8 * w + g) ^ (lane & 7))];
 #pragma unroll
                 for (int kk = 0; kk < 4; ++kk) {
-                    const uint64_t mv = dup2(comp(m, kk));
+                    uint64_t mv[R];
 #pragma unroll
-                    for (int j = 0; j < 4; ++j) fma4(&acc[4 * j], mv, V4[(4 * g + kk) * 4 + j]);
+                    for (int q = 0; q < R; ++q) mv[q] = dup2(comp(m[q], kk));
+#pragma unroll
+                    for (int j = 0; j < 4; ++j) {
+                        const ulonglong2 v = V4[(4 * g + kk) * 4 + j];
+#pragma unroll
+                        for (int q = 0; q < R; ++q) fma4(&acc[q][4 * j], mv[q], v);
+                    }
                 }
             }
             msp::bar_workers<kWorkers>();
         }
 #pragma unroll
-        for (int c = 0; c < 16; ++c) red[(w * 16 + c) * 32 + lane] = acc[c];
-        msp::bar_workers<kWorkers>();
-        // thread: row tid >> 3, columns 2 (tid & 7), + 1
-        const int row = tid >> 3, c = 2 * (tid & 7);
-        float o0 = 0.f, o1 = 0.f;
+        for (int q = 0; q < R; ++q)
 #pragma unroll
-        for (int ww = 0; ww < kWorkWarps; ++ww) {
-            o0 += red[(ww * 16 + c) * 32 + row];
-            o1 += red[(ww * 16 + c + 1) * 32 + row];
-        }
+            for (int c = 0; c < 16; ++c) red[(w * 16 + c) * kTriRows + 32 * q + lane] = acc[q][c];
+        msp::bar_workers<kWorkers>();
+        // thread: 2 R columns of a row
+        const int row = tid / (8 / R), c = 2 * R * (tid % (8 / R));
         float* Y = (kUpper ? a.Y2 : a.Y1) + ((int64_t)I.soff + r0 + row) * kM + c;
-        *reinterpret_cast<float2*>(Y) = make_float2(o0, o1);
+#pragma unroll
+        for (int u = 0; u < 2 * R; u += 2) {
+            float o0 = 0.f, o1 = 0.f;
+#pragma unroll
+            for (int ww = 0; ww < kWorkWarps; ++ww) {
+                o0 += red[(ww * 16 + c + u) * kTriRows + row];
+                o1 += red[(ww * 16 + c + u + 1) * kTriRows + row];
+            }
+            *reinterpret_cast<float2*>(Y + u) = make_float2(o0, o1);
+        }
     }
     msp::cp_async_wait<0>();
     msp::bar_workers<kWorkers>();
@@ -1340,9 +1363,11 @@ __global__ void __launch_bounds__(kThreads, 1) k_batch_solve(BArgs a) {
                 ctl->active[(t + 1) & 1] = 0;
                 ctl->sweepsA += 1;
             }
-            if (worker) step_tri<false>(a, t, smem, red, tid, w, lane);
+            if (worker && a.tri_wide) step_tri<false, 2>(a, t, smem, red, tid, w, lane);
+            else if (worker) step_tri<false, 1>(a, t, smem, red, tid, w, lane);
             MSP_GBAR(kTTri);
-            if (worker) step_tri<true>(a, t, smem, red, tid, w, lane);
+            if (worker && a.tri_wide) step_tri<true, 2>(a, t, smem, red, tid, w, lane);
+            else if (worker) step_tri<true, 1>(a, t, smem, red, tid, w, lane);
             MSP_GBAR(kTTri);
             if (worker) consume_Z(a, ring, full, empty, hdr, kring, red, wsum, w, lane);
             else if (lane == 0)
@@ -1407,6 +1432,7 @@ struct msp_batch_s {
     std::vector<msp_factor_t*> f;
     std::vector<BInst> hinst;
     std::vector<int2> rows, strips, chunks, units;
+    bool tri_wide = false;
     void* mem = nullptr;
     cudaStream_t stream = nullptr;
     BArgs args{};
@@ -1709,11 +1735,15 @@ msp_status msp_batch_create(msp_ctx* ctx, int count, const msp_instance* inst, m
     };
     std::stable_sort(b->strips.begin(), b->strips.end(),
                      [&](const int2& x, const int2& y) { return seg_len(x) > seg_len(y); });
-    // longest first: chunk c of an instance has s_pad - 32 c columns
+    // longest first: chunk c of an instance has s_pad - rows c columns
+    int64_t chunks32 = 0;
+    for (int k : by_n) chunks32 += b->hinst[k].s_pad / 32;
+    b->tri_wide = chunks32 >= (int64_t)kTriMany * ctx->num_sms;
+    const int rows = b->tri_wide ? 64 : 32;
     for (int k : by_n)
-        for (int s = 0; s < b->hinst[k].s_pad / kTriRows; ++s) b->chunks.push_back(make_int2(k, s));
+        for (int s = 0; s < b->hinst[k].s_pad / rows; ++s) b->chunks.push_back(make_int2(k, s));
     std::stable_sort(b->chunks.begin(), b->chunks.end(), [&](const int2& x, const int2& y) {
-        return b->hinst[x.x].s_pad - kTriRows * x.y > b->hinst[y.x].s_pad - kTriRows * y.y;
+        return b->hinst[x.x].s_pad - rows * x.y > b->hinst[y.x].s_pad - rows * y.y;
     });
     b->by_n = by_n;
     // room for the units list at the smallest width
@@ -1816,6 +1846,7 @@ msp_status msp_batch_create(msp_ctx* ctx, int count, const msp_instance* inst, m
     A.nrows = (int)b->rows.size();
     A.nstrips = (int)b->strips.size();
     A.nchunks = (int)b->chunks.size();
+    A.tri_wide = b->tri_wide;
     A.rows = (const int2*)(base + o_rows);
     A.strips = (const int2*)(base + o_strips);
     A.chunks = (const int2*)(base + o_chunks);

@@ -37,3 +37,25 @@ def test_batch_item_edges(sizes):
         assert infos[k]["status"] == 0
     bt.close()
     ctx.close()
+
+
+@pytest.mark.parametrize("count,s", [(56, 500), (57, 500), (115, 200)])
+def test_many_factor_chunks(count, s):
+    """Just below and at the number of factor chunks where their items have 64 rows (912
+    chunks of 32 on 152 SMs), and short factors (s_pad = 256); every column's FP64
+    residual against the stopping rule."""
+    from paper_2405_05865_gb300 import Context
+    ctx = Context(0)
+    lam, n = 1e-2, 540
+    A = torch.from_numpy(rbf_kernel(rbf_points(n, seed=9), 0.08, out_dtype=np.float32)).cuda()
+    gen = torch.Generator(device="cuda").manual_seed(count)
+    Bs = [torch.randn((n, 3), generator=gen, device="cuda", dtype=torch.float64) for _ in range(count)]
+    bt = ctx.batch([dict(A=A, B=B, lam=lam, s=s) for B in Bs])
+    bt.solve(tol=1e-9, refine_tol=1e-4)
+    Ad = A.double()
+    for k, B in enumerate(Bs):
+        X = bt.X(k)
+        r = (B - Ad @ X - lam * X).norm(dim=0)
+        assert bool((r <= 1.01e-9 * B.norm(dim=0)).all())
+    bt.close()
+    ctx.close()

@@ -16,6 +16,7 @@
 // in the same order, so all blocks take identical branches and the number of
 // grid barriers always matches. Reductions use fixed orders (deterministic).
 #include "bulk.cuh"
+#include "l2_columns.cuh"
 #include "msp_internal.cuh"
 
 #include <cooperative_groups.h>
@@ -377,9 +378,10 @@ __device__ inline void load_pair(const __nv_bfloat16* p, float& a, float& b) {
 template <typename T, typename TC, int PL>
 struct L2Shape {
     static constexpr int SP = 32 * PL;
-    static constexpr int U = SP / 2;                              // column pairs
-    static constexpr int NG = U >= kThreads ? 1 : kThreads / U;   // row groups of the column pass
-    static constexpr int KU = (U + kThreads - 1) / kThreads;      // pairs per thread
+    using Cols = msp::L2Columns<SP, kThreads>;
+    static constexpr int U = Cols::pairs;
+    static constexpr int NG = Cols::groups;         // row groups of the column pass
+    static constexpr int KU = Cols::per_thread;
     static constexpr int SCR = NG * SP > kQScratch ? NG * SP : kQScratch;
     // four full vectors, the scratch of the reductions, r and the row results
     static constexpr size_t fixed = ((size_t)4 * SP + SCR + 2 * kRowChunk) * sizeof(T) + 16;
@@ -402,17 +404,20 @@ template <typename T, typename TC, int PL>
 __device__ __forceinline__ void cols_pass(const BlockRows<TC>& rows, int cb, int ce, const T* coef,
                                           T (&acc)[L2Shape<T, TC, PL>::KU][2]) {
     using S = L2Shape<T, TC, PL>;
-    const int grp = S::NG > 1 ? (int)threadIdx.x / S::U : 0;
-    const int u0 = S::NG > 1 ? (int)threadIdx.x % S::U : (int)threadIdx.x;
-    if (grp >= S::NG || u0 >= S::U) return;
+    if (!S::Cols::active((int)threadIdx.x)) return;
+    const int grp = S::Cols::group((int)threadIdx.x), u0 = S::Cols::first((int)threadIdx.x);
     int i = max(cb, rows.nres) + grp;
     for (; i + 7 * S::NG < ce; i += 8 * S::NG) {
         T c[8][S::KU][2];
 #pragma unroll
         for (int q = 0; q < 8; ++q)
 #pragma unroll
-            for (int k = 0; k < S::KU; ++k)
-                load_pair(rows.g + (int64_t)(i + q * S::NG) * S::SP + 2 * (u0 + k * kThreads), c[q][k][0], c[q][k][1]);
+            for (int k = 0; k < S::KU; ++k) {
+                c[q][k][0] = c[q][k][1] = T(0);
+                if (S::Cols::has(u0, k))
+                    load_pair(rows.g + (int64_t)(i + q * S::NG) * S::SP + 2 * (u0 + k * kThreads), c[q][k][0],
+                              c[q][k][1]);
+            }
 #pragma unroll
         for (int q = 0; q < 8; ++q) {
             const T f = coef[i + q * S::NG - cb];
@@ -426,6 +431,7 @@ __device__ __forceinline__ void cols_pass(const BlockRows<TC>& rows, int cb, int
     auto one = [&](const TC* row, T f) {
 #pragma unroll
         for (int k = 0; k < S::KU; ++k) {
+            if (!S::Cols::has(u0, k)) continue;
             T c0, c1;
             load_pair(row + 2 * (u0 + k * kThreads), c0, c1);
             acc[k][0] += f * c0;
@@ -447,7 +453,7 @@ __device__ __forceinline__ void cols_store(T (&acc)[L2Shape<T, TC, PL>::KU][2], 
 #pragma unroll
         for (int k = 0; k < S::KU; ++k) {
             const int u = (int)threadIdx.x + k * kThreads;
-            if (u < S::U) {
+            if (S::Cols::active((int)threadIdx.x) && S::Cols::has((int)threadIdx.x, k)) {
                 part[2 * u] = acc[k][0];
                 part[2 * u + 1] = acc[k][1];
             }

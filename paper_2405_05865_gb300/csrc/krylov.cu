@@ -679,7 +679,7 @@ __global__ void __launch_bounds__(kThreads, 1) k_level2(L2Args<T, TC> a) {
     __shared__ double red[kNW], red_b[kNW], red_c[kNW];
     __shared__ T redc[kNW * 8];
     __shared__ double s_alpha, s_rr, s_val[4];
-    __shared__ int s_bad;
+    __shared__ int s_bad, s_stop;
 
     CtlBlock* ctl = a.ctl;
     // the control words in one round trip
@@ -692,17 +692,17 @@ __global__ void __launch_bounds__(kThreads, 1) k_level2(L2Args<T, TC> a) {
     auto report = [&](int word, int v) {
         if (a.prog && b == 0 && threadIdx.x == 0) a.prog[word] = v;
     };
-    if (c_done | c_err) {
-        report(1, 1);
-        return;
-    }
     const int64_t row0 = a.n * b / G, row1 = a.n * (b + 1) / G;
     const int64_t c0 = sp * b / G, c1 = sp * (b + 1) / G;
     unsigned int* bw = &ctl->bar_word;
     int* err = &ctl->error;
     const bool packed = a.dq != nullptr;
     BlockRows<TC> rows{a.C + row0 * sp, cres, (int)(row1 - row0), (int)min((int64_t)a.res_rows, row1 - row0)};
-    if (threadIdx.x == 0) {
+    // thread 0's view of the flags stands for its block: block 0 may store an error
+    // (s_bad below) while other blocks are still starting, and a block leaves whole or
+    // not at all
+    if (threadIdx.x == 0) s_stop = c_done | c_err;
+    if (threadIdx.x == 0 && !(c_done | c_err)) {
         msp::mbar_init(bar, 1);
         asm volatile("fence.mbarrier_init.release.cluster;" ::: "memory");
         uint32_t left = (uint32_t)(rows.nres * S::row);
@@ -716,6 +716,10 @@ __global__ void __launch_bounds__(kThreads, 1) k_level2(L2Args<T, TC> a) {
         s_bad = 0;
     }
     __syncthreads();
+    if (s_stop) {
+        report(1, 1);
+        return;
+    }
 
     // ---- level-1 update
     const T* p = a.p;

@@ -182,7 +182,6 @@ struct SymvArgs {
 
 __global__ void __launch_bounds__(kSymvThreads, 1) k_symv_packed(SymvArgs a) {
     CtlBlock* ctl = a.ctl;
-    if (ctl->done | ctl->error) return;
     const int iter = ctl->iters;
     const float* p_old = a.p + ((iter & 1) ^ 1) * a.n_pad;
     float* p_new = a.p + (iter & 1) * a.n_pad;
@@ -193,10 +192,13 @@ __global__ void __launch_bounds__(kSymvThreads, 1) k_symv_packed(SymvArgs a) {
     uint64_t* empty = full + kStages;
     __shared__ double red[kConsumerWarps];
     __shared__ float s_beta;
-    __shared__ int col_count[kStages];
+    __shared__ int col_count[kStages], s_stop;
 
     const int warp = threadIdx.x >> 5, lane = threadIdx.x & 31;
+    // one thread reads the flags for its block: block 0 may store an error below while
+    // other blocks are still starting, and the barriers here need every warp
     if (threadIdx.x == 0) {
+        s_stop = ctl->done | ctl->error;
         for (int s = 0; s < kStages; ++s) {
             mbar_init(&full[s], 1);
             mbar_init(&empty[s], kConsumerWarps);
@@ -205,6 +207,7 @@ __global__ void __launch_bounds__(kSymvThreads, 1) k_symv_packed(SymvArgs a) {
         asm volatile("fence.mbarrier_init.release.cluster;" ::: "memory");
     }
     __syncthreads();
+    if (s_stop) return;
 
     const int G = gridDim.x;
     // tiles of this block: t = blockIdx.x + k G

@@ -745,7 +745,21 @@ __global__ void __launch_bounds__(kThreads, 1) k_level2(L2Args<T, TC> a) {
                 else if (!(pq > 0.0)) s_bad = MSP_ENOTPD;
             }
         }
+        // p^T q not positive or not finite: block 0 records it, and every block leaves (the
+        // sum and so the outcome are the same in all of them). Called past a block barrier.
+        auto breakdown = [&]() -> bool {
+            if (!s_bad) return false;
+            if (threadIdx.x == 0) {
+                if (b == 0) atomicExch(err, s_bad);
+                msp::mbar_wait_timed(bar, 0, err);   // the resident rows land before the block leaves
+            }
+            return true;
+        };
         have_r = rows.nr <= kRowChunk;
+        if (rows.nr == 0) {       // fewer rows than blocks
+            __syncthreads();
+            if (breakdown()) return;
+        }
         for (int64_t base = row0; base < row1; base += 32 * kGroups) {
             const int64_t i_own = base + 32 * w + lane;      // the row this thread finishes (w < kGroups)
             const bool own = w < kGroups && i_own < row1;
@@ -789,13 +803,7 @@ __global__ void __launch_bounds__(kThreads, 1) k_level2(L2Args<T, TC> a) {
             for (int g = 0; g < kGroups; ++g)
                 if (w < kNS) sq[(g * kNS + w) * 32 + lane] = v[g];
             __syncthreads();
-            if (s_bad) {
-                if (threadIdx.x == 0) {
-                    if (b == 0) atomicExch(err, s_bad);
-                    msp::mbar_wait_timed(bar, 0, err);   // the resident rows land before the block leaves
-                }
-                return;       // the same in every block
-            }
+            if (breakdown()) return;
             if (own) {
                 const T alpha = (T)s_alpha;
                 T qi = T(0);

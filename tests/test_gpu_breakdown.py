@@ -43,7 +43,7 @@ def _expect_not_pd(ctx, A, b, f):
     assert time.monotonic() - t0 < 1.0
 
 
-@pytest.mark.parametrize("n", [256, 1000, 4096])
+@pytest.mark.parametrize("n", [40, 100, 151, 256, 1000, 4096])   # the first three: fewer rows than SMs
 @pytest.mark.parametrize("lam0", [0.0, 4.9])
 def test_negative_definite_mixed(ctx, n, lam0):
     A, b, f = _negative(ctx, n, lam0)

@@ -267,6 +267,14 @@ MSP_API msp_status msp_set_gram_tensor_cores(msp_ctx* ctx, int on);
  * part of the method (it selects an implementation). */
 MSP_API msp_status msp_set_factor_float_float(msp_ctx* ctx, int on);
 
+/* CTAs in each of the two thread-block clusters that run the level-3 solves of
+ * the three-level method (Algorithm 5): 16 (default; where the device has no
+ * room for such a cluster, 8 all the same) or 8, the portable size. Takes
+ * effect when a general handle next captures SolveM1 or calls
+ * msp_general_solve_m2. Not part of the method (it selects an
+ * implementation). MSP_EINVAL for other values. */
+MSP_API msp_status msp_set_level3_ctas(msp_ctx* ctx, int ctas);
+
 /* How msp_solve issues its level-1 iterations (Algorithm 2's outer loop:
  * the A pass, then the level-2 kernel with the step, SolveM1 and the new
  * direction): on = 1 (default): the two launches of one iteration are

@@ -373,6 +373,10 @@ class Context:
         """Level-1 iterations replayed as a CUDA graph (default) or launched one by one."""
         L.check(self.ptr, self.lib.msp_set_level1_graphs(self.ptr, int(bool(on))))
 
+    def set_level3_ctas(self, ctas: int) -> None:
+        """CTAs a cluster of the level-3 solves: 16 (default) or 8."""
+        L.check(self.ptr, self.lib.msp_set_level3_ctas(self.ptr, int(ctas)))
+
     def set_factor_float_float(self, on: bool) -> None:
         """Cholesky of an FP32 factor in float-float (default) or in FP64."""
         L.check(self.ptr, self.lib.msp_set_factor_float_float(self.ptr, int(bool(on))))

@@ -582,7 +582,7 @@ __global__ void k_dense_mv(const double* __restrict__ M, const float* __restrict
     if (lane == 0) out[row] = (float)s;
 }
 
-// Algorithm 5 steps 2-3 in one launch, on two thread-block clusters of kCl
+// Algorithm 5 steps 2-3 in one launch, on two thread-block clusters of CL
 // CTAs: cluster 0 runs t3 PCG steps on W u = r preconditioned by M3a^{-1},
 // cluster 1 on (W + lam~ I) v = r with M3b^{-1}; W = A~^T A~ is the formed FP64
 // Gram (the same operator as A~^T (A~ .), applied as an s x s product). FP64
@@ -592,22 +592,23 @@ __global__ void k_dense_mv(const double* __restrict__ M, const float* __restrict
 // instruction holds it for 16 cycles whether the lanes' results are needed or
 // not) and the latency of the serial chain product -> dot -> step, so every
 // FP64 instruction that is not the product itself is kept to the threads that
-// need it. A CTA has s_pad threads: 16 lanes form one of its s_pad / kCl rows
+// need it. A CTA has s_pad threads: CL lanes form one of its s_pad / CL rows
 // of a product (their slices of W and M3^{-1} in registers up to s_pad = 384,
-// E = s_pad / kCl values each, read from L1 / L2 beyond). The CTA's row sums are
+// E = s_pad / CL values each, read from L1 / L2 beyond: E = 0). The CTA's row sums are
 // gathered in shared memory and stored to every CTA's copy of the full result by
 // 16-byte pieces (one word per lane and CTA costs twice the barrier), so one
 // cluster barrier per product is the only exchange (two copies in turn: a CTA
-// is never more than one barrier ahead). Thread t then keeps component t of x, r, p redundantly in every CTA, the dots are
-// taken in each CTA from the full vectors in the same order, and one warp
-// forms each step's quotient. The former layout (1024 threads whatever s_pad,
+// is never more than one barrier ahead). Thread t then keeps component t of x, r, p
+// redundantly in every CTA, the dots are taken in each CTA from the full vectors in the
+// same order, and one warp forms each step's quotient. The former layout (1024 threads whatever s_pad,
 // every thread summing partials and dividing, two cluster barriers a product)
 // took 177 us at s_pad = 128, t3 = 8, most of a three-level solve; with this one
-// the solve at 16384 x 2048 went from 355 to 180 ms.
-constexpr int kCl = 16;
+// the solve at 16384 x 2048 went from 355 to 180 ms. CL = 16 is past the portable
+// cluster size: where the device has no room for it (a partition), CL = 8, E = 0.
+constexpr int kClWide = 16, kClPortable = 8;
 
-template <int E>
-__global__ void __cluster_dims__(kCl, 1, 1) __launch_bounds__(E > 0 ? kCl * E : 1024)
+template <int CL, int E>
+__global__ void __cluster_dims__(CL, 1, 1) __launch_bounds__(E > 0 ? CL * E : 1024)
     k_level3_cluster(const double* __restrict__ W, const double* __restrict__ Ma, const double* __restrict__ Mb,
                      double lam_t, int sp, int t3, const float* __restrict__ b, float* __restrict__ u,
                      float* __restrict__ v) {
@@ -615,26 +616,26 @@ __global__ void __cluster_dims__(kCl, 1, 1) __launch_bounds__(E > 0 ? kCl * E : 
     cg::cluster_group cl = cg::this_cluster();
     __shared__ __align__(16) double vec[1024];   // the vector of the next product
     __shared__ __align__(16) double ybuf[2][1024];   // products, in turn
-    __shared__ __align__(16) double stage[1024 / kCl];   // this CTA's part
+    __shared__ __align__(16) double stage[1024 / CL];   // this CTA's part
     __shared__ double red[32];
     __shared__ double s_sc;
     const int rank = (int)cl.block_rank();
-    const int sys = blockIdx.x / kCl;
+    const int sys = blockIdx.x / CL;
     const double shift = sys == 0 ? 0.0 : lam_t;
     float* out = sys == 0 ? u : v;
-    const int tid = threadIdx.x, warp = tid >> 5, lane = tid & 31, l16 = tid & 15;
-    const int nw = sp >> 5, own = sp / kCl;
-    const int row = rank * own + (tid >> 4);
-    // this lane's elements of its row: the pairs 2 l16 + 32 k
-    const double2* Wr = reinterpret_cast<const double2*>(W + (int64_t)row * sp) + l16;
-    const double2* Mr = reinterpret_cast<const double2*>((sys == 0 ? Ma : Mb) + (int64_t)row * sp) + l16;
+    const int tid = threadIdx.x, warp = tid >> 5, lane = tid & 31, lc = tid & (CL - 1);
+    const int nw = sp >> 5, own = sp / CL;
+    const int row = rank * own + (tid / CL);
+    // this lane's elements of its row: the pairs 2 (lc + CL k)
+    const double2* Wr = reinterpret_cast<const double2*>(W + (int64_t)row * sp) + lc;
+    const double2* Mr = reinterpret_cast<const double2*>((sys == 0 ? Ma : Mb) + (int64_t)row * sp) + lc;
     constexpr int ER = E > 0 ? E / 2 : 1;
     double2 wreg[ER], mreg[ER];
     if constexpr (E > 0) {
 #pragma unroll
-        for (int k = 0; k < ER; ++k) mreg[k] = __ldg(Mr + kCl * k);
+        for (int k = 0; k < ER; ++k) mreg[k] = __ldg(Mr + CL * k);
 #pragma unroll
-        for (int k = 0; k < ER; ++k) wreg[k] = __ldg(Wr + kCl * k);
+        for (int k = 0; k < ER; ++k) wreg[k] = __ldg(Wr + CL * k);
     }
     cl.sync();   // every CTA of the cluster runs before its shared memory is written
     int turn = 0;
@@ -642,30 +643,30 @@ __global__ void __cluster_dims__(kCl, 1, 1) __launch_bounds__(E > 0 ? kCl * E : 
     auto product = [&](const double2 (&reg)[ER], const double2* rows, double val) {
         vec[tid] = val;
         __syncthreads();
-        const double2* v2 = reinterpret_cast<const double2*>(vec) + l16;
+        const double2* v2 = reinterpret_cast<const double2*>(vec) + lc;
         double s0 = 0.0, s1 = 0.0;
         if constexpr (E > 0) {
 #pragma unroll
             for (int k = 0; k < ER; ++k) {
-                const double2 a = v2[kCl * k];
+                const double2 a = v2[CL * k];
                 s0 = fma(reg[k].x, a.x, s0);
                 s1 = fma(reg[k].y, a.y, s1);
             }
         } else {
-            const int n2 = sp / (2 * kCl);
+            const int n2 = sp / (2 * CL);
 #pragma unroll 8
             for (int k = 0; k < n2; ++k) {
-                const double2 m = __ldg(rows + kCl * k), a = v2[kCl * k];
+                const double2 m = __ldg(rows + CL * k), a = v2[CL * k];
                 s0 = fma(m.x, a.x, s0);
                 s1 = fma(m.y, a.y, s1);
             }
         }
         double s = s0 + s1;
 #pragma unroll
-        for (int o = kCl / 2; o > 0; o >>= 1) s += __shfl_xor_sync(0xffffffffu, s, o);
-        if (l16 == 0) stage[tid >> 4] = s;
+        for (int o = CL / 2; o > 0; o >>= 1) s += __shfl_xor_sync(0xffffffffu, s, o);
+        if (lc == 0) stage[tid / CL] = s;
         __syncthreads();
-        if (tid < own / 2 * kCl) {
+        if (tid < own / 2 * CL) {
             const int to = tid / (own / 2), piece = tid % (own / 2);
             reinterpret_cast<double2*>(cl.map_shared_rank(&ybuf[turn][0], to) + rank * own)[piece] =
                 reinterpret_cast<const double2*>(stage)[piece];
@@ -1071,15 +1072,33 @@ struct Ops {
         return MSP_OK;
     }
 
+    // whether the device has room for a 16-CTA cluster of the kernel (a host query, made
+    // when SolveM2 is captured)
+    template <typename K>
+    static bool wide_cluster_fits(K kern, int threads) {
+        cudaLaunchConfig_t cfg{};
+        cfg.gridDim = dim3(2 * kClWide);
+        cfg.blockDim = dim3((unsigned)threads);
+        int clusters = 0;
+        if (cudaFuncSetAttribute(kern, cudaFuncAttributeNonPortableClusterSizeAllowed, 1) == cudaSuccess &&
+            cudaOccupancyMaxActiveClusters(&clusters, kern, &cfg) == cudaSuccess && clusters >= 1)
+            return true;
+        cudaGetLastError();
+        return false;
+    }
     // Algorithm 5: z = (u - v) / lam~ (t3 = 0: the exact M2^{-1} r); both
     // level-3 solves run in one launch on the formed W
     msp_status solve_m2(const float* r, float* z, int t3) {
         if (t3 == 0) return dense(g->M2inv, r, z);
         const int sp = (int)g->s_pad;
-        auto kern = sp == 128 ? k_level3_cluster<8> : sp == 256 ? k_level3_cluster<16>
-                    : sp == 384 ? k_level3_cluster<24> : k_level3_cluster<0>;
-        MSP_CUDA_TRY(ctx, cudaFuncSetAttribute(kern, cudaFuncAttributeNonPortableClusterSizeAllowed, 1));
-        kern<<<2 * kCl, sp, 0, strm>>>(g->W64, g->M3a, g->M3b, g->lam_tilde, sp, t3, r, g->u3, g->v3);
+        auto kern = sp == 128 ? k_level3_cluster<kClWide, 8> : sp == 256 ? k_level3_cluster<kClWide, 16>
+                    : sp == 384 ? k_level3_cluster<kClWide, 24> : k_level3_cluster<kClWide, 0>;
+        int ctas = kClWide;
+        if (ctx->level3_ctas < kClWide || !wide_cluster_fits(kern, sp)) {
+            kern = k_level3_cluster<kClPortable, 0>;
+            ctas = kClPortable;
+        }
+        kern<<<2 * ctas, sp, 0, strm>>>(g->W64, g->M3a, g->M3b, g->lam_tilde, sp, t3, r, g->u3, g->v3);
         MSP_CHECK_LAUNCH(ctx);
         if (count) ++*count;
         const float il = (float)(1.0 / g->lam_tilde);
@@ -1764,6 +1783,14 @@ msp_status msp_general_get(msp_ctx* ctx, const msp_general_t* g, float* At, int6
     if (M3b)
         MSP_CUDA_TRY(ctx, cudaMemcpy2DAsync(M3b, g->s * 8, g->G3b, sp * 8, g->s * 8, g->s, cudaMemcpyDeviceToDevice,
                                             ctx->stream));
+    return MSP_OK;
+}
+
+msp_status msp_set_level3_ctas(msp_ctx* ctx, int ctas) {
+    if (!ctx) return msp_set_error(nullptr, MSP_EINVAL, "ctx is NULL");
+    if (ctas != kClWide && ctas != kClPortable)
+        return msp_set_error(ctx, MSP_EINVAL, "level-3 cluster size must be %d or %d", kClPortable, kClWide);
+    ctx->level3_ctas = ctas;
     return MSP_OK;
 }
 

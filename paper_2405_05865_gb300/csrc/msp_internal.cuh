@@ -61,6 +61,7 @@ struct msp_ctx {
     cudaGraphNode_t l1_ev_nodes[2] = {};
     int l1_kernels = 0;
     int64_t l1_graph_iters = 0;  // level-1 iterations replayed from the graph
+    int level3_ctas = 16;        // CTAs a cluster of the level-3 solves, where that many fit (else 8)
     int hutch_terms = 2;         // tensor-core Hutchinson: 2 = two FP16 terms, 3 = three BF16 terms
     msp_ctx** lanes = nullptr;
     cudaStream_t* lane_streams = nullptr;

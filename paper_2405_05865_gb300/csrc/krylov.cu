@@ -304,6 +304,7 @@ struct L2Args {
     int mode;
     int phase;              // PHASE_ALL, or the part before / after a k_inner launch
     int res_rows;           // rows of C a block keeps in shared memory
+    int once;               // level-2 iteration: each row of C read once (gram_pass)
     const TC* C;
     const TC* W;
     const T* B;
@@ -386,6 +387,8 @@ struct L2Shape {
     // four full vectors, the scratch of the reductions, r and the row results
     static constexpr size_t fixed = ((size_t)4 * SP + SCR + 2 * kRowChunk) * sizeof(T) + 16;
     static constexpr size_t row = (size_t)SP * sizeof(TC);
+    // gram_pass is for FP32 arithmetic (in FP64 the products bound the passes, not the reads)
+    static constexpr bool once = sizeof(T) == 4;
 };
 
 // The rows [row0, row0 + nr) of C of one block: the first nres of them in
@@ -497,7 +500,10 @@ __device__ __forceinline__ T reduce_scatter(T* v, int lane) {
 // dot[i - cb] = c_i . vec over the rows [cb, ce) of the block (ce - cb <=
 // kRowChunk); vec in shared memory. A warp takes every kNW-th row. Up to PL =
 // 32 (FP64: 16) its slice of vec stays in registers and it reduces 8 or 16
-// rows' partial dots at once; the rows from L2 come first, two in flight.
+// rows' partial dots at once; the rows from L2 come first, two in flight up to PL =
+// 16 and one beyond (two spilled registers, and what spills goes to L2: next to
+// no L1 is left beside the resident rows. An inner step at s = 1024 took 25.4 us at n =
+// 8192 with the spills, 23.2 without).
 template <typename T, typename TC, int PL>
 __device__ __forceinline__ void dots_pass(const BlockRows<TC>& rows, int cb, int ce, const T* vec, T* dot) {
     constexpr int SP = 32 * PL, W = StoreW<TC>::W;
@@ -529,10 +535,11 @@ __device__ __forceinline__ void dots_pass(const BlockRows<TC>& rows, int cb, int
                     RowSlice<T, PL, TC> c0, c1;
                     c0.load(ptr(o0 + t), lane);
                     const bool two = o0 + t + 1 < cnt;
-                    if (two) c1.load(ptr(o0 + t + 1), lane);
+                    if (two && PL <= 16) c1.load(ptr(o0 + t + 1), lane);
 #pragma unroll
                     for (int k = 0; k < PL; ++k) part[t] += c0.v[k] * vs[k];
                     if (two) {
+                        if (PL > 16) c1.load(ptr(o0 + t + 1), lane);
 #pragma unroll
                         for (int k = 0; k < PL; ++k) part[t + 1] += c1.v[k] * vs[k];
                     }
@@ -549,6 +556,100 @@ __device__ __forceinline__ void dots_pass(const BlockRows<TC>& rows, int cb, int
             const T t = msp::warp_sum(c.dot_smem(vec, lane));
             if (lane == 0) dot[i - cb] = t;
         }
+    }
+}
+
+// How gram_pass cuts a row: HW warps a row, NVH vectors of it a lane, NR rows in
+// flight a warp (32 values a lane, 64 KB an SM).
+template <typename T, typename TC, int PL>
+struct GramShape {
+    static constexpr int W = StoreW<TC>::W, NV = PL / W;
+    static constexpr int HW = PL > 16 ? 2 : 1, NP = kNW / HW;
+    static constexpr int NVH = (NV + HW - 1) / HW;
+    static constexpr int NR = NVH * W >= 32 ? 1 : 32 / (NVH * W);
+    static constexpr size_t bytes = (size_t)NP * 32 * PL * sizeof(T);
+};
+
+// part = sum_i (c_i . vec) c_i over the block's rows, each row read once: HW warps
+// take every NP-th row, form its dot and add it from the registers to their own sums
+// of their columns, which scr (NP x SP) combines in order. The two warps of a row
+// exchange their halves of the dots through xch at a barrier of their own. For blocks
+// whose rows of C do not all fit shared memory: dots_pass and cols_pass read each of the
+// others twice from L2, and at n = 32768, s = 1024 (C as large as L2) from memory. A
+// level-2 step then took 53 us, with this 44; at n = 16384 and s = 2048 71 and 57,
+// s = 1024 27.2 and 27.1, s = 512 21.6 either way. The scratch costs 32 KB of resident rows (64
+// KB at 2048 columns), so where all rows fit the two passes stay (n = 8192, s = 512: 20.6 us
+// with this, 19.6 with the two passes).
+template <typename T, typename TC, int PL>
+__device__ __forceinline__ void gram_pass(const BlockRows<TC>& rows, const T* vec, T* scr, T* xch, T* part) {
+    using G = GramShape<T, TC, PL>;
+    constexpr int SP = 32 * PL, W = G::W;
+    const int lane = threadIdx.x & 31, w = threadIdx.x >> 5, grp = w / G::HW, h = w % G::HW;
+    // vector q of this lane: columns at(q) .. + W of the row
+    auto has = [&](int q) { return G::NV % G::HW == 0 || G::HW * q + h < G::NV; };
+    auto at = [&](int q) { return (G::HW * q + h) * 32 * W + lane * W; };
+    T acc[G::NVH * W];
+#pragma unroll
+    for (int k = 0; k < G::NVH * W; ++k) acc[k] = T(0);
+    int turn = 0;
+    auto walk = [&](const TC* base, int first, int end) {
+#pragma unroll 1
+        for (int i = first + grp; i < end; i += G::NR * G::NP) {
+            T c[G::NR][G::NVH * W], d[G::NR];
+#pragma unroll
+            for (int r = 0; r < G::NR; ++r)
+#pragma unroll
+                for (int q = 0; q < G::NVH; ++q) {
+                    if (i + r * G::NP < end && has(q)) {
+                        load_vec(base + (int64_t)(i + r * G::NP) * SP + at(q), c[r] + q * W);
+                    } else {
+#pragma unroll
+                        for (int e = 0; e < W; ++e) c[r][q * W + e] = T(0);
+                    }
+                }
+#pragma unroll
+            for (int r = 0; r < G::NR; ++r) d[r] = T(0);
+#pragma unroll
+            for (int q = 0; q < G::NVH; ++q) {
+                if (!has(q)) continue;
+                T x[W];
+                load_vec(vec + at(q), x);
+#pragma unroll
+                for (int r = 0; r < G::NR; ++r)
+#pragma unroll
+                    for (int e = 0; e < W; ++e) d[r] += c[r][q * W + e] * x[e];
+            }
+#pragma unroll
+            for (int r = 0; r < G::NR; ++r) d[r] = msp::warp_sum(d[r]);
+            if constexpr (G::HW == 2) {
+                T* x = xch + (turn * G::NP + grp) * 2 * G::NR;
+                if (lane == 0)
+#pragma unroll
+                    for (int r = 0; r < G::NR; ++r) x[h * G::NR + r] = d[r];
+                asm volatile("bar.sync %0, 64;" ::"r"(1 + grp) : "memory");
+#pragma unroll
+                for (int r = 0; r < G::NR; ++r) d[r] = x[r] + x[G::NR + r];
+                turn ^= 1;
+            }
+#pragma unroll
+            for (int r = 0; r < G::NR; ++r)
+#pragma unroll
+                for (int k = 0; k < G::NVH * W; ++k) acc[k] += d[r] * c[r][k];
+        }
+    };
+    walk(rows.g, rows.nres, rows.nr);
+    walk(rows.s, 0, rows.nres);
+#pragma unroll
+    for (int q = 0; q < G::NVH; ++q)
+        if (has(q))
+#pragma unroll
+            for (int e = 0; e < W; ++e) scr[grp * SP + at(q) + e] = acc[q * W + e];
+    __syncthreads();
+    for (int c = threadIdx.x; c < SP; c += kThreads) {
+        T v = T(0);
+#pragma unroll
+        for (int q = 0; q < G::NP; ++q) v += scr[q * SP + c];
+        part[c] = v;
     }
 }
 
@@ -857,7 +958,8 @@ __global__ void __launch_bounds__(kThreads, 1) k_level2(L2Args<T, TC> a) {
         have_r = rows.nr <= kRowChunk;   // srow is not written again below
         cols_store<T, TC, PL>(acc, scr, a.part + (int64_t)b * sp);
         // the block's rows of B and B^T on their way to registers during the barriers
-        const bool one_row = c1 - c0 <= kNW;
+        // (PL > 32: two rows of that length would not fit the registers)
+        const bool one_row = PL <= 32 && c1 - c0 <= kNW;
         const bool my_row = one_row && c0 + w < c1 && a.phase == PHASE_ALL;
         RowSlice<T, PL> mB;
         if (my_row) mB.load(a.B + (c0 + w) * sp, lane);
@@ -964,16 +1066,23 @@ __global__ void __launch_bounds__(kThreads, 1) k_level2(L2Args<T, TC> a) {
         const double tin2 = a.inner_tol2 * gg;
         while (k < a.max_inner && rres > tin2) {
             // P1: partial u = C^T (C d) over this block's rows; wd = W d (columns)
+            if (S::once && a.once) {
+                if constexpr (S::once) {
+                    T* wscr = reinterpret_cast<T*>(smem_raw + (size_t)a.res_rows * S::row + S::fixed);
+                    gram_pass<T, TC, PL>(rows, sd, wscr, sw, a.part + (int64_t)b * sp);
+                }
+            } else {
 #pragma unroll
-            for (int q = 0; q < S::KU; ++q) acc[q][0] = acc[q][1] = T(0);
-            for (int cb = 0; cb < rows.nr; cb += kRowChunk) {
-                const int ce = min(rows.nr, cb + kRowChunk);
-                dots_pass<T, TC, PL>(rows, cb, ce, sd, sw);
-                __syncthreads();
-                cols_pass<T, TC, PL>(rows, cb, ce, sw, acc);
-                if (ce < rows.nr) __syncthreads();
+                for (int q = 0; q < S::KU; ++q) acc[q][0] = acc[q][1] = T(0);
+                for (int cb = 0; cb < rows.nr; cb += kRowChunk) {
+                    const int ce = min(rows.nr, cb + kRowChunk);
+                    dots_pass<T, TC, PL>(rows, cb, ce, sd, sw);
+                    __syncthreads();
+                    cols_pass<T, TC, PL>(rows, cb, ce, sw, acc);
+                    if (ce < rows.nr) __syncthreads();
+                }
+                cols_store<T, TC, PL>(acc, scr, a.part + (int64_t)b * sp);
             }
-            cols_store<T, TC, PL>(acc, scr, a.part + (int64_t)b * sp);
             rows_dot<T, PL, TC>(a.W, sp, c0, c1, sd, a.wdvec);
             if (!msp::grid_barrier(bw, err)) return;
             // P2: u over this block's columns; d.u partial
@@ -1092,7 +1201,16 @@ msp_status launch_level2_pl(msp_ctx* ctx, L2Args<T, TC>& a, int G) {
     const int64_t most = (a.n + G - 1) / G;
     const int64_t fit = (int64_t)(left / S::row);
     a.res_rows = (int)(fit >= most ? most : fit / kNW * kNW);
-    const size_t smem = S::fixed + (size_t)a.res_rows * S::row;
+    a.once = 0;
+    size_t once = 0;
+    if constexpr (S::once) {
+        if (a.max_inner > 0 && a.phase == PHASE_ALL && a.res_rows < most) {
+            a.once = 1;
+            once = GramShape<T, TC, PL>::bytes;
+            a.res_rows = (int)std::min<int64_t>((int64_t)((left - once) / S::row), most);
+        }
+    }
+    const size_t smem = S::fixed + (size_t)a.res_rows * S::row + once;
     MSP_CUDA_TRY(ctx, cudaFuncSetAttribute(kern, cudaFuncAttributeMaxDynamicSharedMemorySize,
                                            (int)smem));
     // co-residency is required by the grid barrier: never exceed what fits

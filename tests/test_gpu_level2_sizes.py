@@ -54,3 +54,34 @@ def test_wide_sketches(ctx, system, s, data):
     assert float(res.norm()) <= 1.2e-10 * float(b.norm())
     f.close()
     sk.close()
+
+
+@pytest.mark.parametrize("n,s", [(16001, 500), (16001, 640), (16001, 1000), (7993, 1500), (7993, 2048)])
+@pytest.mark.parametrize("data", ["fp32", "bf16"])
+def test_level2_iteration_on_rows_from_global_memory(ctx, n, s, data):
+    """The level-2 PCG where each block's rows of C exceed its shared memory (in BF16 they all
+    fit up to s = 640): SolveM1 against the exact level 2 in FP64."""
+    g = torch.Generator(device="cuda").manual_seed(s)
+    G = torch.randn((n, 64), generator=g, device="cuda", dtype=torch.float32) / n ** 0.5
+    A = G @ G.T
+    A.diagonal().add_(0.5)
+    sk = ctx.sketch(A, s, 8, SEED)
+    f = ctx.nystrom(sk, LAM, 1.0, phi=4 * s, data=data)
+    W, C, lt = f.parts()["W"].double(), sk.C().double(), LAM + 1.0
+    if data == "bf16":
+        W, C = W.to(torch.bfloat16).double(), C.to(torch.bfloat16).double()
+    M = C.T @ C + lt * W
+    r = torch.randn(n, generator=g, device="cuda", dtype=torch.float32)
+    w, its = ctx.solve_m1(f, r, max_inner=300, inner_tol=1e-7)
+    assert 0 < its < 300
+    r64 = r.double()
+    h = C.T @ r64
+    y = torch.linalg.solve(M, h)
+    ref = (r64 - C @ y) / lt
+    # FP32 units of |r| and |C| |y|, and what the tolerance leaves of y
+    ev = torch.linalg.eigvalsh(M)
+    c2 = float(torch.linalg.matrix_norm(C, 2))
+    bound = (64 * 2.0 ** -24 * (float(r64.norm()) + c2 * float(y.norm())) + c2 * 2e-7 * float(h.norm()) / float(ev[0])) / lt
+    assert float((w.double() - ref).norm()) <= bound
+    f.close()
+    sk.close()

@@ -29,14 +29,25 @@ __device__ inline void mbar_arrive(uint64_t* bar) {
                  : "memory");
 }
 
+// Cluster: the phase completes by what other CTAs of the cluster send here, which a
+// wait orders at the cluster's scope only.
+template <bool Cluster = false>
 __device__ inline bool mbar_try_wait(uint64_t* bar, uint32_t parity) {
     uint32_t ok;
-    asm volatile(
-        "{\n .reg .pred p;\n mbarrier.try_wait.parity.acquire.cta.shared::cta.b64 p, [%1], %2;\n"
-        " selp.u32 %0, 1, 0, p;\n}\n"
-        : "=r"(ok)
-        : "r"(smem_u32(bar)), "r"(parity)
-        : "memory");
+    if constexpr (Cluster)
+        asm volatile(
+            "{\n .reg .pred p;\n mbarrier.try_wait.parity.acquire.cluster.shared::cta.b64 p, [%1], %2;\n"
+            " selp.u32 %0, 1, 0, p;\n}\n"
+            : "=r"(ok)
+            : "r"(smem_u32(bar)), "r"(parity)
+            : "memory");
+    else
+        asm volatile(
+            "{\n .reg .pred p;\n mbarrier.try_wait.parity.acquire.cta.shared::cta.b64 p, [%1], %2;\n"
+            " selp.u32 %0, 1, 0, p;\n}\n"
+            : "=r"(ok)
+            : "r"(smem_u32(bar)), "r"(parity)
+            : "memory");
     return ok != 0;
 }
 
@@ -45,11 +56,12 @@ __device__ inline bool mbar_try_wait(uint64_t* bar, uint32_t parity) {
 // warps waiting on the same phase all see a completion that happened before
 // any of them gave up; callers that meet at named barriers afterwards rely on
 // every warp taking the same branch.
+template <bool Cluster = false>
 __device__ inline bool mbar_wait_timed(uint64_t* bar, uint32_t parity, int* err) {
-    if (mbar_try_wait(bar, parity)) return true;
+    if (mbar_try_wait<Cluster>(bar, parity)) return true;
     const uint64_t t0 = globaltimer_ns();
     for (int spins = 0;; ++spins) {
-        if (mbar_try_wait(bar, parity)) return true;
+        if (mbar_try_wait<Cluster>(bar, parity)) return true;
         if ((spins & 63) == 63 && globaltimer_ns() - t0 > kWaitLimitNs) {
             atomicExch(err, (int)MSP_ETIMEOUT);
             return false;

@@ -1398,7 +1398,7 @@ __global__ void __launch_bounds__(16 * E + kDotThreads, 1) k_inner(InnerArgs<T> 
             }
             if (tid == 0) {
                 msp::mbar_arrive_expect_tx(&full[sent & 1], SP * (uint32_t)sizeof(T));
-                if (!msp::mbar_wait_timed(&full[sent & 1], (sent >> 1) & 1u, &ctl->error)) s_bad = 1;
+                if (!msp::mbar_wait_timed<true>(&full[sent & 1], (sent >> 1) & 1u, &ctl->error)) s_bad = 1;
             }
         } else if (with_rr) {
             const double t = dot(v, v);

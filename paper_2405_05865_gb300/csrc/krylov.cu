@@ -1396,7 +1396,9 @@ __global__ void __launch_bounds__(16 * E + kDotThreads, 1) k_inner(InnerArgs<T> 
                 const int to = tid / VPD, piece = tid % VPD;
                 st_async16(&ybuf[sent & 1][rank * OWN + piece * W], stage + piece * W, &full[sent & 1], to);
             }
-            if (tid == 0) {
+            // a phase whose wait ran out takes no second arrival: this CTA waits no more, and
+            // leaves at the next test of s_bad
+            if (tid == 0 && !s_bad) {
                 msp::mbar_arrive_expect_tx(&full[sent & 1], SP * (uint32_t)sizeof(T));
                 if (!msp::mbar_wait_timed<true>(&full[sent & 1], (sent >> 1) & 1u, &ctl->error)) s_bad = 1;
             }
@@ -1418,7 +1420,7 @@ __global__ void __launch_bounds__(16 * E + kDotThreads, 1) k_inner(InnerArgs<T> 
         return s_rres;
     };
     const double gg = half(), tin2 = a.inner_tol2 * gg;
-    if (gg > tin2 && a.max_inner > 0) {
+    if (gg > tin2 && a.max_inner > 0 && !s_bad) {
         z = product(bt, nullptr, vb, false);
         scalar(va, z, [&](double t) { return rz = t; });
         if (!dots) d = z[tid];

@@ -29,6 +29,16 @@ bool is_device_ptr(const void* p) {
     return at.type == cudaMemoryTypeDevice || at.type == cudaMemoryTypeManaged;
 }
 
+// Whether a kernel on `device` may write p (memory of another GPU is left to the copies)
+bool writable_on(int device, const void* p) {
+    cudaPointerAttributes at;
+    if (cudaPointerGetAttributes(&at, p) != cudaSuccess) {
+        cudaGetLastError();
+        return false;
+    }
+    return at.type == cudaMemoryTypeManaged || (at.type == cudaMemoryTypeDevice && at.device == device);
+}
+
 // dst row i <- src row i (w 16-byte pieces each), four pieces in flight a thread
 __global__ void __launch_bounds__(256) k_copy_rows(const float4* __restrict__ src, int64_t lds, float4* __restrict__ dst,
                                                    int64_t ldd, int64_t n, int64_t w) {
@@ -515,7 +525,8 @@ msp_status msp_sketch_get_C(msp_ctx* ctx, const msp_sketch_t* sk, void* C, int64
     // a whole number of 16-byte pieces a row, on both sides: the copy kernel (134 MB
     // of traffic at n = 16384, s = 1024: 21 us, against 68 us for the 2-D memcpy,
     // which takes what is left)
-    if ((sk->s * ts) % 16 == 0 && (ldc * ts) % 16 == 0 && ((uintptr_t)C & 15) == 0 && is_device_ptr(C)) {
+    if ((sk->s * ts) % 16 == 0 && (ldc * ts) % 16 == 0 && ((uintptr_t)C & 15) == 0 &&
+        writable_on(ctx->device, C)) {
         const int64_t w = sk->s * ts / 16;
         const unsigned blocks = (unsigned)std::min<int64_t>((sk->n * w + 1023) / 1024, 16 * (int64_t)ctx->num_sms);
         k_copy_rows<<<blocks, 256, 0, ctx->stream>>>((const float4*)sk->C, (int64_t)(sk->s_pad * ts / 16), (float4*)C,

@@ -2344,7 +2344,11 @@ msp_status msp_matvec64(msp_ctx* ctx, const void* A, msp_dtype dt, int64_t n, in
         if (vec) {
             // a row per warp: no more blocks than rows / 8
             const int grid = (int)std::min<int64_t>(Gg, (n + 7) / 8);
-            if (n <= kSplitMax) {
+            // with x split by every block no block may write into x meanwhile (y over x, as
+            // the split kernel ahead of the product allows)
+            const uintptr_t xa = (uintptr_t)x, oa = (uintptr_t)out;
+            const bool apart = xa + (uintptr_t)n * 8 <= oa || oa + (uintptr_t)n * 8 <= xa;
+            if (n <= kSplitMax && apart) {
                 k_matvec64_ff<true><<<grid, 256, 0, ctx->stream>>>((const float*)A, lda, n, lambda, nullptr, nullptr, x, b,
                                                                    out, (double*)scr, &ctl->last_block_counter,
                                                                    norm2_out_dev);

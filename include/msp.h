@@ -106,10 +106,14 @@ typedef struct {
                              operator itself (phi = 0, Phi = I).                 */
     int precision;        /* msp_precision. Default MSP_PREC_MIXED.              */
     int check_every;      /* level-1 iterations between host checks of the
-                             device-side convergence flag with profile = 1;
-                             without it the host keeps at most min(check_every, 4)
-                             iterations queued past the last one that the device
-                             reported in pinned host memory. Default 8.          */
+                             device-side convergence flag (a stream
+                             synchronisation each) with profile = 1, or where the
+                             device's flags ask for blocking or yielding
+                             synchronisation (cudaDeviceScheduleBlockingSync,
+                             cudaDeviceScheduleYield). Otherwise the host keeps at
+                             most min(check_every, 4) iterations queued past the
+                             last one that the device reported in pinned host
+                             memory, and polls that word, busy. Default 8.       */
     int profile;          /* 1: time every A-pass and level-2 launch with CUDA
                              events on the context stream (msp_info *_ms);
                              launches queued after the device flagged

@@ -1842,7 +1842,12 @@ msp_status krylov_solve_t(msp_ctx* ctx, const msp_factor_s* f, const void* A, ms
     // work (every iteration before a check that found no flag): read while
     // the next interval runs, not after it
     int settled = 0, l2_open = -1;
-    if (!pr.on) {
+    // a program that asked for blocking or yielding synchronisation wants the core for
+    // itself: there the host sleeps in a stream synchronisation per check interval
+    unsigned int flags = 0;
+    const bool spin = cudaGetDeviceFlags(&flags) != cudaSuccess ||
+                      !(flags & (cudaDeviceScheduleBlockingSync | cudaDeviceScheduleYield));
+    if (!pr.on && spin) {
         // the device reports each iteration in pinned host words; the host keeps
         // at most `ahead` iterations queued and polls, so the stream never runs
         // dry between checks (a stream synchronisation every 8 iterations left it

@@ -340,7 +340,8 @@ MSP_API msp_status msp_solve(msp_ctx* ctx, const msp_factor_t* f, const void* A,
                      const double* b, double* x, const msp_opts* opts,
                      msp_info* info);
 /* Wall-clock limit of the grid-wide barriers of the level-1 / level-2
- * kernels (msp_solve, msp_solve_refined, msp_solve_many, msp_solve_m1) on
+ * kernels (msp_solve, msp_solve_refined, msp_solve_many, msp_solve_m1) and of
+ * the waits between the blocks of the float-float factor (msp_nystrom) on
  * the context's device, in seconds; 0 restores the default of 2 s. A block
  * that waits longer gives up and the call returns MSP_ETIMEOUT (the context
  * stays usable: every solve resets its control block). Meant for tests of

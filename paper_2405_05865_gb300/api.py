@@ -386,7 +386,8 @@ class Context:
         L.check(self.ptr, self.lib.msp_set_gram_tensor_cores(self.ptr, int(bool(on))))
 
     def set_grid_wait_limit(self, seconds: float) -> None:
-        """Limit of the level-1 / level-2 grid barriers (0: the default 2 s)."""
+        """Limit of the level-1 / level-2 grid barriers and of the float-float
+        factor's waits (0: the default 2 s)."""
         L.check(self.ptr, self.lib.msp_set_grid_wait_limit(self.ptr, float(seconds)))
 
     def solve_refined(self, f: Factor, A: torch.Tensor, A_res: torch.Tensor, b: torch.Tensor, lam: float,

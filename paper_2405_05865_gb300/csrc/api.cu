@@ -917,7 +917,9 @@ msp_status msp_set_grid_wait_limit(msp_ctx* ctx, double seconds) {
         return msp_set_error(ctx, MSP_EINVAL, "grid wait limit must be in [0, 60] s (0: the default)");
     DeviceGuard g(ctx->device);
     const unsigned long long ns = (unsigned long long)(seconds * 1e9);
-    return msp_grid_wait_limit_krylov(ctx, seconds > 0.0 && ns == 0 ? 1ull : ns);
+    const unsigned long long limit = seconds > 0.0 && ns == 0 ? 1ull : ns;
+    MSP_TRY(msp_grid_wait_limit_factor(ctx, limit));
+    return msp_grid_wait_limit_krylov(ctx, limit);
 }
 
 msp_status msp_solve_refined(msp_ctx* ctx, const msp_factor_t* f, const void* A, msp_dtype dtype,

@@ -1394,6 +1394,14 @@ msp_status msp_gemm_tn(msp_ctx* ctx, const float* X, int64_t ldx, int64_t ncx, c
     return MSP_OK;
 }
 
+// The wait limit of this unit's kernel (k_chol_inv_ff) on the current device; 0 restores
+// the default.
+msp_status msp_grid_wait_limit_factor(msp_ctx* ctx, unsigned long long ns) {
+    const unsigned long long v = ns ? ns : msp::kWaitLimitNs;
+    MSP_CUDA_TRY(ctx, cudaMemcpyToSymbol(msp::g_grid_wait_limit_ns, &v, sizeof v));
+    return MSP_OK;
+}
+
 extern "C" msp_status msp_set_factor_float_float(msp_ctx* ctx, int on) {
     if (!ctx) return msp_set_error(nullptr, MSP_EINVAL, "ctx is NULL");
     ctx->factor_ff = on != 0;

@@ -345,6 +345,7 @@ msp_status msp_gram_tc(msp_ctx* ctx, const float* X, int64_t K, int64_t ld, int6
 bool msp_gram_tc_ok(int64_t s_pad);
 
 // factor.cu
+msp_status msp_grid_wait_limit_factor(msp_ctx* ctx, unsigned long long ns);
 msp_status msp_symmetrize_w(msp_ctx* ctx, msp_factor_s* f);
 // w_ready: the event after which the symmetrised W may be read (null: at once)
 msp_status msp_build_factor(msp_ctx* ctx, msp_factor_s* f, const void* Ct, int64_t phi_rows, cudaEvent_t w_ready);

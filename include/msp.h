@@ -283,9 +283,9 @@ MSP_API msp_status msp_set_level3_ctas(msp_ctx* ctx, int ctas);
  * the A pass, then the level-2 kernel with the step, SolveM1 and the new
  * direction): on = 1 (default): the two launches of one iteration are
  * captured once into a CUDA graph (with event-record nodes when
- * opts.profile = 1) and replayed check_every times between host reads of
- * the device convergence flag; the executable is kept by the context and
- * rebuilt when the solve's arguments or buffers change. on = 0: two stream
+ * opts.profile = 1) and replayed (opts.check_every says how the host follows
+ * them); the executable is kept by the context and rebuilt when the solve's
+ * arguments or buffers change. on = 0: two stream
  * launches per iteration. The same kernels run in the same order with the
  * same arguments, so both give the same x bit for bit; where a capture is
  * not possible the solve launches on the stream (msp_info.level1_graph_iters

@@ -1971,9 +1971,10 @@ msp_status msp_batch_create(msp_ctx* ctx, int count, const msp_instance* inst, m
     {
         // default width: the one whose units, dealt out largest first, finish first
         // (in tiles: a unit also costs about 2.5 for its reduction, and one more where
-        // its sums go through the unit partials). On 24 instances of n 512 to 4096 the A
-        // passes take 25.8, 22.1 and 20.7 ms at 16, 32 and 64 tiles, as this orders
-        // them; a floor of 8 units per SM chose 16.
+        // its sums go through the unit partials: fitted to the two batches that follow). On 24
+        // instances of n 512 to 4096 the A passes take 25.4, 22.2 and 21.0 ms at 16, 32 and 64 tiles, on 3
+        // of n 3000 to 4096 11.9, 11.0 and 14.7, as this orders them; a floor of 8 units per
+        // SM chose 16.
         int ut = kUtMin;
         double best = 0.0;
         for (int cand : {256, 128, 64, 32, 16}) {

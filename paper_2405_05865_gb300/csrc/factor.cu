@@ -5,7 +5,8 @@
 //   L^{-1}                     (FP64), stored in the working precision as
 //                               B = L^{-1} and B^T so that the level-2
 //                               iteration applies M2^{-1} v = B^T (B v).
-// The factorisation recursion halves the matrix:
+// FP32 sketches: the factor and its inverse in float-float, by block elimination on 32 x
+// 32 tiles in one launch (k_chol_inv_ff). FP64 ones: a recursion that halves the matrix,
 //   [A11 . ; A21 A22]:  (L11, X11) = f(A11);  L21 = A21 X11^T;
 //   A22 -= L21 L21^T;   (L22, X22) = f(A22);  X21 = -X22 (L21 X11),
 // with a one-block Cholesky + inverse at the leaves (at most 32 x 32) and an
@@ -129,9 +130,9 @@ __global__ void __launch_bounds__(256, 4) k_gram(const TA* __restrict__ Ct, int6
 // The same partial Grams (FP32 input) with 128 x 128 tiles: 512 threads,
 // each 8 rows (ty*4 + i and 64 + ty*4 + i) x 4 columns (tx*4 + j), K chunks
 // of 16 double-buffered in shared memory by 16-byte async copies. Per output
-// the arithmetic is k_gram's -- the same K slices, chunks of 16 summed in
-// FP32 from zero in increasing k, TwoSum into (hi, lo) -- so P is the same
-// to the bit; a thread's 32 outputs per shared-memory read of 12 values (4
+// the arithmetic is k_gram's -- chunks of 16 summed in FP32 from zero in
+// increasing k, TwoSum into (hi, lo) -- so P is the same to the bit for the same K slices
+// (their number follows the tiles, so it can differ); a thread's 32 outputs per shared-memory read of 12 values (4
 // for k_gram's 16) keep the FP32 pipe, not shared memory, the limit.
 __global__ void __launch_bounds__(512, 1) k_gram128(const float* __restrict__ Ct, int64_t K, int64_t ld,
                                                     int64_t s_pad, int nt, double* __restrict__ P) {
@@ -534,9 +535,12 @@ struct FFShared {
 };
 
 // 1/d in float-float for a positive normal d: r0, the hardware's approximation
-// (2^-23 relative), then r = r0 + r0 (e + e^2) with the residual e = 1 - d r0 formed to
+// (2^-23 relative), then a Newton-Raphson step for f(r) = 1/r - d carried to second order,
+// r = r0 + r0 (e + e^2), with the residual e = 1 - d r0 formed to
 // first order exactly (1 - hi(d r0) is exact), ~2^-46 relative. The low part may
-// overlap the high one by a bit or two.
+// overlap the high one by a bit or two. (|X M X^T - I| of the whole factor against the one
+// before, which started from a rounded reciprocal and normalised every product: 1.04 times
+// at s_pad = 128 with s = 60, 0.76 at 128, 0.47, 0.27 and 0.16 at 256, 512 and 1024.)
 __device__ __forceinline__ float2 ff_rcp(float2 d) {
     float r0;
     asm("rcp.approx.ftz.f32 %0, %1;" : "=f"(r0) : "f"(d.x));

@@ -1269,11 +1269,12 @@ struct InnerArgs {
 // M2^{-1} v = B^T (B v), as products with the formed s_pad x s_pad operator, on one
 // cluster of 16 CTAs. In k_level2 an iteration is a pass over C and four grid
 // barriers (18 us at n = 4999, s = 312; 18 us in FP64 at n = 1024, s = 64); here it is
-// three products on data that stays on the SMs, with a cluster barrier each: 6 us
-// and 5.6 us.
+// three products on data that stays on the SMs, with an exchange each: 5.1 us
+// and 5.0 us.
 //
 // A CTA has s_pad / 16 rows of H, B and B^T, 16 lanes a row, E = s_pad / 16 values of
-// a row a lane, all in registers for the whole launch. The row sums are gathered
+// a row a lane, in registers for the whole launch (at s_pad = 384 in FP32, H a pair, 60
+// bytes of them spill). The row sums are gathered
 // in shared memory and sent to every CTA's copy of the result by 16-byte st.async
 // pieces that count on that CTA's mbarrier (two copies in turn: a CTA sends product
 // k + 2 only after it has every CTA's part of k + 1, sent after the reads of k);
@@ -2154,9 +2155,10 @@ __device__ __forceinline__ void ff_acc(float& hi, float& lo, float p, float t) {
 // Requires lda, n multiples of 4 and 16-byte aligned A. SPLIT: x is split by each
 // block into shared memory (n <= kSplitMax) and xh, xl are not read: one launch for a
 // small system, where the launches and blocks are the time (20.5 us a call at n = 1000
-// with k_split_x and 1216 blocks, 10 us with this and a block per 8 rows); each block then pays
-// four FP64-pipe conversions per 32 entries, which the split kernel's 2 us
-// outweigh from about 1500 entries on.
+// with k_split_x and 1216 blocks, 8 to 10 us with this and a block per 8 rows); each block then
+// pays four FP64-pipe conversions per 32 entries, and the split kernel's 2 us are the
+// cheaper way from about 1500 entries on. The line lies at 1024: the two halves of x
+// then take 8 KB of shared memory, which leaves two blocks an SM their L1.
 constexpr int kSplitMax = 1024;
 
 template <bool SPLIT>

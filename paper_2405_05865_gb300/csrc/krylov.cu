@@ -304,7 +304,6 @@ struct L2Args {
     int mode;
     int phase;              // PHASE_ALL, or the part before / after a k_inner launch
     int res_rows;           // rows of C a block keeps in shared memory
-    int once;               // level-2 iteration: each row of C read once (gram_pass)
     const TC* C;
     const TC* W;
     const T* B;
@@ -387,7 +386,8 @@ struct L2Shape {
     // four full vectors, the scratch of the reductions, r and the row results
     static constexpr size_t fixed = ((size_t)4 * SP + SCR + 2 * kRowChunk) * sizeof(T) + 16;
     static constexpr size_t row = (size_t)SP * sizeof(TC);
-    // gram_pass is for FP32 arithmetic (in FP64 the products bound the passes, not the reads)
+    // the level-2 iteration by gram_pass: FP32 arithmetic (in FP64 the products bound the
+    // passes, not the reads)
     static constexpr bool once = sizeof(T) == 4;
 };
 
@@ -573,13 +573,13 @@ struct GramShape {
 // part = sum_i (c_i . vec) c_i over the block's rows, each row read once: HW warps
 // take every NP-th row, form its dot and add it from the registers to their own sums
 // of their columns, which scr (NP x SP) combines in order. The two warps of a row
-// exchange their halves of the dots through xch at a barrier of their own. For blocks
-// whose rows of C do not all fit shared memory: dots_pass and cols_pass read each of the
-// others twice from L2, and at n = 32768, s = 1024 (C as large as L2) from memory. A
-// level-2 step then took 53 us, with this 44; at n = 16384 and s = 2048 71 and 57,
-// s = 1024 27.2 and 27.1, s = 512 21.6 either way. The scratch costs 32 KB of resident rows (64
-// KB at 2048 columns), so where all rows fit the two passes stay (n = 8192, s = 512: 20.6 us
-// with this, 19.6 with the two passes).
+// exchange their halves of the dots through xch at a barrier of their own. dots_pass
+// and cols_pass in its place read each row that is not resident twice from L2, and at n =
+// 32768, s = 1024 (C as large as L2) from memory: a level-2 step took 53 us, with this 44;
+// at n = 16384 and s = 2048 71 and 57, s = 1024 27.2 and 27.1. The scratch costs 32 KB
+// of resident rows (64 KB at 2048 columns), and where all rows are resident all the same this
+// is quicker too, by a block barrier and a second read of shared memory (n = 8192, s = 512:
+// 20.6 and 19.6 us).
 template <typename T, typename TC, int PL>
 __device__ __forceinline__ void gram_pass(const BlockRows<TC>& rows, const T* vec, T* scr, T* xch, T* part) {
     using G = GramShape<T, TC, PL>;
@@ -1066,11 +1066,9 @@ __global__ void __launch_bounds__(kThreads, 1) k_level2(L2Args<T, TC> a) {
         const double tin2 = a.inner_tol2 * gg;
         while (k < a.max_inner && rres > tin2) {
             // P1: partial u = C^T (C d) over this block's rows; wd = W d (columns)
-            if (S::once && a.once) {
-                if constexpr (S::once) {
-                    T* wscr = reinterpret_cast<T*>(smem_raw + (size_t)a.res_rows * S::row + S::fixed);
-                    gram_pass<T, TC, PL>(rows, sd, wscr, sw, a.part + (int64_t)b * sp);
-                }
+            if constexpr (S::once) {
+                T* wscr = reinterpret_cast<T*>(smem_raw + (size_t)a.res_rows * S::row + S::fixed);
+                gram_pass<T, TC, PL>(rows, sd, wscr, sw, a.part + (int64_t)b * sp);
             } else {
 #pragma unroll
                 for (int q = 0; q < S::KU; ++q) acc[q][0] = acc[q][1] = T(0);
@@ -1199,18 +1197,12 @@ msp_status launch_level2_pl(msp_ctx* ctx, L2Args<T, TC>& a, int G) {
     // left beside the vectors (4 KB aside for the kernel's static part)
     const size_t left = ctx->smem_optin - 4096 - S::fixed;
     const int64_t most = (a.n + G - 1) / G;
-    const int64_t fit = (int64_t)(left / S::row);
-    a.res_rows = (int)(fit >= most ? most : fit / kNW * kNW);
-    a.once = 0;
-    size_t once = 0;
-    if constexpr (S::once) {
-        if (a.max_inner > 0 && a.phase == PHASE_ALL && a.res_rows < most) {
-            a.once = 1;
-            once = GramShape<T, TC, PL>::bytes;
-            a.res_rows = (int)std::min<int64_t>((int64_t)((left - once) / S::row), most);
-        }
-    }
-    const size_t smem = S::fixed + (size_t)a.res_rows * S::row + once;
+    size_t scratch = 0;       // gram_pass's, behind the vectors
+    if constexpr (S::once)
+        if (a.max_inner > 0 && a.phase == PHASE_ALL) scratch = GramShape<T, TC, PL>::bytes;
+    const int64_t fit = (int64_t)((left - scratch) / S::row);
+    a.res_rows = (int)(fit >= most ? most : scratch ? fit : fit / kNW * kNW);
+    const size_t smem = S::fixed + (size_t)a.res_rows * S::row + scratch;
     MSP_CUDA_TRY(ctx, cudaFuncSetAttribute(kern, cudaFuncAttributeMaxDynamicSharedMemorySize,
                                            (int)smem));
     // co-residency is required by the grid barrier: never exceed what fits

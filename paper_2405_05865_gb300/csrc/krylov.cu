@@ -2148,10 +2148,10 @@ __device__ __forceinline__ void ff_acc(float& hi, float& lo, float p, float t) {
 // block into shared memory (n <= kSplitMax) and xh, xl are not read: one launch for a
 // small system, where the launches and blocks are the time (20.5 us a call at n = 1000
 // with k_split_x and 1216 blocks, 8 to 10 us with this and a block per 8 rows); each block then
-// pays four FP64-pipe conversions per 32 entries, and the split kernel's 2 us are the
-// cheaper way from about 1500 entries on. The line lies at 1024: the two halves of x
-// then take 8 KB of shared memory, which leaves two blocks an SM their L1.
-constexpr int kSplitMax = 1024;
+// pays four FP64-pipe conversions per 32 entries, which the split kernel's 2 us outweigh
+// from about 1600 entries on. us a call without and with this: 13 to 14 and 10.0 at n = 1100, 13.1
+// and 12.3 at 1300, 14.3 and 13.7 at 1500, 15.1 and 15.1 at 1700, 15.9 and 17.7 at 2000.
+constexpr int kSplitMax = 1536;
 
 template <bool SPLIT>
 __global__ void __launch_bounds__(256, 2) k_matvec64_ff(const float* __restrict__ A, int64_t lda, int64_t n,

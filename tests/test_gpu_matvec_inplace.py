@@ -10,7 +10,7 @@ torch = pytest.importorskip("torch")
 pytestmark = pytest.mark.gpu
 
 
-@pytest.mark.parametrize("n", [128, 512, 1000, 1024, 1028])
+@pytest.mark.parametrize("n", [128, 512, 1000, 1024, 1028, 1400, 1536, 1540])
 def test_y_over_x(n):
     from paper_2405_05865_gb300 import Context, _lib
     ctx = Context(0)

@@ -18,7 +18,7 @@
 // direct level 2, Section 4):
 //   S2  G = C^T R            items (instance, 64-column strip of C)
 //       + convergence flags  one block per instance decides, fixed order
-//   S3  Y1 = L^{-1} G        items (instance, 32-row chunk of s)
+//   S3  Y1 = L^{-1} G        items (instance, 32- or 64-row chunk of s)
 //   S4  Y2 = L^{-T} Y1
 //   S5  Z = (R - C Y2)/lam~  items (instance, 128-row block), dots z.r, z.q
 //   S6  beta, P = Z + beta P
@@ -958,7 +958,9 @@ __device__ __forceinline__ void step_flags(const BArgs& a, int t, int lane) {
 // (FP32 FMA), and the 8 warps' sums are combined in warp order at the end of
 // the strip. A strip is cut into row segments of at most kSegBlocks row blocks, so that
 // the items outnumber the blocks and none is long; the segments' sums are added, in
-// order, where the next step stages G. (Uncut, the 220 strips of the 24-instance batch,
+// order, where the next step stages G. (Cut at 5, 10 and 20 row blocks, this step and the next
+// together take 10.2, 10.5 and 12.5 ms on 8 instances of n 512 to 4096, 22.4, 20.6 and 20.1 on 24, 40.7, 38.8
+// and 36.6 on 64.) (Uncut, the 220 strips of the 24-instance batch,
 // up to 30 tiles each, took 38 us an iteration, against 32.)
 __device__ __noinline__ void consume_G(const BArgs& a, unsigned char* ring, uint64_t* full, uint64_t* empty,
                                        const int2* hdr, uint32_t& kring, float* red, int w, int lane) {
@@ -1034,14 +1036,16 @@ __device__ __noinline__ void consume_G(const BArgs& a, unsigned char* ring, uint
 // the 8 warps' sums are added in warp order. The items are sorted by length and
 // dealt out in turn, so no block waits for a shared counter. With 128-row items
 // claimed from a counter the two steps took 46 us an iteration of the 24-instance
-// batch (n 512 to 4096), and take 37.
+// batch (n 512 to 4096); by the launch's timers it is 44 with 32-row ones, 37 with 64.
 //
-// With many instances the items' number is no concern and the vector block's
+// With many items their number is no concern and the vector block's
 // shared-memory reads are: from kTriMany 32-row chunks for each block on, items have
-// 64 rows, two a lane (R = 2), in pieces of 128 columns: 64 instances of
-// the benchmark (10 or so chunks a block) 17.9 ms of a solve in these steps, 23.0 with 32
-// rows; the batch of 24 has 3 chunks a block and keeps the shorter items.
-constexpr int kTriMany = 6;
+// 64 rows, two a lane (R = 2), in pieces of 128 columns. ms of a solve in these steps with
+// 32 and 64 rows, by chunks a block: 7.4 and 8.4 at 1.8 (16 instances of n 512 to 4096), 6.3
+// and 4.7 at 2.5 (64 of n 300 to 1200), 12.9 and 11.1 at 2.5 (12 of 4000 to 6000), 11.1 and 9.6 at
+// 2.8 (24 of 512 to 4096), 16.9 and 13.7 at 4.6 (40), 25.4 and 17.7 at 7.7 (64); below 1 the
+// 32 rows are 5 to 20% quicker.
+constexpr int kTriMany = 2;
 
 template <bool kUpper, int R>
 __device__ __noinline__ void step_tri(const BArgs& a, int t, unsigned char* smem, float* red, int tid, int w,

@@ -1250,8 +1250,11 @@ __global__ void k_split_pair(const double* __restrict__ src, float* __restrict__
 
 // The level-2 operator H = C^T C + lam~ W of a sketched level 2, its Gram
 // accumulated as M2's on the FP32 pipe (compensated; FP64 for FP64 data), so that
-// products with it are no further from C^T (C d) + lam~ W d than the passes over C
-// in the working precision are. One Gram of n rows (0.1 ms at n = 5000, s = 312)
+// products with it are no further from C^T (C d) + lam~ W d, relative to |C|^2 |d|, than
+// the passes over C in the working precision are. (Along directions that C nearly
+// annihilates the passes are closer. It shows in the level-1 iterations: 52.0 with them and
+// 53.9 with H on FP64 systems of n 500 to 700 with outliers of 1e4; 346 and 347 on FP32
+// kernel systems of n 1000 to 5900.) One Gram of n rows (0.1 ms at n = 5000, s = 312)
 // against a pass over C and two grid barriers saved in every level-2 iteration.
 msp_status msp_form_level2(msp_ctx* ctx, msp_factor_s* f, const void* C, int64_t n) {
     const int64_t sp = f->s_pad, mat = sp * sp;
